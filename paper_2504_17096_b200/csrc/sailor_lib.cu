@@ -19,6 +19,7 @@
 #include "sailor_mixed.cuh"
 #include "sailor_mixed_search.cuh"
 #include "sailor_peaks.cuh"
+#include "sailor_plan_setup.cuh"
 
 using namespace sailor;
 
@@ -473,29 +474,18 @@ uint32_t chunk_of(const sailor_ctx* ctx, uint64_t f) {
     return sc.chunk_start[lo] + (uint32_t)(item / PLAN_THREADS);
 }
 
-using PlanKernel = void (*)(const PlanParams);
-
 constexpr int PLAN_VARIANTS = 15;      // objective x constraint x fused, then the three screened kernels
 
 uint32_t variant_of(uint32_t obj, bool constr, bool fused, bool screen = false) {
     return screen ? 12 + obj : (obj * 2 + (constr ? 1 : 0)) * 2 + (fused ? 1 : 0);
 }
 
-template <bool FUSED>
-PlanKernel pick_kernel_of(uint32_t obj, bool constr) {
-    switch (obj) {
-        case SAILOR_OBJ_MAX_THROUGHPUT: return constr ? plan_kernel<0, true, FUSED> : plan_kernel<0, false, FUSED>;
-        case SAILOR_OBJ_MIN_COST: return constr ? plan_kernel<1, true, FUSED> : plan_kernel<1, false, FUSED>;
-        default: return constr ? plan_kernel<2, true, FUSED> : plan_kernel<2, false, FUSED>;
-    }
-}
-
 PlanKernel pick_kernel(uint32_t obj, bool constr, bool fused, bool screen = false) {
-    if (screen)        // unconstrained searches only; they end their pass in finish_kernel
-        return obj == SAILOR_OBJ_MAX_THROUGHPUT ? plan_kernel<0, false, false, true>
-               : obj == SAILOR_OBJ_MIN_COST     ? plan_kernel<1, false, false, true>
-                                                : plan_kernel<2, false, false, true>;
-    return fused ? pick_kernel_of<true>(obj, constr) : pick_kernel_of<false>(obj, constr);
+    switch (obj) {
+        case SAILOR_OBJ_MAX_THROUGHPUT: return plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT>(constr, fused, screen);
+        case SAILOR_OBJ_MIN_COST: return plan_kernel_of<SAILOR_OBJ_MIN_COST>(constr, fused, screen);
+        default: return plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT_PER_USD>(constr, fused, screen);
+    }
 }
 
 // Searches of up to this many chunks per resident block end their pass inside the search kernel; longer ones
