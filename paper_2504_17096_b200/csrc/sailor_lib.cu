@@ -6,6 +6,7 @@
 #include <cstddef>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -156,6 +157,14 @@ simulate_mixed_kernel(const unsigned char* __restrict__ blob, const uint16_t* __
 
 // ---- host state -----------------------------------------------------------------------------
 
+struct MixedTables {
+    sailor_mixed_space key;                    // the space the tables are of
+    MixedSpaceDesc desc;
+    std::vector<uint64_t> combs;
+    std::vector<uint64_t> flat_base;           // [n_config + 1]
+    uint32_t n_config = 0;
+};
+
 struct SpaceCache {
     bool valid = false;
     sailor_space key;
@@ -219,9 +228,13 @@ struct sailor_ctx {
     // explicit-batch staging (grow-only)
     unsigned char* d_stage = nullptr;
     size_t stage_bytes = 0;
-    // working memory of the search over plans with mixed replicas (grow-only)
+    // the search over plans with mixed replicas: tables of the space last searched, working memory (grow-only)
+    MixedTables* mix = nullptr;
     unsigned char* d_mix = nullptr;
     size_t mix_bytes = 0;
+    bool mix_dirty = true;                 // the counters must be cleared from the host (fresh memory, or a failed search)
+    MixedOut* h_mix_out = nullptr;         // mapped pinned memory
+    MixedOut* d_mix_out = nullptr;
     // tables of the dynamic-programming search (grow-only)
     unsigned char* d_dp = nullptr;
     size_t dp_bytes = 0;
@@ -926,9 +939,8 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
     CUF(cudaFuncSetAttribute(simulate_mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 64) * 1024));
     CUF(cudaFuncSetAttribute(simulate_mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 64) * 1024));
     CUF(cudaFuncSetAttribute(finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 8) * 1024));
-    CUF(cudaFuncSetAttribute(plan_mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 24) * 1024));
-    CUF(cudaFuncSetAttribute(plan_mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 24) * 1024));
-    CUF(cudaFuncSetAttribute(mixed_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 24) * 1024));
+    CUF(cudaFuncSetAttribute(mixed_finish_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 80) * 1024));
+    CUF(cudaFuncSetAttribute(mixed_finish_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 40) * 1024));
 #undef CUF
     *out = ctx;
     return SAILOR_OK;
@@ -955,7 +967,9 @@ int sailor_destroy(sailor_ctx* ctx) {
     cudaFree(ctx->space.d_groups);
     cudaFree(ctx->space.d_cfg_cache);
     cudaFree(ctx->d_stage);
+    delete ctx->mix;
     cudaFree(ctx->d_mix);
+    cudaFreeHost(ctx->h_mix_out);
     cudaFree(ctx->d_dp);
     for (cudaEvent_t e : {ctx->ev0, ctx->ev1, ctx->ev2, ctx->evh0, ctx->evh1, ctx->ev_chunk, ctx->ev_join, ctx->ev_slot[0],
                           ctx->ev_slot[1], ctx->ev_slot[2]})
@@ -1959,13 +1973,6 @@ void list_combinations(uint32_t T, uint32_t units, std::vector<uint64_t>& out) {
     Rec::go(T, 0, units, 0, 0, out);
 }
 
-struct MixedTables {
-    MixedSpaceDesc desc;
-    std::vector<uint64_t> combs;
-    std::vector<uint64_t> flat_base;           // [n_config + 1]
-    uint32_t n_config = 0;
-};
-
 int build_mixed_tables(const sailor_ctx* ctx, const sailor_mixed_space* s, MixedTables& mt) {
     if (!ctx || !s) return SAILOR_E_ARG;
     if (s->n_p == 0 || s->n_mbs == 0 || s->n_rc == 0 || s->n_d == 0 || s->granularity == 0) return SAILOR_E_ARG;
@@ -2025,6 +2032,52 @@ int build_mixed_tables(const sailor_ctx* ctx, const sailor_mixed_space* s, Mixed
     return SAILOR_OK;
 }
 
+bool same_mixed_space(const sailor_mixed_space& a, const sailor_mixed_space& b, uint32_t n_types) {
+    if (a.n_p != b.n_p || a.n_mbs != b.n_mbs || a.n_rc != b.n_rc || a.n_d != b.n_d || a.seg_max != b.seg_max ||
+        a.granularity != b.granularity)
+        return false;
+    return !memcmp(a.p_values, b.p_values, a.n_p) && !memcmp(a.mbs_idx, b.mbs_idx, a.n_mbs) &&
+           !memcmp(a.rc_values, b.rc_values, a.n_rc) && !memcmp(a.tp_idx_of_type, b.tp_idx_of_type, n_types) &&
+           !memcmp(a.d_values, b.d_values, a.n_d * sizeof(uint16_t));
+}
+
+// The device pointers of a mixed search inside the context's working memory; returns the bytes it takes.
+size_t mixed_carve(const sailor_ctx* ctx, const MixedTables& mt, MixedSearchParams& mp) {
+    Bump bump{ctx->d_mix};
+    mp.counters = bump.take<unsigned long long>(MIXC_N);
+    mp.combs = bump.take<uint64_t>(mt.combs.size());
+    mp.cfg_flat_base = bump.take<uint64_t>(mt.flat_base.size());
+    mp.partial = bump.take<Hit>((size_t)SAILOR_K_MAX * ctx->sm_count * 4);
+    mp.queue = bump.take<uint32_t>(std::min<uint64_t>(mt.flat_base[mt.n_config], MIXED_RANGE));
+    return bump.at;
+}
+
+// Working memory for a mixed space and its tables on the device.
+int mixed_workspace(sailor_ctx* ctx, const MixedTables& mt) {
+    if (!ctx->h_mix_out) {
+        CU(ctx, cudaHostAlloc(&ctx->h_mix_out, sizeof(MixedOut), cudaHostAllocMapped));
+        CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->d_mix_out), ctx->h_mix_out, 0));
+    }
+    MixedSearchParams mp;
+    const size_t need = mixed_carve(ctx, mt, mp);
+    if (need > ctx->mix_bytes) {
+        CU(ctx, stream_sync(ctx));
+        cudaFree(ctx->d_mix);
+        ctx->d_mix = nullptr;
+        ctx->mix_bytes = 0;
+        cudaError_t e = cudaMalloc(&ctx->d_mix, need);
+        if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SAILOR_E_NOMEM; }
+        ctx->mix_bytes = need;
+        ctx->mix_dirty = true;
+        mixed_carve(ctx, mt, mp);
+    }
+    CU(ctx, cudaMemcpyAsync(const_cast<uint64_t*>(mp.combs), mt.combs.data(), mt.combs.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
+    CU(ctx, cudaMemcpyAsync(const_cast<uint64_t*>(mp.cfg_flat_base), mt.flat_base.data(), mt.flat_base.size() * 8,
+                            cudaMemcpyHostToDevice, ctx->stream));
+    CU(ctx, stream_sync(ctx));         // the tables are pageable host memory
+    return SAILOR_OK;
+}
+
 }  // namespace
 
 static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const sailor_objective* o, uint32_t k,
@@ -2034,64 +2087,63 @@ static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const s
     if (o->flags != 0 || o->budget_factor_over_cheapest > 0.0 || std::isnan(o->budget_usd_per_iter) ||
         std::isnan(o->min_iters_per_s) || std::isnan(o->budget_factor_over_cheapest))
         return SAILOR_E_ARG;
-    MixedTables mt;
-    int rc = build_mixed_tables(ctx, s, mt);
-    if (rc) return rc;
-    const uint64_t n_total = mt.flat_base[mt.n_config];
     DeviceGuard guard(ctx->device);
-    const uint32_t R = ctx->hdr.R;
-    const size_t smem = ctx->hdr.static_bytes + sizeof(unsigned long long) * MIXS_WARPS * R + sizeof(sailor_mixed_plan) * MIXS_WARPS;
-    const uint64_t want_blocks = (n_total + MIXS_WARPS - 1) / MIXS_WARPS;
-    const uint32_t grid = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(want_blocks, 1), (uint64_t)ctx->sm_count * 4);
-    const size_t total = padded(mt.combs.size() * 8) + padded(mt.flat_base.size() * 8) + padded(sizeof(Hit) * SAILOR_K_MAX * grid) +
-                         padded(sizeof(sailor_mixed_result) * SAILOR_K_MAX) + padded(9 * 8) + 1024;
-    if (total > ctx->mix_bytes) {
-        CU(ctx, stream_sync(ctx));
-        cudaFree(ctx->d_mix);
-        ctx->d_mix = nullptr;
-        ctx->mix_bytes = 0;
-        cudaError_t e = cudaMalloc(&ctx->d_mix, total);
-        if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SAILOR_E_NOMEM; }
-        ctx->mix_bytes = total;
-    }
-    Bump bump{ctx->d_mix};
-    uint64_t* d_combs = bump.take<uint64_t>(mt.combs.size());
-    uint64_t* d_base = bump.take<uint64_t>(mt.flat_base.size());
-    Hit* d_partial = bump.take<Hit>((size_t)SAILOR_K_MAX * grid);
-    sailor_mixed_result* d_results = bump.take<sailor_mixed_result>(SAILOR_K_MAX);
-    unsigned long long* d_counters = bump.take<unsigned long long>(9);
-
-    {
-        const int rc_up = upload_availability(ctx);
+    const bool known = ctx->mix && same_mixed_space(ctx->mix->key, *s, ctx->hdr.T);
+    if (!known) {                      // a space not searched last: its tables, laid out once
+        std::unique_ptr<MixedTables> fresh(new MixedTables());
+        const int rc = build_mixed_tables(ctx, s, *fresh);
+        if (rc) return rc;
+        fresh->key = *s;
+        delete ctx->mix;               // nothing of it is in flight: every search ends synchronised
+        ctx->mix = nullptr;
+        const int rc_up = mixed_workspace(ctx, *fresh);
         if (rc_up) return rc_up;
+        ctx->mix = fresh.release();
     }
-    CU(ctx, cudaMemcpyAsync(d_combs, mt.combs.data(), mt.combs.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-    CU(ctx, cudaMemcpyAsync(d_base, mt.flat_base.data(), mt.flat_base.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-    CU(ctx, cudaMemsetAsync(d_counters, 0, 9 * 8, ctx->stream));
-    CU(ctx, cudaMemsetAsync(d_counters + 6, 0x7f, 8, ctx->stream));           // the cheapest cost starts above every cost
-    CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
+    const MixedTables& mt = *ctx->mix;
+    const uint64_t n_total = mt.flat_base[mt.n_config];
+    const uint32_t R = ctx->hdr.R, grid = (uint32_t)ctx->sm_count * 4;
     MixedSearchParams mp;
     memset(&mp, 0, sizeof(mp));
-    mp.blob = ctx->d_blob; mp.avail = ctx->d_avail; mp.cfg_flat_base = d_base; mp.combs = d_combs; mp.partial = d_partial;
-    mp.counters = d_counters; mp.results = d_results; mp.sp = mt.desc; mp.n_config = mt.n_config; mp.k = k; mp.obj = o->kind;
+    mixed_carve(ctx, mt, mp);
+    if (ctx->mix_dirty) {              // afterwards every search leaves the counters at their starting values
+        CU(ctx, cudaMemsetAsync(mp.counters, 0, MIXC_N * 8, ctx->stream));
+        CU(ctx, cudaMemsetAsync(mp.counters + MIXC_MIN_COST, 0x7f, 8, ctx->stream));
+    }
+    ctx->mix_dirty = true;             // until this call has gone through
+    if (stats) CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
+    mp.blob = ctx->d_blob; mp.out = ctx->d_mix_out; mp.sp = mt.desc; mp.n_config = mt.n_config; mp.k = k; mp.obj = o->kind;
+    memcpy(mp.avail, ctx->h_avail, sizeof(mp.avail));
     mp.n_partial = grid; mp.n_total = n_total; mp.budget = o->budget_usd_per_iter; mp.min_rate = o->min_iters_per_s;
     bool deep = false;                                           // pipelines of more than 32 stages in the space
     for (uint32_t i = 0; i < s->n_p; ++i) deep = deep || s->p_values[i] > 32;
-    if (deep) plan_mixed_kernel<true><<<grid, MIXS_THREADS, smem, ctx->stream>>>(mp);
-    else plan_mixed_kernel<false><<<grid, MIXS_THREADS, smem, ctx->stream>>>(mp);
+    uint32_t launches = 0;
+    for (uint64_t lo = 0; lo < n_total; lo += MIXED_RANGE) {
+        mp.range_lo = lo;
+        mp.range_hi = std::min(n_total, lo + MIXED_RANGE);
+        mp.carry_lists = lo ? 1u : 0u;
+        if (lo) CU(ctx, cudaMemsetAsync(mp.counters + MIXC_QUEUED, 0, 8, ctx->stream));
+        // a block takes at least a few rounds of candidates, since it sets its configuration up first
+        const uint64_t stretches = (mp.range_hi - lo + 2 * MIXS_THREADS - 1) / (2 * MIXS_THREADS);
+        const uint32_t class_grid = (uint32_t)std::min<uint64_t>(stretches, (uint64_t)ctx->sm_count * 8);
+        mixed_class_kernel<<<class_grid, MIXS_THREADS, 0, ctx->stream>>>(mp);
+        CU(ctx, cudaGetLastError());
+        plan_mixed_kernel<<<grid, MIXS_THREADS, 0, ctx->stream>>>(mp);
+        CU(ctx, cudaGetLastError());
+        launches += 2;
+    }
+    if (deep) mixed_finish_kernel<true><<<1, 32 * MIXF_WARPS<true>, mixed_smem(ctx->hdr.static_bytes, R, MIXF_WARPS<true>), ctx->stream>>>(mp);
+    else mixed_finish_kernel<false><<<1, 32 * MIXF_WARPS<false>, mixed_smem(ctx->hdr.static_bytes, R, MIXF_WARPS<false>), ctx->stream>>>(mp);
     CU(ctx, cudaGetLastError());
-    mixed_finish_kernel<<<1, MIXS_THREADS, smem, ctx->stream>>>(mp);
-    CU(ctx, cudaGetLastError());
-    CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
-    unsigned long long counters[9];
-    std::vector<sailor_mixed_result> host_out(k);
-    CU(ctx, cudaMemcpyAsync(counters, d_counters, sizeof(counters), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(ctx, cudaMemcpyAsync(host_out.data(), d_results, sizeof(sailor_mixed_result) * k, cudaMemcpyDeviceToHost, ctx->stream));
-    CU(ctx, stream_sync(ctx));                                 // also: the host tables are pageable
-    if (counters[7]) return SAILOR_E_DEVICE;
-    if (counters[8] > k) return SAILOR_E_DEVICE;
-    *n_found = (uint32_t)counters[8];
-    memcpy(topk, host_out.data(), sizeof(sailor_mixed_result) * counters[8]);
+    ++launches;
+    if (stats) CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
+    CU(ctx, stream_sync(ctx));
+    const unsigned long long* counters = ctx->h_mix_out->counters;
+    if (counters[MIXC_ERROR]) return SAILOR_E_DEVICE;
+    if (counters[MIXC_FOUND] > k) return SAILOR_E_DEVICE;
+    ctx->mix_dirty = false;
+    *n_found = (uint32_t)counters[MIXC_FOUND];
+    memcpy(topk, ctx->h_mix_out->results, sizeof(sailor_mixed_result) * counters[MIXC_FOUND]);
     if (stats) {
         memset(stats, 0, sizeof(*stats));
         stats->n_total = counters[0];
@@ -2102,10 +2154,10 @@ static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const s
         stats->n_feasible = counters[5];
         stats->budget_used = o->budget_usd_per_iter;
         double mc;
-        memcpy(&mc, &counters[6], sizeof(mc));
+        memcpy(&mc, &counters[MIXC_MIN_COST], sizeof(mc));
         stats->min_feasible_cost = counters[5] ? mc : 0.0;
         CU(ctx, cudaEventElapsedTime(&stats->kernel_ms, ctx->ev0, ctx->ev1));
-        stats->n_launches = 2;
+        stats->n_launches = launches;
         stats->n_configs = stats->n_configs_evaluated = mt.n_config;
     }
     return SAILOR_OK;

@@ -38,6 +38,15 @@ __device__ __forceinline__ double warp_max_f64(double x) {
     return __longlong_as_double((long long)m);
 }
 
+// Smallest of the warp's positive binary64 values (they order like their bit patterns).
+__device__ __forceinline__ double warp_min_positive(double x) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+    const uint32_t mh = __reduce_min_sync(MIX_FULL, hi);
+    const uint32_t ml = __reduce_min_sync(MIX_FULL, hi == mh ? lo : 0xffffffffu);
+    return __longlong_as_double((long long)((uint64_t)mh << 32 | ml));
+}
+
 // `cnt` points to this warp's per-digit GPU counters (R of them, shared memory).  Every lane of the warp
 // calls with the same record and gets the same result.
 __device__ inline SimOut simulate_mixed_warp(const TabView& v, const uint16_t* __restrict__ avail,

@@ -974,6 +974,77 @@ __device__ __forceinline__ void run_items(const PlanParams& pp, const CfgShared&
     }
 }
 
+// The k best of `n_lists` sorted lists of SAILOR_K_MAX slots (all k slots written, empty ones as (+inf, ~0)), merged by a
+// whole block of NW warps into s_hits[0]; returns how many there are (at most k).  `sel` (SAILOR_K_MAX words) and `s_n`
+// are scratch in shared memory.  Ends synchronised.
+template <uint32_t NW>
+__device__ __forceinline__ uint32_t merge_block_lists(const Hit* partial, uint32_t n_lists, uint32_t k, Hit (*s_hits)[SAILOR_K_MAX],
+                                                      uint32_t* sel, uint32_t* s_n) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // The k best of all lists lie in the k lists with the best first elements: k elements (those heads) are at
+    // least as good as the k-th best head, and a list whose head is worse holds nothing better than its head.
+    // So: the k best heads first (one element per list, all loads in flight together), then only those lists.
+    // (Other SMs wrote the lists: read them in L2.)
+    auto load_hit = [&](uint32_t b, uint32_t slot, double& sc, uint64_t& fl) {
+        const double2 raw = __ldcg(reinterpret_cast<const double2*>(&partial[(size_t)b * SAILOR_K_MAX + slot]));
+        sc = raw.x;
+        fl = (uint64_t)__double_as_longlong(raw.y);
+    };
+    WarpTopK top;
+    top.init();
+    const uint32_t rounds = (n_lists + 32 * NW - 1) / (32 * NW);
+    for (uint32_t r = 0; r < rounds; ++r) {
+        const uint32_t b = r * 32 * NW + tid;
+        double hs = make_inf();
+        uint64_t hf = ~0ull;
+        if (b < n_lists) load_hit(b, 0, hs, hf);
+        top.offer(hf != ~0ull && (hs < top.thr_score || (hs == top.thr_score && hf < top.thr_flat)), hs, hf, k, lane);
+    }
+    auto tree_merge = [&]() {          // the warps' lists into warp 0's, through shared memory
+        s_hits[warp][lane].score = top.score;
+        s_hits[warp][lane].flat = top.flat;
+        __syncthreads();
+        for (uint32_t step = 1; step < NW; step <<= 1) {
+            if ((warp & (2 * step - 1)) == 0 && warp + step < NW) {
+                top.merge_sorted(s_hits[warp + step][lane].score, s_hits[warp + step][lane].flat, k, lane);
+                s_hits[warp][lane].score = top.score;
+                s_hits[warp][lane].flat = top.flat;
+            }
+            __syncthreads();
+        }
+    };
+    tree_merge();
+    const double cut_s = s_hits[0][k - 1].score;             // the k-th best head (or (+inf, ~0): fewer than k lists hold anything)
+    const uint64_t cut_f = s_hits[0][k - 1].flat;
+    if (tid == 0) *s_n = 0;
+    __syncthreads();
+    for (uint32_t r = 0; r < rounds; ++r) {
+        const uint32_t b = r * 32 * NW + tid;
+        double hs = make_inf();
+        uint64_t hf = ~0ull;
+        if (b < n_lists) load_hit(b, 0, hs, hf);
+        if (hf != ~0ull && (hs < cut_s || (hs == cut_s && hf <= cut_f))) sel[atomicAdd(s_n, 1u)] = b;
+    }
+    __syncthreads();
+    const uint32_t n_sel = *s_n;
+    top.init();
+    for (uint32_t q = warp; q < n_sel; q += NW) {
+        double ls = make_inf();
+        uint64_t lf = ~0ull;
+        if (lane < k) load_hit(sel[q], lane, ls, lf);
+        top.merge_sorted(ls, lf, k, lane);
+    }
+    __syncthreads();                                           // `sel` has been read by everyone
+    tree_merge();
+    if (warp == 0) {
+        const bool have = lane < k && top.flat != ~0ull;
+        const uint32_t n = __popc(__ballot_sync(FULL, have));
+        if (lane == 0) *s_n = n;
+    }
+    __syncthreads();
+    return *s_n;
+}
+
 // End of a pass, run by the one block that hands in its list last (no block waits for another: every block
 // adds one to Ctrl::blocks_done after its list is written, and the block that reads gridDim.x - 1 knows all the
 // lists are in memory).  Merges the blocks' lists, simulates the winners in full for the result records, copies
@@ -1003,72 +1074,10 @@ static __device__ __noinline__ void finish_pass(const PlanParams& pp, const TabV
         }
         return;
     }
-    // The k best of all lists lie in the k lists with the best first elements: k elements (those heads) are at
-    // least as good as the k-th best head, and a list whose head is worse holds nothing better than its head.
-    // So: the k best heads first (one element per list, all loads in flight together), then only those lists.
-    // (Every block writes all k slots of its list, empty ones as (+inf, ~0); read them in L2, other SMs wrote them.)
-    auto load_hit = [&](uint32_t b, uint32_t slot, double& sc, uint64_t& fl) {
-        const double2 raw = __ldcg(reinterpret_cast<const double2*>(&pp.partial[(size_t)b * SAILOR_K_MAX + slot]));
-        sc = raw.x;
-        fl = (uint64_t)__double_as_longlong(raw.y);
-    };
-    WarpTopK top;
-    top.init();
-    const uint32_t rounds = (n_partial + PLAN_THREADS - 1) / PLAN_THREADS;
-    for (uint32_t r = 0; r < rounds; ++r) {
-        const uint32_t b = r * PLAN_THREADS + tid;
-        double hs = make_inf();
-        uint64_t hf = ~0ull;
-        if (b < n_partial) load_hit(b, 0, hs, hf);
-        top.offer(hf != ~0ull && (hs < top.thr_score || (hs == top.thr_score && hf < top.thr_flat)), hs, hf, pp.k, lane);
-    }
-    auto tree_merge = [&]() {          // the warps' lists into warp 0's, through shared memory
-        s_hits[warp][lane].score = top.score;
-        s_hits[warp][lane].flat = top.flat;
-        __syncthreads();
-        for (uint32_t step = 1; step < nw; step <<= 1) {
-            if ((warp & (2 * step - 1)) == 0 && warp + step < nw) {
-                top.merge_sorted(s_hits[warp + step][lane].score, s_hits[warp + step][lane].flat, pp.k, lane);
-                s_hits[warp][lane].score = top.score;
-                s_hits[warp][lane].flat = top.flat;
-            }
-            __syncthreads();
-        }
-    };
-    tree_merge();
-    const double cut_s = s_hits[0][pp.k - 1].score;          // the k-th best head (or (+inf, ~0): fewer than k lists hold anything)
-    const uint64_t cut_f = s_hits[0][pp.k - 1].flat;
-    uint32_t* sel = s_cnt;                                    // the chosen lists (at most k), then reused as counters
-    if (tid == 0) *s_n = 0;
-    __syncthreads();
-    for (uint32_t r = 0; r < rounds; ++r) {
-        const uint32_t b = r * PLAN_THREADS + tid;
-        double hs = make_inf();
-        uint64_t hf = ~0ull;
-        if (b < n_partial) load_hit(b, 0, hs, hf);
-        if (hf != ~0ull && (hs < cut_s || (hs == cut_s && hf <= cut_f))) sel[atomicAdd(s_n, 1u)] = b;
-    }
-    __syncthreads();
-    const uint32_t n_sel = *s_n;
-    top.init();
-    for (uint32_t q = warp; q < n_sel; q += nw) {
-        double ls = make_inf();
-        uint64_t lf = ~0ull;
-        if (lane < pp.k) load_hit(sel[q], lane, ls, lf);
-        top.merge_sorted(ls, lf, pp.k, lane);
-    }
-    __syncthreads();                                           // `sel` has been read by everyone
-    tree_merge();
-    if (warp == 0) {
-        const bool have = lane < pp.k && top.flat != ~0ull;
-        const uint32_t n = __popc(__ballot_sync(FULL, have));
-        if (lane == 0) *s_n = n;
-    }
-    __syncthreads();
+    const uint32_t n = merge_block_lists<PLAN_WARPS>(pp.partial, n_partial, pp.k, s_hits, s_cnt, s_n);   // s_cnt: scratch first, counters then
     // the winners are simulated in full for the result records, all at once: winner j by lane j / PLAN_WARPS of warp
     // j % PLAN_WARPS (each is a long single-thread dependency chain of table look-ups; spread over the warps, at
     // most four different plans share a warp's instruction stream)
-    const uint32_t n = *s_n;
     {
         const uint32_t j = lane * nw + warp;
         if (lane < (SAILOR_K_MAX + nw - 1) / nw && j < n) {

@@ -103,6 +103,40 @@ def test_one_part_per_stage_is_the_plain_search():
             assert {k: int(getattr(pst, k)) for k in COUNT_KEYS} == {k: int(getattr(mst, k)) for k in COUNT_KEYS}
 
 
+@pytest.mark.parametrize("p_values,n_d", [([8], 6), ([1, 2, 3, 8], 8), ([48], 8)])
+def test_spaces_on_both_sides_of_one_range_are_the_plain_search(p_values, n_d):
+    """The classes are taken 2^23 candidates at a time: 9.6e6 and more candidates need a second range, whose lists go on
+    from the first's (48 stages: through the evaluation of deep pipelines).  Same check as above, index by index."""
+    w = W.config3()
+    w.p_values, w.tp_idx, w.d_values = p_values, [2], w.d_values[:n_d]
+    with Ctx(w) as cx:
+        sp = B.make_mixed_space(w, 1, [2] * w.n_types)
+        n = B.sailor_mixed_space_size(cx.ctx, sp)
+        assert n == B.sailor_space_size(cx.ctx, B.make_space(w)) and n > 1 << 23
+        obj = B.Objective(2, 0, 0.0, 0.0, 0.0)
+        plain, pst = B.sailor_plan(cx.ctx, B.make_space(w), obj, 32)
+        for _ in range(2):                                # the second search finds the counters as the first left them
+            mixed, mst = B.sailor_plan_mixed(cx.ctx, sp, obj, 32)
+            assert [(r.flat, r.score, r.cost, r.peak_mem) for r in plain] == [(r.flat, r.score, r.cost, r.peak_mem) for r in mixed]
+            assert {k: int(getattr(pst, k)) for k in COUNT_KEYS} == {k: int(getattr(mst, k)) for k in COUNT_KEYS}
+
+
+@pytest.mark.parametrize("n_types,n_zones,gbs", [(5, 2, 48), (8, 1, 48), (7, 1, 50)])
+def test_classes_with_more_than_four_types(n_types, n_zones, gbs):
+    """Types 4..7 are counted in the second word of 16-bit lanes; gbs = 50 makes some configurations invalid as a whole,
+    and the degrees of the types some combinations."""
+    w = W.tiny(seed=17, n_types=n_types, n_zones=n_zones, L=6, p_values=[1, 3], d_values=(2, 4), mbs_values=(1, 3), rc_values=(0,), seg_max=2, gbs=gbs)
+    tps = [(g * 2) % 3 for g in range(n_types)]
+    w.gpus_per_node[n_types - 1] = 1                      # its degree does not fit a node unless it is 1
+    o = Oracle(w)
+    osp = o.mixed_space(2, tps)
+    with Ctx(w) as cx:
+        for kind, k in ((0, 32), (1, 5)):
+            hits, counts = o.search_mixed(osp, kind, k)
+            res, st = B.sailor_plan_mixed(cx.ctx, B.make_mixed_space(w, 2, tps), B.Objective(kind, 0, 0.0, 0.0, 0.0), k)
+            assert_same(res, st, hits, counts, o, osp, f"{n_types} types, kind {kind}")
+
+
 def test_mixed_search_on_workload_2_with_mixes_beats_or_equals_one_type_per_stage():
     """Workload 2's model and cluster, two pipeline depths: the search over halves and quarters of D contains the
     one-type-per-stage plans of the same tensor-parallel degrees, so its best is at least as good; winners are
