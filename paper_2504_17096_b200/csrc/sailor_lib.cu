@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <array>
 #include <map>
+#include <mutex>
 
 #include "sailor_batch.cuh"
 #include "sailor_dp.cuh"
@@ -173,6 +174,7 @@ struct SpaceCache {
     uint64_t n_total = 0;
     std::vector<uint32_t> chunk_start;     // host copies, for range -> chunk lookup
     std::vector<uint64_t> flat_base;
+    unsigned char* d_mem = nullptr;        // one piece of device memory that holds everything below
     uint32_t* d_chunk_start = nullptr;
     uint64_t* d_flat_base = nullptr;
     size_t smem = 0, smem_screen = 0;      // dynamic shared memory of a search block, without and with the binary32 tables
@@ -190,6 +192,14 @@ struct SpaceCache {
     uint32_t cache_head16 = 0, cache_arr16 = 0;
 };
 
+// What a context keeps in pinned host memory the device can write.
+struct HostBlock {
+    PlanOut out;                           // results of a search
+    SurveyOut survey;                      // what the survey of a space found
+    uint16_t avail[R_MAX];                 // the availability snapshot last set
+    MixedOut mixed;                        // results of a search over plans with mixed replicas
+};
+
 constexpr size_t CFG_CACHE_MAX_BYTES = 512ull << 20;
 
 constexpr uint64_t WAVE_CONFIG_MAX = 1u << 16;
@@ -204,14 +214,16 @@ struct sailor_ctx {
     int last_cuda = 0;
     int sm_count = 0;
     TabHdr hdr;                            // host copy of the header
+    unsigned char* d_mem = nullptr;        // one piece of device memory: the blob and the small buffers below
     unsigned char* d_blob = nullptr;
     uint16_t* d_avail = nullptr;           // device copy for the kernels that take a pointer (brought up to date lazily)
-    uint16_t* h_avail = nullptr;           // pinned; the snapshot last set
+    HostBlock* host = nullptr;             // pinned, one of the process's few such blocks
+    uint16_t* h_avail = nullptr;           // host->avail
     bool avail_dirty = false;              // d_avail is older than h_avail
     PlanOut* d_out_mapped = nullptr;       // device address of h_out (mapped pinned memory)
     Ctrl* d_ctrl = nullptr;
     unsigned int* d_sim_error = nullptr;   // error word of the explicit-batch kernels, then the "deep plans seen" word
-    PlanOut* h_out = nullptr;              // pinned
+    PlanOut* h_out = nullptr;              // &host->out
     bool ctrl_dirty = true;                // the counters must be cleared from the host (first call, or after a failed one)
     uint64_t sync_epoch = 1;               // stream synchronisations by this context so far
     uint64_t avail_epoch = 0;              // sync_epoch when the pinned availability buffer was last handed to a copy
@@ -233,8 +245,6 @@ struct sailor_ctx {
     unsigned char* d_mix = nullptr;
     size_t mix_bytes = 0;
     bool mix_dirty = true;                 // the counters must be cleared from the host (fresh memory, or a failed search)
-    MixedOut* h_mix_out = nullptr;         // mapped pinned memory
-    MixedOut* d_mix_out = nullptr;
     // tables of the dynamic-programming search (grow-only)
     unsigned char* d_dp = nullptr;
     size_t dp_bytes = 0;
@@ -257,6 +267,113 @@ cudaError_t stream_sync(sailor_ctx* ctx) {
     if (e == cudaSuccess) ++ctx->sync_epoch;
     return e;
 }
+
+struct Bump {                       // carves 256-byte aligned pieces out of one device buffer
+    unsigned char* base;
+    size_t at = 0;
+    template <typename T>
+    T* take(size_t n) {
+        T* p = reinterpret_cast<T*>(base + at);
+        at += (n * sizeof(T) + 255) & ~(size_t)255;
+        return p;
+    }
+};
+
+size_t padded(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
+
+// Device memory comes from one memory pool per device that the library owns: a context's first buffers then cost
+// microseconds where cudaMalloc and cudaFree of a megabyte cost 0.3 ms each (up to 12 ms seen).  The pool keeps at most
+// POOL_KEEP bytes that no context uses (what is beyond goes back to the device when a stream is next synchronised).
+// Allocation and release are ordered on the context's stream; the pool itself is safe to use from any thread.
+constexpr uint64_t POOL_KEEP = 64ull << 20;
+constexpr int POOL_DEVICES_MAX = 64;
+
+int device_pool(sailor_ctx* ctx, cudaMemPool_t* out) {
+    static std::mutex lock;
+    static cudaMemPool_t pools[POOL_DEVICES_MAX];
+    if (ctx->device < 0 || ctx->device >= POOL_DEVICES_MAX) return SAILOR_E_RANGE;
+    std::lock_guard<std::mutex> hold(lock);
+    if (!pools[ctx->device]) {
+        cudaMemPoolProps props;
+        memset(&props, 0, sizeof(props));
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = ctx->device;
+        cudaMemPool_t pool;
+        CU(ctx, cudaMemPoolCreate(&pool, &props));
+        uint64_t keep = POOL_KEEP;
+        CU(ctx, cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+        pools[ctx->device] = pool;
+    }
+    *out = pools[ctx->device];
+    return SAILOR_OK;
+}
+
+int device_alloc(sailor_ctx* ctx, unsigned char** p, size_t bytes) {
+    cudaMemPool_t pool;
+    const int rc = device_pool(ctx, &pool);
+    if (rc) return rc;
+    void* got = nullptr;
+    const cudaError_t e = cudaMallocFromPoolAsync(&got, bytes, pool, ctx->stream);
+    if (e != cudaSuccess) {
+        ctx->last_cuda = (int)e;
+        (void)cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? SAILOR_E_NOMEM : SAILOR_E_CUDA;
+    }
+    *p = static_cast<unsigned char*>(got);
+    return SAILOR_OK;
+}
+
+// The work that uses the memory is on the context's stream (or has been joined with it).
+void device_free(sailor_ctx* ctx, unsigned char* p) {
+    if (p) cudaFreeAsync(p, ctx->stream);
+}
+
+// A working buffer that only grows: at least `need` bytes after a successful call.
+int device_grow(sailor_ctx* ctx, unsigned char** p, size_t* have, size_t need) {
+    if (need <= *have) return SAILOR_OK;
+    device_free(ctx, *p);
+    *p = nullptr;
+    *have = 0;
+    const int rc = device_alloc(ctx, p, need);
+    if (rc == SAILOR_OK) *have = need;
+    return rc;
+}
+
+// Pinned host blocks (68 KB each): allocating one can cost a millisecond, so the process keeps a few that no context
+// uses at the moment.
+class HostBlocks {
+  public:
+    int take(sailor_ctx* ctx, HostBlock** out) {
+        {
+            std::lock_guard<std::mutex> hold(lock_);
+            if (n_) { *out = kept_[--n_]; return SAILOR_OK; }
+        }
+        void* p = nullptr;
+        const cudaError_t e = cudaHostAlloc(&p, sizeof(HostBlock), cudaHostAllocMapped | cudaHostAllocPortable);
+        if (e != cudaSuccess) {
+            ctx->last_cuda = (int)e;
+            return e == cudaErrorMemoryAllocation ? SAILOR_E_NOMEM : SAILOR_E_CUDA;
+        }
+        *out = static_cast<HostBlock*>(p);
+        return SAILOR_OK;
+    }
+    void give_back(HostBlock* b) {
+        if (!b) return;
+        {
+            std::lock_guard<std::mutex> hold(lock_);
+            if (n_ < KEEP) { kept_[n_++] = b; return; }
+        }
+        cudaFreeHost(b);
+    }
+
+  private:
+    static constexpr int KEEP = 8;
+    std::mutex lock_;
+    HostBlock* kept_[KEEP] = {};
+    int n_ = 0;
+};
+HostBlocks g_host_blocks;
 
 struct DeviceGuard {
     int prev = -1;
@@ -375,91 +492,71 @@ int prepare_space(sailor_ctx* ctx, const sailor_space* s) {
     if (smem > (size_t)PLAN_SMEM_CEILING) return SAILOR_E_RANGE;
 
     sc.valid = false;
-    cudaFree(sc.d_chunk_start);
-    cudaFree(sc.d_flat_base);
-    sc.d_chunk_start = nullptr;
-    sc.d_flat_base = nullptr;
-    CU(ctx, cudaMalloc(&sc.d_chunk_start, cs.size() * sizeof(uint32_t)));
-    CU(ctx, cudaMalloc(&sc.d_flat_base, fb.size() * sizeof(uint64_t)));
-    CU(ctx, cudaMemcpyAsync(sc.d_chunk_start, cs.data(), cs.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-    CU(ctx, cudaMemcpyAsync(sc.d_flat_base, fb.data(), fb.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, ctx->stream));
-    CU(ctx, stream_sync(ctx));       // the vectors are pageable
-    {   // survey the space once: live chunks per configuration and the closed-form class counts
-        cudaFree(sc.d_live_start);
-        cudaFree(sc.d_cfg_closed);
-        cudaFree(sc.d_wave_start);
-        cudaFree(sc.d_cfg_best);
-        cudaFree(sc.d_groups);
-        cudaFree(sc.d_cfg_cache);
-        sc.d_cfg_cache = nullptr;
-        sc.d_live_start = nullptr;
-        sc.d_cfg_closed = nullptr;
-        sc.d_wave_start = nullptr;
-        sc.d_cfg_best = nullptr;
-        sc.d_groups = nullptr;
-        unsigned long long* d_closed = nullptr;
-        CU(ctx, cudaMalloc(&sc.d_live_start, (n_config + 1) * sizeof(uint32_t)));
-        if (n_config <= WAVE_CONFIG_MAX) {
-            CU(ctx, cudaMalloc(&sc.d_cfg_closed, n_config * 3 * sizeof(unsigned long long)));
-            CU(ctx, cudaMalloc(&sc.d_wave_start, (n_config + 1) * sizeof(uint32_t)));
-            CU(ctx, cudaMalloc(&sc.d_cfg_best, n_config * sizeof(unsigned long long)));
-            CU(ctx, cudaMalloc(&sc.d_groups, (n_config / d.n_d) * sizeof(GroupState)));
-        }
-        CU(ctx, cudaMalloc(&d_closed, 3 * sizeof(unsigned long long)));
-        cudaError_t e = cudaMemsetAsync(d_closed, 0, 3 * sizeof(unsigned long long), ctx->stream);
-        const uint32_t grid = (uint32_t)(n_config < 2048 ? n_config : 2048);
-        if (e == cudaSuccess) {
-            survey_kernel<<<grid, SURVEY_THREADS, 0, ctx->stream>>>(ctx->d_blob, d, (uint32_t)n_config, sc.d_live_start, d_closed,
-                                                                    sc.d_cfg_closed);
-            e = cudaGetLastError();
-        }
-        std::vector<uint32_t> live(n_config + 1, 0);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(live.data(), sc.d_live_start, n_config * sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(sc.closed, d_closed, sizeof(sc.closed), cudaMemcpyDeviceToHost, ctx->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        cudaFree(d_closed);
-        if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SAILOR_E_CUDA; }
-        uint64_t run = 0;                              // exclusive scan on the host: once per space
-        for (uint64_t j = 0; j < n_config; ++j) { const uint32_t v = live[j]; live[j] = (uint32_t)run; run += v; }
-        live[n_config] = (uint32_t)run;
-        sc.live_chunks = (uint32_t)run;
-        CU(ctx, cudaMemcpyAsync(sc.d_live_start, live.data(), (n_config + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-        CU(ctx, stream_sync(ctx));
+    sc.cache_head16 = cache_head16();
+    sc.cache_arr16 = cache_arr16(ctx->hdr.T, ctx->hdr.Z);
+    const bool with_waves = n_config <= WAVE_CONFIG_MAX;
+    // the tables of every configuration, built once: later searches copy them instead of building them
+    const size_t cache_bytes = n_config * 16 * ((size_t)sc.cache_head16 + sc.cache_arr16);
+    bool with_cache = cache_bytes <= CFG_CACHE_MAX_BYTES;
+    unsigned long long* d_closed = nullptr;
+    auto carve_space = [&](unsigned char* base) {
+        Bump bump{base};
+        d_closed = bump.take<unsigned long long>(3);
+        sc.d_chunk_start = bump.take<uint32_t>(n_config + 1);
+        sc.d_flat_base = bump.take<uint64_t>(n_config);
+        sc.d_live_start = bump.take<uint32_t>(n_config + 1);
+        sc.d_cfg_closed = with_waves ? bump.take<unsigned long long>(n_config * 3) : nullptr;
+        sc.d_wave_start = with_waves ? bump.take<uint32_t>(n_config + 1) : nullptr;
+        sc.d_cfg_best = with_waves ? bump.take<unsigned long long>(n_config) : nullptr;
+        sc.d_groups = with_waves ? bump.take<GroupState>(n_config / d.n_d) : nullptr;
+        sc.d_cfg_cache = with_cache ? bump.take<uint4>(cache_bytes / 16) : nullptr;
+        return bump.at;
+    };
+    device_free(ctx, sc.d_mem);
+    sc.d_mem = nullptr;
+    if (device_alloc(ctx, &sc.d_mem, carve_space(nullptr)) != SAILOR_OK) {
+        with_cache = false;                // no room for the tables: searches build them themselves
+        rc = device_alloc(ctx, &sc.d_mem, carve_space(nullptr));
+        if (rc) return rc;
     }
-    {   // the tables of every configuration, once: later searches copy them instead of building them
-        sc.cache_head16 = cache_head16();
-        sc.cache_arr16 = cache_arr16(ctx->hdr.T, ctx->hdr.Z);
-        const size_t rec_bytes = 16 * ((size_t)sc.cache_head16 + sc.cache_arr16);
-        if (n_config * rec_bytes <= CFG_CACHE_MAX_BYTES && cudaMalloc(&sc.d_cfg_cache, n_config * rec_bytes) == cudaSuccess) {
-            // (setting the attribute twice from two threads is harmless: both set the same value)
-            static std::atomic<bool> optin_done[64];
-            const bool tracked = ctx->device >= 0 && ctx->device < 64;
-            if (!tracked || !optin_done[ctx->device].load(std::memory_order_acquire)) {
-                CU(ctx, cudaFuncSetAttribute(cfg_cache_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PLAN_SMEM_CEILING));
-                if (tracked) optin_done[ctx->device].store(true, std::memory_order_release);
-            }
-            PlanParams pp;
-            memset(&pp, 0, sizeof(pp));
-            pp.blob = ctx->d_blob;
-            memcpy(pp.avail, ctx->h_avail, sizeof(pp.avail));
-            pp.ctrl = ctx->d_ctrl;
-            pp.cfg_flat_base = sc.d_flat_base;
-            pp.sp = d;
-            pp.n_config = (uint32_t)n_config;
-            pp.p_max = p_max;
-            pp.live_mode = 1;                  // the lists of usable digits are part of a record
-            pp.min_tp_only = 1;                // and so are the masks of the smaller tensor-parallel degrees
-            pp.cache_head16 = sc.cache_head16;
-            pp.cache_arr16 = sc.cache_arr16;
-            const uint32_t grid = (uint32_t)(n_config < (uint64_t)ctx->sm_count * 2 ? n_config : (uint64_t)ctx->sm_count * 2);
-            cfg_cache_kernel<<<grid, PLAN_THREADS, smem, ctx->stream>>>(pp, sc.d_cfg_cache);
-            CU(ctx, cudaGetLastError());
-            CU(ctx, stream_sync(ctx));
-        } else {
-            sc.d_cfg_cache = nullptr;          // too large (or no memory): searches build the tables themselves
-            (void)cudaGetLastError();
+    carve_space(sc.d_mem);
+    // survey the space: chunk and flat-index offsets, live chunks per configuration, the closed-form class counts
+    CU(ctx, cudaMemsetAsync(d_closed, 0, 3 * sizeof(unsigned long long), ctx->stream));
+    survey_kernel<<<(uint32_t)std::min<uint64_t>(n_config, 2048), SURVEY_THREADS, 0, ctx->stream>>>(
+        ctx->d_blob, d, (uint32_t)n_config, sc.d_live_start, sc.d_chunk_start, sc.d_flat_base, d_closed, sc.d_cfg_closed);
+    CU(ctx, cudaGetLastError());
+    SurveyOut* d_survey = nullptr;
+    CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&d_survey), &ctx->host->survey, 0));
+    live_scan_kernel<<<1, SCAN_THREADS, 0, ctx->stream>>>(sc.d_live_start, (uint32_t)n_config, d_closed, d_survey);
+    CU(ctx, cudaGetLastError());
+    if (sc.d_cfg_cache) {
+        // (setting the attribute twice from two threads is harmless: both set the same value)
+        static std::atomic<bool> optin_done[64];
+        const bool tracked = ctx->device >= 0 && ctx->device < 64;
+        if (!tracked || !optin_done[ctx->device].load(std::memory_order_acquire)) {
+            CU(ctx, cudaFuncSetAttribute(cfg_cache_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PLAN_SMEM_CEILING));
+            if (tracked) optin_done[ctx->device].store(true, std::memory_order_release);
         }
+        PlanParams pp;
+        memset(&pp, 0, sizeof(pp));
+        pp.blob = ctx->d_blob;
+        memcpy(pp.avail, ctx->h_avail, sizeof(pp.avail));
+        pp.ctrl = ctx->d_ctrl;
+        pp.cfg_flat_base = sc.d_flat_base;
+        pp.sp = d;
+        pp.n_config = (uint32_t)n_config;
+        pp.p_max = p_max;
+        pp.live_mode = 1;                  // the lists of usable digits are part of a record
+        pp.min_tp_only = 1;                // and so are the masks of the smaller tensor-parallel degrees
+        pp.cache_head16 = sc.cache_head16;
+        pp.cache_arr16 = sc.cache_arr16;
+        const uint32_t grid = (uint32_t)(n_config < (uint64_t)ctx->sm_count * 2 ? n_config : (uint64_t)ctx->sm_count * 2);
+        cfg_cache_kernel<<<grid, PLAN_THREADS, smem, ctx->stream>>>(pp, sc.d_cfg_cache);
+        CU(ctx, cudaGetLastError());
     }
+    CU(ctx, stream_sync(ctx));             // the host needs the number of live chunks
+    sc.live_chunks = ctx->host->survey.live_chunks;
+    memcpy(sc.closed, ctx->host->survey.closed, sizeof(sc.closed));
     sc.key = *s;
     sc.desc = d;
     sc.n_config = (uint32_t)n_config;
@@ -686,14 +783,15 @@ int host_batch(sailor_ctx* ctx, const unsigned char* recs, size_t rec_bytes, uin
     const size_t slot_bytes = (slot_records * (rec_bytes + 32) + 255) / 256 * 256;
     const uint64_t n_chunks = (n + chunk - 1) / chunk;
     const size_t need = slot_bytes * (split ? (n_chunks < HOST_SLOTS ? n_chunks : HOST_SLOTS) : 1);
-    if (need > ctx->stage_bytes) {
-        CU(ctx, stream_sync(ctx));
-        cudaFree(ctx->d_stage);
-        ctx->d_stage = nullptr;
-        ctx->stage_bytes = 0;
-        cudaError_t e = cudaMalloc(&ctx->d_stage, need);
-        if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SAILOR_E_NOMEM; }
-        ctx->stage_bytes = need;
+    {
+        const int rc_mem = device_grow(ctx, &ctx->d_stage, &ctx->stage_bytes, need);
+        if (rc_mem) return rc_mem;
+    }
+    if (split && !ctx->out_stream) {       // made when the first batch that needs them arrives
+        CU(ctx, cudaEventCreateWithFlags(&ctx->ev_chunk, cudaEventDisableTiming));
+        CU(ctx, cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
+        for (cudaEvent_t& e : ctx->ev_slot) CU(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        CU(ctx, cudaStreamCreateWithFlags(&ctx->out_stream, cudaStreamNonBlocking));
     }
     {
         const int rc_up = upload_availability(ctx);
@@ -869,21 +967,27 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
         delete ctx;
         return SAILOR_E_RANGE;
     }
-    h.off_chain_f = put<double>(blob, nullptr, c4);
-    h.off_chain_b = put<double>(blob, nullptr, c4);
-    h.off_chain_u = put<double>(blob, nullptr, c3);
-    h.off_cmp_params = put<uint64_t>(blob, nullptr, n_comp);
-    h.off_cmp_grad = put<double>(blob, nullptr, cmp_grad);
-    h.off_cmp_mem = put<uint64_t>(blob, nullptr, cmp_mem);
-    h.off_cmp_fb = put<double>(blob, nullptr, cmp_fb);
-    h.off_cmp_upd = put<double>(blob, nullptr, cmp_upd);
-    blob.resize((blob.size() + 31) & ~(size_t)31);         // a table entry is one 32-byte sector
-    h.off_piece = put<PieceRec>(blob, nullptr, cmp_fb);
-    h.off_lnk_intra2 = put<double>(blob, nullptr, R * n_mbs);
-    h.off_lnk_inter2 = put<double>(blob, nullptr, R * n_mbs);
-    h.off_lnk_zone2 = put<double>(blob, nullptr, (size_t)Z * Z * n_mbs);
-    h.total_bytes = align16((uint32_t)blob.size());
-    blob.resize(h.total_bytes);
+    // what the kernels below form from the static part lies behind it, on the device only
+    size_t at = h.static_bytes;
+    auto reserve = [&](size_t bytes, size_t align) {
+        at = (at + align - 1) / align * align;
+        const uint32_t off = (uint32_t)at;
+        at += bytes;
+        return off;
+    };
+    h.off_chain_f = reserve(c4 * 8, 16);
+    h.off_chain_b = reserve(c4 * 8, 16);
+    h.off_chain_u = reserve(c3 * 8, 16);
+    h.off_cmp_params = reserve(n_comp * 8, 16);
+    h.off_cmp_grad = reserve(cmp_grad * 8, 16);
+    h.off_cmp_mem = reserve(cmp_mem * 8, 16);
+    h.off_cmp_fb = reserve(cmp_fb * 8, 16);
+    h.off_cmp_upd = reserve(cmp_upd * 8, 16);
+    h.off_piece = reserve(cmp_fb * sizeof(PieceRec), 32);  // a table entry is one 32-byte sector
+    h.off_lnk_intra2 = reserve(R * n_mbs * 8, 16);
+    h.off_lnk_inter2 = reserve(R * n_mbs * 8, 16);
+    h.off_lnk_zone2 = reserve((size_t)Z * Z * n_mbs * 8, 16);
+    h.total_bytes = align16((uint32_t)at);
     memcpy(blob.data(), &h, sizeof(h));
 
     auto fail = [&](int code) { sailor_destroy(ctx); return code; };
@@ -895,34 +999,35 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
             return fail(e_ == cudaErrorMemoryAllocation ? SAILOR_E_NOMEM : SAILOR_E_CUDA); \
         }                                                           \
     } while (0)
-    cudaDeviceProp prop;
-    CUF(cudaGetDeviceProperties(&prop, cuda_device));
-    ctx->sm_count = prop.multiProcessorCount;
+    CUF(cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, cuda_device));
     ctx->max_grid = (uint32_t)ctx->sm_count * 8;
-    CUF(cudaMalloc(&ctx->d_blob, h.total_bytes));
-    CUF(cudaMalloc(&ctx->d_avail, R_MAX * sizeof(uint16_t)));
-    CUF(cudaMallocHost(&ctx->h_avail, R_MAX * sizeof(uint16_t)));
-    memset(ctx->h_avail, 0, R_MAX * sizeof(uint16_t));       // availability starts at zero on both sides
-    CUF(cudaMalloc(&ctx->d_ctrl, sizeof(Ctrl)));
-    CUF(cudaMalloc(&ctx->d_sim_error, 2 * sizeof(unsigned int)));
-    CUF(cudaHostAlloc(&ctx->h_out, sizeof(PlanOut), cudaHostAllocMapped));
+    int rc = g_host_blocks.take(ctx, &ctx->host);
+    if (rc) return fail(rc);
+    memset(static_cast<void*>(ctx->host), 0, offsetof(HostBlock, mixed));     // availability starts at zero on both sides
+    ctx->h_avail = ctx->host->avail;
+    ctx->h_out = &ctx->host->out;
     CUF(cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->d_out_mapped), ctx->h_out, 0));
-    memset(ctx->h_out, 0, sizeof(PlanOut));
-    CUF(cudaMalloc(&ctx->d_partial, sizeof(Hit) * SAILOR_K_MAX * ctx->max_grid));
-    CUF(cudaMalloc(&ctx->d_partial_n, sizeof(uint32_t) * ctx->max_grid));
+    auto carve_ctx = [&](unsigned char* base) {              // returns (bytes that start from zero, all bytes)
+        Bump bump{base};
+        ctx->d_avail = bump.take<uint16_t>(R_MAX);
+        ctx->d_ctrl = bump.take<Ctrl>(1);
+        ctx->d_sim_error = bump.take<unsigned int>(2);
+        const size_t zeroed = bump.at;
+        ctx->d_blob = bump.take<unsigned char>(h.total_bytes);
+        ctx->d_partial = bump.take<Hit>((size_t)SAILOR_K_MAX * ctx->max_grid);
+        ctx->d_partial_n = bump.take<uint32_t>(ctx->max_grid);
+        return std::make_pair(zeroed, bump.at);
+    };
+    rc = device_alloc(ctx, &ctx->d_mem, carve_ctx(nullptr).second);
+    if (rc) return fail(rc);
+    const size_t zeroed = carve_ctx(ctx->d_mem).first;
     CUF(cudaEventCreate(&ctx->ev0));
     CUF(cudaEventCreate(&ctx->ev1));
     CUF(cudaEventCreate(&ctx->ev2));
     CUF(cudaEventCreate(&ctx->evh0));
     CUF(cudaEventCreate(&ctx->evh1));
-    CUF(cudaStreamCreateWithFlags(&ctx->out_stream, cudaStreamNonBlocking));
-    CUF(cudaEventCreateWithFlags(&ctx->ev_chunk, cudaEventDisableTiming));
-    CUF(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
-    for (cudaEvent_t& e : ctx->ev_slot) CUF(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    CUF(cudaMemcpyAsync(ctx->d_blob, blob.data(), h.total_bytes, cudaMemcpyHostToDevice, ctx->stream));
-    CUF(cudaMemsetAsync(ctx->d_avail, 0, R_MAX * sizeof(uint16_t), ctx->stream));
-    CUF(cudaMemsetAsync(ctx->d_ctrl, 0, sizeof(Ctrl), ctx->stream));
-    CUF(cudaMemsetAsync(ctx->d_sim_error, 0, 2 * sizeof(unsigned int), ctx->stream));
+    CUF(cudaMemsetAsync(ctx->d_mem, 0, zeroed, ctx->stream));
+    CUF(cudaMemcpyAsync(ctx->d_blob, blob.data(), h.static_bytes, cudaMemcpyHostToDevice, ctx->stream));   // returns when `blob` has been read
     {
         const uint32_t n_threads = 4 * T * n_tp * n_mbs + 2 * T * n_tp;
         chain_kernel<<<(n_threads + 127) / 128, 128, 0, ctx->stream>>>(ctx->d_blob);
@@ -934,7 +1039,6 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
         batch_tables_kernel<<<grid, 128, 0, ctx->stream>>>(ctx->d_blob);
         CUF(cudaGetLastError());
     }
-    CUF(cudaStreamSynchronize(ctx->stream));           // `blob` is pageable host memory
     // both kernels stage the static tables in dynamic shared memory; the create-time limit is 96 KB
     CUF(cudaFuncSetAttribute(simulate_mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 64) * 1024));
     CUF(cudaFuncSetAttribute(simulate_mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 64) * 1024));
@@ -949,28 +1053,10 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
 int sailor_destroy(sailor_ctx* ctx) {
     if (!ctx) return SAILOR_OK;
     DeviceGuard guard(ctx->device);
-    if (ctx->d_blob) cudaStreamSynchronize(ctx->stream);
-    cudaFree(ctx->d_blob);
-    cudaFree(ctx->d_avail);
-    cudaFreeHost(ctx->h_avail);
-    cudaFree(ctx->d_ctrl);
-    cudaFree(ctx->d_sim_error);
-    cudaFreeHost(ctx->h_out);
-    cudaFree(ctx->d_partial);
-    cudaFree(ctx->d_partial_n);
-    cudaFree(ctx->space.d_chunk_start);
-    cudaFree(ctx->space.d_flat_base);
-    cudaFree(ctx->space.d_live_start);
-    cudaFree(ctx->space.d_cfg_closed);
-    cudaFree(ctx->space.d_wave_start);
-    cudaFree(ctx->space.d_cfg_best);
-    cudaFree(ctx->space.d_groups);
-    cudaFree(ctx->space.d_cfg_cache);
-    cudaFree(ctx->d_stage);
+    if (ctx->d_mem) cudaStreamSynchronize(ctx->stream);
+    for (unsigned char* p : {ctx->d_mem, ctx->space.d_mem, ctx->d_stage, ctx->d_mix, ctx->d_dp}) device_free(ctx, p);
+    g_host_blocks.give_back(ctx->host);
     delete ctx->mix;
-    cudaFree(ctx->d_mix);
-    cudaFreeHost(ctx->h_mix_out);
-    cudaFree(ctx->d_dp);
     for (cudaEvent_t e : {ctx->ev0, ctx->ev1, ctx->ev2, ctx->evh0, ctx->evh1, ctx->ev_chunk, ctx->ev_join, ctx->ev_slot[0],
                           ctx->ev_slot[1], ctx->ev_slot[2]})
         if (e) cudaEventDestroy(e);
@@ -1402,23 +1488,6 @@ extern "C" int sailor_plan_noalloc(sailor_ctx* ctx, const sailor_space* s, const
 
 // ---- per-stage GPU types by dynamic programming ---------------------------------------------------
 
-namespace {
-
-struct Bump {                       // carves 256-byte aligned pieces out of one device buffer
-    unsigned char* base;
-    size_t at = 0;
-    template <typename T>
-    T* take(size_t n) {
-        T* p = reinterpret_cast<T*>(base + at);
-        at += (n * sizeof(T) + 255) & ~(size_t)255;
-        return p;
-    }
-};
-
-size_t padded(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
-
-}  // namespace
-
 // The recursion steered by the budget (Sec. 4.2.3): one thread per problem, depth first.
 static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor_zone_order* orders, uint32_t n_orders,
                                const sailor_objective* o, uint64_t workspace_bytes, uint32_t k, sailor_dp_result* topk,
@@ -1460,14 +1529,9 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
                          padded(n_problems * DP_BUDGET_P_MAX * sizeof(DpbFrame)) + padded(sizeof(sailor_dp_result) * SAILOR_K_MAX) +
                          padded(40) + 4096;
     if (total > workspace_bytes) return SAILOR_E_RANGE;
-    if (total > ctx->dp_bytes) {
-        CU(ctx, stream_sync(ctx));
-        cudaFree(ctx->d_dp);
-        ctx->d_dp = nullptr;
-        ctx->dp_bytes = 0;
-        cudaError_t e = cudaMalloc(&ctx->d_dp, total);
-        if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SAILOR_E_NOMEM; }
-        ctx->dp_bytes = total;
+    {
+        const int rc_mem = device_grow(ctx, &ctx->d_dp, &ctx->dp_bytes, total);
+        if (rc_mem) return rc_mem;
     }
     Bump bump{ctx->d_dp};
     double* d_tabs = bump.take<double>(tab_bytes / sizeof(double));
@@ -1758,14 +1822,9 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
                          padded(n_problems * sizeof(DpProblem)) +
                          2 * padded((max_blocks + p_max + 16) * sizeof(uint32_t)) + 2 * padded(max_entries * sizeof(DpVal)) +
                          padded(max_choice) + padded(sizeof(sailor_dp_result) * SAILOR_K_MAX) + padded(24) + 4096;
-    if (total > ctx->dp_bytes) {
-        CU(ctx, stream_sync(ctx));
-        cudaFree(ctx->d_dp);
-        ctx->d_dp = nullptr;
-        ctx->dp_bytes = 0;
-        cudaError_t e = cudaMalloc(&ctx->d_dp, total);
-        if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SAILOR_E_NOMEM; }
-        ctx->dp_bytes = total;
+    {
+        const int rc_mem = device_grow(ctx, &ctx->d_dp, &ctx->dp_bytes, total);
+        if (rc_mem) return rc_mem;
     }
     Bump bump{ctx->d_dp};
     double* d_tabs = bump.take<double>(tab_bytes / sizeof(double));
@@ -2054,21 +2113,12 @@ size_t mixed_carve(const sailor_ctx* ctx, const MixedTables& mt, MixedSearchPara
 
 // Working memory for a mixed space and its tables on the device.
 int mixed_workspace(sailor_ctx* ctx, const MixedTables& mt) {
-    if (!ctx->h_mix_out) {
-        CU(ctx, cudaHostAlloc(&ctx->h_mix_out, sizeof(MixedOut), cudaHostAllocMapped));
-        CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->d_mix_out), ctx->h_mix_out, 0));
-    }
     MixedSearchParams mp;
     const size_t need = mixed_carve(ctx, mt, mp);
     if (need > ctx->mix_bytes) {
-        CU(ctx, stream_sync(ctx));
-        cudaFree(ctx->d_mix);
-        ctx->d_mix = nullptr;
-        ctx->mix_bytes = 0;
-        cudaError_t e = cudaMalloc(&ctx->d_mix, need);
-        if (e != cudaSuccess) { ctx->last_cuda = (int)e; return SAILOR_E_NOMEM; }
-        ctx->mix_bytes = need;
         ctx->mix_dirty = true;
+        const int rc = device_grow(ctx, &ctx->d_mix, &ctx->mix_bytes, need);
+        if (rc) return rc;
         mixed_carve(ctx, mt, mp);
     }
     CU(ctx, cudaMemcpyAsync(const_cast<uint64_t*>(mp.combs), mt.combs.data(), mt.combs.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
@@ -2112,7 +2162,8 @@ static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const s
     }
     ctx->mix_dirty = true;             // until this call has gone through
     if (stats) CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
-    mp.blob = ctx->d_blob; mp.out = ctx->d_mix_out; mp.sp = mt.desc; mp.n_config = mt.n_config; mp.k = k; mp.obj = o->kind;
+    CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&mp.out), &ctx->host->mixed, 0));
+    mp.blob = ctx->d_blob; mp.sp = mt.desc; mp.n_config = mt.n_config; mp.k = k; mp.obj = o->kind;
     memcpy(mp.avail, ctx->h_avail, sizeof(mp.avail));
     mp.n_partial = grid; mp.n_total = n_total; mp.budget = o->budget_usd_per_iter; mp.min_rate = o->min_iters_per_s;
     bool deep = false;                                           // pipelines of more than 32 stages in the space
@@ -2138,12 +2189,12 @@ static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const s
     ++launches;
     if (stats) CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
     CU(ctx, stream_sync(ctx));
-    const unsigned long long* counters = ctx->h_mix_out->counters;
+    const unsigned long long* counters = ctx->host->mixed.counters;
     if (counters[MIXC_ERROR]) return SAILOR_E_DEVICE;
     if (counters[MIXC_FOUND] > k) return SAILOR_E_DEVICE;
     ctx->mix_dirty = false;
     *n_found = (uint32_t)counters[MIXC_FOUND];
-    memcpy(topk, ctx->h_mix_out->results, sizeof(sailor_mixed_result) * counters[MIXC_FOUND]);
+    memcpy(topk, ctx->host->mixed.results, sizeof(sailor_mixed_result) * counters[MIXC_FOUND]);
     if (stats) {
         memset(stats, 0, sizeof(*stats));
         stats->n_total = counters[0];

@@ -67,11 +67,13 @@ __global__ void __launch_bounds__(PLAN_THREADS, PLAN_MIN_BLOCKS) cfg_cache_kerne
 // host tp and whose stages fit in memory (H2: independent of availability), hence the number of
 // chunks of prefixes made of such digits only, and -- in closed form -- how many candidates are
 // invalid or out of memory.  Runs once per (context, space); the plan search then enumerates only
-// the live prefixes.  One block per configuration at a time.
+// the live prefixes.  One block per configuration at a time.  The same pass lays down where every
+// configuration's candidates and chunks start when nothing is pruned.
 constexpr int SURVEY_THREADS = 128;
 
 __global__ void __launch_bounds__(SURVEY_THREADS)
 survey_kernel(const unsigned char* __restrict__ blob, SpaceDesc sp, uint32_t n_config, uint32_t* __restrict__ live_chunks,
+              uint32_t* __restrict__ chunk_start /* [n_config + 1] */, uint64_t* __restrict__ flat_base /* [n_config] */,
               unsigned long long* __restrict__ closed /* total, invalid, oom */,
               unsigned long long* __restrict__ cfg_closed /* [n_config][3], the same per configuration; may be null */) {
     __shared__ uint32_t oom_stage[SAILOR_P_MAX];
@@ -134,7 +136,66 @@ survey_kernel(const unsigned char* __restrict__ blob, SpaceDesc sp, uint32_t n_c
                 if (cfg_closed) cfg_closed[3 * (size_t)c + j] = mine[j];
             }
             live_chunks[c] = chunks;
+            // candidates and chunks of the configurations before this one: whole sub-spaces, then equal ones
+            const uint32_t per_p = sp.n_mbs * sp.n_tp * sp.n_rc * sp.n_d;
+            uint64_t flat = 0;
+            uint32_t chunk = 0;
+            for (uint32_t j = 0; j <= c / per_p; ++j) {
+                const uint32_t before = j < c / per_p ? per_p : c - j * per_p;
+                const uint64_t items = ipow64(R, nseg_of(sp.p_values[j], sp.seg_max) - 1);
+                const uint32_t per_cfg = (uint32_t)((items + PLAN_THREADS - 1) / PLAN_THREADS);
+                flat += before * items * R;
+                chunk += before * per_cfg;
+                if (c + 1 == n_config && j == c / per_p) chunk_start[n_config] = chunk + per_cfg;
+            }
+            flat_base[c] = flat;
+            chunk_start[c] = chunk;
         }
+    }
+}
+
+// Live chunks per configuration -> where each configuration's live chunks start, in place (exclusive scan, one
+// block); the total and the closed-form counts go to the host.
+struct SurveyOut {
+    uint32_t live_chunks, _pad;
+    unsigned long long closed[3];
+};
+constexpr int SCAN_THREADS = 1024;
+
+__global__ void __launch_bounds__(SCAN_THREADS)
+live_scan_kernel(uint32_t* __restrict__ live, uint32_t n_config, const unsigned long long* __restrict__ closed, SurveyOut* out) {
+    __shared__ uint32_t warp_sum[SCAN_THREADS / 32];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t per = (n_config + SCAN_THREADS - 1) / SCAN_THREADS;
+    const uint32_t c0 = min(tid * per, n_config), c1 = min(c0 + per, n_config);
+    uint32_t mine = 0;
+    for (uint32_t c = c0; c < c1; ++c) mine += live[c];
+    uint32_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(FULL, incl, o);
+        if (lane >= (uint32_t)o) incl += up;
+    }
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t w = warp_sum[lane];
+        uint32_t wi = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t up = __shfl_up_sync(FULL, wi, o);
+            if (lane >= (uint32_t)o) wi += up;
+        }
+        warp_sum[lane] = wi - w;
+        if (lane == 31) { live[n_config] = wi; out->live_chunks = wi; }
+        if (lane < 3) out->closed[lane] = closed[lane];
+    }
+    __syncthreads();
+    uint32_t at = warp_sum[warp] + incl - mine;
+    for (uint32_t c = c0; c < c1; ++c) {
+        const uint32_t here = live[c];
+        live[c] = at;
+        at += here;
     }
 }
 

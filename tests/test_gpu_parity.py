@@ -650,3 +650,41 @@ def test_config5_sampled_candidates_match_oracle_one_by_one(make_ctx):
     assert set(np.unique(packed["P"]).tolist()) == set(w.p_values)
     s = orc[0]
     assert (s == 0).any() and (s & B.ST_OOM).any() and (s & B.ST_OVER_AVAIL).any() and (s & B.ST_INVALID).any()
+
+
+@pytest.mark.parametrize("n_threads,own_stream", [(1, False), (4, True)])
+def test_contexts_come_and_go_on_threads_and_streams(n_threads, own_stream, torch_cuda):
+    """Contexts take their memory from a pool that outlives them: whatever an earlier context of any thread or stream
+    left in it must not show in the results of a fresh one, for spaces and batches of different sizes in turn."""
+    import threading
+    torch = torch_cuda
+    loads = [W.config1(), W.tiny(seed=21, n_types=3, n_zones=2), W.config6()]
+    want = []
+    for w in loads:
+        o = Oracle(w)
+        recs = W.random_plans(w, 300, seed=9)
+        want.append((o.search(w.objective, 8, min_rate=w.min_iters_per_s)[0], recs, o.simulate_records(recs)))
+    wrong = []
+
+    def work(t):
+        stream = torch.cuda.Stream() if own_stream else torch.cuda.current_stream()
+        for rnd in range(6):
+            w, (hits, recs, sim) = loads[(t + rnd) % len(loads)], want[(t + rnd) % len(loads)]
+            ctx = B.sailor_create(w, 0, stream.cuda_stream)
+            try:
+                B.sailor_set_availability(ctx, w.avail)
+                res, _ = B.sailor_plan(ctx, B.make_space(w), B.make_objective(w), 8)
+                if [(r.flat, r.t_iter, r.cost) for r in res] != [(h["flat"], h["t_iter"], h["cost"]) for h in hits]:
+                    wrong.append((t, rnd, "search"))
+                ti, mem, cost, st = B.sailor_simulate(ctx, B.pack_records(recs))
+                if not (np.array_equal(st, sim[0]) and np.array_equal(mem, sim[3]) and np.array_equal(ti, sim[1], equal_nan=True)):
+                    wrong.append((t, rnd, "records"))
+            finally:
+                B.sailor_destroy(ctx)
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(n_threads)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not wrong, wrong
