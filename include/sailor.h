@@ -498,16 +498,15 @@ int sailor_plan_mixed(sailor_ctx* ctx, const sailor_mixed_space* s, const sailor
  * check of the simulator's cost against the budget still follows, as without the flag.  n_states then counts the
  * calls of the recursion.
  *
- * On the device every problem is a dense table over its states (stage, type, zone position,
+ * On the device every problem is a table over the states a stage can be in (stage, type, zone position,
  * stages per type already placed in that zone; a type with room for all P stages in a zone is not
- * counted there), filled from the last stage to the first, one launch per stage for all problems
- * of a batch together; batches are cut so that the tables fit `workspace_bytes`. */
-/* How sailor_plan_dp lays out and walks its tables, in sailor_objective.flags.  The results do not
- * depend on them; they exist so that every code path can be selected (and tested) through this
- * interface.  Index of a zone position's count vectors: the smaller of the two ways (default), mixed
- * radix whenever it fits (DENSE), by rank whenever it fits (COMPACT).  Threads of a stage's launch: one
- * per reachable count vector for all its types (default), one per reachable count vector and type
- * (BY_TYPE), one per table entry (BY_ENTRY). */
+ * counted there, a type that fits no stage's memory is left out), filled from the last stage to the first: small
+ * problems by one block each, the others together, one launch per stage; batches are cut so that the tables fit
+ * `workspace_bytes`. */
+/* Flags of sailor_plan_dp that once chose between table layouts and thread assignments, in sailor_objective.flags.
+ * There is one layout now and the results never depended on them; they are still accepted, at most one of each pair.
+ * With INDEX_DENSE a problem whose tables in mixed radix over all scarce types would exceed `workspace_bytes` or 2^31
+ * entries is still refused (E_RANGE), as before. */
 #define SAILOR_DP_FLAG_INDEX_DENSE    0x100u
 #define SAILOR_DP_FLAG_INDEX_COMPACT  0x200u
 #define SAILOR_DP_FLAG_ENUM_BY_TYPE   0x400u

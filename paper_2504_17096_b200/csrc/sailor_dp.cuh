@@ -4,17 +4,25 @@
 // (stage i, type g of stage i, zone position zp of stage i, u = stages per type already placed in
 // that zone, stage i included).  Zones before zp are never revisited and zones after it are
 // untouched (first fit), so nothing else of the past matters.  A type that a zone could give to all
-// P stages is not counted in u.  For every zone position and type there is a slice of S[zp] entries
-// indexed by u, in one of two ways chosen per zone position: densely in mixed radix (radix cap + 1 per
-// counted type), or compactly by the rank of u among the count vectors that respect the caps and add
-// up to at most P (a zone never holds more than P stages); the compact index is much smaller when
-// many types are scarce at once.  The value of a state is the best plan of stages i.. from it:
-// (sum of stage times, straggler, slowest synchronisation, slowest update).
+// P stages is not counted in u, and a type that fits no stage's memory is never placed.  The value of
+// a state is the best plan of stages i.. from it: (sum of stage times, straggler, slowest
+// synchronisation, slowest update).
 //
-// The tables are filled from the last stage to the first.  One launch handles one stage distance
-// from the end for every problem of a batch (problems are sorted by depth, so the launch for
-// distance s covers a prefix of the block list); a thread owns one state and tries every type for
-// the next stage.  Per-configuration quantities (stage times per type, synchronisation per digit,
+// Only states that stage i can be in are visited.  First fit leaves a zone only when one of its types
+// is used up, so position zp is reached after at least lo(zp) = sum of the smallest caps of the earlier
+// positions and after at most mx(zp) = sum of all their caps stages: a stage i in position zp has
+//     max(0 or 1, i + 1 - mx(zp))  <=  stages counted in u  <=  i + 1 - lo(zp)
+// behind it (in the first zone of counted types only: exactly i + 1).  The count vectors of a position are
+// numbered sum by sum (within a sum in lexicographic order), so the vectors of a stage are one contiguous range
+// per position, and a move of one stage is a look-up: `nxt` holds, per vector and type, the vector with one more
+// stage of that type.  Vectors, ranges and moves depend on (P, D * tp, zone order, types that fit) only -- a
+// *layout*, shared by all problems alike in these and laid down once per call by dp_layout_kernel.
+// A problem without a type for some stage's memory has no plan and no tables.
+//
+// Tables are filled from the last stage to the first: a thread owns one count vector for all types of stage i,
+// tries every type for the next stage, and each value of the next stage is read by exactly one vector of the same
+// position.  Small problems take one block through all their stages; the others advance together, a launch per
+// distance from the last stage.  Per-configuration quantities (stage times per type, synchronisation per digit,
 // message times per digit pair) are formed once per configuration by dp_tables_kernel.
 #pragma once
 
@@ -24,39 +32,44 @@ namespace sailor {
 
 constexpr int DP_THREADS = 256;
 constexpr uint8_t DP_NONE = 255;
-constexpr uint32_t DP_DENSE = 0xffffffffu;
+constexpr uint32_t DP_SELF = 0x80000000u;        // in a row of `nxt`: the vector holds a stage of this type (or need not count it)
+constexpr uint32_t DP_NO_VEC = 0x7fffffffu;      // no room for one more stage of this type in the position
+constexpr uint32_t DP_NO_STATE = 0xffffffffu;
+constexpr uint32_t DP_SMALL = 2048;              // most vectors a stage of a small problem has: eight rounds of one block
 
 struct alignas(32) DpVal {           // best plan of stages i.. from a state; sum = +inf: there is none.  Aligned to its
                                      // size: a value then moves in one load or store
     double sum, mx, sy, up;
 };
 
-struct DpProblem {
-    uint64_t val_off;                // first entry of this problem in the two level buffers of its batch
-    uint64_t choice_off;             // first byte of its choices: [stage][entry]
-    uint32_t config, order, index;   // index = config * n_orders + order
-    uint32_t n_lvl;                  // entries per stage
-    uint32_t P, nz, need;            // need = D * tp GPUs per stage
+struct DpLayout {
+    uint32_t P, nz;                  // positions that a pipeline of P stages can reach
+    uint32_t nxt_off;                // first row of `nxt`
+    uint32_t live_off;               // first word of its live rows
+    uint32_t vec_base[SAILOR_Z_MAX + 1];           // first vector of each position
+    uint32_t sum_max[SAILOR_Z_MAX];  // largest sum a position's vectors have
+    uint32_t w_off[SAILOR_Z_MAX];    // its rank table: W[j][s], j = 0 .. n_counted, s = 0 .. P (vectors of the counted
+                                     // types from the j-th on that add up to at most s)
+    uint32_t first_vec[SAILOR_Z_MAX][SAILOR_T_MAX];     // the vector of "one stage, of this type"
     uint8_t zone[SAILOR_Z_MAX];      // zone of each position of the order
-    uint8_t cap[SAILOR_Z_MAX][SAILOR_T_MAX];       // stages a (position, type) can host, saturated at 255
-    uint8_t first_later[SAILOR_Z_MAX][SAILOR_T_MAX];   // first position after zp that can host a stage of the type
-    uint32_t stride[SAILOR_Z_MAX][SAILOR_T_MAX];   // mixed-radix stride of a counted type; 0: not counted
-    uint32_t S[SAILOR_Z_MAX];        // entries of one (position, type) slice
-    uint32_t zp_base[SAILOR_Z_MAX + 1];            // first entry of each position's T slices
-    uint32_t vt_lo;                  // the problem's rank tables are vtabs[vt_lo .. vt_lo + vt_len)
-    uint32_t first_idx[SAILOR_Z_MAX][SAILOR_T_MAX];    // index of "one stage, of this type" inside a slice
-    uint32_t vt_off[SAILOR_Z_MAX];   // compact index: offset of the position's rank table in `vtabs`; DP_DENSE: mixed radix
-    uint32_t rank_off[SAILOR_Z_MAX]; // the position's rank table whatever its index (DP_DENSE: no counted type, or
-                                     // none built): lets a launch enumerate only the count vectors a stage can reach
-    uint32_t vt_len, _pad;
-    uint8_t n_counted[SAILOR_Z_MAX]; // counted types of each position
-    uint64_t magic[SAILOR_Z_MAX][SAILOR_T_MAX];    // ceil(2^64 / (cap + 1)) of a counted type: for 32-bit x,
-                                                   // x / (cap + 1) == high 64 bits of x * magic
+    uint8_t n_counted[SAILOR_Z_MAX];
+    uint8_t counted[SAILOR_Z_MAX];   // bit g: type g is counted
+    uint8_t cap[SAILOR_Z_MAX][SAILOR_T_MAX];            // stages a (position, type) can host, saturated at 255
+    uint8_t first_later[SAILOR_Z_MAX][SAILOR_T_MAX];    // first position after zp that can host a stage of the type
 };
-static_assert(sizeof(DpProblem) % 8 == 0, "copied word by word");
+static_assert(sizeof(DpLayout) % 4 == 0, "copied word by word");
+// A live row (one per stage): count of live vectors, count before this stage, then per position (first vector, slot of
+// that vector); a vector's slot is its place among the live vectors of the stage.
+__host__ __device__ inline uint32_t dp_live_words(uint32_t nz) { return 2 + 2 * nz; }
+constexpr uint32_t DP_LIVE_WORDS_MAX = 2 + 2 * SAILOR_Z_MAX;
 
-struct DpResult {                    // per problem, written by dp_finish_kernel
-    double value;                    // +inf: no plan
+struct DpJob {                       // a problem that has tables
+    uint64_t val_off;                // first entry of its two level buffers
+    uint64_t succ_off;               // first word of its successors: [stage][slot][type]
+    uint32_t config, index, layout, P;   // index = config * n_orders + order
+};
+
+struct DpResult {                    // per problem that has a plan, written by dp_finish_kernel
     double t_iter, cost;             // the simulator's figures for the plan (stage order)
     uint64_t peak_mem;
     uint32_t status, _pad;
@@ -79,8 +92,9 @@ struct DpTabLayout {
 };
 
 __global__ void __launch_bounds__(DP_THREADS)
-dp_tables_kernel(const unsigned char* __restrict__ blob, SpaceDesc sp, uint32_t n_config, DpTabLayout lay,
-                 double* __restrict__ tabs) {
+dp_tables_kernel(const unsigned char* __restrict__ blob, SpaceDesc sp, uint32_t n_config, uint32_t n_orders, DpTabLayout lay,
+                 const uint8_t* __restrict__ wanted /* [n_config], null: all */, double* __restrict__ tabs,
+                 double* __restrict__ value /* [n_config * n_orders]: +inf, no plan so far */) {
     __shared__ uint64_t s_params[SAILOR_P_MAX];
     __shared__ uint32_t s_ok[SAILOR_P_MAX];
     TabView v;
@@ -89,6 +103,8 @@ dp_tables_kernel(const unsigned char* __restrict__ blob, SpaceDesc sp, uint32_t 
     const uint32_t T = h->T, R = h->R, tid = threadIdx.x;
     for (uint32_t c = blockIdx.x; c < n_config; c += gridDim.x) {
         __syncthreads();
+        for (uint32_t q = tid; q < n_orders; q += DP_THREADS) value[(size_t)c * n_orders + q] = make_inf();
+        if (wanted && !wanted[c]) continue;
         const Config k = config_of(sp, c);
         double* tab = tabs + (size_t)c * lay.stride();
         const uint32_t tp = h->tp_values[k.tpi];
@@ -131,400 +147,205 @@ dp_tables_kernel(const unsigned char* __restrict__ blob, SpaceDesc sp, uint32_t 
     }
 }
 
-// ---- the index of a count vector inside a slice -------------------------------------------------------
+// ---- layouts -------------------------------------------------------------------------------------------
 //
-// Compact index of zone position zp: the counted types j = 0 .. m-1 (ascending type) have caps c_j.  With
-// W[j][s] = number of (u_j .. u_{m-1}) within the caps that add up to at most s, and V[j][s] = W[j][0] + .. +
-// W[j][s], the rank of u in lexicographic order is sum_j (V[j+1][s_j] - V[j+1][s_j - u_j]), s_0 = P,
-// s_{j+1} = s_j - u_j.  The table holds V[j][s] for j = 0 .. m, s = 0 .. P, row after row.
+// With W[j][s] as above, the vectors with exactly `s` stages of the types from j on whose first count is below x are
+// W[j + 1][s] - W[j + 1][s - x] many, and the vectors of sum s start behind the W[0][s - 1] with a smaller sum.
 
-// One digit of an unranking: the count x of a type, given the rank r among the vectors that agree on the types
-// before it and have s stages left for this type and the later ones.  `row` = V[j + 1][.] of the type's successor:
-// below(x) = row[s] - row[s - x] vectors start with a smaller count, and x is the largest count <= lim with
-// below(x) <= r.  After the last counted type nothing varies (V = s + 1), so below(x) = x there; elsewhere below is
-// non-decreasing in x and a bisection finds x.
-__device__ __forceinline__ void dp_digit(const uint32_t* __restrict__ row, uint32_t s, uint32_t lim, uint32_t r, bool last,
-                                         uint32_t& x, uint32_t& below) {
-    if (last) {
-        x = min(lim, r);
-        below = x;
-        return;
-    }
-    const uint32_t top = row[s];
-    uint32_t lo = 0, hi = lim;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi + 1) >> 1;                 // 1 <= mid <= lim <= s
-        if (top - row[s - mid] <= r) lo = mid; else hi = mid - 1;
-    }
-    x = lo;
-    below = lo ? top - row[s - lo] : 0u;
-}
+struct DpLayoutParams {
+    const DpLayout* layouts;
+    const uint32_t* blk_prefix;      // [n_layouts + 1] blocks before each layout
+    const uint32_t* wtab;
+    uint32_t* nxt;                   // [vector][TM]
+    uint32_t n_layouts, T;
+};
 
-// counts of a slice index: u[t] for counted types, 0 for the others.  Returns false, possibly before all counts
-// are known, as soon as they add up to more than `limit`.
-__device__ __forceinline__ bool dp_counts(const DpProblem& pb, const uint32_t* __restrict__ vtabs, uint32_t zp, uint32_t T,
-                                          uint32_t ui, uint32_t (&u)[SAILOR_T_MAX], uint32_t limit) {
-    uint32_t total = 0;
-    if (pb.vt_off[zp] == DP_DENSE) {
-        uint32_t rem = ui;
-#pragma unroll
-        for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) {
-            u[t] = 0;
-            if (t < T && pb.stride[zp][t]) {
-                const uint32_t q = (uint32_t)__umul64hi((uint64_t)rem, pb.magic[zp][t]);
-                u[t] = rem - q * (pb.cap[zp][t] + 1u);
-                rem = q;
-                total += u[t];
-            }
+template <uint32_t TM>
+__global__ void __launch_bounds__(DP_THREADS) dp_layout_kernel(const __grid_constant__ DpLayoutParams lp) {
+    __shared__ DpLayout L;
+    const uint32_t tid = threadIdx.x, T = lp.T;
+    uint32_t which = 0;
+    {
+        uint32_t hi = lp.n_layouts;
+        while (hi - which > 1) {
+            const uint32_t mid = (which + hi) >> 1;
+            if (lp.blk_prefix[mid] <= blockIdx.x) which = mid; else hi = mid;
         }
-        return total <= limit;
-    } else {
-        const uint32_t* vt = vtabs + pb.vt_off[zp];
-        const uint32_t w = pb.P + 1;
-        uint32_t r = ui, s = pb.P, j = 0;
-#pragma unroll
-        for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) {
-            u[t] = 0;
-            if (t < T && pb.stride[zp][t]) {
-                const uint32_t lim = min((uint32_t)pb.cap[zp][t], s);
-                uint32_t x, below;                               // `below`: vectors that start with a count smaller than x
-                dp_digit(vt + (j + 1) * w, s, lim, r, j + 1 == pb.n_counted[zp], x, below);
-                u[t] = x;
-                total += x;
-                if (total > limit) return false;                 // the walks of the remaining types are not needed
-                r -= below;
-                s -= x;
-                ++j;
-            }
-        }
-        return true;
     }
-}
-
-// The r-th count vector (lexicographic) among those within the caps that add up to at most `budget`.
-__device__ __forceinline__ void dp_unrank(const DpProblem& pb, const uint32_t* __restrict__ vt, uint32_t zp, uint32_t T,
-                                          uint32_t r, uint32_t budget, uint32_t (&u)[SAILOR_T_MAX]) {
-    const uint32_t w = pb.P + 1;
-    uint32_t s = budget, j = 0;
+    for (uint32_t x = tid; x < sizeof(DpLayout) / 4; x += DP_THREADS)
+        reinterpret_cast<uint32_t*>(&L)[x] = reinterpret_cast<const uint32_t*>(lp.layouts + which)[x];
+    __syncthreads();
+    const uint32_t v = (blockIdx.x - lp.blk_prefix[which]) * DP_THREADS + tid;
+    if (v >= L.vec_base[L.nz]) return;
+    uint32_t zp = 0;
+    while (v >= L.vec_base[zp + 1]) ++zp;
+    const uint32_t w = L.P + 1, base = L.vec_base[zp], e = v - base, most = L.sum_max[zp], counted = L.counted[zp];
+    const uint32_t* W = lp.wtab + L.w_off[zp];
+    uint32_t s = 0;                                          // the sum: the smallest with W[0][s] > e
+    for (uint32_t hi = most; s < hi;) {
+        const uint32_t mid = (s + hi) >> 1;
+        if (W[mid] > e) hi = mid; else s = mid + 1;
+    }
+    uint32_t u[SAILOR_T_MAX], r = e - (s ? W[s - 1] : 0u), rem = s, j = 0;
 #pragma unroll
     for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) {
         u[t] = 0;
-        if (t < T && pb.stride[zp][t]) {
-            const uint32_t lim = min((uint32_t)pb.cap[zp][t], s);
-            uint32_t x, below;
-            dp_digit(vt + (j + 1) * w, s, lim, r, j + 1 == pb.n_counted[zp], x, below);
-            u[t] = x;
-            r -= below;
-            s -= x;
+        if ((counted >> t) & 1u) {
+            const uint32_t* row = W + (j + 1) * w;
+            const uint32_t top = row[rem];
+            uint32_t lo = 0, hi = min((uint32_t)L.cap[zp][t], rem);
+            while (lo < hi) {                                // the largest count that leaves at most r vectors before it
+                const uint32_t mid = (lo + hi + 1) >> 1;
+                if (top - row[rem - mid] <= r) lo = mid; else hi = mid - 1;
+            }
+            r -= top - row[rem - lo];
+            u[t] = lo;
+            rem -= lo;
             ++j;
         }
     }
-}
-
-// slice index of the count vector u with one more stage of type `plus_one` (compact index only)
-__device__ __forceinline__ uint32_t dp_rank(const DpProblem& pb, const uint32_t* __restrict__ vtabs, uint32_t zp, uint32_t T,
-                                            const uint32_t (&u)[SAILOR_T_MAX], uint32_t plus_one) {
-    const uint32_t* vt = vtabs + pb.vt_off[zp];
-    const uint32_t w = pb.P + 1;
-    uint32_t r = 0, s = pb.P, j = 0;
+    uint32_t out[TM];
 #pragma unroll
-    for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) {
-        if (t < T && pb.stride[zp][t]) {
-            const uint32_t x = u[t] + (t == plus_one ? 1u : 0u);
-            const uint32_t* row = vt + (j + 1) * w;
-            if (x) r += row[s] - row[s - x];                     // the caller keeps the counts within P in total
-            s -= x;
-            ++j;
+    for (uint32_t g = 0; g < TM; ++g) {
+        out[g] = DP_NO_VEC;
+        if (g >= T) continue;
+        if ((counted >> g) & 1u) {
+            if (u[g] < L.cap[zp][g] && s < most) {
+                uint32_t at = W[s], left = s + 1, q = 0;
+#pragma unroll
+                for (uint32_t t = 0; t < SAILOR_T_MAX; ++t)
+                    if ((counted >> t) & 1u) {
+                        const uint32_t x = u[t] + (t == g ? 1u : 0u);
+                        const uint32_t* row = W + (q + 1) * w;
+                        at += row[left] - row[left - x];
+                        left -= x;
+                        ++q;
+                    }
+                out[g] = base + at;
+            }
+            if (u[g]) out[g] |= DP_SELF;
+        } else if (L.cap[zp][g]) {
+            out[g] = v | DP_SELF;                            // room for every stage: not counted
         }
     }
-    return r;
-}
-
-// Where does a stage of type g2 go when the previous stage sits at position zp with counts u (slice index ui)?
-// Returns the position (DP_NONE: nowhere) and the entry index of the state that results.
-struct DpMove { uint32_t zp, entry; };
-
-__device__ __forceinline__ DpMove dp_move(const DpProblem& pb, const uint32_t* __restrict__ vtabs, uint32_t T, uint32_t zp,
-                                          uint32_t ui, const uint32_t (&u)[SAILOR_T_MAX], uint32_t g2) {
-    DpMove m;
-    const uint32_t cap = pb.cap[zp][g2];
-    uint32_t u_g2 = 0, placed = 0;
+    uint4* dst = reinterpret_cast<uint4*>(lp.nxt + (size_t)(L.nxt_off + v) * TM);
 #pragma unroll
-    for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) {
-        u_g2 = t == g2 ? u[t] : u_g2;
-        placed += u[t];
-    }
-    // first fit: this zone while it has room for one more stage of the type, else the next zone that has
-    const bool counted = pb.stride[zp][g2] != 0;
-    const bool here = counted ? u_g2 < cap : cap >= 1;           // not counted: room for every stage, or none at all
-    if (here) {
-        m.zp = zp;
-        uint32_t idx = ui;
-        if (counted) {
-            if (pb.vt_off[zp] == DP_DENSE) idx = ui + pb.stride[zp][g2];
-            else if (placed >= pb.P) { m.zp = DP_NONE; m.entry = 0; return m; }      // more than P stages: no such state
-            else idx = dp_rank(pb, vtabs, zp, T, u, g2);
-        }
-        m.entry = pb.zp_base[zp] + g2 * pb.S[zp] + idx;
-        return m;
-    }
-    const uint32_t p = pb.first_later[zp][g2];
-    m.zp = p;
-    m.entry = p == DP_NONE ? 0u : pb.zp_base[p] + g2 * pb.S[p] + pb.first_idx[p][g2];      // the new zone holds this stage only
-    return m;
+    for (uint32_t q = 0; q < TM / 4; ++q) dst[q] = make_uint4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
 }
+
+// ---- the stages ----------------------------------------------------------------------------------------
 
 struct DpLevelParams {
-    const DpProblem* problems;
-    const uint32_t* blk_problem;     // entries mode: block -> problem of the batch
-    const uint32_t* blk_first;       // entries mode: block -> first entry it covers
-    const uint32_t* blk_prefix;      // live mode: [n_active + 1] blocks before each problem of this launch
-    uint32_t n_active;               // live mode: problems of this launch (a prefix of the batch)
-    uint32_t per_thread;             // vector kernel: count vectors a thread takes, a block's width apart
+    const DpLayout* layouts;
+    const DpJob* jobs;
+    const uint32_t* live;
+    const uint32_t* nxt;
     const double* tabs;
-    const uint32_t* vtabs;           // rank tables of the compactly indexed zone positions
-    DpVal* val[2];                   // level buffers; stage i lives in val[(P - 1 - i) & 1]
-    uint8_t* choice;
+    DpVal* val[2];                   // level buffers [slot][type]; stage i lives in val[(P - 1 - i) & 1]
+    uint32_t* succ;                  // [stage][slot][type]: slot * T + type of the best next state
+    const uint32_t* blk_prefix;      // per-stage launches: [n_active + 1] blocks before each job of this launch
     DpTabLayout lay;
-    uint32_t T;
+    uint32_t T, n_active;
     uint32_t dist;                   // stage i = P - 1 - dist
 };
 
-// LIVE = false: a thread per table entry (block map over entries); entries no stage sequence can reach at this
-// stage leave early.  LIVE = true: a thread per count vector that stage i can have reached (at most i + 1 stages
-// in the zone), enumerated by rank with that budget through the positions' rank tables (block map over those).
-template <bool LIVE>
-__global__ void __launch_bounds__(DP_THREADS, 5) dp_level_kernel(const __grid_constant__ DpLevelParams lp) {
-    __shared__ DpProblem pb;
-    const uint32_t tid = threadIdx.x;
-    uint32_t which, first;
-    if (LIVE) {                                              // the problem whose blocks include this one (all threads alike)
-        uint32_t lo = 0, hi = lp.n_active;
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (lp.blk_prefix[mid] <= blockIdx.x) lo = mid; else hi = mid;
-        }
-        which = lo;
-        first = (blockIdx.x - lp.blk_prefix[lo]) * DP_THREADS;
-    } else {
-        which = lp.blk_problem[blockIdx.x];
-        first = lp.blk_first[blockIdx.x];
-    }
-    {
-        const DpProblem* src = lp.problems + which;
-        for (uint32_t x = tid; x < sizeof(DpProblem) / 4; x += DP_THREADS)
-            reinterpret_cast<uint32_t*>(&pb)[x] = reinterpret_cast<const uint32_t*>(src)[x];
-    }
-    __syncthreads();
-    const uint32_t T = lp.T, P = pb.P, i = P - 1 - lp.dist;
-    const double* tab = lp.tabs + (size_t)pb.config * lp.lay.stride();
-    const uint32_t* okv = reinterpret_cast<const uint32_t*>(tab + lp.lay.off_ok());
-    const double nb = (double)*reinterpret_cast<const uint64_t*>(tab + lp.lay.off_nb());
-    uint32_t zp = 0, g = 0, ui, e;
-    uint32_t u[SAILOR_T_MAX];
-    uint32_t S;
-    if (LIVE) {
-        // live index -> (zone position, type, r-th count vector with at most i + 1 stages) -> its table entry
-        uint32_t l = first + tid;
-        const uint32_t budget = i + 1;                       // <= P
-        uint32_t wz = 0;
-        for (;; ++zp) {
-            if (zp == pb.nz) return;                             // past the last live vector of this stage
-            wz = 1;
-            if (pb.rank_off[zp] != DP_DENSE) {
-                const uint32_t* row0 = lp.vtabs + pb.rank_off[zp];   // V[0][s]: vectors of all counted types up to sum s
-                wz = row0[budget] - row0[budget - 1];
-            }
-            if (l < T * wz) break;
-            l -= T * wz;
-        }
-        while (l >= wz) { l -= wz; ++g; }
-        S = pb.S[zp];
-        if (pb.rank_off[zp] != DP_DENSE) dp_unrank(pb, lp.vtabs + pb.rank_off[zp], zp, T, l, budget, u);
-        else {
-#pragma unroll
-            for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) u[t] = 0;
-        }
-        if (pb.vt_off[zp] != DP_DENSE) ui = dp_rank(pb, lp.vtabs, zp, T, u, 0xffffffffu);
-        else {
-            ui = 0;
-#pragma unroll
-            for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) ui += (t < T) ? u[t] * pb.stride[zp][t] : 0u;
-        }
-        e = pb.zp_base[zp] + g * S + ui;
-    } else {
-        e = first + tid;
-        if (e >= pb.n_lvl) return;
-        // entry -> (zone position, type, counts); no division by run-time values: the slices of a position are
-        // stepped through, and the counts come off by reciprocal multiplication or by a walk through the rank table
-        while (zp + 1 < pb.nz && e >= pb.zp_base[zp + 1]) ++zp;
-        ui = e - pb.zp_base[zp];
-        S = pb.S[zp];
-        while (ui >= S) { ui -= S; ++g; }
-        // stage i is at most the (i+1)-th stage of its zone: entries that count more are never reached, and
-        // since a move raises the count by one per stage, no entry that passes this test ever reads one that fails it
-        if (!dp_counts(pb, lp.vtabs, zp, T, ui, u, i + 1)) return;
-    }
-    DpVal* cur = lp.val[lp.dist & 1] + pb.val_off;
-    const DpVal* nxt = lp.val[(lp.dist & 1) ^ 1] + pb.val_off;
-    uint8_t* choice = lp.choice + pb.choice_off + (size_t)i * pb.n_lvl;
-    DpVal best;
-    best.sum = make_inf(); best.mx = best.sy = best.up = 0.0;
-    uint8_t pick = DP_NONE;
-    // a state holds stage i itself: its type must be usable there and, when counted, counted at least once
-    uint32_t u_g = 0;
-#pragma unroll
-    for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) u_g = t == g ? u[t] : u_g;
-    const bool self = ((okv[i] >> g) & 1u) && pb.cap[zp][g] >= 1 && (pb.stride[zp][g] == 0 || u_g >= 1);
-    if (self) {
-        const uint32_t d = pb.zone[zp] * T + g;
-        const double fb = tab[lp.lay.off_fb() + i * T + g], upd = tab[lp.lay.off_upd() + i * T + g];
-        const double sync = tab[lp.lay.off_sync() + (size_t)i * lp.lay.R + d];
-        if (lp.dist == 0) {                                      // the last stage sends nothing
-            best.sum = fb; best.mx = fb; best.sy = sync; best.up = upd;
-        } else {
-            double best_v = make_inf();
-            const uint32_t ok_next = okv[i + 1];
-#pragma unroll
-            for (uint32_t g2 = 0; g2 < SAILOR_T_MAX; ++g2) {
-                if (g2 >= T) break;
-                if (!((ok_next >> g2) & 1u)) continue;
-                const DpMove mv = dp_move(pb, lp.vtabs, T, zp, ui, u, g2);
-                if (mv.zp == DP_NONE) continue;
-                const uint32_t zp2 = mv.zp, entry = mv.entry;
-                const DpVal n = nxt[entry];
-                if (!(n.sum < make_inf())) continue;
-                const uint32_t d2 = pb.zone[zp2] * T + g2;
-                const double t = add_rn(fb, tab[lp.lay.off_c2x() + (size_t)d2 * lp.lay.R + d]);
-                DpVal c;
-                c.sum = add_rn(t, n.sum);
-                c.mx = dmax(t, n.mx);
-                c.sy = dmax(sync, n.sy);
-                c.up = dmax(upd, n.up);
-                const double val = add_rn(add_rn(add_rn(c.sum, mul_rn(nb, c.mx)), c.sy), c.up);
-                if (pick == DP_NONE || val < best_v) { best = c; best_v = val; pick = (uint8_t)g2; }
-            }
-        }
-    }
-    cur[e] = best;
-    choice[e] = pick;
-}
-
-// A thread per reachable count vector, all types of stage i at once (TM >= T types).  The T entries that share a
-// count vector share its unranking, its table index and, for every type of the next stage, the moved vector's entry:
-// those are formed once, the next stage's values are gathered together, and only the T x T combinations remain per
-// type.  Same arithmetic per (type, next type) pair and the same order of the next types as dp_level_kernel.
-
-constexpr uint32_t DP_VEC_PER_THREAD = 4;       // in launches large enough to fill the GPU several times over
-
-// The work of one stage (distance `dist` from the last) of the problem `pb` for the count vectors first + tid,
-// first + DP_THREADS + tid, ... (`rounds` of them): see dp_level_vec_kernel.  `vtabs` addresses the problem's rank
-// tables by their offsets from the start of all tables.
+// Stage i of a job for the vector in `slot` of the stage, all its types at once (TM >= T types).  `here` and `then` are
+// the live rows of stages i and i + 1 (shared memory).
 template <uint32_t TM>
-__device__ __forceinline__ void dp_vec_level(const DpLevelParams& lp, const DpProblem& pb, const uint32_t* vtabs, uint32_t dist,
-                                             uint32_t first, uint32_t rounds) {
-    const uint32_t tid = threadIdx.x;
-    const uint32_t T = lp.T, P = pb.P, i = P - 1 - dist;
-    const double* tab = lp.tabs + (size_t)pb.config * lp.lay.stride();
+__device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayout& L, const DpJob& job, const uint32_t* here,
+                                          const uint32_t* then, uint32_t i, uint32_t slot) {
+    const uint32_t T = lp.T, dist = job.P - 1 - i;
+    const double* tab = lp.tabs + (size_t)job.config * lp.lay.stride();
     const uint32_t* okv = reinterpret_cast<const uint32_t*>(tab + lp.lay.off_ok());
     const double nb = (double)*reinterpret_cast<const uint64_t*>(tab + lp.lay.off_nb());
-    DpVal* cur = lp.val[dist & 1] + pb.val_off;
-    const DpVal* nxt = lp.val[(dist & 1) ^ 1] + pb.val_off;
-    uint8_t* choice = lp.choice + pb.choice_off + (size_t)i * pb.n_lvl;
-    const uint32_t budget = i + 1;                           // <= P
-    const uint32_t ok_here = okv[i];
-    // several vectors per thread, a block's width apart: the block's set-up (its problem, the rank tables) is paid once
-    for (uint32_t round = 0; round < rounds; ++round) {
-        uint32_t zp = 0, ui;
-        uint32_t u[SAILOR_T_MAX];
-        uint32_t l = first + round * DP_THREADS + tid;
-        for (;; ++zp) {
-            if (zp == pb.nz) return;                             // past the last reachable vector (later rounds too)
-            uint32_t wz = 1;
-            if (pb.rank_off[zp] != DP_DENSE) {
-                const uint32_t* row0 = vtabs + pb.rank_off[zp];
-                wz = row0[budget] - row0[budget - 1];
-            }
-            if (l < wz) break;
-            l -= wz;
-        }
-        const uint32_t S = pb.S[zp];
-        if (pb.rank_off[zp] != DP_DENSE) dp_unrank(pb, vtabs + pb.rank_off[zp], zp, T, l, budget, u);
-        else {
+    uint32_t zp = 0;
+    while (zp + 1 < L.nz && here[3 + 2 * (zp + 1)] <= slot) ++zp;
+    const uint32_t v = here[2 + 2 * zp] + (slot - here[3 + 2 * zp]);
+    uint32_t nx[TM];
+    {
+        const uint4* row = reinterpret_cast<const uint4*>(lp.nxt + (size_t)(L.nxt_off + v) * TM);
 #pragma unroll
-            for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) u[t] = 0;
+        for (uint32_t q = 0; q < TM / 4; ++q) {
+            const uint4 x = __ldg(row + q);
+            nx[4 * q] = x.x; nx[4 * q + 1] = x.y; nx[4 * q + 2] = x.z; nx[4 * q + 3] = x.w;
         }
-        if (pb.vt_off[zp] != DP_DENSE) ui = dp_rank(pb, vtabs, zp, T, u, 0xffffffffu);
-        else {
-            ui = 0;
+    }
+    // what follows a stage of each type g2: the state it leads to (the same for every type of stage i) and its value
+    const DpVal* nxt = lp.val[(dist & 1) ^ 1] + job.val_off;
+    DpVal n[TM];
+    uint32_t code[TM], d2[TM];
 #pragma unroll
-            for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) ui += (t < T) ? u[t] * pb.stride[zp][t] : 0u;
-        }
-        const uint32_t e0 = pb.zp_base[zp] + ui;
-        // what follows a stage of each type g2: the entry it leads to (the same for every type of stage i) and its value
-        DpVal n[TM];
-        uint32_t d2v[TM];
+    for (uint32_t g2 = 0; g2 < TM; ++g2) {
+        code[g2] = DP_NO_STATE;
+        d2[g2] = 0;
+        n[g2].sum = make_inf(); n[g2].mx = n[g2].sy = n[g2].up = 0.0;
+    }
+    if (dist != 0) {
+        const uint32_t ok_next = okv[i + 1];
 #pragma unroll
         for (uint32_t g2 = 0; g2 < TM; ++g2) {
-            d2v[g2] = DP_NONE;
-            n[g2].sum = make_inf(); n[g2].mx = n[g2].sy = n[g2].up = 0.0;
+            if (g2 >= T || !((ok_next >> g2) & 1u)) continue;
+            // first fit: this position while it has room for one more stage of the type, else the next that has
+            uint32_t zp2 = zp, id = nx[g2] & DP_NO_VEC;
+            if (id == DP_NO_VEC) {
+                zp2 = L.first_later[zp][g2];
+                if (zp2 == DP_NONE) continue;
+                id = L.first_vec[zp2][g2];
+            }
+            const uint32_t slot2 = then[3 + 2 * zp2] + (id - then[2 + 2 * zp2]);
+            if (slot2 >= then[0]) continue;                  // (a move of a live state leads to a live state)
+            code[g2] = slot2 * T + g2;
+            d2[g2] = L.zone[zp2] * T + g2;
+            n[g2] = nxt[code[g2]];
         }
-        if (dist != 0) {
-            const uint32_t ok_next = okv[i + 1];
+    }
+    const uint32_t ok_here = okv[i];
+    DpVal* cur = lp.val[dist & 1] + job.val_off + (size_t)slot * T;
+    uint32_t* succ = lp.succ + job.succ_off + (size_t)(here[1] + slot) * T;
+#pragma unroll
+    for (uint32_t g = 0; g < TM; ++g) {
+        if (g >= T) break;
+        // a state holds stage i itself: its type must fit the stage and, when counted, be counted at least once
+        if (!((ok_here >> g) & 1u) || !(nx[g] & DP_SELF)) continue;
+        const uint32_t d = L.zone[zp] * T + g;
+        const double fb = tab[lp.lay.off_fb() + i * T + g], upd = tab[lp.lay.off_upd() + i * T + g];
+        const double sync = tab[lp.lay.off_sync() + (size_t)i * lp.lay.R + d];
+        DpVal best;
+        uint32_t pick = DP_NO_STATE;
+        if (dist == 0) {                                     // the last stage sends nothing
+            best.sum = fb; best.mx = fb; best.sy = sync; best.up = upd;
+        } else {
+            best.sum = make_inf(); best.mx = best.sy = best.up = 0.0;
+            double best_v = make_inf();
 #pragma unroll
             for (uint32_t g2 = 0; g2 < TM; ++g2) {
-                if (g2 >= T || !((ok_next >> g2) & 1u)) continue;
-                const DpMove mv = dp_move(pb, vtabs, T, zp, ui, u, g2);
-                if (mv.zp == DP_NONE) continue;
-                n[g2] = nxt[mv.entry];
-                d2v[g2] = pb.zone[mv.zp] * T + g2;
+                if (code[g2] == DP_NO_STATE || !(n[g2].sum < make_inf())) continue;
+                const double t = add_rn(fb, tab[lp.lay.off_c2x() + (size_t)d2[g2] * lp.lay.R + d]);
+                DpVal c;
+                c.sum = add_rn(t, n[g2].sum);
+                c.mx = dmax(t, n[g2].mx);
+                c.sy = dmax(sync, n[g2].sy);
+                c.up = dmax(upd, n[g2].up);
+                const double val = add_rn(add_rn(add_rn(c.sum, mul_rn(nb, c.mx)), c.sy), c.up);
+                if (pick == DP_NO_STATE || val < best_v) { best = c; best_v = val; pick = code[g2]; }
             }
         }
-#pragma unroll
-        for (uint32_t g = 0; g < TM; ++g) {
-            if (g >= T) break;
-            DpVal best;
-            best.sum = make_inf(); best.mx = best.sy = best.up = 0.0;
-            uint8_t pick = DP_NONE;
-            // a state holds stage i itself: its type must be usable there and, when counted, counted at least once
-            const bool self = ((ok_here >> g) & 1u) && pb.cap[zp][g] >= 1 && (pb.stride[zp][g] == 0 || u[g] >= 1);
-            if (self) {
-                const uint32_t d = pb.zone[zp] * T + g;
-                const double fb = tab[lp.lay.off_fb() + i * T + g], upd = tab[lp.lay.off_upd() + i * T + g];
-                const double sync = tab[lp.lay.off_sync() + (size_t)i * lp.lay.R + d];
-                if (dist == 0) {                                  // the last stage sends nothing
-                    best.sum = fb; best.mx = fb; best.sy = sync; best.up = upd;
-                } else {
-                    double best_v = make_inf();
-#pragma unroll
-                    for (uint32_t g2 = 0; g2 < TM; ++g2) {
-                        if (d2v[g2] == DP_NONE || !(n[g2].sum < make_inf())) continue;
-                        const double t = add_rn(fb, tab[lp.lay.off_c2x() + (size_t)d2v[g2] * lp.lay.R + d]);
-                        DpVal c;
-                        c.sum = add_rn(t, n[g2].sum);
-                        c.mx = dmax(t, n[g2].mx);
-                        c.sy = dmax(sync, n[g2].sy);
-                        c.up = dmax(upd, n[g2].up);
-                        const double val = add_rn(add_rn(add_rn(c.sum, mul_rn(nb, c.mx)), c.sy), c.up);
-                        if (pick == DP_NONE || val < best_v) { best = c; best_v = val; pick = (uint8_t)g2; }
-                    }
-                }
-            }
-            cur[e0 + g * S] = best;
-            choice[e0 + g * S] = pick;
-        }
+        cur[g] = best;
+        succ[g] = pick;
     }
 }
 
+// One stage (a distance from the last) of every job of the launch; a thread per live vector.
 template <uint32_t TM>
-__global__ void __launch_bounds__(DP_THREADS, TM <= 4 ? 3 : 2) dp_level_vec_kernel(const __grid_constant__ DpLevelParams lp) {
-    extern __shared__ uint32_t s_vt[];                       // the problem's rank tables
-    __shared__ DpProblem pb;
+__global__ void __launch_bounds__(DP_THREADS, TM <= 4 ? 3 : 2) dp_level_kernel(const __grid_constant__ DpLevelParams lp) {
+    __shared__ DpLayout L;
+    __shared__ DpJob job;
+    __shared__ uint32_t rows[2][DP_LIVE_WORDS_MAX];
     __shared__ uint32_t s_lo;
     const uint32_t tid = threadIdx.x;
     uint32_t which = 0;
-    // the problem whose blocks include this one: a search with DP_THREADS probes per round instead of two, so that
-    // a block waits for one or two loads, not for a chain of them
+    // the job whose blocks include this one: a search with DP_THREADS probes per round, so that a block waits for one or
+    // two loads, not for a chain of them
     {
         uint32_t lo = 0, n = lp.n_active;                    // invariant: prefix[lo] <= block < prefix[lo + n]
         while (n > 1) {
@@ -539,97 +360,107 @@ __global__ void __launch_bounds__(DP_THREADS, TM <= 4 ? 3 : 2) dp_level_vec_kern
         }
         which = lo;
     }
-    const uint32_t first = (blockIdx.x - lp.blk_prefix[which]) * (DP_THREADS * lp.per_thread);
-    {
-        const DpProblem* src = lp.problems + which;
-        for (uint32_t x = tid; x < sizeof(DpProblem) / 4; x += DP_THREADS)
-            reinterpret_cast<uint32_t*>(&pb)[x] = reinterpret_cast<const uint32_t*>(src)[x];
+    const uint32_t slot = (blockIdx.x - lp.blk_prefix[which]) * DP_THREADS + tid;
+    const DpJob& gj = lp.jobs[which];
+    const DpLayout* gl = lp.layouts + gj.layout;
+    const uint32_t i = gj.P - 1 - lp.dist;
+    if (tid < sizeof(DpJob) / 8) reinterpret_cast<uint64_t*>(&job)[tid] = reinterpret_cast<const uint64_t*>(&gj)[tid];
+    for (uint32_t x = tid; x < sizeof(DpLayout) / 4; x += DP_THREADS)
+        reinterpret_cast<uint32_t*>(&L)[x] = reinterpret_cast<const uint32_t*>(gl)[x];
+    const uint32_t words = dp_live_words(gl->nz);
+    if (tid < words) {
+        const uint32_t* row = lp.live + gl->live_off + (size_t)i * words + tid;
+        rows[0][tid] = row[0];
+        rows[1][tid] = lp.dist ? row[words] : 0u;
     }
     __syncthreads();
-    for (uint32_t x = tid; x < pb.vt_len; x += DP_THREADS) s_vt[x] = lp.vtabs[pb.vt_lo + x];
-    __syncthreads();
-    // offsets into the rank tables count from the start of all tables: the staged copy is addressed the same way
-    const uint32_t* const vtabs = s_vt - pb.vt_lo;
-    dp_vec_level<TM>(lp, pb, vtabs, lp.dist, first, lp.per_thread);
+    if (slot < rows[0][0]) dp_vector<TM>(lp, L, job, rows[0], rows[1], i, slot);
 }
 
-// Small problems: a block takes one problem through all its stages, from the last to the first, with a barrier
-// between stages (a stage reads only what the same block wrote for the stage after it): one launch per batch
-// instead of one per stage.
+// Small problems: a block takes one job through all its stages, from the last to the first, with a barrier between
+// stages (a stage reads only what the same block wrote for the stage after it).
 template <uint32_t TM>
 __global__ void __launch_bounds__(DP_THREADS, TM <= 4 ? 3 : 2) dp_problem_kernel(const __grid_constant__ DpLevelParams lp) {
-    extern __shared__ uint32_t s_vt[];                       // the problem's rank tables
-    __shared__ DpProblem pb;
+    __shared__ DpLayout L;
+    __shared__ DpJob job;
+    __shared__ uint32_t rows[2][DP_LIVE_WORDS_MAX];
     const uint32_t tid = threadIdx.x;
-    {
-        const DpProblem* src = lp.problems + blockIdx.x;
-        for (uint32_t x = tid; x < sizeof(DpProblem) / 4; x += DP_THREADS)
-            reinterpret_cast<uint32_t*>(&pb)[x] = reinterpret_cast<const uint32_t*>(src)[x];
-    }
+    const DpJob& gj = lp.jobs[blockIdx.x];
+    const DpLayout* gl = lp.layouts + gj.layout;
+    if (tid < sizeof(DpJob) / 8) reinterpret_cast<uint64_t*>(&job)[tid] = reinterpret_cast<const uint64_t*>(&gj)[tid];
+    for (uint32_t x = tid; x < sizeof(DpLayout) / 4; x += DP_THREADS)
+        reinterpret_cast<uint32_t*>(&L)[x] = reinterpret_cast<const uint32_t*>(gl)[x];
     __syncthreads();
-    for (uint32_t x = tid; x < pb.vt_len; x += DP_THREADS) s_vt[x] = lp.vtabs[pb.vt_lo + x];
-    __syncthreads();
-    const uint32_t* const vtabs = s_vt - pb.vt_lo;
-    for (uint32_t dist = 0; dist < pb.P; ++dist) {
-        const uint32_t budget = pb.P - dist;                 // stage i = P - 1 - dist has at most i + 1 stages behind it
-        uint32_t vectors = 0;
-        for (uint32_t zp = 0; zp < pb.nz; ++zp) {
-            uint32_t wz = 1;
-            if (pb.rank_off[zp] != DP_DENSE) {
-                const uint32_t* row0 = vtabs + pb.rank_off[zp];
-                wz = row0[budget] - row0[budget - 1];
-            }
-            vectors += wz;
-        }
-        dp_vec_level<TM>(lp, pb, vtabs, dist, 0, (vectors + DP_THREADS - 1) / DP_THREADS);
+    const uint32_t words = dp_live_words(L.nz);
+    for (uint32_t dist = 0; dist < job.P; ++dist) {
+        const uint32_t i = job.P - 1 - dist;
+        uint32_t* here = rows[dist & 1];
+        if (tid < words) here[tid] = lp.live[L.live_off + (size_t)i * words + tid];
+        __syncthreads();                                     // the row, and the values of the stage after this one
+        for (uint32_t slot = tid; slot < here[0]; slot += DP_THREADS)
+            dp_vector<TM>(lp, L, job, here, rows[(dist & 1) ^ 1], i, slot);
         __syncthreads();
     }
 }
 
-// Stage 0 and the walk through the kept choices: one thread per problem.
+// Stage 0 and the walk through the kept successors: one thread per job.  The walk is a chain of one dependent load per
+// stage (a successor is the next state's own address).
 struct DpFinishParams {
     const unsigned char* blob;
     const uint16_t* avail;
     SpaceDesc sp;
-    const DpProblem* problems;
+    const DpLayout* layouts;
+    const DpJob* jobs;
+    const uint32_t* live;
     const double* tabs;
-    const uint32_t* vtabs;
     const DpVal* val[2];
-    const uint8_t* choice;
+    const uint32_t* succ;
+    double* value;                   // indexed by problem index
     DpResult* results;               // indexed by problem index
     DpTabLayout lay;
-    uint32_t n_problems, T;
+    uint32_t n_jobs, T;
 };
 
-__global__ void __launch_bounds__(128) dp_finish_kernel(const __grid_constant__ DpFinishParams fp) {
+constexpr int DP_FINISH_THREADS = 32;
+
+__global__ void __launch_bounds__(DP_FINISH_THREADS) dp_finish_kernel(const __grid_constant__ DpFinishParams fp) {
     const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= fp.n_problems) return;
-    const DpProblem& pb = fp.problems[x];
-    DpResult& out = fp.results[pb.index];
-    const uint32_t T = fp.T, P = pb.P;
-    const double* tab = fp.tabs + (size_t)pb.config * fp.lay.stride();
+    if (x >= fp.n_jobs) return;
+    const DpJob job = fp.jobs[x];
+    const DpLayout& L = fp.layouts[job.layout];
+    DpResult& out = fp.results[job.index];
+    const uint32_t T = fp.T, P = job.P, nz = L.nz, words = dp_live_words(nz);
+    const uint32_t* live = fp.live + L.live_off;
+    const double* tab = fp.tabs + (size_t)job.config * fp.lay.stride();
     const uint32_t* okv = reinterpret_cast<const uint32_t*>(tab + fp.lay.off_ok());
     const double nb = (double)*reinterpret_cast<const uint64_t*>(tab + fp.lay.off_nb());
-    const DpVal* lvl0 = fp.val[(P - 1) & 1] + pb.val_off;
+    const DpVal* lvl0 = fp.val[(P - 1) & 1] + job.val_off;
     double best_v = make_inf();
-    uint32_t g = DP_NONE, zp = 0, entry = 0;
+    uint32_t code = DP_NO_STATE;
     for (uint32_t g0 = 0; g0 < T; ++g0) {                    // stage 0 by first fit from the first zone of the order
         if (!((okv[0] >> g0) & 1u)) continue;
-        const uint32_t p = pb.cap[0][g0] >= 1 ? 0u : pb.first_later[0][g0];
+        const uint32_t p = L.cap[0][g0] >= 1 ? 0u : L.first_later[0][g0];
         if (p == DP_NONE) continue;
-        const uint32_t e = pb.zp_base[p] + g0 * pb.S[p] + pb.first_idx[p][g0];
-        const DpVal v = lvl0[e];
+        const uint32_t slot = live[3 + 2 * p] + (L.first_vec[p][g0] - live[2 + 2 * p]);
+        if (slot >= live[0]) continue;
+        const DpVal v = lvl0[slot * T + g0];
         if (!(v.sum < make_inf())) continue;
         const double val = add_rn(add_rn(add_rn(v.sum, mul_rn(nb, v.mx)), v.sy), v.up);
-        if (g == DP_NONE || val < best_v) { best_v = val; g = g0; zp = p; entry = e; }
+        if (code == DP_NO_STATE || val < best_v) { best_v = val; code = slot * T + g0; }
     }
-    out.value = best_v;
-    if (g == DP_NONE) return;
-    const Config k = config_of(fp.sp, pb.config);
+    if (code == DP_NO_STATE) return;                         // the value stays at "no plan"
+    fp.value[job.index] = best_v;
+    const Config k = config_of(fp.sp, job.config);
     sailor_run runs[SAILOR_P_MAX];
     uint32_t n_runs = 0;
+    const uint32_t* succ = fp.succ + job.succ_off;
     for (uint32_t i = 0; i < P; ++i) {
-        const uint8_t z = pb.zone[zp];
+        const uint32_t* row = live + (size_t)i * words;
+        const uint32_t now = code, slot = now / T, g = now - slot * T;
+        if (i + 1 < P) code = succ[(size_t)row[1] * T + now];
+        uint32_t zp = 0;
+        while (zp + 1 < nz && row[3 + 2 * (zp + 1)] <= slot) ++zp;
+        const uint8_t z = L.zone[zp];
         out.type[i] = (uint8_t)g;
         out.zone[i] = z;
         if (n_runs && runs[n_runs - 1].type == g && runs[n_runs - 1].zone == z) runs[n_runs - 1].n_stages++;
@@ -638,13 +469,6 @@ __global__ void __launch_bounds__(128) dp_finish_kernel(const __grid_constant__ 
             runs[n_runs].tp_idx = (uint8_t)k.tpi; runs[n_runs].n_stages = 1;
             ++n_runs;
         }
-        if (i + 1 == P) break;
-        const uint8_t g2 = fp.choice[pb.choice_off + (size_t)i * pb.n_lvl + entry];
-        const uint32_t ui = (entry - pb.zp_base[zp]) % pb.S[zp];
-        uint32_t u[SAILOR_T_MAX];
-        dp_counts(pb, fp.vtabs, zp, T, ui, u, P);
-        const DpMove mv = dp_move(pb, fp.vtabs, T, zp, ui, u, g2);
-        g = g2; zp = mv.zp; entry = mv.entry;
     }
     // the plan written out, through the simulator (Sec. 4.3): what a caller compares with a constraint
     TabView v;
@@ -658,10 +482,17 @@ __global__ void __launch_bounds__(128) dp_finish_kernel(const __grid_constant__ 
 }
 
 // The k best problems by (value, problem index), then the simulator's figures for their plans.
+struct DpOut {                       // what a search leaves for the host, in mapped pinned memory
+    unsigned long long counters[5];  // [0] problems with a plan, [1] number written to results, [2] plans over the constraint,
+                                     // [3], [4] of the budget loop: problems given up, calls
+    sailor_dp_result results[SAILOR_K_MAX];
+};
+
 struct DpSelectParams {
+    const double* value;             // [n_problems]
     const DpResult* results;
-    sailor_dp_result* out;           // [k] device
-    unsigned long long* counters;    // [0] problems with a plan, [1] number written to out, [2] plans over the constraint
+    const unsigned long long* counters;   // null, or the budget loop's [3] and [4]
+    DpOut* out;
     SpaceDesc sp;
     uint32_t n_problems, n_orders, k;
     double budget, min_rate;         // <= 0: none
@@ -681,10 +512,10 @@ __global__ void __launch_bounds__(DP_SELECT_THREADS) dp_select_kernel(const __gr
     uint32_t solved = 0, over = 0;
     for (uint32_t base = warp * 32; base < sp.n_problems; base += nw * 32) {
         const uint32_t j = base + lane;
-        const double v = j < sp.n_problems ? sp.results[j].value : make_inf();
+        const double v = j < sp.n_problems ? sp.value[j] : make_inf();
         bool have = v < make_inf();
         solved += have;
-        if (have) {                                           // the planner keeps a plan only within the constraint
+        if (have && (sp.budget > 0.0 || sp.min_rate > 0.0)) {  // the planner keeps a plan only within the constraint
             const DpResult& r = sp.results[j];
             const bool out_of = (sp.budget > 0.0 && r.cost > sp.budget) || (sp.min_rate > 0.0 && 1.0 / r.t_iter < sp.min_rate);
             over += out_of;
@@ -715,33 +546,35 @@ __global__ void __launch_bounds__(DP_SELECT_THREADS) dp_select_kernel(const __gr
         const uint32_t n = __popc(__ballot_sync(FULL, lane < sp.k && top.flat != ~0ull));
         if (lane == 0) {
             s_n = n;
-            sp.counters[0] = s_solved;
-            sp.counters[1] = n;
-            sp.counters[2] = s_over;
+            sp.out->counters[0] = s_solved;
+            sp.out->counters[1] = n;
+            sp.out->counters[2] = s_over;
+            sp.out->counters[3] = sp.counters ? sp.counters[3] : 0;
+            sp.out->counters[4] = sp.counters ? sp.counters[4] : 0;
         }
     }
     __syncthreads();
     for (uint32_t j = warp; j < s_n; j += nw) {
-        if (lane != 0) continue;
         const uint32_t idx = (uint32_t)s_hits[0][j].flat;
         const DpResult& r = sp.results[idx];
         const uint32_t c = idx / sp.n_orders;
         const Config k = config_of(sp.sp, c);
-        sailor_dp_result o;
-        for (int q = 0; q < (int)sizeof(o); ++q) reinterpret_cast<unsigned char*>(&o)[q] = 0;
-        o.config = c;
-        o.order = idx % sp.n_orders;
-        o.value = r.value;
-        o.P = (uint8_t)k.P; o.mbs_idx = (uint8_t)k.mi; o.tp_idx = (uint8_t)k.tpi; o.rc = (uint8_t)k.rc; o.D = (uint16_t)k.D;
-        for (uint32_t i = 0; i < k.P; ++i) {
-            o.type[i] = r.type[i];
-            o.zone[i] = r.zone[i];
+        sailor_dp_result& o = sp.out->results[j];
+        if (lane == 0) {
+            o.config = c;
+            o.order = idx % sp.n_orders;
+            o.value = s_hits[0][j].score;
+            o.t_iter = r.t_iter;
+            o.cost = r.cost;
+            o.peak_mem = r.peak_mem;
+            o.status = r.status;
+            o.P = (uint8_t)k.P; o.mbs_idx = (uint8_t)k.mi; o.tp_idx = (uint8_t)k.tpi; o.rc = (uint8_t)k.rc; o.D = (uint16_t)k.D;
+            o._pad = 0;
         }
-        o.t_iter = r.t_iter;
-        o.cost = r.cost;
-        o.peak_mem = r.peak_mem;
-        o.status = r.status;
-        sp.out[j] = o;
+        for (uint32_t i = lane; i < SAILOR_P_MAX; i += 32) {
+            o.type[i] = i < k.P ? r.type[i] : 0;
+            o.zone[i] = i < k.P ? r.zone[i] : 0;
+        }
     }
 }
 

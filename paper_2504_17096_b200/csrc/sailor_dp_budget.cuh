@@ -20,6 +20,14 @@ namespace sailor {
 
 constexpr uint32_t DP_BUDGET_P_MAX = 32;     // deepest pipeline the limited recursion takes
 
+struct DpProblem {                   // what first fit needs of a (configuration, zone order)
+    uint32_t config, order, index;   // index = config * n_orders + order
+    uint32_t P, nz, need;            // need = D * tp GPUs per stage
+    uint8_t zone[SAILOR_Z_MAX];      // zone of each position of the order
+    uint8_t cap[SAILOR_Z_MAX][SAILOR_T_MAX];       // stages a (position, type) can host, saturated at 255
+    uint8_t first_later[SAILOR_Z_MAX][SAILOR_T_MAX];   // first position after zp that can host a stage of the type
+};
+
 struct DpbFrame {                    // one call of the recursion: stage `level` on type g at zone position zp
     double limit;                    // what stages level.. may be charged
     double rate, sync, fb, upd;      // of this stage on its GPUs
@@ -38,7 +46,8 @@ struct DpBudgetParams {
     SpaceDesc sp;
     const DpProblem* problems;
     const double* tabs;
-    DpResult* results;               // indexed by problem index
+    double* value;                   // indexed by problem index; +inf: no plan
+    DpResult* results;
     DpbFrame* frames;                // [n_problems][DP_BUDGET_P_MAX]
     unsigned long long* counters;    // [3] += problems given up, [4] += calls of the recursion
     DpTabLayout lay;
@@ -56,7 +65,6 @@ __global__ void __launch_bounds__(64) dp_budget_kernel(const __grid_constant__ D
     if (x >= bp.n_problems) return;
     const DpProblem& pb = bp.problems[x];
     DpResult& out = bp.results[pb.index];
-    out.value = make_inf();
     const uint32_t T = bp.T, P = pb.P;
     const double* tab = bp.tabs + (size_t)pb.config * bp.lay.stride();
     if (*reinterpret_cast<const uint32_t*>(tab + bp.lay.off_nb() + 1) == 0 || P > DP_BUDGET_P_MAX) return;   // no valid plan here
@@ -222,7 +230,7 @@ __global__ void __launch_bounds__(64) dp_budget_kernel(const __grid_constant__ D
     atomicAdd(&bp.counters[4], nodes);
     if (gave_up) { atomicAdd(&bp.counters[3], 1ull); return; }
     if (!best_found) return;
-    out.value = best_v;
+    bp.value[pb.index] = best_v;
     // zones by first fit, as the recursion placed them; then the plan through the simulator (Sec. 4.3)
     sailor_run runs[DP_BUDGET_P_MAX];
     uint32_t n_runs = 0, zp = 0;

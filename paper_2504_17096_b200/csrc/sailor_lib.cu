@@ -198,6 +198,7 @@ struct HostBlock {
     SurveyOut survey;                      // what the survey of a space found
     uint16_t avail[R_MAX];                 // the availability snapshot last set
     MixedOut mixed;                        // results of a search over plans with mixed replicas
+    DpOut dp;                              // results of a search over per-stage GPU types
 };
 
 constexpr size_t CFG_CACHE_MAX_BYTES = 512ull << 20;
@@ -240,6 +241,7 @@ struct sailor_ctx {
     // explicit-batch staging (grow-only)
     unsigned char* d_stage = nullptr;
     size_t stage_bytes = 0;
+    std::vector<unsigned char> h_static;   // host copy of the blob's static part
     // the search over plans with mixed replicas: tables of the space last searched, working memory (grow-only)
     MixedTables* mix = nullptr;
     unsigned char* d_mix = nullptr;
@@ -248,6 +250,8 @@ struct sailor_ctx {
     // tables of the dynamic-programming search (grow-only)
     unsigned char* d_dp = nullptr;
     size_t dp_bytes = 0;
+    unsigned char* d_dp_up = nullptr;      // layouts, jobs and block lists of a batch
+    size_t dp_up_bytes = 0;
 };
 
 namespace {
@@ -340,7 +344,7 @@ int device_grow(sailor_ctx* ctx, unsigned char** p, size_t* have, size_t need) {
     return rc;
 }
 
-// Pinned host blocks (68 KB each): allocating one can cost a millisecond, so the process keeps a few that no context
+// Pinned host blocks (76 KB each): allocating one can cost a millisecond, so the process keeps a few that no context
 // uses at the moment.
 class HostBlocks {
   public:
@@ -1028,6 +1032,7 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
     CUF(cudaEventCreate(&ctx->evh1));
     CUF(cudaMemsetAsync(ctx->d_mem, 0, zeroed, ctx->stream));
     CUF(cudaMemcpyAsync(ctx->d_blob, blob.data(), h.static_bytes, cudaMemcpyHostToDevice, ctx->stream));   // returns when `blob` has been read
+    ctx->h_static.swap(blob);
     {
         const uint32_t n_threads = 4 * T * n_tp * n_mbs + 2 * T * n_tp;
         chain_kernel<<<(n_threads + 127) / 128, 128, 0, ctx->stream>>>(ctx->d_blob);
@@ -1054,7 +1059,7 @@ int sailor_destroy(sailor_ctx* ctx) {
     if (!ctx) return SAILOR_OK;
     DeviceGuard guard(ctx->device);
     if (ctx->d_mem) cudaStreamSynchronize(ctx->stream);
-    for (unsigned char* p : {ctx->d_mem, ctx->space.d_mem, ctx->d_stage, ctx->d_mix, ctx->d_dp}) device_free(ctx, p);
+    for (unsigned char* p : {ctx->d_mem, ctx->space.d_mem, ctx->d_stage, ctx->d_mix, ctx->d_dp, ctx->d_dp_up}) device_free(ctx, p);
     g_host_blocks.give_back(ctx->host);
     delete ctx->mix;
     for (cudaEvent_t e : {ctx->ev0, ctx->ev1, ctx->ev2, ctx->evh0, ctx->evh1, ctx->ev_chunk, ctx->ev_join, ctx->ev_slot[0],
@@ -1488,6 +1493,164 @@ extern "C" int sailor_plan_noalloc(sailor_ctx* ctx, const sailor_space* s, const
 
 // ---- per-stage GPU types by dynamic programming ---------------------------------------------------
 
+namespace {
+
+// A layout as the host lays it down (see DpLayout), its positions' rank tables and its live rows.
+struct LayoutInfo {
+    DpLayout l;
+    std::vector<uint32_t> w;           // rank tables, position after position
+    std::vector<uint32_t> live;        // [P][dp_live_words(nz)]
+    uint64_t total_live = 0;           // live vectors of all stages
+    uint32_t max_live = 0;
+    int batch = -1;                    // the last batch it was put into, and its place there
+    uint32_t place = 0;
+};
+
+// The layout of pipelines of P stages of `need` GPUs each over the zones of `order`, with the types of `usable`.
+// Returns SAILOR_E_RANGE when a position has more than 2^31 vectors; a stage without live vectors leaves max_live at 0.
+int build_layout(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_zone_order& order, uint32_t usable, LayoutInfo& info) {
+    const uint32_t T = ctx->hdr.T, w = P + 1;
+    DpLayout& l = info.l;
+    memset(&l, 0, sizeof(l));
+    memset(l.first_later, DP_NONE, sizeof(l.first_later));
+    l.P = P;
+    uint64_t lo = 0, mx = 0;               // stages before a position: at least, at most
+    uint64_t lo_of[SAILOR_Z_MAX], mx_of[SAILOR_Z_MAX], n_vec = 0;
+    bool uncounted_of[SAILOR_Z_MAX], hosts[SAILOR_Z_MAX];
+    std::vector<uint64_t> W((size_t)(T + 1) * w), first_sum(order.n, 0);
+    for (uint32_t zp = 0; zp < order.n && lo < P; ++zp) {
+        l.nz = zp + 1;
+        l.zone[zp] = order.zone[zp];
+        uint32_t types[SAILOR_T_MAX], m = 0;
+        uint64_t least = ~0ull, all = 0;
+        uncounted_of[zp] = hosts[zp] = false;
+        for (uint32_t g = 0; g < T; ++g) {
+            if (!((usable >> g) & 1u)) continue;
+            const uint64_t cap = ctx->h_avail[order.zone[zp] * T + g] / need;
+            l.cap[zp][g] = (uint8_t)(cap > 255 ? 255 : cap);
+            least = cap < least ? cap : least;
+            all += cap;
+            hosts[zp] = hosts[zp] || cap > 0;
+            if (cap >= P) uncounted_of[zp] = true;
+            else if (cap > 0) { types[m++] = g; l.counted[zp] |= (uint8_t)(1u << g); }
+        }
+        l.n_counted[zp] = (uint8_t)m;
+        lo_of[zp] = lo;
+        mx_of[zp] = mx;
+        const uint32_t most = P - (uint32_t)lo;              // largest sum a stage here can have behind it
+        l.sum_max[zp] = most;
+        // W[j][s]: vectors of the counted types from the j-th on, within the caps, that add up to at most s
+        for (uint32_t s = 0; s < w; ++s) W[(size_t)m * w + s] = 1;
+        for (uint32_t j = m; j-- > 0;) {
+            const uint64_t cj = l.cap[zp][types[j]];
+            const uint64_t* below = &W[(size_t)(j + 1) * w];
+            uint64_t* row = &W[(size_t)j * w];
+            // exact counts N[j][s] = sum over x <= cj of N[j + 1][s - x] = W[j + 1][s] - W[j + 1][s - cj - 1]
+            uint64_t run = 0;
+            for (uint32_t s = 0; s < w; ++s) {
+                run += below[s] - (s > cj ? below[s - cj - 1] : 0);
+                row[s] = run < (1ull << 40) ? run : (1ull << 40);        // (beyond the limit below: only kept from running over)
+            }
+        }
+        if (W[most] > (1ull << 31)) return SAILOR_E_RANGE;
+        l.w_off[zp] = (uint32_t)info.w.size();
+        for (size_t x = 0; x < (size_t)(m + 1) * w; ++x) info.w.push_back((uint32_t)(W[x] < 0xffffffffull ? W[x] : 0xffffffffull));
+        l.vec_base[zp] = (uint32_t)n_vec;
+        for (uint32_t j = 0; j < m; ++j)
+            l.first_vec[zp][types[j]] = (uint32_t)(n_vec + W[0] + (P >= 1 ? W[(size_t)(j + 1) * w + 1] - W[(size_t)(j + 1) * w] : 0));
+        for (uint32_t g = 0; g < T; ++g)
+            if (l.cap[zp][g] && !((l.counted[zp] >> g) & 1u)) l.first_vec[zp][g] = (uint32_t)n_vec;
+        n_vec += W[most];
+        if (n_vec > (1ull << 31)) return SAILOR_E_RANGE;
+        lo += least == ~0ull ? P : least;
+        mx = uncounted_of[zp] ? (uint64_t)1 << 32 : mx + all;
+    }
+    l.vec_base[l.nz] = (uint32_t)n_vec;
+    for (uint32_t zp = 0; zp < l.nz; ++zp)
+        for (uint32_t g = 0; g < T; ++g)
+            for (uint32_t q = zp + 1; q < l.nz; ++q)
+                if (l.cap[q][g] >= 1) { l.first_later[zp][g] = (uint8_t)q; break; }
+    const uint32_t words = dp_live_words(l.nz);
+    info.live.assign((size_t)P * words, 0);
+    for (uint32_t i = 0; i < P; ++i) {
+        uint32_t* row = &info.live[(size_t)i * words];
+        row[1] = (uint32_t)info.total_live;
+        uint64_t slots = 0;
+        for (uint32_t zp = 0; zp < l.nz; ++zp) {
+            const uint32_t* W0 = &info.w[l.w_off[zp]];
+            uint64_t first = 0, count = 0;
+            if (hosts[zp] && i + 1 > lo_of[zp]) {
+                const uint64_t top = i + 1 - lo_of[zp];
+                uint64_t bottom = uncounted_of[zp] ? 0 : 1;
+                if (!uncounted_of[zp] && i + 1 > mx_of[zp] && i + 1 - mx_of[zp] > bottom) bottom = i + 1 - mx_of[zp];
+                if (bottom <= top) {
+                    first = bottom ? W0[bottom - 1] : 0;
+                    count = W0[top] - first;
+                }
+            }
+            row[2 + 2 * zp] = (uint32_t)(l.vec_base[zp] + first);
+            row[3 + 2 * zp] = (uint32_t)slots;
+            slots += count;
+        }
+        row[0] = (uint32_t)slots;
+        info.total_live += slots;
+        if (slots == 0 || (slots + 1) * ctx->hdr.T >= 0xffffffffull || info.total_live >= 0xffffffffull) {
+            const bool none = slots == 0;
+            info.max_live = 0;
+            return none ? SAILOR_OK : SAILOR_E_RANGE;
+        }
+        info.max_live = std::max(info.max_live, (uint32_t)slots);
+    }
+    return SAILOR_OK;
+}
+
+// The GPU types that fit the memory of some stage of a configuration; 0 when a stage fits none.  Inside a stretch of
+// stages of one make-up the first keeps the most microbatches and the last the fewest.
+uint32_t usable_types(const sailor_ctx* ctx, const TabView& v, const Config& k, uint64_t n_b) {
+    const TabHdr& h = ctx->hdr;
+    const uint32_t P = k.P, base = h.n_blocks / P, extra = h.n_blocks % P, tp = h.tp_values[k.tpi];
+    auto fits = [&](uint32_t i) {
+        const bool e = (i == 0) && h.has_embed, hd = (i == P - 1) && h.has_head;
+        const uint64_t inflight = (uint64_t)(P - i) < n_b ? (uint64_t)(P - i) : n_b;
+        const StageMem sm = stage_memory(v, k.tpi, k.mi, k.rc, base + (i < extra ? 1u : 0u), e, hd, inflight);
+        uint32_t mask = 0;
+        for (uint32_t g = 0; g < h.T; ++g)
+            if (sm.mem + h.reserved[g] <= h.capacity[g] && tp <= h.gpn[g]) mask |= 1u << g;
+        return mask;
+    };
+    uint32_t all = 0;
+    for (uint32_t i = 0; i < P;) {
+        uint32_t end = P;
+        if (i == 0 && h.has_embed) end = 1;
+        else {
+            if (i < extra && extra < end) end = extra;
+            if (h.has_head && i < P - 1 && P - 1 < end) end = P - 1;
+        }
+        if (!fits(i)) return 0;
+        all |= fits(end - 1);
+        i = end;
+    }
+    return all;
+}
+
+// SAILOR_DP_FLAG_INDEX_DENSE: the size the tables of a problem would have in mixed radix over all its scarce types.
+int dense_fits(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_zone_order& order, uint64_t workspace_bytes) {
+    const uint32_t T = ctx->hdr.T;
+    uint64_t entries = 0;
+    for (uint32_t zp = 0; zp < order.n; ++zp) {
+        uint64_t box = T;
+        for (uint32_t g = 0; g < T; ++g) {
+            const uint64_t cap = ctx->h_avail[order.zone[zp] * T + g] / need;
+            if (cap >= 1 && cap < P) box *= cap + 1;
+            if (box > (1ull << 31)) return SAILOR_E_RANGE;
+        }
+        entries += box;
+    }
+    return entries > (1ull << 31) || entries * (2 * sizeof(DpVal) + P) > workspace_bytes ? SAILOR_E_RANGE : SAILOR_OK;
+}
+
+}  // namespace
+
 // The recursion steered by the budget (Sec. 4.2.3): one thread per problem, depth first.
 static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor_zone_order* orders, uint32_t n_orders,
                                const sailor_objective* o, uint64_t workspace_bytes, uint32_t k, sailor_dp_result* topk,
@@ -1526,7 +1689,7 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     lay.p_max = p_max; lay.T = T; lay.R = h.R;
     const size_t tab_bytes = (size_t)n_config * lay.stride() * sizeof(double);
     const size_t total = padded(tab_bytes) + padded(n_problems * sizeof(DpResult)) + padded(n_problems * sizeof(DpProblem)) +
-                         padded(n_problems * DP_BUDGET_P_MAX * sizeof(DpbFrame)) + padded(sizeof(sailor_dp_result) * SAILOR_K_MAX) +
+                         padded(n_problems * DP_BUDGET_P_MAX * sizeof(DpbFrame)) + padded(n_problems * sizeof(double)) +
                          padded(40) + 4096;
     if (total > workspace_bytes) return SAILOR_E_RANGE;
     {
@@ -1538,8 +1701,10 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     DpResult* d_results = bump.take<DpResult>(n_problems);
     DpProblem* d_problems = bump.take<DpProblem>(n_problems);
     DpbFrame* d_frames = bump.take<DpbFrame>(n_problems * DP_BUDGET_P_MAX);
-    sailor_dp_result* d_out = bump.take<sailor_dp_result>(SAILOR_K_MAX);
+    double* d_value = bump.take<double>(n_problems);
     unsigned long long* d_counters = bump.take<unsigned long long>(5);
+    DpOut* d_out = nullptr;
+    CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&d_out), &ctx->host->dp, 0));
 
     uint32_t launches = 0;
     {
@@ -1547,19 +1712,18 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
         if (rc_up) return rc_up;
     }
     CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
-    CU(ctx, cudaMemsetAsync(d_tabs, 0, tab_bytes, ctx->stream));
     CU(ctx, cudaMemsetAsync(d_counters, 0, 40, ctx->stream));
     CU(ctx, cudaMemcpyAsync(d_problems, prob.data(), n_problems * sizeof(DpProblem), cudaMemcpyHostToDevice, ctx->stream));
     {
         const uint32_t grid = (uint32_t)(n_config < 4096 ? n_config : 4096);
-        dp_tables_kernel<<<grid, DP_THREADS, 0, ctx->stream>>>(ctx->d_blob, d, (uint32_t)n_config, lay, d_tabs);
+        dp_tables_kernel<<<grid, DP_THREADS, 0, ctx->stream>>>(ctx->d_blob, d, (uint32_t)n_config, n_orders, lay, nullptr, d_tabs, d_value);
         CU(ctx, cudaGetLastError());
         ++launches;
     }
     DpBudgetParams bp;
     memset(&bp, 0, sizeof(bp));
     bp.blob = ctx->d_blob; bp.avail = ctx->d_avail; bp.sp = d; bp.problems = d_problems; bp.tabs = d_tabs;
-    bp.results = d_results; bp.frames = d_frames; bp.counters = d_counters; bp.lay = lay;
+    bp.value = d_value; bp.results = d_results; bp.frames = d_frames; bp.counters = d_counters; bp.lay = lay;
     bp.n_problems = (uint32_t)n_problems; bp.T = T;
     bp.limit = o->budget_usd_per_iter;
     bp.node_limit = 1ull << 24;
@@ -1568,21 +1732,18 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     ++launches;
     DpSelectParams sel;
     memset(&sel, 0, sizeof(sel));
-    sel.results = d_results; sel.out = d_out; sel.counters = d_counters;
+    sel.value = d_value; sel.results = d_results; sel.out = d_out; sel.counters = d_counters;
     sel.sp = d; sel.n_problems = (uint32_t)n_problems; sel.n_orders = n_orders; sel.k = k;
     sel.budget = o->budget_usd_per_iter; sel.min_rate = o->min_iters_per_s;
     dp_select_kernel<<<1, DP_SELECT_THREADS, 0, ctx->stream>>>(sel);
     CU(ctx, cudaGetLastError());
     ++launches;
     CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
-    unsigned long long counters[5] = {0, 0, 0, 0, 0};
-    std::vector<sailor_dp_result> host_out(k);
-    CU(ctx, cudaMemcpyAsync(counters, d_counters, sizeof(counters), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(ctx, cudaMemcpyAsync(host_out.data(), d_out, sizeof(sailor_dp_result) * k, cudaMemcpyDeviceToHost, ctx->stream));
     CU(ctx, stream_sync(ctx));                                 // also: `prob` is pageable
+    const unsigned long long* counters = ctx->host->dp.counters;
     if (counters[1] > k) return SAILOR_E_DEVICE;
     *n_found = (uint32_t)counters[1];
-    memcpy(topk, host_out.data(), sizeof(sailor_dp_result) * counters[1]);
+    memcpy(topk, ctx->host->dp.results, sizeof(sailor_dp_result) * counters[1]);
     if (stats) {
         stats->n_problems = n_problems;
         stats->n_solved = counters[0];
@@ -1637,362 +1798,244 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
         return plan_dp_budget_impl(ctx, d, orders, n_orders, o, workspace_bytes, k, topk, n_found, stats);
     }
 
-    // every problem's table layout, from the availability last set (host copy)
+    // problems that can have a plan, and the layouts they share
     const uint64_t n_problems = n_config * n_orders;
-    std::vector<DpProblem> prob(n_problems);
-    std::vector<uint32_t> vtabs;        // rank tables of the compactly indexed zone positions, all problems
-    // how a zone position's count vectors are indexed: 0 = the smaller of the two ways, 1 = mixed radix whenever it
-    // fits, 2 = by rank whenever it fits (SAILOR_DP_FLAG_INDEX_*)
-    const int index_mode = (o->flags & SAILOR_DP_FLAG_INDEX_DENSE) ? 1 : (o->flags & SAILOR_DP_FLAG_INDEX_COMPACT) ? 2 : 0;
-    // which threads a stage's launch has: one per count vector the stage can have reached ("live", whenever every
-    // zone position has its rank table), or one per table entry (SAILOR_DP_FLAG_ENUM_BY_ENTRY)
-    bool all_live = !(o->flags & SAILOR_DP_FLAG_ENUM_BY_ENTRY);
-    std::vector<uint64_t> V, live_stage;                     // scratch of the loop below
-    std::vector<uint64_t> live_off(n_problems + 1, 0);      // per problem: where its per-stage live counts start
-    std::vector<uint32_t> live_cnt;                          // count vectors stage i can have reached, all positions
+    TabView hv;
+    hv.bind(ctx->h_static.data(), ctx->h_static.data());
+    std::vector<LayoutInfo> layouts;
+    std::map<std::pair<uint64_t, uint64_t>, uint32_t> layout_of;
+    struct Problem { uint32_t config, index, layout, place; };   // place: of the layout among its batch's
+    std::vector<Problem> by_depth[SAILOR_P_MAX + 1];         // deepest first, so that a stage's launch covers a prefix
+    std::vector<uint8_t> wanted(n_config, 0);                // configurations whose per-configuration tables are needed
     uint64_t n_states = 0;
-    uint32_t vt_len_max = 0;                                 // words of the largest problem's rank tables
-    std::map<std::array<uint64_t, 3>, uint64_t> same_states;
     for (uint64_t c = 0; c < n_config; ++c) {
         const Config cf = config_of(d, (uint32_t)c);
         const uint32_t tp = h.tp_values[cf.tpi];
         const uint64_t dm = (uint64_t)cf.D * h.mbs_values[cf.mi];
-        const bool valid = h.gbs % dm == 0 && h.heads % tp == 0;
         const uint64_t need = (uint64_t)cf.D * tp;
+        if (h.gbs % dm != 0 || h.heads % tp != 0) continue;  // no valid plan
+        if (o->flags & SAILOR_DP_FLAG_INDEX_DENSE)
+            for (uint32_t q = 0; q < n_orders; ++q)
+                if (dense_fits(ctx, cf.P, need, orders[q], workspace_bytes) != SAILOR_OK) return SAILOR_E_RANGE;
+        const uint32_t usable = usable_types(ctx, hv, cf, h.gbs / dm);
+        if (!usable) continue;                               // some stage fits no type
         for (uint32_t q = 0; q < n_orders; ++q) {
-            DpProblem& pb = prob[c * n_orders + q];
-            memset(&pb, 0, sizeof(pb));
-            pb.config = (uint32_t)c; pb.order = q; pb.index = (uint32_t)(c * n_orders + q);
-            pb.P = cf.P; pb.nz = orders[q].n; pb.need = (uint32_t)(need > 0xffffffffull ? 0xffffffffull : need);
-            memset(pb.first_later, DP_NONE, sizeof(pb.first_later));
-            live_off[c * n_orders + q] = live_cnt.size();
-            if (!valid) continue;                           // no entries: the finish step finds no plan
-            // the states, their index and the rank tables depend on (P, D * tp, zone order) only: configurations
-            // that differ in the microbatch size or in recomputation take them from the first such problem
-            const std::array<uint64_t, 3> key = {cf.P, need, q};
-            const auto seen = same_states.find(key);
-            if (seen != same_states.end()) {
-                const DpProblem& first = prob[seen->second];
-                const uint32_t config = pb.config, index = pb.index;
-                pb = first;
-                pb.config = config; pb.index = index;
-                live_off[c * n_orders + q] = live_off[seen->second];
-                n_states += (uint64_t)pb.n_lvl * cf.P;
-                continue;
+            const std::pair<uint64_t, uint64_t> key((uint64_t)q << 8 | cf.P, need << SAILOR_T_MAX | usable);
+            const auto seen = layout_of.emplace(key, (uint32_t)layouts.size());
+            if (seen.second) {
+                layouts.emplace_back();
+                const int rc_lay = build_layout(ctx, cf.P, need, orders[q], usable, layouts.back());
+                if (rc_lay) return rc_lay;
             }
-            same_states.emplace(key, c * n_orders + q);
-            uint64_t n_lvl = 0;
-            pb.vt_lo = (uint32_t)vtabs.size();
-            live_stage.assign(cf.P, 0);
-            for (uint32_t zp = 0; zp < pb.nz; ++zp) {
-                pb.zone[zp] = orders[q].zone[zp];
-                // counted types: the zone can host some but not all P stages of them
-                uint32_t counted[SAILOR_T_MAX], m = 0;
-                uint64_t dense = 1;
-                bool dense_ok = true;
-                for (uint32_t g = 0; g < T; ++g) {
-                    const uint64_t cap = ctx->h_avail[pb.zone[zp] * T + g] / need;
-                    pb.cap[zp][g] = (uint8_t)(cap > 255 ? 255 : cap);
-                    if (cap >= 1 && cap < cf.P) {
-                        counted[m++] = g;
-                        if (dense_ok) dense *= cap + 1;
-                        if (dense > (1ull << 31)) dense_ok = false;
-                    }
-                }
-                pb.n_counted[zp] = (uint8_t)m;
-                // compact index: count vectors within the caps that add up to at most P (rank tables V[j][s])
-                const uint32_t w = cf.P + 1;
-                V.assign((size_t)(m + 1) * w, 0);
-                for (uint32_t sgm = 0; sgm < w; ++sgm) V[(size_t)m * w + sgm] = sgm + 1;           // W = 1 each
-                bool compact_ok = true;
-                for (uint32_t j = m; j-- > 0;) {
-                    const uint64_t cj = pb.cap[zp][counted[j]];
-                    uint64_t run = 0;
-                    for (uint32_t sgm = 0; sgm < w; ++sgm) {
-                        const uint64_t lo = sgm > cj ? V[(size_t)(j + 1) * w + (sgm - cj - 1)] : 0;
-                        run += V[(size_t)(j + 1) * w + sgm] - lo;                                  // W[j][s]
-                        V[(size_t)j * w + sgm] = run;
-                        if (run > (1ull << 31)) compact_ok = false;
-                    }
-                }
-                const uint64_t compact = m ? V[cf.P] - (cf.P ? V[cf.P - 1] : 0) : 1;                // W[0][P]
-                if (!dense_ok && !compact_ok) return SAILOR_E_RANGE;
-                const bool use_compact = index_mode == 2 ? compact_ok && m > 0
-                                         : index_mode == 1 ? !dense_ok
-                                                           : (m > 0 && compact_ok && (!dense_ok || dense > 4 * compact));
-                uint64_t S = 1;
-                pb.rank_off[zp] = DP_DENSE;
-                if (m > 0 && compact_ok) {                   // the rank table serves the live enumeration in any case
-                    pb.rank_off[zp] = (uint32_t)vtabs.size();
-                    for (uint64_t x : V) vtabs.push_back((uint32_t)x);
-                    if (vtabs.size() > (1ull << 30)) return SAILOR_E_RANGE;
-                } else if (m > 0) {
-                    all_live = false;
-                }
-                for (uint32_t st = 0; st < cf.P; ++st) {     // count vectors with at most st + 1 stages
-                    const uint32_t bud = st + 1;
-                    live_stage[st] += m > 0 && compact_ok ? V[bud] - V[bud - 1] : 1;
-                }
-                if (use_compact) {
-                    S = compact;
-                    pb.vt_off[zp] = pb.rank_off[zp];
-                    for (uint32_t j = 0; j < m; ++j) {
-                        // rank of "one stage of type counted[j]": every vector that has a zero there and is zero before it
-                        // comes first: V[j+1][P] - V[j+1][P-1] ... summed by the rank formula with u = e_j
-                        pb.stride[zp][counted[j]] = 1;                                         // marks the type as counted
-                        pb.first_idx[zp][counted[j]] = (uint32_t)(V[(size_t)(j + 1) * w + cf.P] - V[(size_t)(j + 1) * w + cf.P - 1]);
-                    }
-                } else {
-                    pb.vt_off[zp] = DP_DENSE;
-                    for (uint32_t j = 0; j < m; ++j) {
-                        const uint32_t g = counted[j];
-                        pb.magic[zp][g] = ~0ull / (pb.cap[zp][g] + 1ull) + 1;                  // ceil(2^64 / (cap + 1)), cap + 1 >= 2
-                        pb.stride[zp][g] = (uint32_t)S;
-                        pb.first_idx[zp][g] = (uint32_t)S;
-                        S *= pb.cap[zp][g] + 1ull;
-                    }
-                }
-                pb.S[zp] = (uint32_t)S;
-                pb.zp_base[zp] = (uint32_t)n_lvl;
-                n_lvl += (uint64_t)T * S;
-                if (n_lvl > (1ull << 31)) return SAILOR_E_RANGE;
-            }
-            pb.zp_base[pb.nz] = (uint32_t)n_lvl;
-            for (uint32_t zp = 0; zp < pb.nz; ++zp)
-                for (uint32_t g = 0; g < T; ++g)
-                    for (uint32_t q = zp + 1; q < pb.nz; ++q)
-                        if (pb.cap[q][g] >= 1) { pb.first_later[zp][g] = (uint8_t)q; break; }
-            pb.n_lvl = (uint32_t)n_lvl;
-            pb.vt_len = (uint32_t)(vtabs.size() - pb.vt_lo);
-            vt_len_max = pb.vt_len > vt_len_max ? pb.vt_len : vt_len_max;
-            n_states += n_lvl * cf.P;
-            for (uint32_t st = 0; st < cf.P; ++st) live_cnt.push_back((uint32_t)(live_stage[st] > n_lvl ? n_lvl : live_stage[st]));   // <= n_lvl / T
+            const LayoutInfo& info = layouts[seen.first->second];
+            if (info.max_live == 0) continue;                // some stage has nowhere to go
+            by_depth[cf.P].push_back({(uint32_t)c, (uint32_t)(c * n_orders + q), seen.first->second, 0});
+            wanted[c] = 1;
+            n_states += info.total_live * T;
         }
     }
-    // deepest pipelines first, so that the launch for a distance from the last stage covers a prefix
-    std::vector<uint32_t> by_depth;
-    by_depth.reserve(n_problems);
-    for (uint64_t j = 0; j < n_problems; ++j)
-        if (prob[j].n_lvl) by_depth.push_back((uint32_t)j);
-    std::stable_sort(by_depth.begin(), by_depth.end(), [&](uint32_t a, uint32_t b) { return prob[a].P > prob[b].P; });
-    auto work_bytes = [](const DpProblem& pb) { return (uint64_t)pb.n_lvl * (2 * sizeof(DpVal) + pb.P); };
-    struct Batch { size_t first, count; uint64_t entries, choice_bytes, blocks; };
+    std::vector<Problem> todo;
+    for (uint32_t P = SAILOR_P_MAX; P > 0; --P) todo.insert(todo.end(), by_depth[P].begin(), by_depth[P].end());
+
+    // cut into batches that fit the workspace: per problem two level buffers and its successors (padded to 256 bytes
+    // each), per layout its moves
+    const uint32_t TM = T <= 4 ? 4 : SAILOR_T_MAX;
+    struct Batch {
+        size_t first, count;
+        uint64_t val_entries, succ_words, nxt_rows;
+        std::vector<std::pair<uint32_t, uint32_t>> layouts;  // layout, its first row of moves in this batch
+    };
     std::vector<Batch> batches;
-    uint64_t largest = 0;
-    for (size_t j = 0; j < by_depth.size();) {
-        Batch b = {j, 0, 0, 0, 0};
+    uint64_t largest = 0, max_val = 0, max_succ = 0, max_rows = 0;
+    auto pad8 = [](uint64_t x) { return (x + 7) / 8 * 8; };
+    auto pad64 = [](uint64_t x) { return (x + 63) / 64 * 64; };
+    for (size_t j = 0; j < todo.size();) {
+        Batch b = {j, 0, 0, 0, 0, {}};
         uint64_t bytes = 0;
-        while (j < by_depth.size()) {
-            const DpProblem& pb = prob[by_depth[j]];
-            const uint64_t wb = work_bytes(pb) + 512;
-            if (b.count && bytes + wb > workspace_bytes) break;
-            if (wb > workspace_bytes) return SAILOR_E_RANGE;      // one problem alone does not fit
-            bytes += wb;
-            b.entries += pb.n_lvl;
-            b.choice_bytes += (uint64_t)pb.n_lvl * pb.P;
-            b.blocks += all_live ? (uint64_t)pb.P + 1 : (pb.n_lvl + DP_THREADS - 1) / DP_THREADS;   // words of the block lists
-            ++b.count; ++j;
+        for (; j < todo.size(); ++j) {
+            LayoutInfo& info = layouts[todo[j].layout];
+            const uint64_t val = pad8((uint64_t)info.max_live * T), succ = pad64(info.total_live * T);
+            const uint64_t rows = info.batch == (int)batches.size() ? 0 : info.l.vec_base[info.l.nz];
+            const uint64_t more = val * 2 * sizeof(DpVal) + succ * 4 + rows * TM * 4;
+            if (bytes + more > workspace_bytes || b.nxt_rows + rows >= (1ull << 32)) {
+                if (b.count == 0) return SAILOR_E_RANGE;     // one problem alone does not fit
+                break;
+            }
+            if (rows) {
+                info.batch = (int)batches.size();
+                info.place = (uint32_t)b.layouts.size();
+                b.layouts.emplace_back(todo[j].layout, (uint32_t)b.nxt_rows);
+                b.nxt_rows += rows;
+            }
+            todo[j].place = info.place;
+            bytes += more;
+            b.val_entries += val;
+            b.succ_words += succ;
+            ++b.count;
         }
-        largest = bytes > largest ? bytes : largest;
-        batches.push_back(b);
+        largest = std::max(largest, bytes);
+        max_val = std::max(max_val, b.val_entries);
+        max_succ = std::max(max_succ, b.succ_words);
+        max_rows = std::max(max_rows, b.nxt_rows);
+        batches.push_back(std::move(b));
     }
-    uint64_t max_entries = 0, max_choice = 0, max_blocks = 0, max_count = 0;
-    for (const Batch& b : batches) {
-        max_entries = std::max(max_entries, b.entries);
-        max_choice = std::max(max_choice, b.choice_bytes);
-        max_blocks = std::max(max_blocks, b.blocks);
-        max_count = std::max<uint64_t>(max_count, b.count);
-    }
-    if (max_blocks > 0x7fffffffull) return SAILOR_E_RANGE;
-    if (all_live) {                                        // what the launches visit: live count vectors only
-        n_states = 0;
-        for (uint64_t j = 0; j < n_problems; ++j)
-            for (uint32_t st = 0; prob[j].n_lvl && st < prob[j].P; ++st) n_states += (uint64_t)live_cnt[live_off[j] + st] * T;
-    }
-    // a thread per count vector for all its types at once, or a thread per (count vector, type)
-    // (its blocks stage their problem's rank tables in shared memory: at most Z * (T + 1) * (P + 1) words)
-    const bool by_vector = all_live && vt_len_max * 4 <= 40 * 1024 && !(o->flags & SAILOR_DP_FLAG_ENUM_BY_TYPE);
-    const uint32_t live_mult = by_vector ? 1u : T;
 
     DeviceGuard guard(ctx->device);
+    {
+        const int rc_up = upload_availability(ctx);
+        if (rc_up) return rc_up;
+    }
     DpTabLayout lay;
     lay.p_max = p_max; lay.T = T; lay.R = h.R;
     const size_t tab_bytes = (size_t)n_config * lay.stride() * sizeof(double);
-    const size_t total = padded(tab_bytes) + padded(vtabs.size() * sizeof(uint32_t) + 4) + padded(n_problems * sizeof(DpResult)) +
-                         padded(n_problems * sizeof(DpProblem)) +
-                         2 * padded((max_blocks + p_max + 16) * sizeof(uint32_t)) + 2 * padded(max_entries * sizeof(DpVal)) +
-                         padded(max_choice) + padded(sizeof(sailor_dp_result) * SAILOR_K_MAX) + padded(24) + 4096;
+    DpOut* d_out = nullptr;
+    CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&d_out), &ctx->host->dp, 0));
+    const size_t total = padded(tab_bytes) + padded(n_problems * sizeof(DpResult)) + padded(n_problems * sizeof(double)) +
+                         padded(max_rows * TM * 4) + 2 * padded(max_val * sizeof(DpVal)) + padded(max_succ * 4);
     {
         const int rc_mem = device_grow(ctx, &ctx->d_dp, &ctx->dp_bytes, total);
         if (rc_mem) return rc_mem;
     }
     Bump bump{ctx->d_dp};
     double* d_tabs = bump.take<double>(tab_bytes / sizeof(double));
-    uint32_t* d_vtabs = bump.take<uint32_t>(vtabs.size() + 1);
     DpResult* d_results = bump.take<DpResult>(n_problems);
-    DpProblem* d_problems = bump.take<DpProblem>(n_problems);
-    uint32_t* d_blk_problem = bump.take<uint32_t>(max_blocks + p_max + 16);
-    uint32_t* d_blk_first = bump.take<uint32_t>(max_blocks + p_max + 16);
-    DpVal* d_val0 = bump.take<DpVal>(max_entries);
-    DpVal* d_val1 = bump.take<DpVal>(max_entries);
-    uint8_t* d_choice = bump.take<uint8_t>(max_choice);
-    sailor_dp_result* d_out = bump.take<sailor_dp_result>(SAILOR_K_MAX);
-    unsigned long long* d_counters = bump.take<unsigned long long>(3);
+    double* d_value = bump.take<double>(n_problems);
+    DpLevelParams lp;
+    memset(&lp, 0, sizeof(lp));
+    uint32_t* d_nxt = bump.take<uint32_t>(max_rows * TM);
+    lp.nxt = d_nxt;
+    lp.val[0] = bump.take<DpVal>(max_val);
+    lp.val[1] = bump.take<DpVal>(max_val);
+    lp.succ = bump.take<uint32_t>(max_succ);
+    lp.tabs = d_tabs; lp.lay = lay; lp.T = T;
 
     uint32_t launches = 0;
-    {
-        const int rc_up = upload_availability(ctx);
-        if (rc_up) return rc_up;
-    }
-    CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
-    CU(ctx, cudaMemsetAsync(d_tabs, 0, tab_bytes, ctx->stream));
-    CU(ctx, cudaMemsetAsync(d_counters, 0, 24, ctx->stream));
-    if (!vtabs.empty())
-        CU(ctx, cudaMemcpyAsync(d_vtabs, vtabs.data(), vtabs.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-    {
-        const uint32_t grid = (uint32_t)(n_config < 4096 ? n_config : 4096);
-        dp_tables_kernel<<<grid, DP_THREADS, 0, ctx->stream>>>(ctx->d_blob, d, (uint32_t)n_config, lay, d_tabs);
+    if (stats) CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
+    std::vector<unsigned char> up;                           // what a batch uploads, in one copy
+    auto add = [&](const void* p, size_t bytes) {
+        const size_t off = padded(up.size());
+        up.resize(off + bytes);
+        if (bytes) memcpy(up.data() + off, p, bytes);
+        return off;
+    };
+    const size_t off_wanted = add(wanted.data(), wanted.size());         // with the first batch
+    for (size_t bi = 0; bi < std::max<size_t>(batches.size(), 1); ++bi) {
+        const Batch* b = batches.empty() ? nullptr : &batches[bi];       // none: no problem has a plan
+        std::vector<DpLayout> lays;
+        std::vector<DpJob> jobs;
+        std::vector<uint32_t> lay_blk(1, 0), wtab, live, prefix;
+        std::vector<size_t> dist_off;
+        uint32_t n_big = 0;
+        if (b) {
+            for (const auto& used : b->layouts) {            // layouts, with offsets into the joint tables
+                const LayoutInfo& info = layouts[used.first];
+                lays.push_back(info.l);
+                lays.back().nxt_off = used.second;
+                for (uint32_t zp = 0; zp < info.l.nz; ++zp) lays.back().w_off[zp] += (uint32_t)wtab.size();
+                lays.back().live_off = (uint32_t)live.size();
+                wtab.insert(wtab.end(), info.w.begin(), info.w.end());
+                live.insert(live.end(), info.live.begin(), info.live.end());
+                lay_blk.push_back(lay_blk.back() + (info.l.vec_base[info.l.nz] + DP_THREADS - 1) / DP_THREADS);
+            }
+            // jobs: those that go stage by stage first (deepest first), then the small ones
+            jobs.resize(b->count);
+            for (size_t j = 0; j < b->count; ++j) n_big += layouts[todo[b->first + j].layout].max_live > DP_SMALL ? 1u : 0u;
+            uint32_t at_big = 0, at_small = n_big;
+            uint64_t val_off = 0, succ_off = 0;
+            for (size_t j = 0; j < b->count; ++j) {
+                const Problem& pr = todo[b->first + j];
+                const LayoutInfo& info = layouts[pr.layout];
+                DpJob& job = jobs[info.max_live > DP_SMALL ? at_big++ : at_small++];
+                job.val_off = val_off;
+                job.succ_off = succ_off;
+                job.config = pr.config; job.index = pr.index; job.layout = pr.place; job.P = info.l.P;
+                val_off += pad8((uint64_t)info.max_live * T);
+                succ_off += pad64(info.total_live * T);
+            }
+            for (uint32_t dist = 0; n_big && dist < jobs[0].P; ++dist) {     // per distance from the last stage: blocks before each job
+                dist_off.push_back(prefix.size());
+                uint32_t blocks = 0;
+                for (uint32_t j = 0; j < n_big && jobs[j].P > dist; ++j) {
+                    prefix.push_back(blocks);
+                    const DpLayout& l = lays[jobs[j].layout];
+                    blocks += (live[l.live_off + (size_t)(jobs[j].P - 1 - dist) * dp_live_words(l.nz)] + DP_THREADS - 1) / DP_THREADS;
+                }
+                prefix.push_back(blocks);
+            }
+            dist_off.push_back(prefix.size());
+        }
+        const size_t off_lay = add(lays.data(), lays.size() * sizeof(DpLayout)), off_blk = add(lay_blk.data(), lay_blk.size() * 4),
+                     off_w = add(wtab.data(), wtab.size() * 4), off_live = add(live.data(), live.size() * 4),
+                     off_jobs = add(jobs.data(), jobs.size() * sizeof(DpJob)), off_prefix = add(prefix.data(), prefix.size() * 4);
+        {
+            const int rc_mem = device_grow(ctx, &ctx->d_dp_up, &ctx->dp_up_bytes, padded(up.size()));
+            if (rc_mem) return rc_mem;
+        }
+        CU(ctx, cudaMemcpyAsync(ctx->d_dp_up, up.data(), up.size(), cudaMemcpyHostToDevice, ctx->stream));   // returns when `up` has been read
+        if (bi == 0) {
+            dp_tables_kernel<<<(uint32_t)std::min<uint64_t>(n_config, 4096), DP_THREADS, 0, ctx->stream>>>(
+                ctx->d_blob, d, (uint32_t)n_config, n_orders, lay, ctx->d_dp_up + off_wanted, d_tabs, d_value);
+            CU(ctx, cudaGetLastError());
+            ++launches;
+        }
+        if (!b) break;
+        lp.layouts = reinterpret_cast<const DpLayout*>(ctx->d_dp_up + off_lay);
+        lp.live = reinterpret_cast<const uint32_t*>(ctx->d_dp_up + off_live);
+        lp.jobs = reinterpret_cast<const DpJob*>(ctx->d_dp_up + off_jobs);
+        const uint32_t* d_prefix = reinterpret_cast<const uint32_t*>(ctx->d_dp_up + off_prefix);
+        DpLayoutParams yp;
+        memset(&yp, 0, sizeof(yp));
+        yp.layouts = lp.layouts;
+        yp.blk_prefix = reinterpret_cast<const uint32_t*>(ctx->d_dp_up + off_blk);
+        yp.wtab = reinterpret_cast<const uint32_t*>(ctx->d_dp_up + off_w);
+        yp.nxt = d_nxt; yp.n_layouts = (uint32_t)lays.size(); yp.T = T;
+        if (TM == 4) dp_layout_kernel<4><<<lay_blk.back(), DP_THREADS, 0, ctx->stream>>>(yp);
+        else dp_layout_kernel<SAILOR_T_MAX><<<lay_blk.back(), DP_THREADS, 0, ctx->stream>>>(yp);
         CU(ctx, cudaGetLastError());
         ++launches;
-    }
-    // problems that have no entries still get their "no plan" result from the finish step
-    std::vector<DpProblem> stage_buf;
-    std::vector<uint32_t> blk_problem, blk_first;
-    {
-        stage_buf.clear();
-        for (uint64_t j = 0; j < n_problems; ++j)
-            if (!prob[j].n_lvl) stage_buf.push_back(prob[j]);
-        if (!stage_buf.empty()) {
-            CU(ctx, cudaMemcpyAsync(d_problems, stage_buf.data(), stage_buf.size() * sizeof(DpProblem), cudaMemcpyHostToDevice,
-                                    ctx->stream));
-            DpFinishParams fp;
-            memset(&fp, 0, sizeof(fp));
-            fp.blob = ctx->d_blob; fp.avail = ctx->d_avail; fp.sp = d; fp.problems = d_problems; fp.tabs = d_tabs; fp.vtabs = d_vtabs; fp.val[0] = d_val0; fp.val[1] = d_val1; fp.choice = d_choice;
-            fp.results = d_results; fp.lay = lay; fp.n_problems = (uint32_t)stage_buf.size(); fp.T = T;
-            dp_finish_kernel<<<(fp.n_problems + 127) / 128, 128, 0, ctx->stream>>>(fp);
-            CU(ctx, cudaGetLastError());
-            ++launches;
-            CU(ctx, stream_sync(ctx));       // the staging vector is reused below
-        }
-    }
-    for (const Batch& b : batches) {
-        stage_buf.resize(b.count);
-        blk_problem.clear();
-        blk_first.clear();
-        uint64_t val_off = 0, choice_off = 0;
-        uint32_t max_p = 0;
-        std::vector<uint64_t> blocks_upto(p_max + 2, 0);       // entries mode: blocks of problems deeper than a distance
-        std::vector<uint64_t> dist_off(p_max + 2, 0);          // live mode: where the block list of a distance starts
-        for (size_t j = 0; j < b.count; ++j) {
-            DpProblem pb = prob[by_depth[b.first + j]];
-            pb.val_off = val_off;
-            pb.choice_off = choice_off;
-            val_off += pb.n_lvl;
-            choice_off += (uint64_t)pb.n_lvl * pb.P;
-            stage_buf[j] = pb;
-            max_p = pb.P > max_p ? pb.P : max_p;
-            if (!all_live) {
-                const uint32_t nb = (pb.n_lvl + DP_THREADS - 1) / DP_THREADS;
-                for (uint32_t q = 0; q < nb; ++q) { blk_problem.push_back((uint32_t)j); blk_first.push_back(q * DP_THREADS); }
-                for (uint32_t dist = 0; dist < pb.P; ++dist) blocks_upto[dist] += nb;
-            }
-        }
-        std::vector<uint32_t> n_active(p_max + 1, 0), per_thread(p_max + 1, 1);
-        // small problems only (no stage of any problem has more than a few blocks' worth of count vectors): a block
-        // per problem runs all its stages in one launch
-        bool block_per_problem = by_vector;
-        for (size_t j = 0; block_per_problem && j < b.count; ++j) {
-            const uint32_t pj = by_depth[b.first + j];
-            for (uint32_t st = 0; st < prob[pj].P; ++st)
-                if (live_cnt[live_off[pj] + st] > 8u * DP_THREADS) { block_per_problem = false; break; }
-        }
-        if (all_live && !block_per_problem) {                                        // per distance from the last stage: blocks before each problem
-            for (uint32_t dist = 0; dist < max_p; ++dist) {
-                dist_off[dist] = blk_problem.size();
-                uint32_t blocks = 0;
-                if (by_vector) {                               // small launches keep one vector per thread: more blocks
-                    uint64_t vectors = 0;
-                    for (size_t j = 0; j < b.count && prob[by_depth[b.first + j]].P > dist; ++j) {
-                        const uint32_t pj = by_depth[b.first + j];
-                        vectors += live_cnt[live_off[pj] + (prob[pj].P - 1 - dist)];
-                    }
-                    if (vectors >= 16ull * ctx->sm_count * DP_THREADS * DP_VEC_PER_THREAD) per_thread[dist] = DP_VEC_PER_THREAD;
-                }
-                const uint32_t per_block = DP_THREADS * per_thread[dist];
-                for (size_t j = 0; j < b.count; ++j) {
-                    const uint32_t pj = by_depth[b.first + j];
-                    const DpProblem& pb = prob[pj];
-                    if (pb.P <= dist) break;                   // sorted by depth
-                    blk_problem.push_back(blocks);
-                    blocks += (uint32_t)(((uint64_t)live_cnt[live_off[pj] + (pb.P - 1 - dist)] * live_mult + per_block - 1) / per_block);
-                    ++n_active[dist];
-                }
-                blk_problem.push_back(blocks);
-            }
-            dist_off[max_p] = blk_problem.size();
-            blk_first.assign(1, 0);                            // unused in this mode
-        }
-        CU(ctx, cudaMemcpyAsync(d_problems, stage_buf.data(), b.count * sizeof(DpProblem), cudaMemcpyHostToDevice, ctx->stream));
-        if (!blk_problem.empty())
-            CU(ctx, cudaMemcpyAsync(d_blk_problem, blk_problem.data(), blk_problem.size() * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                                    ctx->stream));
-        if (!blk_first.empty())
-            CU(ctx, cudaMemcpyAsync(d_blk_first, blk_first.data(), blk_first.size() * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                                    ctx->stream));
-        DpLevelParams lp;
-        memset(&lp, 0, sizeof(lp));
-        lp.problems = d_problems; lp.blk_problem = d_blk_problem; lp.blk_first = d_blk_first; lp.tabs = d_tabs;
-        lp.vtabs = d_vtabs;
-        lp.val[0] = d_val0; lp.val[1] = d_val1; lp.choice = d_choice; lp.lay = lay; lp.T = T;
-        if (block_per_problem) {
-            if (T <= 4) dp_problem_kernel<4><<<(uint32_t)b.count, DP_THREADS, vt_len_max * 4, ctx->stream>>>(lp);
-            else dp_problem_kernel<SAILOR_T_MAX><<<(uint32_t)b.count, DP_THREADS, vt_len_max * 4, ctx->stream>>>(lp);
+        const uint32_t n_small = (uint32_t)jobs.size() - n_big;
+        if (n_small) {
+            DpLevelParams sp = lp;
+            sp.jobs = lp.jobs + n_big;
+            if (TM == 4) dp_problem_kernel<4><<<n_small, DP_THREADS, 0, ctx->stream>>>(sp);
+            else dp_problem_kernel<SAILOR_T_MAX><<<n_small, DP_THREADS, 0, ctx->stream>>>(sp);
             CU(ctx, cudaGetLastError());
             ++launches;
         }
-        for (uint32_t dist = 0; dist < max_p && !block_per_problem; ++dist) {
+        for (uint32_t dist = 0; dist + 1 < dist_off.size(); ++dist) {
             lp.dist = dist;
-            if (all_live) {
-                const uint32_t n_blk = blk_problem[dist_off[dist] + n_active[dist]];
-                if (n_blk == 0) continue;
-                lp.blk_prefix = d_blk_problem + dist_off[dist];
-                lp.n_active = n_active[dist];
-                lp.per_thread = per_thread[dist];
-                if (by_vector && T <= 4) dp_level_vec_kernel<4><<<n_blk, DP_THREADS, vt_len_max * 4, ctx->stream>>>(lp);
-                else if (by_vector) dp_level_vec_kernel<SAILOR_T_MAX><<<n_blk, DP_THREADS, vt_len_max * 4, ctx->stream>>>(lp);
-                else dp_level_kernel<true><<<n_blk, DP_THREADS, 0, ctx->stream>>>(lp);
-            } else {
-                dp_level_kernel<false><<<(uint32_t)blocks_upto[dist], DP_THREADS, 0, ctx->stream>>>(lp);
-            }
+            lp.blk_prefix = d_prefix + dist_off[dist];
+            lp.n_active = (uint32_t)(dist_off[dist + 1] - dist_off[dist] - 1);
+            const uint32_t n_blk = prefix[dist_off[dist + 1] - 1];
+            if (TM == 4) dp_level_kernel<4><<<n_blk, DP_THREADS, 0, ctx->stream>>>(lp);
+            else dp_level_kernel<SAILOR_T_MAX><<<n_blk, DP_THREADS, 0, ctx->stream>>>(lp);
             CU(ctx, cudaGetLastError());
             ++launches;
         }
         DpFinishParams fp;
         memset(&fp, 0, sizeof(fp));
-        fp.blob = ctx->d_blob; fp.avail = ctx->d_avail; fp.sp = d; fp.problems = d_problems; fp.tabs = d_tabs; fp.vtabs = d_vtabs; fp.val[0] = d_val0; fp.val[1] = d_val1; fp.choice = d_choice;
-        fp.results = d_results; fp.lay = lay; fp.n_problems = (uint32_t)b.count; fp.T = T;
-        dp_finish_kernel<<<(fp.n_problems + 127) / 128, 128, 0, ctx->stream>>>(fp);
+        fp.blob = ctx->d_blob; fp.avail = ctx->d_avail; fp.sp = d; fp.layouts = lp.layouts; fp.jobs = lp.jobs; fp.live = lp.live;
+        fp.tabs = d_tabs; fp.val[0] = lp.val[0]; fp.val[1] = lp.val[1]; fp.succ = lp.succ; fp.value = d_value;
+        fp.results = d_results; fp.lay = lay; fp.n_jobs = (uint32_t)jobs.size(); fp.T = T;
+        dp_finish_kernel<<<(fp.n_jobs + DP_FINISH_THREADS - 1) / DP_FINISH_THREADS, DP_FINISH_THREADS, 0, ctx->stream>>>(fp);
         CU(ctx, cudaGetLastError());
         ++launches;
-        CU(ctx, stream_sync(ctx));           // the host vectors are reused by the next batch
+        up.clear();
     }
     DpSelectParams sel;
     memset(&sel, 0, sizeof(sel));
-    sel.results = d_results; sel.out = d_out; sel.counters = d_counters;
+    sel.value = d_value; sel.results = d_results; sel.out = d_out;
     sel.sp = d; sel.n_problems = (uint32_t)n_problems; sel.n_orders = n_orders; sel.k = k;
     sel.budget = o->budget_usd_per_iter; sel.min_rate = o->min_iters_per_s;
     dp_select_kernel<<<1, DP_SELECT_THREADS, 0, ctx->stream>>>(sel);
     CU(ctx, cudaGetLastError());
     ++launches;
-    CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
-    unsigned long long counters[3] = {0, 0, 0};
-    std::vector<sailor_dp_result> host_out(k);
-    CU(ctx, cudaMemcpyAsync(counters, d_counters, sizeof(counters), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(ctx, cudaMemcpyAsync(host_out.data(), d_out, sizeof(sailor_dp_result) * k, cudaMemcpyDeviceToHost, ctx->stream));
+    if (stats) CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
     CU(ctx, stream_sync(ctx));
+    const unsigned long long* counters = ctx->host->dp.counters;
     if (counters[1] > k) return SAILOR_E_DEVICE;               // cannot happen; never copy past the caller's k records
     *n_found = (uint32_t)counters[1];
-    memcpy(topk, host_out.data(), sizeof(sailor_dp_result) * counters[1]);
+    memcpy(topk, ctx->host->dp.results, sizeof(sailor_dp_result) * counters[1]);
     if (stats) {
         stats->n_problems = n_problems;
         stats->n_solved = counters[0];
@@ -2003,7 +2046,7 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
         CU(ctx, cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
         stats->kernel_ms = ms;
         stats->n_launches = launches;
-        stats->n_batches = (uint32_t)batches.size();
+        stats->n_batches = (uint32_t)std::max<size_t>(batches.size(), 1);
         stats->n_unfinished = 0;
     }
     return SAILOR_OK;

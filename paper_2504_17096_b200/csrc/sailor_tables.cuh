@@ -149,7 +149,7 @@ __host__ __device__ __forceinline__ uint64_t ceil_div64(uint64_t a, uint32_t b) 
 // (Sec. 4.3: M_peak = M_model + M_activation; stage i keeps min(P - i, N_b) microbatches).
 struct StageMem { uint64_t params, mem; };
 
-__device__ __forceinline__ StageMem stage_memory(const TabView& v, uint32_t tpi, uint32_t mi, uint32_t rc,
+__host__ __device__ __forceinline__ StageMem stage_memory(const TabView& v, uint32_t tpi, uint32_t mi, uint32_t rc,
                                                  uint32_t nb, bool e, bool hd, uint64_t inflight) {
     const TabHdr* h = v.h;
     const uint32_t tp = h->tp_values[tpi];

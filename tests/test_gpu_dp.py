@@ -210,6 +210,30 @@ def test_dp_sampled_problems_of_the_large_workloads():
             assert (r.value, r.t_iter, r.cost, r.peak_mem, r.status) == (ref["value"], sim.t_iter, sim.cost, sim.peak_mem, 0)
 
 
+@pytest.mark.parametrize("avail,d_values", [
+    ([[0, 3, 1], [5, 0, 2], [1, 1, 1]], (1,)),             # a zone without some types: passed, or entered by the others only
+    ([[12, 0, 0], [0, 40, 0], [0, 0, 9]], (1, 2)),         # one type per zone, one of them with room for every stage
+    ([[0, 0, 0], [2, 2, 0], [0, 0, 30]], (1, 2)),          # an empty first zone, a tight one, a wide one
+    ([[6, 6, 6], [6, 6, 6], [6, 6, 6]], (1, 6)),           # caps equal to the depth (6) and to one stage
+    ([[5, 7, 60], [3, 3, 3], [60, 60, 60]], (1, 2)),       # counted and uncounted types side by side
+])
+def test_dp_reachable_ranges(avail, d_values):
+    """The ranges of count vectors a stage can have behind it, at their edges: caps of 0, 1, P - 1, P and more; with and
+    without a type too small for any stage."""
+    for small_type in (False, True):
+        w = W.tiny(seed=23, n_types=3, n_zones=3, L=6, p_values=[1, 2, 5, 6], d_values=d_values, tp_values=(1, 2),
+                   mbs_values=(1,), rc_values=(0,))
+        w.avail[...] = np.array(avail, dtype=np.uint16)
+        if small_type:
+            w.capacity[1] = 1                              # fits nothing
+        orders = [[0, 1, 2], [2, 0], [1], [2, 1, 0]]
+        o = Oracle(w)
+        want = oracle_all(w, o, orders)
+        with Ctx(w) as cx:
+            res, st = B.sailor_plan_dp(cx.ctx, cx.space, orders, 32)
+        assert_dp_equal(res, st, want, w, o, orders, 32, f"{avail} {small_type}")
+
+
 def test_dp_constraints_drop_plans_after_the_recursion():
     """A budget or a throughput floor is checked on each problem's plan by the simulator's cost and time."""
     w, orders = W.tiny(seed=3, n_types=3, n_zones=2, L=6, p_values=[1, 2, 3, 6]), [[0, 1], [1, 0]]
