@@ -233,7 +233,7 @@ struct sailor_ctx {
     Hit* d_partial = nullptr;
     uint32_t* d_partial_n = nullptr;
     uint32_t max_grid = 0;                 // capacity of the partial-result buffers
-    uint32_t grid_of[15] = {0};            // resident blocks per kernel variant, for the cached space
+    uint32_t grid_of[30] = {0};            // resident blocks per kernel variant, for the cached space
     SpaceCache space;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr, evh0 = nullptr, evh1 = nullptr;
     cudaStream_t out_stream = nullptr;     // results of a host batch leave on it while the next chunk comes in
@@ -576,29 +576,28 @@ int prepare_space(sailor_ctx* ctx, const sailor_space* s) {
     return SAILOR_OK;
 }
 
-// Chunk that contains flat index f (f < n_total).
-uint32_t chunk_of(const sailor_ctx* ctx, uint64_t f) {
+// Configuration that contains flat index f (f < n_total).
+uint32_t config_at(const sailor_ctx* ctx, uint64_t f) {
     const SpaceCache& sc = ctx->space;
     uint32_t lo = 0, hi = sc.n_config;
     while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) / 2;
         if (sc.flat_base[mid] <= f) lo = mid; else hi = mid;
     }
-    const uint64_t item = (f - sc.flat_base[lo]) / ctx->hdr.R;
-    return sc.chunk_start[lo] + (uint32_t)(item / PLAN_THREADS);
+    return lo;
 }
 
-constexpr int PLAN_VARIANTS = 15;      // objective x constraint x fused, then the three screened kernels
+constexpr int PLAN_VARIANTS = 30;      // (objective x constraint x fused, then the three screened kernels) x every candidate or not
 
-uint32_t variant_of(uint32_t obj, bool constr, bool fused, bool screen = false) {
-    return screen ? 12 + obj : (obj * 2 + (constr ? 1 : 0)) * 2 + (fused ? 1 : 0);
+uint32_t variant_of(uint32_t obj, bool constr, bool fused, bool eval_all, bool screen = false) {
+    return (screen ? 12 + obj : (obj * 2 + (constr ? 1 : 0)) * 2 + (fused ? 1 : 0)) * 2 + (eval_all ? 1 : 0);
 }
 
-PlanKernel pick_kernel(uint32_t obj, bool constr, bool fused, bool screen = false) {
+PlanKernel pick_kernel(uint32_t obj, bool constr, bool fused, bool eval_all, bool screen = false) {
     switch (obj) {
-        case SAILOR_OBJ_MAX_THROUGHPUT: return plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT>(constr, fused, screen);
-        case SAILOR_OBJ_MIN_COST: return plan_kernel_of<SAILOR_OBJ_MIN_COST>(constr, fused, screen);
-        default: return plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT_PER_USD>(constr, fused, screen);
+        case SAILOR_OBJ_MAX_THROUGHPUT: return plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT>(constr, fused, screen, eval_all);
+        case SAILOR_OBJ_MIN_COST: return plan_kernel_of<SAILOR_OBJ_MIN_COST>(constr, fused, screen, eval_all);
+        default: return plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT_PER_USD>(constr, fused, screen, eval_all);
     }
 }
 
@@ -648,7 +647,6 @@ int enqueue_pass(sailor_ctx* ctx, uint32_t obj, double budget, bool budget_from_
     pp.flat_lo = lo;
     pp.flat_hi = hi;
     pp.k = k;
-    pp.eval_all = (flags & SAILOR_FLAG_EVAL_ALL) ? 1u : 0u;
     pp.min_tp_only = (flags & SAILOR_FLAG_MIN_TP_ONLY) ? 1u : 0u;
     pp.cfg_cache = sc.d_cfg_cache;
     pp.cache_head16 = sc.cache_head16;
@@ -674,17 +672,18 @@ int enqueue_pass(sailor_ctx* ctx, uint32_t obj, double budget, bool budget_from_
         pp.live_mode = 1;
         pp.chunk_lo = 0;
         pp.chunk_hi = sc.live_chunks;
-    } else if (hi > lo) {
-        pp.chunk_lo = chunk_of(ctx, lo);
-        pp.chunk_hi = chunk_of(ctx, hi - 1) + 1;
+    } else if (hi > lo) {                 // a range: whole configurations, whose items are not in flat order (run_items)
+        pp.chunk_lo = sc.chunk_start[config_at(ctx, lo)];
+        pp.chunk_hi = sc.chunk_start[config_at(ctx, hi - 1) + 1];
     }
     if (pp.chunk_hi > pp.chunk_lo) {
         const uint32_t n_chunks = waves ? sc.live_chunks : pp.chunk_hi - pp.chunk_lo;
         const bool constr = budget_from_ctrl || budget > 0.0 || min_rate > 0.0;
         const bool screen = (flags & SAILOR_FLAG_F32_SCREEN) != 0;
         const bool fused = !screen && n_chunks <= FUSED_CHUNKS_PER_BLOCK * 2u * (uint32_t)ctx->sm_count;
-        PlanKernel kern = pick_kernel(obj, constr, fused, screen);
-        const uint32_t variant = variant_of(obj, constr, fused, screen);
+        const bool eval_all = (flags & SAILOR_FLAG_EVAL_ALL) != 0;
+        PlanKernel kern = pick_kernel(obj, constr, fused, eval_all, screen);
+        const uint32_t variant = variant_of(obj, constr, fused, eval_all, screen);
         const size_t smem_k = screen ? sc.smem_screen : sc.smem;
         if (smem_k > (size_t)PLAN_SMEM_CEILING) return SAILOR_E_RANGE;
         pp.screen = screen ? 1u : 0u;
@@ -1336,7 +1335,6 @@ int enqueue_pass_noalloc(sailor_ctx* ctx, NoAllocScratch* sc, const SpaceDesc& d
     pp.flat_lo = 0;
     pp.flat_hi = total;
     pp.k = k;
-    pp.eval_all = (flags & SAILOR_FLAG_EVAL_ALL) ? 1u : 0u;
     pp.min_tp_only = (flags & SAILOR_FLAG_MIN_TP_ONLY) ? 1u : 0u;
     pp.budget_from_ctrl = budget_from_ctrl ? 1u : 0u;
     pp.p_max = p_max;
@@ -1350,8 +1348,9 @@ int enqueue_pass_noalloc(sailor_ctx* ctx, NoAllocScratch* sc, const SpaceDesc& d
     pp.cost_only = next_budget_factor > 0.0 ? 1u : 0u;
     const uint32_t n_chunks = chunk_hi - chunk_lo;
     const bool constr = budget_from_ctrl || budget > 0.0 || min_rate > 0.0;
-    PlanKernel kern = pick_kernel(obj, constr, true);
-    const uint32_t variant = variant_of(obj, constr, true);
+    const bool eval_all = (flags & SAILOR_FLAG_EVAL_ALL) != 0;
+    PlanKernel kern = pick_kernel(obj, constr, true, eval_all);
+    const uint32_t variant = variant_of(obj, constr, true, eval_all);
     {
         const int rc_opt = smem_optin(ctx, kern, variant);
         if (rc_opt) return rc_opt;

@@ -73,7 +73,6 @@ struct PlanParams {
     uint32_t chunk_lo, chunk_hi, batch;
     uint64_t flat_lo, flat_hi;
     uint32_t k;
-    uint32_t eval_all;
     uint32_t budget_from_ctrl;         // read the budget from ctrl->budget
     uint32_t p_max;                    // largest P of the space (sizes the stage tables)
     uint32_t live_mode;                // cfg_chunk_start counts only chunks of prefixes made of usable digits
@@ -234,10 +233,13 @@ struct alignas(16) CfgShared {
     uint32_t lower_tpi[SAILOR_TP_MAX];    // their tp indices
     uint64_t lower_fit[SAILOR_TP_MAX][SAILOR_SEG_MAX];   // digit d: every stage of the segment fits at that degree
     uint64_t flat_base;          // flat index of the configuration's first candidate
-    uint64_t _pad_head;
+    uint32_t zone_alike;         // the last segment's records of a type are the same bits in every zone: bit 0 all but
+                                 // the price rate, bit 1 the price rate (what evaluate_zones may share between zones)
+    uint32_t _pad_head;
     // ---- everything above depends on the configuration and the context only, not on availability: it is what a
     // ---- cached record holds (with the arrays rec .. fb_last); everything below belongs to the block or the snapshot
     alignas(16) uint64_t avail_last;     // digit d: need[last] <= avail[d]
+    uint32_t whole;              // all candidates of the configuration lie in the range searched
     uint32_t magic;              // floor(2^32 / R) + 1: x / R == umulhi(x, magic) for x < 2^26
     uint32_t cur_config;
     uint32_t next_chunk, batch_len;
@@ -360,6 +362,7 @@ static __device__ void build_config(const PlanParams& pp, const TabView& v, CfgS
             cs.ar_coef = k.D > 0 ? cs.ar_steps / (double)k.D : 0.0;
             cs.n_items = ipow64(R, k.nseg - 1);
             cs.flat_base = pp.cfg_flat_base[c];
+            cs.zone_alike = 0;
             cs._pad_head = 0;
             cs.packed = 0;             // decided at the end of the build, and only for valid configurations
             cs.cur_config = c;
@@ -483,13 +486,28 @@ static __device__ void build_config(const PlanParams& pp, const TabView& v, CfgS
             if (!((oom_bits >> (8 * (j + 1) + g)) & 1ull))
                 atomicOr(reinterpret_cast<unsigned long long*>(&cs.lower_fit[j][s]), 1ull << d);
     }
-    __syncthreads();                   // the memory masks are complete
+    __syncthreads();                   // the memory masks and the records are complete
+    {
+        const SegRec* recs = a.rec + (k.nseg - 1) * R;
+        bool time_alike = true, rate_alike = true;
+        for (uint32_t d = tid; d < R; d += PLAN_THREADS) {
+            const SegRec &x = recs[d], &y = recs[d % T];
+            for (int q = 0; q < N_RUNS; ++q) time_alike &= x.v[q] == y.v[q];
+            time_alike &= x.tmax == y.tmax && x.sync == y.sync && x.upd == y.upd;
+            rate_alike &= x.rate == y.rate;
+        }
+        const int t_all = __syncthreads_and(time_alike), r_all = __syncthreads_and(rate_alike);
+        if (tid == 0) cs.zone_alike = (t_all ? 1u : 0u) | (r_all ? 2u : 0u);
+    }
     if (tid < 32) {
         const uint32_t last = k.nseg - 1;
         const uint32_t need_last = cs.need[last];
         const uint32_t a_lo = __ballot_sync(FULL, tid < R && need_last <= a.availv[tid < R ? tid : 0]);
         const uint32_t a_hi = __ballot_sync(FULL, tid + 32 < R && need_last <= a.availv[tid + 32 < R ? tid + 32 : 0]);
-        if (tid == 0) cs.avail_last = ((uint64_t)a_hi << 32) | a_lo;
+        if (tid == 0) {
+            cs.avail_last = ((uint64_t)a_hi << 32) | a_lo;
+            cs.whole = cs.flat_base >= pp.flat_lo && cs.flat_base + cs.n_items * R <= pp.flat_hi;
+        }
         if (pp.live_mode) {
             // usable digits per segment (valid type, fits in memory): only prefixes made of them are
             // enumerated; lane d places digit d (and d + 32) at its rank among the set bits
@@ -530,6 +548,7 @@ static __device__ void load_config(const PlanParams& pp, CfgShared& cs, CfgArray
         const uint32_t a_hi = __ballot_sync(FULL, tid + 32 < R && need_last <= a.availv[tid + 32 < R ? tid + 32 : 0]);
         if (tid == 0) {
             cs.avail_last = ((uint64_t)a_hi << 32) | a_lo;
+            cs.whole = cs.flat_base >= pp.flat_lo && cs.flat_base + cs.n_items * R <= pp.flat_hi;
             cs.packed = cs.valid ? pp.live_mode : 0u;
             cs.cur_config = c;
         }
@@ -576,36 +595,61 @@ __device__ __forceinline__ void flush_counters(CfgShared& cs, Counters& cnt, uin
     }
 }
 
-// acc + v + v + ... (n times), one rounding per addition: the stage-by-stage sum of a run.
-__device__ __forceinline__ double add_n(double acc, double v, uint32_t n) {
-#pragma unroll 4
-    for (uint32_t j = 0; j < n; ++j) acc = add_rn(acc, v);
+// The binary32 screen's counterparts of the arithmetic helpers (no NaN occurs).
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float dmax(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ void keep_min(double& least, double x, bool good) { least = (good && x < least) ? x : least; }
+__device__ __forceinline__ void keep_min(float& least, float x, bool good) { least = fminf(least, good ? x : least); }
+
+// acc + v if the (warp-uniform) condition holds: a predicated addition, where the compiler would add and select.
+__device__ __forceinline__ void add_if(double& acc, double v, bool yes) {
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p add.rn.f64 %0, %0, %1;\n\t}" : "+d"(acc) : "d"(v), "r"((uint32_t)yes));
+}
+__device__ __forceinline__ void add_if(float& acc, float v, bool yes) {
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p add.rn.f32 %0, %0, %1;\n\t}" : "+f"(acc) : "f"(v), "r"((uint32_t)yes));
+}
+// acc + v + v + ... (n times, n warp-uniform), one rounding per addition: the stage-by-stage sum of a run.  Runs are
+// mostly short: the first four additions are straight code.
+template <typename F>
+__device__ __forceinline__ F add_n(F acc, F v, uint32_t n) {
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) add_if(acc, v, j < n);
+#pragma unroll 1
+    for (uint32_t j = 4; j < n; ++j) acc = add_rn(acc, v);
     return acc;
 }
 
+// The walk over the last segment's digit is written once for binary64 (F = double) and for the binary32 screen
+// (F = float, from the rounded tables).
+template <typename F> struct RecOf;
+template <> struct RecOf<double> { using type = SegRec; };
+template <> struct RecOf<float> { using type = SegRec32; };
+
 // What a lane carries from its prefix into the walk over the last segment's digit.
+template <typename F>
 struct ItemState {
-    double acc, mx, sy, up, rate, cc;    // running sum / maxima / price rate / transfer cost of the prefix
-    double fb_b;                         // f+b of the prefix's last stage (its message goes to the last digit)
+    F acc, mx, sy, up, rate, cc;         // running sum / maxima / price rate / transfer cost of the prefix
+    F fb_b;                              // f+b of the prefix's last stage (its message goes to the last digit)
     uint64_t ok, walk;                   // per last digit: feasible for this lane / worth visiting for the warp
-    const SegRec* recs;                  // records of the last segment
-    const double* c2x_col;               // c2x[.][d_prev]
-    const double* comm_col;              // commx[.][z_prev]
+    const typename RecOf<F>::type* recs; // records of the last segment
+    const F* c2x_col;                    // c2x[.][d_prev]
+    const F* comm_col;                   // commx[.][z_prev]
 };
 
 // Time and cost of the W candidates that extend item `it` with last digits d .. d+W-1, evaluated
 // side by side (W independent dependency chains; the stage loops run once for all of them).
-template <int NSEG, int N2, int W>
-__device__ __forceinline__ void eval_candidates(const CfgShared& cs, const ItemState& it, uint32_t Z, uint32_t R,
-                                                uint32_t d, double nb, double (&t_iter)[W], double (&cost)[W]) {
+template <int NSEG, int N2, int W, typename F>
+__device__ __forceinline__ void eval_candidates(const CfgShared& cs, const ItemState<F>& it, uint32_t Z, uint32_t R,
+                                                uint32_t d, F nb, F (&t_iter)[W], F (&cost)[W]) {
     constexpr uint32_t last = NSEG - 1;
-    const SegRec* rc = it.recs + d;
-    double t_sum[W], t_max[W], c_comm[W], r[W];
+    const typename RecOf<F>::type* rc = it.recs + d;
+    F t_sum[W], t_max[W], c_comm[W], r[W];
 #pragma unroll
     for (int w = 0; w < W; ++w) {
         t_sum[w] = it.acc; t_max[w] = it.mx; c_comm[w] = it.cc; r[w] = it.rate;
         if (NSEG > 1) {                                   // last stage of the prefix sends to digit d + w
-            const double tb = add_rn(it.fb_b, it.c2x_col[(d + w) * R]);
+            const F tb = add_rn(it.fb_b, it.c2x_col[(d + w) * R]);
             t_sum[w] = add_rn(t_sum[w], tb);
             t_max[w] = dmax(t_max[w], tb);
             c_comm[w] = add_rn(c_comm[w], it.comm_col[(d + w) * Z]);
@@ -636,95 +680,14 @@ __device__ __forceinline__ void eval_candidates(const CfgShared& cs, const ItemS
 #pragma unroll
     for (int w = 0; w < W; ++w) {
         t_max[w] = dmax(t_max[w], rc[w].tmax);
-        const double t_pp = add_rn(t_sum[w], mul_rn(nb, t_max[w]));
+        const F t_pp = add_rn(t_sum[w], mul_rn(nb, t_max[w]));
         t_iter[w] = add_rn(add_rn(t_pp, dmax(it.sy, rc[w].sync)), dmax(it.up, rc[w].upd));
         cost[w] = add_rn(mul_rn(r[w], t_iter[w]), c_comm[w]);
     }
 }
 
-// ---- the binary32 screen: the same walk from the rounded tables ---------------------------------------------
-__device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float fmaxf_sel(float a, float b) { return fmaxf(a, b); }      // one instruction in binary32; no NaN occurs
-
-struct ItemState32 {
-    float acc, mx, sy, up, rate, cc, fb_b;
-    const SegRec32* recs;
-    const float* c2x_col;
-    const float* comm_col;
-};
-
-template <int NSEG, int N2, int W>
-__device__ __forceinline__ void eval_candidates32(const CfgShared& cs, const ItemState32& it, uint32_t Z, uint32_t R,
-                                                  uint32_t d, float nb, float (&t_iter)[W], float (&cost)[W]) {
-    constexpr uint32_t last = NSEG - 1;
-    const SegRec32* rc = it.recs + d;
-    float t_sum[W], t_max[W], c_comm[W], r[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-        t_sum[w] = it.acc; t_max[w] = it.mx; c_comm[w] = it.cc; r[w] = it.rate;
-        if (NSEG > 1) {
-            const float tb = fadd(it.fb_b, it.c2x_col[(d + w) * R]);
-            t_sum[w] = fadd(t_sum[w], tb);
-            t_max[w] = fmaxf_sel(t_max[w], tb);
-            c_comm[w] = fadd(c_comm[w], it.comm_col[(d + w) * Z]);
-        }
-    }
-#define SAILOR_STAGE32(RUN)                                                        \
-    _Pragma("unroll") for (int w = 0; w < W; ++w) {                                \
-        t_sum[w] = fadd(t_sum[w], rc[w].v[RUN]);                                   \
-        r[w] = fadd(r[w], rc[w].rate);                                             \
-    }
-    if (N2 >= 0) {
-#pragma unroll
-        for (int j = 0; j < N2; ++j) { SAILOR_STAGE32(2) }
-        SAILOR_STAGE32(3)
-    } else {
-        const uint32_t n0 = cs.n_run[last][0], n1 = cs.n_run[last][1], n2 = cs.n_run[last][2], n3 = cs.n_run[last][3];
-        if (n0) { SAILOR_STAGE32(0) }
-        for (uint32_t j = 0; j < n1; ++j) { SAILOR_STAGE32(1) }
-        uint32_t j = n2;
-        for (; j >= 4; j -= 4) { SAILOR_STAGE32(2) SAILOR_STAGE32(2) SAILOR_STAGE32(2) SAILOR_STAGE32(2) }
-        if (j & 2) { SAILOR_STAGE32(2) SAILOR_STAGE32(2) }
-        if (j & 1) { SAILOR_STAGE32(2) }
-        if (n3) { SAILOR_STAGE32(3) }
-    }
-#undef SAILOR_STAGE32
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-        t_max[w] = fmaxf_sel(t_max[w], rc[w].tmax);
-        const float t_pp = fadd(t_sum[w], fmul(nb, t_max[w]));
-        t_iter[w] = fadd(fadd(t_pp, fmaxf_sel(it.sy, rc[w].sync)), fmaxf_sel(it.up, rc[w].upd));
-        cost[w] = fadd(fmul(r[w], t_iter[w]), c_comm[w]);
-    }
-}
-
-// Binary32 pass over the candidates of one item: the lane's best score and cheapest cost, both approximate.
-template <int NSEG, int OBJ, int N2>
-__device__ __forceinline__ void walk_fast32(const CfgShared& cs, const ItemState32& it, uint64_t ok, uint64_t walk,
-                                            uint32_t Z, uint32_t R, float& best, float& min_cost) {
-    const float nb = (float)cs.n_b;
-    constexpr uint32_t U = PLAN_DIGITS_PER_STEP;
-    for (uint32_t half = 0; half * 32 < R; ++half) {
-        const uint32_t wm = (uint32_t)(walk >> (32 * half)), om = (uint32_t)(ok >> (32 * half));
-        const uint32_t d_end = min(R - 32 * half, 32u);
-        for (uint32_t dd = 0; dd < d_end; dd += U) {
-            if (!((wm >> dd) & ((1u << U) - 1u))) continue;   // warp-uniform
-            float t[U], c[U];
-            eval_candidates32<NSEG, N2, (int)U>(cs, it, Z, R, 32 * half + dd, nb, t, c);
-#pragma unroll
-            for (uint32_t u = 0; u < U; ++u) {
-                const bool g = (om >> (dd + u)) & 1u;
-                const float sc = OBJ == SAILOR_OBJ_MAX_THROUGHPUT ? t[u] : OBJ == SAILOR_OBJ_MIN_COST ? c[u] : fmul(t[u], c[u]);
-                min_cost = fminf(min_cost, g ? c[u] : min_cost);
-                best = fminf(best, g ? sc : best);
-            }
-        }
-    }
-}
-
-template <int OBJ>
-__device__ __forceinline__ double score_of(double t_iter, double cost) {
+template <int OBJ, typename F>
+__device__ __forceinline__ F score_of(F t_iter, F cost) {
     return OBJ == SAILOR_OBJ_MAX_THROUGHPUT ? t_iter : OBJ == SAILOR_OBJ_MIN_COST ? cost : mul_rn(t_iter, cost);
 }
 
@@ -741,11 +704,11 @@ __device__ __forceinline__ bool within(const PlanParams& pp, double budget, doub
 // Fast pass over the candidates of one item, several digits per step (independent dependency
 // chains per thread): tracks the lane's best score, the feasible count and the cheapest cost.
 // No votes, no list updates.  Tables are padded, so a step may read (and mask out) digits >= R.
-template <int NSEG, int OBJ, bool CONSTR, int N2>
-__device__ __forceinline__ void walk_fast(const PlanParams& pp, const CfgShared& cs, const ItemState& it,
-                                          uint32_t Z, uint32_t R, double budget, double& best, uint32_t& feas,
-                                          double& min_cost) {
-    const double nb = (double)cs.n_b;
+template <int NSEG, int OBJ, bool CONSTR, int N2, typename F>
+__device__ __forceinline__ void walk_fast(const PlanParams& pp, const CfgShared& cs, const ItemState<F>& it,
+                                          uint32_t Z, uint32_t R, double budget, F& best, uint32_t& feas,
+                                          F& min_cost) {
+    const F nb = (F)cs.n_b;
     constexpr uint32_t U = PLAN_DIGITS_PER_STEP;
     for (uint32_t half = 0; half * 32 < R; ++half) {
         const uint32_t wm = (uint32_t)(it.walk >> (32 * half)), om = (uint32_t)(it.ok >> (32 * half));
@@ -753,24 +716,166 @@ __device__ __forceinline__ void walk_fast(const PlanParams& pp, const CfgShared&
         for (uint32_t dd = 0; dd < d_end; dd += U) {
             if (!((wm >> dd) & ((1u << U) - 1u))) continue;   // warp-uniform
             const uint32_t d = 32 * half + dd;
-            double t[U], c[U];
+            F t[U], c[U];
             eval_candidates<NSEG, N2, (int)U>(cs, it, Z, R, d, nb, t, c);
 #pragma unroll
             for (uint32_t u = 0; u < U; ++u) {
                 const bool g = ((om >> (dd + u)) & 1u) && within<CONSTR>(pp, budget, t[u], c[u]);
-                const double sc = score_of<OBJ>(t[u], c[u]);
                 if (CONSTR) feas += (uint32_t)g;
-                min_cost = (g && c[u] < min_cost) ? c[u] : min_cost;
-                best = (g && sc < best) ? sc : best;
+                keep_min(min_cost, c[u], g);
+                keep_min(best, score_of<OBJ>(t[u], c[u]), g);
             }
         }
     }
 }
 
+// The bulk of every space has four segments: call `walk` with the shape of the last one as a constant where it is a
+// common one (N2 >= 0: that many plain stages, then the final stage, nothing else), which makes the candidate loop
+// straight-line code; -1 is the general form.
+template <int N> struct Shape { static constexpr int value = N; };
+template <int NSEG, typename Walk>
+__device__ __forceinline__ void by_shape(const CfgShared& cs, Walk walk) {
+    if (NSEG == SAILOR_SEG_MAX && cs.n_run[3][0] == 0 && cs.n_run[3][1] == 0 && cs.n_run[3][3] == 1) {
+        switch (cs.n_run[3][2]) {
+            case 0: walk(Shape<0>()); return;
+            case 1: walk(Shape<1>()); return;
+            case 2: walk(Shape<2>()); return;
+            case 3: walk(Shape<3>()); return;
+            default: break;
+        }
+    }
+    walk(Shape<-1>());
+}
+
+// ---- items without a feasible candidate, when every candidate's time and cost is asked for ----------------------
+//
+// SAILOR_FLAG_EVAL_ALL wants the time and the cost of every candidate formed, also of those that are invalid, out of
+// memory or over the availability.  Where no lane of the warp has a feasible candidate (98 % of workload 5) nothing is
+// selected from them, so no masks and no minima are formed; the values are only checked for what non-negative tables
+// cannot give, a set sign bit (one three-input OR a candidate).
+__device__ __forceinline__ void evaluated(uint32_t& signs, double t, double c) {
+    signs |= (uint32_t)__double2hiint(t) | (uint32_t)__double2hiint(c);
+}
+__device__ __forceinline__ void evaluated(uint32_t& signs, float t, float c) { signs |= __float_as_uint(t) | __float_as_uint(c); }
+
+// The candidates of W zones that are not the prefix's own and (OWN) of the one that is.  A digit is a (zone, type) pair:
+// the message from the prefix, and with it the running sum, the maximum and the transfer cost up to the last segment,
+// depend on the zone alone unless it is the prefix's own, so these heads are formed once per zone and kept in registers;
+// where a type's record is alike in all zones (CfgShared::zone_alike) it is read once for all of them, and the maxima over
+// synchronisation and update times and (RATE) the price-rate sum are formed once.  n_b x max(a, b) is taken as
+// max(n_b x a, n_b x b): rounding is monotone, so these are the same bits; a transfer cost of zero is not added.  Every
+// candidate still takes its own additions over the segment's stages, in stage order, and its own closing terms: the bits
+// are those of eval_candidates.  N2 >= 0: the segment is N2 plain stages and the final stage (straight code); -1: any.
+// Bound: issue slots (64 % busy) and the FP64 pipe (52 %): 6 + (stages of the segment) FP64 instructions a candidate
+// against 14 + 2 x (stages) digit by digit.  Workload 5, 6.4e9 candidates: 13.89 -> 7.30 ms, 55.9 -> 26.9
+// lane-instructions a candidate, about 7 of them what an item costs before its candidates (digits, masks, prefix sums).
+template <int N2, int W, bool RATE, bool OWN, typename F>
+__device__ __forceinline__ void evaluate_zones(const CfgShared& cs, const ItemState<F>& it, uint32_t T, uint32_t Z, uint32_t R,
+                                               uint32_t z_own, uint32_t first, F nb, uint32_t& signs) {
+    constexpr uint32_t last = SAILOR_SEG_MAX - 1;
+    constexpr int S = W + (OWN ? 1 : 0);
+    F hs[S], hm[S], hc[S];
+    uint32_t dz[S];
+    if (OWN) { dz[S - 1] = z_own * T; hc[S - 1] = it.cc; }
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        const uint32_t j = first + w;
+        dz[w] = (j + (j >= z_own ? 1u : 0u)) * T;
+        const F tb = add_rn(it.fb_b, it.c2x_col[dz[w] * R]);
+        hs[w] = add_rn(it.acc, tb);
+        hm[w] = mul_rn(nb, dmax(it.mx, tb));
+        hc[w] = add_rn(it.cc, it.comm_col[dz[w] * Z]);
+    }
+    const F* own = it.c2x_col + z_own * T * R;
+    // the last of four segments: stages with an extra block, plain stages, the final stage
+    const uint32_t n1 = N2 >= 0 ? 0u : cs.n_run[last][1], n2 = N2 >= 0 ? (uint32_t)N2 : cs.n_run[last][2], n = n1 + n2 + 1;
+#pragma unroll 1
+    for (uint32_t g = 0; g < T; ++g) {
+        const typename RecOf<F>::type* rc = it.recs + g;
+        const F v1 = rc->v[1], v2 = rc->v[2], v3 = rc->v[3];
+        if (OWN) {
+            const F tb = add_rn(it.fb_b, own[g * R]);
+            hs[S - 1] = add_rn(it.acc, tb);
+            hm[S - 1] = mul_rn(nb, dmax(it.mx, tb));
+        }
+        F t_sum[S], r = it.rate;
+        if (N2 >= 0) {
+#pragma unroll
+            for (int w = 0; w < S; ++w) {
+                t_sum[w] = hs[w];
+#pragma unroll
+                for (int j = 0; j < N2; ++j) t_sum[w] = add_rn(t_sum[w], v2);
+                t_sum[w] = add_rn(t_sum[w], v3);
+            }
+            if (RATE)
+#pragma unroll
+                for (int j = 0; j <= N2; ++j) r = add_rn(r, rc->rate);
+        } else {
+            const F v0 = n1 ? v1 : n2 ? v2 : v3;
+#pragma unroll
+            for (int w = 0; w < S; ++w) t_sum[w] = add_rn(hs[w], v0);
+#pragma unroll 1
+            for (uint32_t j = 1; j < n; ++j) {
+                const F v = j < n1 ? v1 : j + 1 < n ? v2 : v3;
+#pragma unroll
+                for (int w = 0; w < S; ++w) t_sum[w] = add_rn(t_sum[w], v);
+            }
+            if (RATE) r = add_n(r, rc->rate, n);
+        }
+        const F tm = mul_rn(nb, rc->tmax), sy = dmax(it.sy, rc->sync), up = dmax(it.up, rc->upd);
+#pragma unroll
+        for (int w = 0; w < S; ++w) {
+            const F t = add_rn(add_rn(add_rn(t_sum[w], dmax(hm[w], tm)), sy), up);
+            if (!RATE) r = add_n(it.rate, rc[dz[w]].rate, n);
+            evaluated(signs, t, add_rn(mul_rn(r, t), hc[w]));
+        }
+    }
+}
+
+// All candidates of an item of a four-segment configuration; `z_prev` is the zone the lane's prefix sends from.  Returns
+// the values' sign bits (bit 31).
+template <typename F>
+__device__ __forceinline__ uint32_t evaluate_only(const CfgShared& cs, const ItemState<F>& it, uint32_t T, uint32_t Z, uint32_t R,
+                                                  bool active, uint32_t z_prev) {
+    constexpr int NSEG = SAILOR_SEG_MAX;
+    const F nb = (F)cs.n_b;
+    const uint32_t lanes = __ballot_sync(FULL, active);
+    const uint32_t z_own = __shfl_sync(FULL, z_prev, lanes ? __ffs(lanes) - 1 : 0);
+    const bool by_zone = (cs.zone_alike & 1u) && __all_sync(FULL, !active || z_prev == z_own);
+    uint32_t signs = 0;
+    if (!by_zone || Z == 1) {
+        constexpr uint32_t U = PLAN_DIGITS_PER_STEP;       // (the tables are padded)
+        for (uint32_t d = 0; d < R; d += U) {
+            F t[U], c[U];
+            eval_candidates<NSEG, -1, (int)U>(cs, it, Z, R, d, nb, t, c);
+#pragma unroll
+            for (uint32_t u = 0; u < U; ++u) evaluated(signs, t[u], c[u]);
+        }
+        return signs;
+    }
+    // the first group takes the prefix's own zone along
+    const bool rate = (cs.zone_alike & 2u) != 0;
+    uint32_t j;
+    if (Z > 7) {
+        if (rate) by_shape<NSEG>(cs, [&](auto shape) { evaluate_zones<decltype(shape)::value, 7, true, true>(cs, it, T, Z, R, z_own, 0, nb, signs); });
+        else evaluate_zones<-1, 7, false, true>(cs, it, T, Z, R, z_own, 0, nb, signs);
+        j = 7;
+    } else if (Z > 4) {
+        if (rate) by_shape<NSEG>(cs, [&](auto shape) { evaluate_zones<decltype(shape)::value, 4, true, true>(cs, it, T, Z, R, z_own, 0, nb, signs); });
+        else evaluate_zones<-1, 4, false, true>(cs, it, T, Z, R, z_own, 0, nb, signs);
+        j = 4;
+    } else {
+        evaluate_zones<-1, 1, false, true>(cs, it, T, Z, R, z_own, 0, nb, signs);
+        j = 1;
+    }
+    for (; j + 1 < Z; ++j) evaluate_zones<-1, 1, false, false>(cs, it, T, Z, R, z_own, j, nb, signs);
+    return signs;
+}
+
 // Rare second pass over an item: the same arithmetic, one digit at a time, and every candidate that
 // may enter the warp's top-k list is offered to it (warp-synchronous).  Nothing is counted.
 template <int NSEG, int OBJ, bool CONSTR, int N2>
-__device__ __forceinline__ void walk_offer(const PlanParams& pp, const CfgShared& cs, const ItemState& it,
+__device__ __forceinline__ void walk_offer(const PlanParams& pp, const CfgShared& cs, const ItemState<double>& it,
                                            uint32_t Z, uint32_t R, double budget, uint64_t item_flat,
                                            WarpTopK& top, uint32_t lane, double outer_thr, double& min_cost) {
     const double nb = (double)cs.n_b;
@@ -788,118 +893,126 @@ __device__ __forceinline__ void walk_offer(const PlanParams& pp, const CfgShared
 }
 
 // One item per lane: fixed prefix digits, walk the last segment's digit.
-// N2 >= 0 fixes the shape of the last segment at compile time (N2 plain stages, then the final
-// stage, nothing else), which makes the candidate loop straight-line code; N2 < 0 is the general form.
-template <int NSEG, int OBJ, bool CONSTR, int N2, bool SCREEN>
+// EVAL: the time and cost of every candidate is wanted (SAILOR_FLAG_EVAL_ALL).
+template <int NSEG, int OBJ, bool CONSTR, bool SCREEN, bool EVAL>
 __device__ __forceinline__ void run_items(const PlanParams& pp, const CfgShared& cs, const CfgArrays& a,
                                           uint32_t T, uint32_t Z, uint32_t R, uint32_t q, bool active,
-                                          uint64_t item_flat, double budget, WarpTopK& top, Counters& cnt,
-                                          uint32_t lane) {
+                                          double budget, WarpTopK& top, Counters& cnt, uint32_t lane) {
     constexpr uint32_t last = NSEG - 1;
     // ---- prefix: segments 0 .. NSEG-2 --------------------------------------------------------
+    // EVAL: the digit of the prefix's last segment varies slowest over the items of a configuration, so that the lanes of
+    // a warp nearly always send to the last segment from one zone (evaluate_only relies on it).  Otherwise it varies
+    // fastest: the lanes' prefixes then share their first digits, and with them most of what makes a prefix fail.
+    constexpr int SLOWEST = EVAL && NSEG > 1 ? NSEG - 2 : 0, FASTEST = EVAL ? NSEG - 3 : NSEG - 2;
     uint32_t dg[NSEG > 1 ? NSEG - 1 : 1];
     {
         uint32_t x = active ? q : 0;
-        if (cs.packed) {                                   // mixed radix over the usable digits of each segment
-#pragma unroll
-            for (int s = NSEG - 2; s >= 0; --s) {
+        auto peel = [&](int s, bool rest) {                // mixed radix, over the usable digits of each segment when packed
+            if (cs.packed) {
                 const uint32_t n = cs.g_cnt[s];
-                const uint32_t y = n > 1 ? __umulhi(x, cs.g_magic[s]) : x;   // x / n
+                const uint32_t y = rest ? 0u : n > 1 ? __umulhi(x, cs.g_magic[s]) : x;   // x / n
                 dg[s] = active ? cs.good_list[s][x - y * n] : 0u;
                 x = y;
-            }
-        } else {
-#pragma unroll
-            for (int s = NSEG - 2; s >= 0; --s) {
-                const uint32_t y = R == 1 ? x : __umulhi(x, cs.magic);     // x / R
+            } else {
+                const uint32_t y = rest ? 0u : R == 1 ? x : __umulhi(x, cs.magic);     // x / R
                 dg[s] = x - y * R;
                 x = y;
             }
+        };
+        if (NSEG > 1) {
+#pragma unroll
+            for (int s = FASTEST; s >= (EVAL ? 0 : 1); --s) peel(s, false);
+            peel(SLOWEST, true);
         }
     }
-    if (cs.packed) {                                       // the item's flat index follows from its digits
+    uint64_t item_flat = cs.flat_base;                     // the item's flat index follows from its digits
+    {
         uint64_t pf = 0;
 #pragma unroll
         for (int s = 0; s < NSEG - 1; ++s) pf = pf * R + dg[s];
-        item_flat = cs.flat_base + pf * R;
+        item_flat += pf * R;
     }
-    // ---- status of the prefix: node validity, memory, availability (integer work only) ------------
-    bool p_inv = false, p_oom = false, p_over = false;
+    // ---- status of the prefix: node validity and memory (integer work only) -------------------------
+    bool p_inv = false, p_oom = false;
 #pragma unroll
     for (int s = 0; s < NSEG - 1; ++s) {
-        const uint32_t d = dg[s];
-        p_inv |= (cs.invalid_mask >> d) & 1;
-        p_oom |= (cs.oom_mask[s] >> d) & 1;
-        uint32_t tot = 0;                                 // demand of this digit over the prefix
-#pragma unroll
-        for (int s2 = 0; s2 < NSEG - 1; ++s2) tot += (dg[s2] == d) ? cs.need[s2] : 0u;
-        p_over |= tot > a.availv[d];
+        p_inv |= (cs.invalid_mask >> dg[s]) & 1;
+        p_oom |= (cs.oom_mask[s] >> dg[s]) & 1;
     }
     // ---- which last digits are in range / valid / fit / available ------------------------------
     uint64_t range = R == 64 ? ~0ull : ((1ull << R) - 1);
-    if (item_flat < pp.flat_lo) {
-        const uint64_t skip = pp.flat_lo - item_flat;
-        range = skip >= 64 ? 0 : range & (~0ull << skip);
-    }
-    if (item_flat + R > pp.flat_hi) {
-        const uint64_t keep = pp.flat_hi > item_flat ? pp.flat_hi - item_flat : 0;
-        range = keep >= 64 ? range : range & ((1ull << keep) - 1);
+    if (!cs.whole) {                                       // (a configuration that lies in the range as a whole skips this)
+        if (item_flat < pp.flat_lo) {
+            const uint64_t skip = pp.flat_lo - item_flat;
+            range = skip >= 64 ? 0 : range & (~0ull << skip);
+        }
+        if (item_flat + R > pp.flat_hi) {
+            const uint64_t keep = pp.flat_hi > item_flat ? pp.flat_hi - item_flat : 0;
+            range = keep >= 64 ? range : range & ((1ull << keep) - 1);
+        }
     }
     if (!active) range = 0;
     const uint64_t valid_l = range & ~cs.invalid_mask;
-    const uint64_t fit_l = valid_l & ~cs.oom_mask[last];
-    uint64_t drop = 0;            // last digits at which the whole plan also fits with a smaller degree
-    if (pp.min_tp_only)
-        for (uint32_t j = 0; j < cs.n_lower; ++j) {
-            bool pf = true;
-#pragma unroll
-            for (int s = 0; s < NSEG - 1; ++s) pf &= (cs.lower_fit[j][s] >> dg[s]) & 1;
-            if (pf) drop |= cs.lower_fit[j][last];
-        }
-    const uint64_t good_l = fit_l & ~drop;
-    uint64_t ok = good_l & cs.avail_last;
-#pragma unroll
-    for (int s = 0; s < NSEG - 1; ++s) {                  // a last digit equal to a prefix digit adds up
-        const uint32_t d = dg[s];
-        uint32_t tot = cs.need[last];
-#pragma unroll
-        for (int s2 = 0; s2 < NSEG - 1; ++s2) tot += (dg[s2] == d) ? cs.need[s2] : 0u;
-        if (tot > a.availv[d]) ok &= ~(1ull << d);
-    }
-    // exactly one class per candidate: invalid, then oom, then over availability
-    const uint32_t n_range = __popcll(range);
-    if (cs.packed) {                                      // total, invalid and oom were added in closed form
-        cnt.pruned += __popcll(fit_l) - __popcll(good_l);
-        if (p_over) { cnt.over_avail += __popcll(good_l); ok = 0; }
-        else cnt.over_avail += __popcll(good_l) - __popcll(ok);
-    } else if (p_inv) { cnt.total += n_range; cnt.invalid += n_range; ok = 0; }
-    else {
+    uint64_t ok = 0;
+    uint32_t n_ok = 0;
+    // exactly one class per candidate: invalid, then oom, then over availability (packed: total, invalid and oom were
+    // added in closed form)
+    if (!cs.packed) {
+        const uint32_t n_range = __popcll(range);
         cnt.total += n_range;
-        cnt.invalid += n_range - __popcll(valid_l);
-        if (p_oom) { cnt.oom += __popcll(valid_l); ok = 0; }
+        if (p_inv) cnt.invalid += n_range;
         else {
-            cnt.oom += __popcll(valid_l) - __popcll(fit_l);
-            cnt.pruned += __popcll(fit_l) - __popcll(good_l);
-            if (p_over) { cnt.over_avail += __popcll(good_l); ok = 0; }
-            else cnt.over_avail += __popcll(good_l) - __popcll(ok);
+            const uint32_t n_valid = __popcll(valid_l);
+            cnt.invalid += n_range - n_valid;
+            cnt.oom += p_oom ? n_valid : (uint32_t)__popcll(valid_l & cs.oom_mask[last]);
         }
     }
-    const uint32_t n_ok = __popcll(ok);
-    if (!CONSTR) cnt.feasible += n_ok;
+    if (__any_sync(FULL, active && !p_inv && !p_oom)) {    // no lane gets further in most warps of an unpruned search
+        const uint64_t fit_l = p_inv || p_oom ? 0ull : valid_l & ~cs.oom_mask[last];
+        uint64_t drop = 0;        // last digits at which the whole plan also fits with a smaller degree
+        if (pp.min_tp_only)
+            for (uint32_t j = 0; j < cs.n_lower; ++j) {
+                bool pf = true;
+#pragma unroll
+                for (int s = 0; s < NSEG - 1; ++s) pf &= (cs.lower_fit[j][s] >> dg[s]) & 1;
+                if (pf) drop |= cs.lower_fit[j][last];
+            }
+        const uint64_t good_l = fit_l & ~drop;
+        cnt.pruned += __popcll(fit_l) - __popcll(good_l);
+        bool p_over = false;
+        uint32_t tot[NSEG > 1 ? NSEG - 1 : 1];             // demand of a prefix digit over the prefix
+#pragma unroll
+        for (int s = 0; s < NSEG - 1; ++s) {
+            tot[s] = 0;
+#pragma unroll
+            for (int s2 = 0; s2 < NSEG - 1; ++s2) tot[s] += (dg[s2] == dg[s]) ? cs.need[s2] : 0u;
+            p_over |= tot[s] > a.availv[dg[s]];
+        }
+        ok = p_over ? 0ull : good_l & cs.avail_last;
+        if (__any_sync(FULL, ok != 0)) {
+#pragma unroll
+            for (int s = 0; s < NSEG - 1; ++s)             // a last digit equal to a prefix digit adds up
+                if (cs.need[last] + tot[s] > a.availv[dg[s]]) ok &= ~(1ull << dg[s]);
+        }
+        n_ok = __popcll(ok);
+        cnt.over_avail += __popcll(good_l) - n_ok;
+        if (!CONSTR) cnt.feasible += n_ok;
+    }
 
     // ---- the candidates -----------------------------------------------------------------------
-    const uint64_t walk = pp.eval_all ? warp_or64(range) : warp_or64(ok);   // warp-uniform: skip dead digits
-    if (walk == 0) {                                      // nothing to evaluate for any lane of the warp
-        return;
-    }
+    const bool none_ok = !__any_sync(FULL, n_ok != 0);     // then a warp goes on only because every candidate is wanted
+    if (none_ok && !(EVAL && __any_sync(FULL, range != 0))) return;
+    const uint64_t walk = warp_or64(EVAL ? range : ok);    // warp-uniform: skip dead digits
     // ---- running sums of the prefix, in stage order ---------------------------------------------
     double acc = 0.0, mx = 0.0, sy = 0.0, up = 0.0, rate = 0.0, cc = 0.0;
 #pragma unroll
     for (int s = 0; s < NSEG - 1; ++s) {
         const uint32_t d = dg[s];
         const SegRec& rc = a.rec[s * R + d];
-#pragma unroll
-        for (int r = 0; r < N_RUNS - 1; ++r) acc = add_n(acc, rc.v[r], cs.n_run[s][r]);   // run 3 is the final stage
+        // (run 0 is the stage with the embedding, so the first segment's; run 3 is the final stage)
+        if (s == 0 && cs.n_run[0][0]) acc = add_rn(acc, rc.v[0]);
+        if (cs.n_run[s][1]) acc = add_n(acc, rc.v[1], cs.n_run[s][1]);
+        acc = add_n(acc, rc.v[2], cs.n_run[s][2]);
         mx = dmax(mx, rc.tmax);
         sy = dmax(sy, rc.sync);
         up = dmax(up, rc.upd);
@@ -912,7 +1025,7 @@ __device__ __forceinline__ void run_items(const PlanParams& pp, const CfgShared&
             cc = add_rn(cc, a.commx[dn * Z + (a.tz[d] >> 8)]);
         }
     }
-    ItemState it;
+    ItemState<double> it;
     it.acc = acc; it.mx = mx; it.sy = sy; it.up = up; it.rate = rate; it.cc = cc;
     it.ok = ok;
     it.walk = walk;
@@ -929,23 +1042,34 @@ __device__ __forceinline__ void run_items(const PlanParams& pp, const CfgShared&
 
     if (SCREEN) {
         // binary32 first; the item is walked exactly only if it may hold a member of the top-k or the cheapest plan
-        ItemState32 s32;
+        ItemState<float> s32;
         s32.acc = __double2float_rn(acc); s32.mx = __double2float_rn(mx); s32.sy = __double2float_rn(sy);
         s32.up = __double2float_rn(up); s32.rate = __double2float_rn(rate); s32.cc = __double2float_rn(cc);
         s32.fb_b = __double2float_rn(it.fb_b);
+        s32.ok = ok;
+        s32.walk = walk;
         s32.recs = a.rec32 + last * R;
         s32.c2x_col = a.c2x32 + d_prev;
         s32.comm_col = a.commx32 + z_prev;
+        if (EVAL && NSEG == SAILOR_SEG_MAX && none_ok) {
+            if ((int)evaluate_only(cs, s32, T, Z, R, active, z_prev) < 0) pp.ctrl->error = 1u;
+            return;
+        }
         const float f_inf = __int_as_float(0x7f800000);
         float best32 = f_inf, minc32 = f_inf;
-        walk_fast32<NSEG, OBJ, N2>(cs, s32, ok, walk, Z, R, best32, minc32);
+        uint32_t none = 0;
+        by_shape<NSEG>(cs, [&](auto shape) {
+            walk_fast<NSEG, OBJ, false, decltype(shape)::value>(pp, cs, s32, Z, R, budget, best32, none, minc32);
+        });
         const double outer_thr = __longlong_as_double((long long)*reinterpret_cast<const volatile unsigned long long*>(&cs.thr_bits));
         const double outer_minc = __longlong_as_double((long long)*reinterpret_cast<const volatile unsigned long long*>(&cs.minc_bits));
         const double thr = top.thr_score < outer_thr ? top.thr_score : outer_thr;
         const bool need = best32 < f_inf && ((double)best32 <= thr * (1.0 + SCREEN_BAND) || (double)minc32 <= outer_minc * (1.0 + SCREEN_BAND));
         if (__any_sync(FULL, need)) {
             const double before = top.thr_score, mc_before = cnt.min_cost;
-            walk_offer<NSEG, OBJ, CONSTR, N2>(pp, cs, it, Z, R, budget, item_flat, top, lane, outer_thr, cnt.min_cost);
+            by_shape<NSEG>(cs, [&](auto shape) {
+                walk_offer<NSEG, OBJ, CONSTR, decltype(shape)::value>(pp, cs, it, Z, R, budget, item_flat, top, lane, outer_thr, cnt.min_cost);
+            });
             if (lane == 0 && top.thr_score < before)
                 atomicMin(const_cast<unsigned long long*>(&cs.thr_bits), (unsigned long long)__double_as_longlong(top.thr_score));
             if (cnt.min_cost < mc_before)
@@ -953,10 +1077,16 @@ __device__ __forceinline__ void run_items(const PlanParams& pp, const CfgShared&
         }
         return;
     }
+    if (EVAL && NSEG == SAILOR_SEG_MAX && none_ok) {
+        if ((int)evaluate_only(cs, it, T, Z, R, active, z_prev) < 0) pp.ctrl->error = 1u;      // cannot happen
+        return;
+    }
     // fast pass: no votes, no list updates; each lane keeps its item's best score
     double best = make_inf();
     uint32_t feas = 0;
-    walk_fast<NSEG, OBJ, CONSTR, N2>(pp, cs, it, Z, R, budget, best, feas, cnt.min_cost);
+    by_shape<NSEG>(cs, [&](auto shape) {
+        walk_fast<NSEG, OBJ, CONSTR, decltype(shape)::value>(pp, cs, it, Z, R, budget, best, feas, cnt.min_cost);
+    });
     cnt.cfg_best = best < cnt.cfg_best ? best : cnt.cfg_best;
     if (CONSTR) {
         cnt.feasible += feas;
@@ -968,7 +1098,9 @@ __device__ __forceinline__ void run_items(const PlanParams& pp, const CfgShared&
     const double outer_thr = __longlong_as_double((long long)*reinterpret_cast<const volatile unsigned long long*>(&cs.thr_bits));
     if (!pp.cost_only && __any_sync(FULL, best < make_inf() && best <= top.thr_score && best <= outer_thr)) {   // best == inf: no feasible candidate
         const double before = top.thr_score;
-        walk_offer<NSEG, OBJ, CONSTR, N2>(pp, cs, it, Z, R, budget, item_flat, top, lane, outer_thr, cnt.min_cost);
+        by_shape<NSEG>(cs, [&](auto shape) {
+            walk_offer<NSEG, OBJ, CONSTR, decltype(shape)::value>(pp, cs, it, Z, R, budget, item_flat, top, lane, outer_thr, cnt.min_cost);
+        });
         if (lane == 0 && top.thr_score < before)
             atomicMin(const_cast<unsigned long long*>(&cs.thr_bits), (unsigned long long)__double_as_longlong(top.thr_score));
     }
@@ -1130,7 +1262,7 @@ static __device__ __noinline__ void finish_pass(const PlanParams& pp, const TabV
 // by launch and hand-over latencies, want).  Not FUSED: the lists are left for finish_kernel (the call inside the
 // kernel costs the candidate loop a few registers, which long searches would pay for in every iteration).
 // SCREEN: candidates are evaluated in binary32 first (unconstrained searches; see SCREEN_BAND).
-template <int OBJ, bool CONSTR, bool FUSED, bool SCREEN = false>
+template <int OBJ, bool CONSTR, bool FUSED, bool EVAL, bool SCREEN = false>
 __global__ void __launch_bounds__(PLAN_THREADS, SCREEN ? PLAN_SCREEN_BLOCKS : PLAN_MIN_BLOCKS) plan_kernel(const __grid_constant__ PlanParams pp) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ CfgShared cs;
@@ -1246,10 +1378,10 @@ __global__ void __launch_bounds__(PLAN_THREADS, SCREEN ? PLAN_SCREEN_BLOCKS : PL
             }
             const uint32_t q = (ch - chunk_start[c]) * PLAN_THREADS + tid;    // < R^3 + 256 <= 2^18 + 256
             const bool active = q < (cs.packed ? cs.live_items : cs.n_items);
-            const uint64_t item_flat = cs.flat_base + (uint64_t)q * R;
             if (!cs.valid) {
                 // every candidate of the configuration is invalid; count those in range
                 if (active) {
+                    const uint64_t item_flat = cs.flat_base + (uint64_t)q * R;
                     const uint64_t lo = item_flat > pp.flat_lo ? item_flat : pp.flat_lo;
                     const uint64_t hi = item_flat + R < pp.flat_hi ? item_flat + R : pp.flat_hi;
                     const uint32_t n = hi > lo ? (uint32_t)(hi - lo) : 0u;
@@ -1258,25 +1390,12 @@ __global__ void __launch_bounds__(PLAN_THREADS, SCREEN ? PLAN_SCREEN_BLOCKS : PL
                 }
                 continue;
             }
-            // the bulk of every space has four segments: pick the straight-line loop for its common shapes
-            const int fixed = (cs.n_run[3][0] == 0 && cs.n_run[3][1] == 0 && cs.n_run[3][3] == 1 && cs.n_run[3][2] <= 3)
-                                  ? (int)cs.n_run[3][2] : -1;
-#define SAILOR_RUN(NS, NF) run_items<NS, OBJ, CONSTR, NF, SCREEN>(pp, cs, a, T, Z, R, q, active, item_flat, budget, top, cnt, lane)
             switch (cs.cfg.nseg) {
-                case 1: SAILOR_RUN(1, -1); break;
-                case 2: SAILOR_RUN(2, -1); break;
-                case 3: SAILOR_RUN(3, -1); break;
-                default:
-                    switch (fixed) {
-                        case 0: SAILOR_RUN(4, 0); break;
-                        case 1: SAILOR_RUN(4, 1); break;
-                        case 2: SAILOR_RUN(4, 2); break;
-                        case 3: SAILOR_RUN(4, 3); break;
-                        default: SAILOR_RUN(4, -1); break;
-                    }
-                    break;
+                case 1: run_items<1, OBJ, CONSTR, SCREEN, EVAL>(pp, cs, a, T, Z, R, q, active, budget, top, cnt, lane); break;
+                case 2: run_items<2, OBJ, CONSTR, SCREEN, EVAL>(pp, cs, a, T, Z, R, q, active, budget, top, cnt, lane); break;
+                case 3: run_items<3, OBJ, CONSTR, SCREEN, EVAL>(pp, cs, a, T, Z, R, q, active, budget, top, cnt, lane); break;
+                default: run_items<4, OBJ, CONSTR, SCREEN, EVAL>(pp, cs, a, T, Z, R, q, active, budget, top, cnt, lane); break;
             }
-#undef SAILOR_RUN
         }
         // per-thread counters are 32 bits wide: hand them to the block's 64-bit sums in time
         if (__any_sync(FULL, cnt.total > (1u << 30))) flush_counters(cs, cnt, lane);
@@ -1335,11 +1454,15 @@ using PlanKernel = void (*)(const PlanParams);
 
 // The search kernels of one objective.  Each objective is compiled in a file of its own (sailor_plan_obj*.cu), side
 // by side: the straight-line variants of the candidate loop are what the library takes longest to compile.
+template <int OBJ, bool EVAL>
+PlanKernel plan_kernel_with(bool constr, bool fused, bool screen) {
+    if (screen) return plan_kernel<OBJ, false, false, EVAL, true>;     // unconstrained searches only; they end their pass in finish_kernel
+    if (fused) return constr ? plan_kernel<OBJ, true, true, EVAL> : plan_kernel<OBJ, false, true, EVAL>;
+    return constr ? plan_kernel<OBJ, true, false, EVAL> : plan_kernel<OBJ, false, false, EVAL>;
+}
 template <int OBJ>
-PlanKernel plan_kernel_of(bool constr, bool fused, bool screen) {
-    if (screen) return plan_kernel<OBJ, false, false, true>;      // unconstrained searches only; they end their pass in finish_kernel
-    if (fused) return constr ? plan_kernel<OBJ, true, true> : plan_kernel<OBJ, false, true>;
-    return constr ? plan_kernel<OBJ, true, false> : plan_kernel<OBJ, false, false>;
+PlanKernel plan_kernel_of(bool constr, bool fused, bool screen, bool eval_all) {
+    return eval_all ? plan_kernel_with<OBJ, true>(constr, fused, screen) : plan_kernel_with<OBJ, false>(constr, fused, screen);
 }
 
 }  // namespace sailor

@@ -6,9 +6,9 @@
 
 namespace sailor {
 
-extern template PlanKernel plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT>(bool, bool, bool);
-extern template PlanKernel plan_kernel_of<SAILOR_OBJ_MIN_COST>(bool, bool, bool);
-extern template PlanKernel plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT_PER_USD>(bool, bool, bool);
+extern template PlanKernel plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT>(bool, bool, bool, bool);
+extern template PlanKernel plan_kernel_of<SAILOR_OBJ_MIN_COST>(bool, bool, bool, bool);
+extern template PlanKernel plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT_PER_USD>(bool, bool, bool, bool);
 
 // The end of a pass as a launch of its own (one block), after a search kernel that is not FUSED.
 __global__ void __launch_bounds__(PLAN_THREADS) finish_kernel(const __grid_constant__ PlanParams pp, uint32_t n_partial) {

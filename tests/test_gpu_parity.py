@@ -688,3 +688,35 @@ def test_contexts_come_and_go_on_threads_and_streams(n_threads, own_stream, torc
     for th in threads:
         th.join()
     assert not wrong, wrong
+
+
+@pytest.mark.parametrize("n_types,n_zones,zoned,poly", [(1, 8, False, False), (2, 5, True, False), (2, 7, False, False), (3, 3, False, True),
+                                                        (1, 2, True, False), (4, 1, False, False)])
+def test_every_candidate_over_zone_shapes(n_types, n_zones, zoned, poly, make_ctx):
+    """SAILOR_FLAG_EVAL_ALL takes the zones of the last segment in groups of seven, four and one, with shared or own price
+    rates, and digit by digit where links differ between zones: same lists and counts as the oracle and as the pruned
+    search, over whole spaces and ranges that begin and end inside configurations."""
+    w = W.tiny(seed=29, n_types=n_types, n_zones=n_zones, L=9, p_values=[4, 9], d_values=(1, 4), tp_values=(1, 2), mbs_values=(2,),
+               rc_values=(0,))
+    if zoned:
+        w.price_per_hour = w.price_per_hour * np.linspace(0.8, 1.2, n_zones)[:, None]
+    if poly:
+        w = W.with_bandwidth_polynomials(w, seed=3)
+    o, ctx = Oracle(w), make_ctx(w).ctx
+    sp = B.make_space(w)
+    n = B.sailor_space_size(ctx, sp)
+    for kind in (0, 1, 2):
+        hits, counts = o.search(kind, 16)
+        flags = [B.FLAG_EVAL_ALL, 0, B.FLAG_EVAL_ALL | B.FLAG_F32_SCREEN]
+        for f in flags:
+            res, st = B.sailor_plan(ctx, sp, B.Objective(kind, f, 0.0, 0.0, 0.0), 16)
+            assert [(r.flat, r.score, r.cost) for r in res] == [(h["flat"], h["score"], h["cost"]) for h in hits], (kind, f)
+            assert (st.n_invalid, st.n_oom, st.n_over_avail, st.n_feasible) == tuple(
+                counts[k] for k in ("n_invalid", "n_oom", "n_over_avail", "n_feasible")), (kind, f)
+    lo, hi = n // 3 + 1, n - n // 5 - 3
+    hits, counts = o.search(0, 16, lo=lo, hi=hi)
+    for f in (B.FLAG_EVAL_ALL, 0):
+        res, st = B.sailor_plan_range(ctx, sp, B.Objective(0, f, 0.0, 0.0, 0.0), lo, hi, 16)
+        assert [r.flat for r in res] == [h["flat"] for h in hits] and st.n_total == hi - lo
+        assert (st.n_invalid, st.n_oom, st.n_over_avail, st.n_feasible) == tuple(
+            counts[k] for k in ("n_invalid", "n_oom", "n_over_avail", "n_feasible"))
