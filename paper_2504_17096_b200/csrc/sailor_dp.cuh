@@ -94,13 +94,14 @@ struct DpTabLayout {
 __global__ void __launch_bounds__(DP_THREADS)
 dp_tables_kernel(const unsigned char* __restrict__ blob, SpaceDesc sp, uint32_t n_config, uint32_t n_orders, DpTabLayout lay,
                  const uint8_t* __restrict__ wanted /* [n_config], null: all */, double* __restrict__ tabs,
-                 double* __restrict__ value /* [n_config * n_orders]: +inf, no plan so far */) {
+                 double* __restrict__ value /* [n_config * n_orders]: +inf, no plan so far */, DeviceSpan* span) {
     __shared__ uint64_t s_params[SAILOR_P_MAX];
     __shared__ uint32_t s_ok[SAILOR_P_MAX];
     TabView v;
     v.bind(blob, blob);
     const TabHdr* h = v.h;
     const uint32_t T = h->T, R = h->R, tid = threadIdx.x;
+    if (blockIdx.x == 0 && tid == 0) span->start = device_ns();          // the call's first kernel
     for (uint32_t c = blockIdx.x; c < n_config; c += gridDim.x) {
         __syncthreads();
         for (uint32_t q = tid; q < n_orders; q += DP_THREADS) value[(size_t)c * n_orders + q] = make_inf();
@@ -485,6 +486,7 @@ __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_finish_kernel(const __gr
 struct DpOut {                       // what a search leaves for the host, in mapped pinned memory
     unsigned long long counters[5];  // [0] problems with a plan, [1] number written to results, [2] plans over the constraint,
                                      // [3], [4] of the budget loop: problems given up, calls
+    DeviceSpan span;
     sailor_dp_result results[SAILOR_K_MAX];
 };
 
@@ -576,6 +578,7 @@ __global__ void __launch_bounds__(DP_SELECT_THREADS) dp_select_kernel(const __gr
             o.zone[i] = i < k.P ? r.zone[i] : 0;
         }
     }
+    if (tid == 0) sp.out->span.end = device_ns();
 }
 
 }  // namespace sailor

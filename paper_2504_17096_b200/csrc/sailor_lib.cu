@@ -289,7 +289,7 @@ size_t padded(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
 // microseconds where cudaMalloc and cudaFree of a megabyte cost 0.3 ms each (up to 12 ms seen).  The pool keeps at most
 // POOL_KEEP bytes that no context uses (what is beyond goes back to the device when a stream is next synchronised).
 // Allocation and release are ordered on the context's stream; the pool itself is safe to use from any thread.
-constexpr uint64_t POOL_KEEP = 64ull << 20;
+constexpr uint64_t POOL_KEEP = 256ull << 20;
 constexpr int POOL_DEVICES_MAX = 64;
 
 int device_pool(sailor_ctx* ctx, cudaMemPool_t* out) {
@@ -390,6 +390,8 @@ struct DeviceGuard {
         if (prev >= 0) cudaSetDevice(prev);
     }
 };
+
+float span_ms(const DeviceSpan& s) { return s.end > s.start ? (float)((double)(s.end - s.start) * 1e-6) : 0.f; }
 
 bool finite_nonneg(const double* p, size_t n) {
     for (size_t i = 0; i < n; ++i)
@@ -657,6 +659,7 @@ int enqueue_pass(sailor_ctx* ctx, uint32_t obj, double budget, bool budget_from_
     pp.min_rate = min_rate;
     pp.out = ctx->d_out_mapped;        // the block that ends the pass writes the results straight into pinned host memory
     pp.finish = 1;
+    pp.first = *n_launches == 0 && !waves ? 1u : 0u;
     pp.next_budget_factor = next_budget_factor;
     pp.cost_only = next_budget_factor > 0.0 ? 1u : 0u;
     uint32_t grid = 0;
@@ -714,6 +717,7 @@ int enqueue_pass(sailor_ctx* ctx, uint32_t obj, double budget, bool budget_from_
             wp.cfg_best = sc.d_cfg_best;
             wp.groups = sc.d_groups;
             wp.ctrl = ctx->d_ctrl;
+            wp.out = ctx->d_out_mapped;
             wp.n_config = sc.n_config;
             wp.n_d = sc.desc.n_d;
             // H3: largest degree first when throughput is maximised; H4: smallest first when cost is minimised
@@ -731,6 +735,7 @@ int enqueue_pass(sailor_ctx* ctx, uint32_t obj, double budget, bool budget_from_
             }
             for (uint32_t w = 0; w < wp.n_d; ++w) {
                 wp.wave = w;
+                wp.first = *n_launches == 0 ? 1u : 0u;
                 wave_step_kernel<<<1, WAVE_THREADS, 0, ctx->stream>>>(wp);
                 CU(ctx, cudaGetLastError());
                 pp.carry_lists = w ? 1u : 0u;
@@ -741,7 +746,7 @@ int enqueue_pass(sailor_ctx* ctx, uint32_t obj, double budget, bool budget_from_
             }
         }
         if (!fused) {              // the end of the pass as a launch of its own
-            finish_kernel<<<1, PLAN_THREADS, ctx->hdr.static_bytes + sizeof(uint32_t) * SAILOR_K_MAX * ctx->hdr.R, ctx->stream>>>(pp, grid);
+            finish_kernel<<<1, PLAN_THREADS, ctx->hdr.static_bytes + sizeof(uint32_t) * SAILOR_K_MAX, ctx->stream>>>(pp, grid);
             CU(ctx, cudaGetLastError());
             ++*n_launches;
         }
@@ -1205,7 +1210,6 @@ static int plan_range_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_
         CU(ctx, cudaMemsetAsync(&ctx->d_ctrl->min_cost_bits, 0x7f, 2 * sizeof(unsigned long long), ctx->stream));
     }
     ctx->ctrl_dirty = true;            // until this call has gone through
-    if (stats) CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
     const bool two_pass = o->budget_factor_over_cheapest > 0.0;
     // a whole-space search with pruning on walks only the prefixes the survey found live
     const bool live = !(o->flags & SAILOR_FLAG_EVAL_ALL) && flat_lo == 0 && flat_hi == total;
@@ -1219,7 +1223,6 @@ static int plan_range_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_
     rc = enqueue_pass(ctx, o->kind, o->budget_usd_per_iter, two_pass, o->min_iters_per_s, o->flags, flat_lo,
                       flat_hi, live, k, 0.0, &launches, &launched);
     if (rc) return rc;
-    if (stats) CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
     if (!launched) memset(&ctx->h_out->ctrl, 0, sizeof(Ctrl));    // an empty range: nothing ran, nothing was found
     CU(ctx, stream_sync(ctx));                                      // the results are in h_out once the kernels are done
     ctx->ctrl_dirty = false;
@@ -1247,9 +1250,7 @@ static int plan_range_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_
         double mc;
         memcpy(&mc, &cr.min_cost_bits, sizeof(mc));
         stats->min_feasible_cost = cr.stats[5] ? mc : 0.0;
-        float ms = 0.f;
-        CU(ctx, cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
-        stats->kernel_ms = ms;
+        stats->kernel_ms = launched ? span_ms(ctx->h_out->span) : 0.f;
         stats->n_launches = launches;
         stats->d2h_ms = 0.f;               // no copy of its own: the results were written in place
         if (ctx->h2d_fresh) {              // an upload for another entry point was enqueued before this search: complete by now
@@ -1710,12 +1711,11 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
         const int rc_up = upload_availability(ctx);
         if (rc_up) return rc_up;
     }
-    CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
     CU(ctx, cudaMemsetAsync(d_counters, 0, 40, ctx->stream));
     CU(ctx, cudaMemcpyAsync(d_problems, prob.data(), n_problems * sizeof(DpProblem), cudaMemcpyHostToDevice, ctx->stream));
     {
         const uint32_t grid = (uint32_t)(n_config < 4096 ? n_config : 4096);
-        dp_tables_kernel<<<grid, DP_THREADS, 0, ctx->stream>>>(ctx->d_blob, d, (uint32_t)n_config, n_orders, lay, nullptr, d_tabs, d_value);
+        dp_tables_kernel<<<grid, DP_THREADS, 0, ctx->stream>>>(ctx->d_blob, d, (uint32_t)n_config, n_orders, lay, nullptr, d_tabs, d_value, &d_out->span);
         CU(ctx, cudaGetLastError());
         ++launches;
     }
@@ -1737,7 +1737,6 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     dp_select_kernel<<<1, DP_SELECT_THREADS, 0, ctx->stream>>>(sel);
     CU(ctx, cudaGetLastError());
     ++launches;
-    CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
     CU(ctx, stream_sync(ctx));                                 // also: `prob` is pageable
     const unsigned long long* counters = ctx->host->dp.counters;
     if (counters[1] > k) return SAILOR_E_DEVICE;
@@ -1749,9 +1748,7 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
         stats->n_over_constraint = counters[2];
         stats->n_states = counters[4];
         stats->workspace_used = total;
-        float ms = 0.f;
-        CU(ctx, cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
-        stats->kernel_ms = ms;
+        stats->kernel_ms = span_ms(ctx->host->dp.span);
         stats->n_launches = launches;
         stats->n_batches = 1;
         stats->n_unfinished = (uint32_t)counters[3];
@@ -1909,7 +1906,6 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
     lp.tabs = d_tabs; lp.lay = lay; lp.T = T;
 
     uint32_t launches = 0;
-    if (stats) CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
     std::vector<unsigned char> up;                           // what a batch uploads, in one copy
     auto add = [&](const void* p, size_t bytes) {
         const size_t off = padded(up.size());
@@ -1973,7 +1969,7 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
         CU(ctx, cudaMemcpyAsync(ctx->d_dp_up, up.data(), up.size(), cudaMemcpyHostToDevice, ctx->stream));   // returns when `up` has been read
         if (bi == 0) {
             dp_tables_kernel<<<(uint32_t)std::min<uint64_t>(n_config, 4096), DP_THREADS, 0, ctx->stream>>>(
-                ctx->d_blob, d, (uint32_t)n_config, n_orders, lay, ctx->d_dp_up + off_wanted, d_tabs, d_value);
+                ctx->d_blob, d, (uint32_t)n_config, n_orders, lay, ctx->d_dp_up + off_wanted, d_tabs, d_value, &d_out->span);
             CU(ctx, cudaGetLastError());
             ++launches;
         }
@@ -2029,7 +2025,6 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
     dp_select_kernel<<<1, DP_SELECT_THREADS, 0, ctx->stream>>>(sel);
     CU(ctx, cudaGetLastError());
     ++launches;
-    if (stats) CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
     CU(ctx, stream_sync(ctx));
     const unsigned long long* counters = ctx->host->dp.counters;
     if (counters[1] > k) return SAILOR_E_DEVICE;               // cannot happen; never copy past the caller's k records
@@ -2041,9 +2036,7 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
         stats->n_over_constraint = counters[2];
         stats->n_states = n_states;
         stats->workspace_used = largest;
-        float ms = 0.f;
-        CU(ctx, cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
-        stats->kernel_ms = ms;
+        stats->kernel_ms = span_ms(ctx->host->dp.span);
         stats->n_launches = launches;
         stats->n_batches = (uint32_t)std::max<size_t>(batches.size(), 1);
         stats->n_unfinished = 0;
@@ -2203,7 +2196,6 @@ static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const s
         CU(ctx, cudaMemsetAsync(mp.counters + MIXC_MIN_COST, 0x7f, 8, ctx->stream));
     }
     ctx->mix_dirty = true;             // until this call has gone through
-    if (stats) CU(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
     CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&mp.out), &ctx->host->mixed, 0));
     mp.blob = ctx->d_blob; mp.sp = mt.desc; mp.n_config = mt.n_config; mp.k = k; mp.obj = o->kind;
     memcpy(mp.avail, ctx->h_avail, sizeof(mp.avail));
@@ -2229,7 +2221,6 @@ static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const s
     else mixed_finish_kernel<false><<<1, 32 * MIXF_WARPS<false>, mixed_smem(ctx->hdr.static_bytes, R, MIXF_WARPS<false>), ctx->stream>>>(mp);
     CU(ctx, cudaGetLastError());
     ++launches;
-    if (stats) CU(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
     CU(ctx, stream_sync(ctx));
     const unsigned long long* counters = ctx->host->mixed.counters;
     if (counters[MIXC_ERROR]) return SAILOR_E_DEVICE;
@@ -2249,7 +2240,7 @@ static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const s
         double mc;
         memcpy(&mc, &counters[MIXC_MIN_COST], sizeof(mc));
         stats->min_feasible_cost = counters[5] ? mc : 0.0;
-        CU(ctx, cudaEventElapsedTime(&stats->kernel_ms, ctx->ev0, ctx->ev1));
+        stats->kernel_ms = span_ms(ctx->host->mixed.span);
         stats->n_launches = launches;
         stats->n_configs = stats->n_configs_evaluated = mt.n_config;
     }

@@ -90,6 +90,7 @@ enum { MIXC_MIN_COST = 6, MIXC_ERROR = 7, MIXC_FOUND = 8, MIXC_QUEUED = 9, MIXC_
 // What a search leaves for the host, written by mixed_finish_kernel into mapped pinned memory.
 struct MixedOut {
     unsigned long long counters[MIXC_N];
+    DeviceSpan span;
     sailor_mixed_result results[SAILOR_K_MAX];
 };
 
@@ -185,6 +186,7 @@ __global__ void __launch_bounds__(MIXS_THREADS) mixed_class_kernel(const __grid_
     uint64_t pos = mp.range_lo + share * blockIdx.x;
     const uint64_t stop = pos + share < mp.range_hi ? pos + share : mp.range_hi;
     uint32_t n_inv = 0, n_oom = 0, n_over = 0;
+    if (mp.range_lo == 0 && blockIdx.x == 0 && tid == 0) mp.out->span.start = device_ns();
     if (tid < 3) s_class[tid] = 0;
     uint32_t cfg = 0;
     if (pos < stop) {
@@ -609,6 +611,7 @@ __global__ void __launch_bounds__(32 * MIXF_WARPS<DEEP>) mixed_finish_kernel(con
         mp.out->counters[tid] = tid == 0 ? mp.n_total : tid == MIXC_FOUND ? n : live[tid];
         live[tid] = tid == MIXC_MIN_COST ? COST_BITS_START : 0ull;
     }
+    if (tid == 0) mp.out->span.end = device_ns();
 }
 
 // Shared memory of `warps` evaluating warps: the static tables, R counters and a record per warp.

@@ -54,6 +54,7 @@ struct Ctrl {                       // one per context, device memory
 // or the next call needs no clearing from the host.
 struct PlanOut {
     Ctrl ctrl;
+    DeviceSpan span;
     sailor_result results[SAILOR_K_MAX];
 };
 
@@ -81,6 +82,7 @@ struct PlanParams {
     const uint32_t* chunk_hi_dev;      // non-null: chunks [0, *chunk_hi_dev) instead of [chunk_lo, chunk_hi)
     unsigned long long* cfg_best;      // non-null: [n_config] best feasible score per configuration (ordered bits)
     PlanOut* out;                      // where the block that finishes the pass leaves the results
+    uint32_t first;                    // this launch is the call's first: it stamps the start
     uint32_t finish;                   // this launch ends a pass: its last block merges the lists and writes `out`
     double next_budget_factor;         // > 0: the finishing block writes ctrl->budget = factor * best cost (next pass)
     uint32_t cost_only;                // the pass only looks for the cheapest feasible cost (no lists, no result records)
@@ -163,6 +165,21 @@ struct WarpTopK {
             const bool upper = lane & stride;
             if (other_less != upper) { score = os; flat = of; }     // lower lane keeps the smaller, upper the larger
         }
+        thr_score = __shfl_sync(FULL, score, k - 1);
+        thr_flat = __shfl_sync(FULL, flat, k - 1);
+    }
+    // Sort the lanes' elements (empty slots are (+inf, ~0)) ascending: a bitonic network, fifteen compare-exchanges.
+    __device__ __forceinline__ void sort(uint32_t k, uint32_t lane) {
+#pragma unroll
+        for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+            for (int stride = size >> 1; stride; stride >>= 1) {
+                const double os = __shfl_xor_sync(FULL, score, stride);
+                const uint64_t of = __shfl_xor_sync(FULL, flat, stride);
+                const bool other_less = os < score || (os == score && of < flat);
+                const bool keep_larger = ((lane & stride) != 0) != ((lane & size) != 0);
+                if (other_less != keep_larger) { score = os; flat = of; }
+            }
         thr_score = __shfl_sync(FULL, score, k - 1);
         thr_flat = __shfl_sync(FULL, flat, k - 1);
     }
@@ -1122,15 +1139,17 @@ __device__ __forceinline__ uint32_t merge_block_lists(const Hit* partial, uint32
         sc = raw.x;
         fl = (uint64_t)__double_as_longlong(raw.y);
     };
-    WarpTopK top;
+    WarpTopK top, more;
     top.init();
     const uint32_t rounds = (n_lists + 32 * NW - 1) / (32 * NW);
     for (uint32_t r = 0; r < rounds; ++r) {
         const uint32_t b = r * 32 * NW + tid;
-        double hs = make_inf();
-        uint64_t hf = ~0ull;
-        if (b < n_lists) load_hit(b, 0, hs, hf);
-        top.offer(hf != ~0ull && (hs < top.thr_score || (hs == top.thr_score && hf < top.thr_flat)), hs, hf, k, lane);
+        more.init();
+        if (b < n_lists) load_hit(b, 0, more.score, more.flat);
+        if (more.flat == ~0ull) more.score = make_inf();       // an empty list (only its first slot need be written)
+        more.sort(k, lane);
+        if (r == 0) top = more;
+        else top.merge_sorted(more.score, more.flat, k, lane);
     }
     auto tree_merge = [&]() {          // the warps' lists into warp 0's, through shared memory
         s_hits[warp][lane].score = top.score;
@@ -1158,14 +1177,20 @@ __device__ __forceinline__ uint32_t merge_block_lists(const Hit* partial, uint32
         if (hf != ~0ull && (hs < cut_s || (hs == cut_s && hf <= cut_f))) sel[atomicAdd(s_n, 1u)] = b;
     }
     __syncthreads();
-    const uint32_t n_sel = *s_n;
+    const uint32_t n_sel = *s_n;                               // at most k
     top.init();
-    for (uint32_t q = warp; q < n_sel; q += NW) {
-        double ls = make_inf();
-        uint64_t lf = ~0ull;
-        if (lane < k) load_hit(sel[q], lane, ls, lf);
-        top.merge_sorted(ls, lf, k, lane);
+    constexpr uint32_t PER_WARP = (SAILOR_K_MAX + NW - 1) / NW;
+    double ls[PER_WARP];
+    uint64_t lf[PER_WARP];
+#pragma unroll
+    for (uint32_t x = 0; x < PER_WARP; ++x) {                  // all loads in flight before the first merge
+        ls[x] = make_inf();
+        lf[x] = ~0ull;
+        if (warp + x * NW < n_sel && lane < k) load_hit(sel[warp + x * NW], lane, ls[x], lf[x]);
     }
+#pragma unroll
+    for (uint32_t x = 0; x < PER_WARP; ++x)
+        if (warp + x * NW < n_sel) top.merge_sorted(ls[x], lf[x], k, lane);
     __syncthreads();                                           // `sel` has been read by everyone
     tree_merge();
     if (warp == 0) {
@@ -1177,15 +1202,138 @@ __device__ __forceinline__ uint32_t merge_block_lists(const Hit* partial, uint32
     return *s_n;
 }
 
+// The result record of candidate `hit.flat`: decoded, simulated and written by one warp, lane i taking stage i (then
+// i + 32, ...).  Per-stage terms are formed side by side; the sums whose order is part of the result run over the lanes'
+// terms in stage order, so the bits are those of simulate_runs.  Bound by latency: a thread alone waits for one table
+// after another (9.4 us from decoding to the record for plans of up to 24 stages, 5.0 us here).
+__device__ __forceinline__ void write_result(const PlanParams& pp, const TabView& v, const Hit& hit, sailor_result* out, uint32_t lane) {
+    const TabHdr* h = v.h;
+    const SpaceDesc& sp = pp.sp;
+    const uint32_t T = h->T, Z = h->Z, R = h->R;
+    // the sub-space (number of stages) that holds the index: lane j knows the size of the j-th
+    const uint32_t per_p = sp.n_mbs * sp.n_tp * sp.n_rc * sp.n_d;
+    uint64_t size = 0;
+    if (lane < sp.n_p) size = (uint64_t)per_p * ipow64(R, nseg_of(sp.p_values[lane], sp.seg_max));
+    uint64_t end = size;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t up = __shfl_up_sync(FULL, end, o);
+        if (lane >= (uint32_t)o) end += up;
+    }
+    const uint32_t sub = __ffs(__ballot_sync(FULL, lane < sp.n_p && hit.flat < end)) - 1;
+    const uint64_t rem = hit.flat - __shfl_sync(FULL, end - size, sub);
+    const uint32_t nseg = nseg_of(sp.p_values[sub], sp.seg_max);
+    const uint32_t block = (uint32_t)ipow64(R, nseg);       // candidates of a configuration: at most 64^4
+    const uint32_t cfg = (uint32_t)(rem / block);
+    uint32_t x = (uint32_t)(rem - (uint64_t)cfg * block), dg[SAILOR_SEG_MAX];
+#pragma unroll
+    for (int q = SAILOR_SEG_MAX - 1; q >= 0; --q) {
+        dg[q] = 0;
+        if ((uint32_t)q < nseg) { const uint32_t y = x / R; dg[q] = x - y * R; x = y; }
+    }
+    const Config k = config_of(sp, sub * per_p + cfg);
+    const uint32_t P = k.P, D = k.D, mi = k.mi, tp = h->tp_values[k.tpi];
+    uint32_t seg_end[SAILOR_SEG_MAX], gz[SAILOR_SEG_MAX];   // per segment: past its last stage; type | zone << 8
+#pragma unroll
+    for (uint32_t q = 0; q < SAILOR_SEG_MAX; ++q) {
+        seg_end[q] = q < nseg ? ((q + 1) * P + nseg - 1) / nseg : P;
+        gz[q] = dg[q] / T;
+        gz[q] = (dg[q] - gz[q] * T) | gz[q] << 8;
+    }
+    auto of_stage = [&](uint32_t i, const uint32_t (&seg)[SAILOR_SEG_MAX]) {
+        return i < seg_end[0] ? seg[0] : i < seg_end[1] ? seg[1] : i < seg_end[2] ? seg[2] : seg[3];
+    };
+    const uint64_t dm = (uint64_t)D * h->mbs_values[mi], n_b = h->gbs / dm;
+    uint32_t status = (n_b * dm != h->gbs || !((h->heads_ok >> k.tpi) & 1u)) ? SAILOR_ST_INVALID : 0u;
+#pragma unroll
+    for (uint32_t q = 0; q < SAILOR_SEG_MAX; ++q) {         // GPUs of every (zone, type) used, over all segments that use it
+        uint32_t stages = 0;
+#pragma unroll
+        for (uint32_t q2 = 0; q2 < SAILOR_SEG_MAX; ++q2)
+            if (q2 < nseg && dg[q2] == dg[q]) stages += seg_end[q2] - (q2 ? seg_end[q2 - 1] : 0u);
+        if (q < nseg && (uint64_t)stages * D * tp > pp.avail[dg[q]]) status |= SAILOR_ST_OVER_AVAIL;
+    }
+    const uint32_t base = h->n_blocks / P, extra = h->n_blocks - base * P;
+    const double msg = (double)v.p2p[mi], steps = (double)(2 * (uint64_t)(D - 1)), coef = steps / (double)D;
+    const double xbytes = (double)(2 * n_b * (uint64_t)D * v.p2p[mi]);
+    double sum_t = 0.0, max_t = 0.0, max_sync = 0.0, max_u = 0.0, rate = 0.0, c_comm = 0.0;
+    uint64_t peak = 0;
+    for (uint32_t at = 0; at < P; at += 32) {
+        const uint32_t i = at + lane;
+        double t = 0.0, gpu_rate = 0.0, comm = 0.0;
+        bool crosses = false;
+        if (i < P) {
+            const uint32_t x_i = of_stage(i, gz), g = x_i & 0xff, z = x_i >> 8, d = z * T + g;
+            const bool e = (i == 0) && h->has_embed, hd = (i == P - 1) && h->has_head;
+            const size_t comp = (size_t)((e ? 2u : 0u) + (hd ? 1u : 0u)) * h->chain_len + base + (i < extra ? 1u : 0u);
+            const size_t ct = comp * h->n_tp + k.tpi;
+            t = v.cmp_fb[(((comp * T + g) * h->n_tp + k.tpi) * h->n_mbs + mi) * 2 + k.rc];
+            max_u = dmax(max_u, v.cmp_upd[(comp * T + g) * h->n_tp + k.tpi]);
+            const uint64_t* mm = v.cmp_mem + ((ct * h->n_mbs + mi) * 2 + k.rc) * 2;
+            const uint64_t inflight = (uint64_t)(P - i) < n_b ? (uint64_t)(P - i) : n_b;
+            const uint64_t m = mm[0] + h->reserved[g] + inflight * mm[1];
+            if (m > h->capacity[g]) status |= SAILOR_ST_OOM;
+            if (tp > h->gpn[g]) status |= SAILOR_ST_INVALID;
+            peak = m > peak ? m : peak;
+            if (D > 1) max_sync = dmax(max_sync, allreduce_bytes_time(v, d, (uint64_t)D * tp <= h->gpn[g], v.cmp_grad[ct], D, steps, coef));
+            gpu_rate = mul_rn((double)(D * tp), v.price_s[d]);
+            if (i + 1 < P) {
+                const uint32_t x_n = of_stage(i + 1, gz), zn = x_n >> 8;
+                t = add_rn(t, mul_rn(2.0, boundary_time(v, g, z, tp, x_n & 0xff, zn, tp, D, msg)));
+                crosses = zn != z;
+                if (crosses) comm = mul_rn(xbytes, v.egress[z * Z + zn]);
+            }
+            max_t = dmax(max_t, t);
+        }
+        const uint32_t n = P - at < 32 ? P - at : 32;
+        for (uint32_t l = 0; l < n; ++l) {                   // in stage order
+            sum_t = add_rn(sum_t, __shfl_sync(FULL, t, l));
+            rate = add_rn(rate, __shfl_sync(FULL, gpu_rate, l));
+        }
+        for (uint32_t m = __ballot_sync(FULL, crosses); m; m &= m - 1) c_comm = add_rn(c_comm, __shfl_sync(FULL, comm, __ffs(m) - 1));
+    }
+#pragma unroll 1
+    for (int o = 16; o; o >>= 1) {
+        max_t = dmax(max_t, __shfl_xor_sync(FULL, max_t, o));
+        max_sync = dmax(max_sync, __shfl_xor_sync(FULL, max_sync, o));
+        max_u = dmax(max_u, __shfl_xor_sync(FULL, max_u, o));
+        const uint64_t other = __shfl_xor_sync(FULL, peak, o);
+        peak = other > peak ? other : peak;
+    }
+    status = __reduce_or_sync(FULL, status);
+    const double t_iter = add_rn(add_rn(add_rn(sum_t, mul_rn((double)n_b, max_t)), max_sync), max_u);
+    if (lane == 0) {
+        out->flat = hit.flat;
+        out->score = hit.score;
+        out->t_iter = t_iter;
+        out->cost = add_rn(mul_rn(rate, t_iter), c_comm);
+        out->peak_mem = peak;
+        out->status = status;
+        out->_pad = 0;
+    }
+    if (lane < sizeof(sailor_plan_rec) / 4) {                // the record word by word: header, then a run per segment
+        uint32_t word = 0;
+        if (lane == 0) word = P | mi << 8 | k.rc << 16 | nseg << 24;
+        else if (lane == 1) word = D;
+        else if (lane - 2 < nseg) {
+            const uint32_t q = lane - 2, x_q = q == 0 ? gz[0] : q == 1 ? gz[1] : q == 2 ? gz[2] : gz[3];
+            const uint32_t a = q == 0 ? 0u : q == 1 ? seg_end[0] : q == 2 ? seg_end[1] : seg_end[2];
+            const uint32_t e = q == 0 ? seg_end[0] : q == 1 ? seg_end[1] : q == 2 ? seg_end[2] : seg_end[3];
+            word = x_q | k.tpi << 16 | (e - a) << 24;
+        }
+        reinterpret_cast<uint32_t*>(&out->plan)[lane] = word;
+    }
+}
+
 // End of a pass, run by the one block that hands in its list last (no block waits for another: every block
 // adds one to Ctrl::blocks_done after its list is written, and the block that reads gridDim.x - 1 knows all the
 // lists are in memory).  Merges the blocks' lists, simulates the winners in full for the result records, copies
 // the counters next to them, hands `factor x best cost` to a following pass, and puts the counters back to
 // their starting values.  `v` is the block's own view of the static tables (already in shared memory); `s_hits`
-// (PLAN_WARPS lists) and `s_cnt` (R x SAILOR_K_MAX words) are scratch in shared memory.
+// (PLAN_WARPS lists) and `s_cnt` (SAILOR_K_MAX words) are scratch in shared memory.
 static __device__ __noinline__ void finish_pass(const PlanParams& pp, const TabView& v, Hit (*s_hits)[SAILOR_K_MAX],
                                          uint32_t* s_cnt, uint32_t* s_n, uint32_t n_partial) {
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = PLAN_WARPS;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (pp.cost_only) {
         // the cheapest-plan pass of a budget-factor search: all the next pass needs is factor x the cheapest feasible
         // cost, which every block has already folded into Ctrl::min_cost_bits (the same bits a full simulation of
@@ -1206,29 +1354,10 @@ static __device__ __noinline__ void finish_pass(const PlanParams& pp, const TabV
         }
         return;
     }
-    const uint32_t n = merge_block_lists<PLAN_WARPS>(pp.partial, n_partial, pp.k, s_hits, s_cnt, s_n);   // s_cnt: scratch first, counters then
-    // the winners are simulated in full for the result records, all at once: winner j by lane j / PLAN_WARPS of warp
-    // j % PLAN_WARPS (each is a long single-thread dependency chain of table look-ups; spread over the warps, at
-    // most four different plans share a warp's instruction stream)
-    {
-        const uint32_t j = lane * nw + warp;
-        if (lane < (SAILOR_K_MAX + nw - 1) / nw && j < n) {
-            sailor_result r;
-            r.flat = s_hits[0][j].flat;
-            r.score = s_hits[0][j].score;
-            r._pad = 0;
-            decode_flat(pp.sp, v.h->T, v.h->Z, r.flat, &r.plan);
-            const SimOut o = simulate_record(v, pp.avail, r.plan, s_cnt + j, SAILOR_K_MAX);
-            r.t_iter = o.t_iter;
-            r.cost = o.cost;
-            r.peak_mem = o.peak_mem;
-            r.status = o.status;
-            pp.out->results[j] = r;
-            if (j == 0 && pp.next_budget_factor > 0.0) pp.ctrl->budget = mul_rn(pp.next_budget_factor, o.cost);
-        }
-    }
+    const uint32_t n = merge_block_lists<PLAN_WARPS>(pp.partial, n_partial, pp.k, s_hits, s_cnt, s_n);
+    // the winners are simulated in full for the result records, a warp each
+    for (uint32_t j = warp; j < n; j += PLAN_WARPS) write_result(pp, v, s_hits[0][j], pp.out->results + j, lane);
     if (tid == 0) {
-        if (n == 0 && pp.next_budget_factor > 0.0) pp.ctrl->budget = make_inf();
         // the counters as they stand (every block's contribution is in: atomics, then its blocks_done increment)
         volatile Ctrl* live = pp.ctrl;
         Ctrl c;
@@ -1253,7 +1382,8 @@ static __device__ __noinline__ void finish_pass(const PlanParams& pp, const TabV
         live->n_cfg_evaluated = 0;
         live->min_cost_bits = COST_BITS_START;
         live->thr_bits = COST_BITS_START;
-        if (!(pp.next_budget_factor > 0.0)) live->error = 0;   // a following pass of the same call keeps the flag
+        live->error = 0;               // (a cheapest-plan pass before this one kept the flag)
+        pp.out->span.end = device_ns();
         live->n_found = 0;
     }
 }
@@ -1271,6 +1401,7 @@ __global__ void __launch_bounds__(PLAN_THREADS, SCREEN ? PLAN_SCREEN_BLOCKS : PL
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const TabHdr* gh = reinterpret_cast<const TabHdr*>(pp.blob);
     const uint32_t static_bytes = gh->static_bytes;
+    if (pp.first && blockIdx.x == 0 && tid == 0) pp.out->span.start = device_ns();
 
     // stage the static tables: one bulk copy, bounded wait, plain-load fallback
     if (!bulk_load(dyn, pp.blob, static_bytes, &cs.mbar)) {

@@ -12,7 +12,7 @@ extern template PlanKernel plan_kernel_of<SAILOR_OBJ_MAX_THROUGHPUT_PER_USD>(boo
 
 // The end of a pass as a launch of its own (one block), after a search kernel that is not FUSED.
 __global__ void __launch_bounds__(PLAN_THREADS) finish_kernel(const __grid_constant__ PlanParams pp, uint32_t n_partial) {
-    extern __shared__ __align__(16) unsigned char dyn[];      // the static tables, then R x SAILOR_K_MAX counters
+    extern __shared__ __align__(16) unsigned char dyn[];      // the static tables, then SAILOR_K_MAX words
     __shared__ Hit s_hits[PLAN_WARPS][SAILOR_K_MAX];
     __shared__ uint64_t mbar;
     __shared__ uint32_t s_n;
@@ -220,7 +220,9 @@ struct WaveParams {
     unsigned long long* cfg_best;      // [n_config]
     GroupState* groups;                // [n_config / n_d]
     Ctrl* ctrl;
+    PlanOut* out;
     uint32_t n_config, n_d, wave;
+    uint32_t first;                    // this launch is the call's first: it stamps the start
     uint8_t order[SAILOR_ND_MAX];      // positions in d_values, in the order they are tried
 };
 
@@ -235,6 +237,7 @@ __global__ void __launch_bounds__(WAVE_THREADS) wave_step_kernel(const __grid_co
     const unsigned long long inf_bits = (unsigned long long)__double_as_longlong(make_inf());
     if (tid < 3) s_closed[tid] = 0;
     if (tid == 0) s_eval = 0;
+    if (wp.first && tid == 0) wp.out->span.start = device_ns();
     // the rule, applied to what the previous wave found
     for (uint32_t g = tid; g < n_groups; g += WAVE_THREADS) {
         GroupState gs = wp.groups[g];

@@ -235,6 +235,17 @@ __device__ __forceinline__ double sync_time(const TabView& v, uint32_t g, uint32
     return allreduce_time(v, g, z * v.h->T + g, tp, D, params, steps, steps / (double)D);
 }
 
+// Nanoseconds of the device's clock: a search stamps where its first kernel starts and its last ends (two events around
+// the launches cost the call 8 us).
+__device__ __forceinline__ unsigned long long device_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+struct DeviceSpan {
+    unsigned long long start, end;
+};
+
 struct SimOut {
     double t_iter, cost;
     uint64_t peak_mem;
