@@ -491,8 +491,8 @@ int sailor_plan_mixed(sailor_ctx* ctx, const sailor_mixed_space* s, const sailor
  * is slower, the stage is charged again with that straggler and they are solved again with the smaller remainder.
  * The last stage is its own straggler and counts when its charge is within its limit.  Candidates combine and
  * compare as above.  The remaining budget is an argument of the recursion (a state reached with two different
- * remainders is solved twice), so the tables above do not apply: each problem is walked depth-first by one GPU
- * thread, problems in parallel.  The work can grow as T^P: a branch is cut when what is left cannot pay the
+ * remainders is solved twice), so the tables above do not apply: each problem is walked depth-first, problems and
+ * the types of their first stages in parallel.  The work can grow as T^P: a branch is cut when what is left cannot pay the
  * cheapest conceivable rest of the pipeline (this changes no result), and a problem that needs more than 2^24 calls
  * of the recursion is given up and counted in n_unfinished.  The charge underestimates the simulator's cost (it
  * leaves out warm-up, cool-down, synchronisation and update time, as the paper's simplification does), so the

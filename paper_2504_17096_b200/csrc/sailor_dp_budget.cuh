@@ -6,9 +6,9 @@
 // slower the stage is charged again with that one and they are solved again, until the assumption holds,
 // nothing is left, or they have no plan.  The remaining limit is an argument of the recursion, so a state has no
 // single value and the tables of the unlimited search do not apply: every problem (configuration x zone order) is
-// walked depth-first by one thread with an explicit stack in global memory.  Problems are independent, which is
-// where the parallelism is; a problem's own walk is sequential by nature (each call's limit depends on the
-// charges before it).  A branch is cut when what is left cannot pay even the cheapest conceivable rest of the
+// walked depth-first with an explicit stack.  Problems, and the types of a problem's first stage, are independent, which
+// is where the parallelism is; a walk itself is sequential by nature (each call's limit depends on the charges before
+// it).  A branch is cut when what is left cannot pay even the cheapest conceivable rest of the
 // pipeline (every later stage alone on its cheapest GPUs, charged for its own compute time): such a branch has no
 // plan, so the cut changes nothing but the work.  A problem that would take more than `node_limit` calls is given
 // up and reported as unfinished.
@@ -40,6 +40,12 @@ struct DpbFrame {                    // one call of the recursion: stage `level`
     uint8_t b_type[DP_BUDGET_P_MAX]; // types of stages level.. of the best plan (indexed by stage)
 };
 
+struct DpbRoot {                     // what the walk from one type of stage 0 found
+    double value;                    // +inf: no plan
+    unsigned long long nodes;        // calls of the recursion; above the limit: given up
+    uint8_t type[DP_BUDGET_P_MAX];
+};
+
 struct DpBudgetParams {
     const unsigned char* blob;
     const uint16_t* avail;
@@ -48,10 +54,10 @@ struct DpBudgetParams {
     const double* tabs;
     double* value;                   // indexed by problem index; +inf: no plan
     DpResult* results;
-    DpbFrame* frames;                // [n_problems][DP_BUDGET_P_MAX]
+    DpbRoot* roots;                  // [n_problems][T]
     unsigned long long* counters;    // [3] += problems given up, [4] += calls of the recursion
     DpTabLayout lay;
-    uint32_t n_problems, T;
+    uint32_t n_problems, T, p_max;
     double limit;
     unsigned long long node_limit;
 };
@@ -60,12 +66,28 @@ __device__ __forceinline__ double dpb_value(double nb, double sum, double mx, do
     return add_rn(add_rn(add_rn(sum, mul_rn(nb, mx)), sy), up);
 }
 
-__global__ void __launch_bounds__(64) dp_budget_kernel(const __grid_constant__ DpBudgetParams bp) {
-    const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= bp.n_problems) return;
+// A warp per (problem, type of stage 0).  The walk is one lane's: problems differ too much in what they try to share
+// instructions (a thread per problem ran a warp's 32 walks one after the other), and its stack sits in shared memory.
+// Bound by the latency of one chain of calls.  Workload 2, pipelines of up to eight stages, all orders, budget 1.2 x
+// cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.64 ms a call.
+constexpr int DPB_WARPS = 4;
+
+__host__ __device__ inline size_t dpb_smem(uint32_t p_max) {
+    return DPB_WARPS * (p_max * sizeof(DpbFrame) + (p_max + 1) * sizeof(double));
+}
+
+__global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_constant__ DpBudgetParams bp) {
+    extern __shared__ __align__(16) unsigned char dyn[];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t unit = blockIdx.x * DPB_WARPS + warp, T = bp.T;
+    if (unit >= bp.n_problems * T) return;
+    const uint32_t x = unit / T, g0 = unit - x * T;
+    DpbFrame* const fr = reinterpret_cast<DpbFrame*>(dyn) + warp * bp.p_max;
+    double* const lb = reinterpret_cast<double*>(reinterpret_cast<DpbFrame*>(dyn) + DPB_WARPS * bp.p_max) + warp * (bp.p_max + 1);
     const DpProblem& pb = bp.problems[x];
-    DpResult& out = bp.results[pb.index];
-    const uint32_t T = bp.T, P = pb.P;
+    DpbRoot& root = bp.roots[unit];
+    if (lane == 0) { root.value = make_inf(); root.nodes = 0; }
+    const uint32_t P = pb.P;
     const double* tab = bp.tabs + (size_t)pb.config * bp.lay.stride();
     if (*reinterpret_cast<const uint32_t*>(tab + bp.lay.off_nb() + 1) == 0 || P > DP_BUDGET_P_MAX) return;   // no valid plan here
     TabView v;
@@ -73,6 +95,9 @@ __global__ void __launch_bounds__(64) dp_budget_kernel(const __grid_constant__ D
     const TabHdr* h = v.h;
     const uint32_t R = h->R, Z = h->Z;
     const uint32_t* okv = reinterpret_cast<const uint32_t*>(tab + bp.lay.off_ok());
+    if (!((okv[0] >> g0) & 1u)) return;
+    const uint32_t p0 = pb.cap[0][g0] >= 1 ? 0u : pb.first_later[0][g0];     // by first fit from the first zone of the order
+    if (p0 == DP_NONE) return;
     const uint64_t n_b = *reinterpret_cast<const uint64_t*>(tab + bp.lay.off_nb());
     const double nb = (double)n_b;
     const Config k = config_of(bp.sp, pb.config);
@@ -82,155 +107,162 @@ __global__ void __launch_bounds__(64) dp_budget_kernel(const __grid_constant__ D
     const double* updt = tab + bp.lay.off_upd();
     const double* synct = tab + bp.lay.off_sync();
     const double* c2x = tab + bp.lay.off_c2x();
-    DpbFrame* fr = bp.frames + (size_t)x * DP_BUDGET_P_MAX;
 
     // the least any plan of stages j.. can be charged: every stage alone on the cheapest GPUs it fits, for its own
     // compute time; added up from the last stage backwards, as the recursion adds its charges
-    double lb[DP_BUDGET_P_MAX + 1];
-    lb[P] = 0.0;
-    for (uint32_t j = P; j-- > 0;) {
+    if (lane < P) {
         double least = make_inf();
         for (uint32_t g = 0; g < T; ++g) {
-            if (!((okv[j] >> g) & 1u)) continue;
+            if (!((okv[lane] >> g) & 1u)) continue;
             for (uint32_t q = 0; q < pb.nz; ++q) {
-                const double c = mul_rn(mul_rn(gpus, v.price_s[pb.zone[q] * T + g]), mul_rn(nb, fbt[j * T + g]));
+                const double c = mul_rn(mul_rn(gpus, v.price_s[pb.zone[q] * T + g]), mul_rn(nb, fbt[lane * T + g]));
                 least = c < least ? c : least;
             }
         }
-        lb[j] = add_rn(least, lb[j + 1]);
+        lb[lane] = least;
     }
+    __syncwarp();
+    if (lane != 0) return;
+    lb[P] = 0.0;
+    for (uint32_t j = P; j-- > 0;) lb[j] = add_rn(lb[j], lb[j + 1]);
+    if (bp.limit < lb[0]) return;
 
     unsigned long long nodes = 0;
     bool gave_up = false;
     // result of the call that has just returned
     bool r_found = false;
     double r_sum = 0.0, r_mx = 0.0, r_sy = 0.0, r_up = 0.0, r_cost = 0.0;
-    // stage 0: every type, by first fit from the first zone of the order
-    bool best_found = false;
-    double best_v = make_inf();
-    uint8_t best_type[DP_BUDGET_P_MAX];
-    for (uint32_t g0 = 0; g0 < T && !gave_up; ++g0) {
-        if (!((okv[0] >> g0) & 1u)) continue;
-        const uint32_t p0 = pb.cap[0][g0] >= 1 ? 0u : pb.first_later[0][g0];
-        if (p0 == DP_NONE) continue;
-        if (bp.limit < lb[0]) continue;
-        int level = 0;
-        {
-            DpbFrame& f = fr[0];
-            f.g = (uint8_t)g0; f.zp = (uint8_t)p0; f.limit = bp.limit;
-            for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) f.u[t] = 0;
-            f.u[g0] = 1;
+    int level = 0;
+    {
+        DpbFrame& f = fr[0];
+        f.g = (uint8_t)g0; f.zp = (uint8_t)p0; f.limit = bp.limit;
+        for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) f.u[t] = 0;
+        f.u[g0] = 1;
+    }
+    enum { ENTER, NEXT_TYPE, CHARGE, RESUME } state = ENTER;
+    while (level >= 0) {
+        DpbFrame& f = fr[level];
+        const uint32_t i = (uint32_t)level, g = f.g, z = pb.zone[f.zp], d = z * T + g;
+        if (state == ENTER) {
+            if (++nodes > bp.node_limit) { gave_up = true; break; }
+            f.b_found = 0;
+            f.rate = mul_rn(gpus, v.price_s[d]);
+            f.sync = synct[i * R + d];
+            f.fb = fbt[i * T + g];
+            f.upd = updt[i * T + g];
+            if (i == P - 1) {                    // the last stage sends nothing and is its own straggler
+                const double charge = mul_rn(f.rate, mul_rn(nb, f.fb));
+                r_found = charge <= f.limit;
+                r_sum = f.fb; r_mx = f.fb; r_sy = f.sync; r_up = f.upd; r_cost = charge;
+                f.b_type[i] = (uint8_t)g;
+                --level;
+                state = RESUME;
+                continue;
+            }
+            f.g2 = 0;
+            state = NEXT_TYPE;
         }
-        enum { ENTER, NEXT_TYPE, CHARGE, RESUME } state = ENTER;
-        while (level >= 0) {
-            DpbFrame& f = fr[level];
-            const uint32_t i = (uint32_t)level, g = f.g, z = pb.zone[f.zp], d = z * T + g;
-            if (state == ENTER) {
-                if (++nodes > bp.node_limit) { gave_up = true; break; }
-                f.b_found = 0;
-                f.rate = mul_rn(gpus, v.price_s[d]);
-                f.sync = synct[i * R + d];
-                f.fb = fbt[i * T + g];
-                f.upd = updt[i * T + g];
-                if (i == P - 1) {                    // the last stage sends nothing and is its own straggler
-                    const double charge = mul_rn(f.rate, mul_rn(nb, f.fb));
-                    r_found = charge <= f.limit;
-                    r_sum = f.fb; r_mx = f.fb; r_sy = f.sync; r_up = f.upd; r_cost = charge;
-                    f.b_type[i] = (uint8_t)g;
-                    --level;
-                    state = RESUME;
-                    continue;
-                }
-                f.g2 = 0;
-                state = NEXT_TYPE;
-            }
-            if (state == NEXT_TYPE) {
-                bool placed = false;
-                while (f.g2 < T) {
-                    const uint32_t g2 = f.g2;
-                    if ((okv[i + 1] >> g2) & 1u) {
-                        // first fit: this zone while it has room for one more stage of the type, else the next that has
-                        uint32_t zp2 = f.zp;
-                        if (!(f.u[g2] < pb.cap[f.zp][g2])) zp2 = pb.first_later[f.zp][g2];
-                        if (zp2 != DP_NONE) {
-                            f.zp2 = (uint8_t)zp2;
-                            for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) f.u2[t] = zp2 == f.zp ? f.u[t] : 0;
-                            f.u2[g2]++;
-                            const uint32_t z2 = pb.zone[zp2], dn = z2 * T + g2;
-                            f.t = add_rn(f.fb, c2x[dn * R + d]);
-                            f.comm = z2 != z ? mul_rn(xbytes, v.egress[z * Z + z2]) : 0.0;
-                            f.assumed = f.t;                 // first: this stage is the straggler
-                            placed = true;
-                            break;
-                        }
-                    }
-                    ++f.g2;
-                }
-                if (!placed) {                               // every type tried: hand the best plan back
-                    r_found = f.b_found != 0;
-                    r_sum = f.b_sum; r_mx = f.b_mx; r_sy = f.b_sy; r_up = f.b_up; r_cost = f.b_cost;
-                    --level;
-                    state = RESUME;
-                    continue;
-                }
-                state = CHARGE;
-            }
-            if (state == CHARGE) {
-                f.charge = add_rn(mul_rn(f.rate, mul_rn(nb, f.assumed)), f.comm);
-                const double rest = f.limit - f.charge;
-                if (!(rest > 0.0) || rest < lb[i + 1]) {    // nothing left, or not enough for any rest of the pipeline
-                    ++f.g2;
-                    state = NEXT_TYPE;
-                    continue;
-                }
-                DpbFrame& c = fr[level + 1];
-                c.g = f.g2; c.zp = f.zp2; c.limit = rest;
-                for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) c.u[t] = f.u2[t];
-                ++level;
-                state = ENTER;
-                continue;
-            }
-            // RESUME: the call for stages i + 1.. has returned
-            if (!r_found) {
-                ++f.g2;
-                state = NEXT_TYPE;
-                continue;
-            }
-            if (r_mx <= f.assumed) {                         // the assumption holds
-                const double all = add_rn(f.charge, r_cost);
-                if (all <= f.limit) {
-                    const double c_sum = add_rn(f.t, r_sum), c_mx = dmax(f.t, r_mx), c_sy = dmax(f.sync, r_sy),
-                                 c_up = dmax(f.upd, r_up);
-                    if (!f.b_found || dpb_value(nb, c_sum, c_mx, c_sy, c_up) < dpb_value(nb, f.b_sum, f.b_mx, f.b_sy, f.b_up)) {
-                        f.b_found = 1;
-                        f.b_sum = c_sum; f.b_mx = c_mx; f.b_sy = c_sy; f.b_up = c_up; f.b_cost = all;
-                        const DpbFrame& c = fr[level + 1];
-                        for (uint32_t j = i + 1; j < P; ++j) f.b_type[j] = c.b_type[j];
-                        f.b_type[i] = (uint8_t)g;
+        if (state == NEXT_TYPE) {
+            bool placed = false;
+            while (f.g2 < T) {
+                const uint32_t g2 = f.g2;
+                if ((okv[i + 1] >> g2) & 1u) {
+                    // first fit: this zone while it has room for one more stage of the type, else the next that has
+                    uint32_t zp2 = f.zp;
+                    if (!(f.u[g2] < pb.cap[f.zp][g2])) zp2 = pb.first_later[f.zp][g2];
+                    if (zp2 != DP_NONE) {
+                        f.zp2 = (uint8_t)zp2;
+                        for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) f.u2[t] = zp2 == f.zp ? f.u[t] : 0;
+                        f.u2[g2]++;
+                        const uint32_t z2 = pb.zone[zp2], dn = z2 * T + g2;
+                        f.t = add_rn(f.fb, c2x[dn * R + d]);
+                        f.comm = z2 != z ? mul_rn(xbytes, v.egress[z * Z + z2]) : 0.0;
+                        f.assumed = f.t;                 // first: this stage is the straggler
+                        placed = true;
+                        break;
                     }
                 }
                 ++f.g2;
-                state = NEXT_TYPE;
+            }
+            if (!placed) {                               // every type tried: hand the best plan back
+                r_found = f.b_found != 0;
+                r_sum = f.b_sum; r_mx = f.b_mx; r_sy = f.b_sy; r_up = f.b_up; r_cost = f.b_cost;
+                --level;
+                state = RESUME;
                 continue;
             }
-            f.assumed = r_mx;                                // charge again with the straggler that was found
             state = CHARGE;
         }
-        if (gave_up) break;
-        // the call for stage 0 on g0 has returned (level == -1)
-        if (r_found) {
-            const double val = dpb_value(nb, r_sum, r_mx, r_sy, r_up);
-            if (!best_found || val < best_v) {
-                best_found = true;
-                best_v = val;
-                for (uint32_t j = 0; j < P; ++j) best_type[j] = fr[0].b_type[j];
+        if (state == CHARGE) {
+            f.charge = add_rn(mul_rn(f.rate, mul_rn(nb, f.assumed)), f.comm);
+            const double rest = f.limit - f.charge;
+            if (!(rest > 0.0) || rest < lb[i + 1]) {    // nothing left, or not enough for any rest of the pipeline
+                ++f.g2;
+                state = NEXT_TYPE;
+                continue;
             }
+            DpbFrame& c = fr[level + 1];
+            c.g = f.g2; c.zp = f.zp2; c.limit = rest;
+            for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) c.u[t] = f.u2[t];
+            ++level;
+            state = ENTER;
+            continue;
         }
+        // RESUME: the call for stages i + 1.. has returned
+        if (!r_found) {
+            ++f.g2;
+            state = NEXT_TYPE;
+            continue;
+        }
+        if (r_mx <= f.assumed) {                         // the assumption holds
+            const double all = add_rn(f.charge, r_cost);
+            if (all <= f.limit) {
+                const double c_sum = add_rn(f.t, r_sum), c_mx = dmax(f.t, r_mx), c_sy = dmax(f.sync, r_sy),
+                             c_up = dmax(f.upd, r_up);
+                if (!f.b_found || dpb_value(nb, c_sum, c_mx, c_sy, c_up) < dpb_value(nb, f.b_sum, f.b_mx, f.b_sy, f.b_up)) {
+                    f.b_found = 1;
+                    f.b_sum = c_sum; f.b_mx = c_mx; f.b_sy = c_sy; f.b_up = c_up; f.b_cost = all;
+                    const DpbFrame& c = fr[level + 1];
+                    for (uint32_t j = i + 1; j < P; ++j) f.b_type[j] = c.b_type[j];
+                    f.b_type[i] = (uint8_t)g;
+                }
+            }
+            ++f.g2;
+            state = NEXT_TYPE;
+            continue;
+        }
+        f.assumed = r_mx;                                // charge again with the straggler that was found
+        state = CHARGE;
     }
-    atomicAdd(&bp.counters[4], nodes);
-    if (gave_up) { atomicAdd(&bp.counters[3], 1ull); return; }
-    if (!best_found) return;
+    root.nodes = nodes;
+    if (gave_up || !r_found) return;
+    root.value = dpb_value(nb, r_sum, r_mx, r_sy, r_up);
+    for (uint32_t j = 0; j < P; ++j) root.type[j] = fr[0].b_type[j];
+}
+
+// Per problem the best of its first stage's types (the lowest among equals), written out and simulated; one thread each.
+__global__ void __launch_bounds__(DP_FINISH_THREADS) dp_budget_finish_kernel(const __grid_constant__ DpBudgetParams bp) {
+    const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= bp.n_problems) return;
+    const DpProblem& pb = bp.problems[x];
+    const uint32_t T = bp.T, P = pb.P;
+    const DpbRoot* roots = bp.roots + (size_t)x * T;
+    unsigned long long nodes = 0;
+    double best_v = make_inf();
+    uint32_t best = DP_NONE;
+    for (uint32_t g = 0; g < T; ++g) {
+        nodes += roots[g].nodes;
+        if (roots[g].value < best_v) { best_v = roots[g].value; best = g; }
+    }
+    if (nodes) atomicAdd(&bp.counters[4], nodes);
+    if (nodes > bp.node_limit) { atomicAdd(&bp.counters[3], 1ull); return; }
+    if (best == DP_NONE) return;
     bp.value[pb.index] = best_v;
+    const uint8_t* best_type = roots[best].type;
+    DpResult& out = bp.results[pb.index];
+    TabView v;
+    v.bind(bp.blob, bp.blob);
+    const Config k = config_of(bp.sp, pb.config);
     // zones by first fit, as the recursion placed them; then the plan through the simulator (Sec. 4.3)
     sailor_run runs[DP_BUDGET_P_MAX];
     uint32_t n_runs = 0, zp = 0;

@@ -1689,7 +1689,7 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     lay.p_max = p_max; lay.T = T; lay.R = h.R;
     const size_t tab_bytes = (size_t)n_config * lay.stride() * sizeof(double);
     const size_t total = padded(tab_bytes) + padded(n_problems * sizeof(DpResult)) + padded(n_problems * sizeof(DpProblem)) +
-                         padded(n_problems * DP_BUDGET_P_MAX * sizeof(DpbFrame)) + padded(n_problems * sizeof(double)) +
+                         padded(n_problems * T * sizeof(DpbRoot)) + padded(n_problems * sizeof(double)) +
                          padded(40) + 4096;
     if (total > workspace_bytes) return SAILOR_E_RANGE;
     {
@@ -1700,7 +1700,7 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     double* d_tabs = bump.take<double>(tab_bytes / sizeof(double));
     DpResult* d_results = bump.take<DpResult>(n_problems);
     DpProblem* d_problems = bump.take<DpProblem>(n_problems);
-    DpbFrame* d_frames = bump.take<DpbFrame>(n_problems * DP_BUDGET_P_MAX);
+    DpbRoot* d_roots = bump.take<DpbRoot>(n_problems * T);
     double* d_value = bump.take<double>(n_problems);
     unsigned long long* d_counters = bump.take<unsigned long long>(5);
     DpOut* d_out = nullptr;
@@ -1722,13 +1722,15 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     DpBudgetParams bp;
     memset(&bp, 0, sizeof(bp));
     bp.blob = ctx->d_blob; bp.avail = ctx->d_avail; bp.sp = d; bp.problems = d_problems; bp.tabs = d_tabs;
-    bp.value = d_value; bp.results = d_results; bp.frames = d_frames; bp.counters = d_counters; bp.lay = lay;
-    bp.n_problems = (uint32_t)n_problems; bp.T = T;
+    bp.value = d_value; bp.results = d_results; bp.roots = d_roots; bp.counters = d_counters; bp.lay = lay;
+    bp.n_problems = (uint32_t)n_problems; bp.T = T; bp.p_max = p_max;
     bp.limit = o->budget_usd_per_iter;
     bp.node_limit = 1ull << 24;
-    dp_budget_kernel<<<(uint32_t)((n_problems + 63) / 64), 64, 0, ctx->stream>>>(bp);
+    dp_budget_kernel<<<(uint32_t)((n_problems * T + DPB_WARPS - 1) / DPB_WARPS), 32 * DPB_WARPS, dpb_smem(p_max), ctx->stream>>>(bp);
     CU(ctx, cudaGetLastError());
-    ++launches;
+    dp_budget_finish_kernel<<<(uint32_t)((n_problems + DP_FINISH_THREADS - 1) / DP_FINISH_THREADS), DP_FINISH_THREADS, 0, ctx->stream>>>(bp);
+    CU(ctx, cudaGetLastError());
+    launches += 2;
     DpSelectParams sel;
     memset(&sel, 0, sizeof(sel));
     sel.value = d_value; sel.results = d_results; sel.out = d_out; sel.counters = d_counters;
