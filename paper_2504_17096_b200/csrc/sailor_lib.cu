@@ -27,7 +27,6 @@ using namespace sailor;
 
 namespace {
 
-constexpr int SIM_THREADS = 256;
 constexpr int PLAN_SMEM_CEILING = 200 * 1024;    // dynamic shared memory any search may ask for
 
 // ---- kernels of the explicit-batch path -----------------------------------------------------
@@ -102,13 +101,15 @@ __global__ void compose_kernel(unsigned char* blob) {
     }
 }
 
-// One warp per plan with mixed replicas (records `stride` bytes apart holding `max_stages` stages, read in place,
-// lane i reading stage i).  Tables in shared memory, then R 64-bit GPU counters per warp.  Plans of up to 32 stages
-// are evaluated by the DEEP = false launch, which leaves deeper ones alone and notes in `deep_seen` that there are
-// some; the DEEP = true launch that follows returns at once when there are none and evaluates only those otherwise
-// (a lane then owns up to three stages; the state of that evaluation does not fit the registers of the first).
+// One warp per plan with mixed replicas (records `stride` bytes apart holding `max_stages` stages, read in place).
+// Tables in shared memory, then a scratch area per warp.  Plans of up to 32 stages are evaluated by the DEEP = false
+// launch, which leaves deeper ones alone and notes in `deep_seen` that there are some; the DEEP = true launch that follows
+// returns at once when there are none and evaluates only those otherwise (three times the scratch per warp).
+template <bool DEEP> constexpr uint32_t MIX_WARPS = DEEP ? 4 : 8;
+template <bool DEEP> constexpr uint32_t MIX_STAGES = DEEP ? SAILOR_MIX_P_MAX : 32;
+
 template <bool DEEP>
-__global__ void __launch_bounds__(SIM_THREADS, DEEP ? 2 : 4)
+__global__ void __launch_bounds__(32 * MIX_WARPS<DEEP>, 4)
 simulate_mixed_kernel(const unsigned char* __restrict__ blob, const uint16_t* __restrict__ avail,
                       const unsigned char* __restrict__ plans, uint32_t stride, uint32_t max_stages, uint64_t n,
                       double* __restrict__ t_iter, uint64_t* __restrict__ peak_mem, double* __restrict__ cost,
@@ -117,33 +118,31 @@ simulate_mixed_kernel(const unsigned char* __restrict__ blob, const uint16_t* __
     __shared__ uint64_t mbar;
     if (DEEP && *reinterpret_cast<volatile unsigned int*>(deep_seen) == 0) return;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    constexpr uint32_t WARPS = SIM_THREADS / 32;
+    constexpr uint32_t WARPS = MIX_WARPS<DEEP>;
     const uint32_t static_bytes = reinterpret_cast<const TabHdr*>(blob)->static_bytes;
     if (!bulk_load(dyn, blob, static_bytes, &mbar)) {
         if (tid == 0) atomicOr(error, SIM_ERR_DEVICE);
-        for (uint32_t x = tid; x < static_bytes / 16; x += SIM_THREADS)
+        for (uint32_t x = tid; x < static_bytes / 16; x += 32 * WARPS)
             reinterpret_cast<uint4*>(dyn)[x] = reinterpret_cast<const uint4*>(blob)[x];
         __syncthreads();
     }
     TabView v;
     v.bind(dyn, blob);
-    unsigned long long* counters = reinterpret_cast<unsigned long long*>(dyn + static_bytes) + (size_t)warp * v.h->R;
+    auto& scratch = reinterpret_cast<MixScratch<MIX_STAGES<DEEP>>*>(dyn + static_bytes)[warp];
     for (uint64_t j = (uint64_t)blockIdx.x * WARPS + warp; j < n; j += (uint64_t)gridDim.x * WARPS) {
         const sailor_mixed_plan& r = *reinterpret_cast<const sailor_mixed_plan*>(plans + j * stride);
         const uint32_t P = r.P;
         SimOut o;
-        if (DEEP) {
-            if (P <= 32 || P > max_stages) continue;             // done by the first launch
-            o = simulate_mixed_tiles<SAILOR_MIX_P_MAX / 32>(v, avail, r, counters, lane);
-        } else if (P > max_stages) {                             // more stages than the record has room for
+        if (DEEP && (P <= 32 || P > max_stages)) continue;       // done by the first launch
+        if (P > max_stages) {                                    // more stages than the record has room for
             o.t_iter = o.cost = make_nan();
             o.peak_mem = 0;
             o.status = SAILOR_ST_BAD_RECORD;
-        } else if (P > 32) {
+        } else if (!DEEP && P > 32) {
             if (lane == 0) *reinterpret_cast<volatile unsigned int*>(deep_seen) = 1u;
             continue;
         } else {
-            o = simulate_mixed_warp(v, avail, r, counters, lane);
+            o = simulate_mixed_warp(v, blob, avail, r, scratch, lane);
         }
         if (lane == 0) {
             if (t_iter) t_iter[j] = o.t_iter;
@@ -155,6 +154,11 @@ simulate_mixed_kernel(const unsigned char* __restrict__ blob, const uint16_t* __
         __syncwarp();
     }
 }
+
+template <bool DEEP>
+size_t mixed_smem(const TabHdr& h) { return h.static_bytes + sizeof(MixScratch<MIX_STAGES<DEEP>>) * MIX_WARPS<DEEP>; }
+template <bool DEEP>
+size_t mixed_finish_smem(const TabHdr& h) { return h.static_bytes + sizeof(MixFinishWarp<DEEP>) * MIXF_WARPS<DEEP>; }
 
 // ---- host state -----------------------------------------------------------------------------
 
@@ -1049,11 +1053,11 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
         CUF(cudaGetLastError());
     }
     // both kernels stage the static tables in dynamic shared memory; the create-time limit is 96 KB
-    CUF(cudaFuncSetAttribute(simulate_mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 64) * 1024));
-    CUF(cudaFuncSetAttribute(simulate_mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 64) * 1024));
+    CUF(cudaFuncSetAttribute(simulate_mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixScratch<MIX_STAGES<false>>) * MIX_WARPS<false>));
+    CUF(cudaFuncSetAttribute(simulate_mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixScratch<MIX_STAGES<true>>) * MIX_WARPS<true>));
     CUF(cudaFuncSetAttribute(finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 8) * 1024));
-    CUF(cudaFuncSetAttribute(mixed_finish_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 80) * 1024));
-    CUF(cudaFuncSetAttribute(mixed_finish_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 40) * 1024));
+    CUF(cudaFuncSetAttribute(mixed_finish_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixFinishWarp<false>) * MIXF_WARPS<false>));
+    CUF(cudaFuncSetAttribute(mixed_finish_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixFinishWarp<true>) * MIXF_WARPS<true>));
 #undef CUF
     *out = ctx;
     return SAILOR_OK;
@@ -1132,19 +1136,16 @@ int sailor_simulate_mixed_strided(sailor_ctx* ctx, const void* plans_v, uint64_t
     DeviceGuard guard(ctx->device);
     auto launch = [ctx, record_bytes, max_stages](const unsigned char* d_plans, uint64_t m, double* d_t, uint64_t* d_m, double* d_c,
                                                   uint32_t* d_s, uint32_t report_bad) {
-        const uint64_t tiles = (m + SIM_THREADS / 32 - 1) / (SIM_THREADS / 32);     // a warp per plan
-        const uint64_t cap = (uint64_t)ctx->sm_count * 32;
-        const uint32_t grid = (uint32_t)(tiles < cap ? tiles : cap);
-        const size_t smem = ctx->hdr.static_bytes + sizeof(unsigned long long) * (SIM_THREADS / 32) * ctx->hdr.R;
+        // a warp per plan; blocks take several plans per warp in larger batches
+        const uint64_t blocks = (m + MIX_WARPS<false> - 1) / MIX_WARPS<false>, cap = (uint64_t)ctx->sm_count * 32;
         unsigned int* deep_seen = ctx->d_sim_error + 1;
         if (max_stages > 32) CU(ctx, cudaMemsetAsync(deep_seen, 0, sizeof(unsigned int), ctx->stream));
-        simulate_mixed_kernel<false><<<grid, SIM_THREADS, smem, ctx->stream>>>(ctx->d_blob, ctx->d_avail, d_plans, record_bytes,
-                                                                                max_stages, m, d_t, d_m, d_c, d_s, ctx->d_sim_error,
-                                                                                deep_seen, report_bad);
+        simulate_mixed_kernel<false><<<(uint32_t)std::min(blocks, cap), 32 * MIX_WARPS<false>, mixed_smem<false>(ctx->hdr), ctx->stream>>>(
+            ctx->d_blob, ctx->d_avail, d_plans, record_bytes, max_stages, m, d_t, d_m, d_c, d_s, ctx->d_sim_error, deep_seen, report_bad);
         CU(ctx, cudaGetLastError());
         if (max_stages > 32) {                                   // the plans of more than 32 stages, if the first launch saw any
-            const uint64_t cap2 = (uint64_t)ctx->sm_count * 16;
-            simulate_mixed_kernel<true><<<(uint32_t)(tiles < cap2 ? tiles : cap2), SIM_THREADS, smem, ctx->stream>>>(
+            const uint64_t blocks2 = (m + MIX_WARPS<true> - 1) / MIX_WARPS<true>, cap2 = (uint64_t)ctx->sm_count * 16;
+            simulate_mixed_kernel<true><<<(uint32_t)std::min(blocks2, cap2), 32 * MIX_WARPS<true>, mixed_smem<true>(ctx->hdr), ctx->stream>>>(
                 ctx->d_blob, ctx->d_avail, d_plans, record_bytes, max_stages, m, d_t, d_m, d_c, d_s, ctx->d_sim_error, deep_seen,
                 report_bad);
             CU(ctx, cudaGetLastError());
@@ -2189,7 +2190,7 @@ static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const s
     }
     const MixedTables& mt = *ctx->mix;
     const uint64_t n_total = mt.flat_base[mt.n_config];
-    const uint32_t R = ctx->hdr.R, grid = (uint32_t)ctx->sm_count * 4;
+    const uint32_t grid = (uint32_t)ctx->sm_count * 4;
     MixedSearchParams mp;
     memset(&mp, 0, sizeof(mp));
     mixed_carve(ctx, mt, mp);
@@ -2219,8 +2220,8 @@ static int plan_mixed_impl(sailor_ctx* ctx, const sailor_mixed_space* s, const s
         CU(ctx, cudaGetLastError());
         launches += 2;
     }
-    if (deep) mixed_finish_kernel<true><<<1, 32 * MIXF_WARPS<true>, mixed_smem(ctx->hdr.static_bytes, R, MIXF_WARPS<true>), ctx->stream>>>(mp);
-    else mixed_finish_kernel<false><<<1, 32 * MIXF_WARPS<false>, mixed_smem(ctx->hdr.static_bytes, R, MIXF_WARPS<false>), ctx->stream>>>(mp);
+    if (deep) mixed_finish_kernel<true><<<1, 32 * MIXF_WARPS<true>, mixed_finish_smem<true>(ctx->hdr), ctx->stream>>>(mp);
+    else mixed_finish_kernel<false><<<1, 32 * MIXF_WARPS<false>, mixed_finish_smem<false>(ctx->hdr), ctx->stream>>>(mp);
     CU(ctx, cudaGetLastError());
     ++launches;
     CU(ctx, stream_sync(ctx));

@@ -12,7 +12,6 @@
 // mixed_finish_kernel, which merges them and writes the winners out with their records.
 #pragma once
 
-#include "sailor_batch.cuh"
 #include "sailor_mixed.cuh"
 
 namespace sailor {
@@ -113,10 +112,10 @@ struct MixedSearchParams {
 constexpr int MIXS_THREADS = 256;
 constexpr int MIXS_WARPS = MIXS_THREADS / 32;
 
-// The record of candidate `flat` into `plan` (shared memory, one per warp), by all lanes of the warp; the stages past
-// the last are all zero, as the host decoder leaves them.
+// The record of candidate `flat` into `plan` (shared memory, one per warp, room for `stages` stages), by all lanes of the
+// warp; the stages past the last are all zero, as the host decoder leaves them.
 __device__ __forceinline__ void mixed_candidate(const MixedSearchParams& mp, uint32_t T, uint32_t Z, uint64_t flat,
-                                                sailor_mixed_plan* plan, uint32_t lane) {
+                                                sailor_mixed_plan* plan, uint32_t stages, uint32_t lane) {
     uint32_t lo = 0, hi = mp.n_config;                       // the configuration whose block holds the index
     while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) >> 1;
@@ -131,7 +130,7 @@ __device__ __forceinline__ void mixed_candidate(const MixedSearchParams& mp, uin
         plan->P = (uint8_t)k.P; plan->mbs_idx = (uint8_t)k.mi; plan->rc = (uint8_t)k.rc; plan->_pad = 0;
         plan->D = (uint16_t)k.D; plan->_pad2 = 0;
     }
-    for (uint32_t i = lane; i < SAILOR_MIX_P_MAX; i += 32) {
+    for (uint32_t i = lane; i < stages; i += 32) {
         if (i < k.P) mixed_build_stage(mp.sp, k, T, mp.combs, digit, i, &plan->stage[i]);
         else {
             uint32_t* z = reinterpret_cast<uint32_t*>(&plan->stage[i]);
@@ -564,10 +563,16 @@ __global__ void __launch_bounds__(MIXS_THREADS, 2) plan_mixed_kernel(const __gri
     }
 }
 
-// Merge the blocks' lists; the winners are built and simulated again for the result records, a warp each and all at
-// once (32 warps of 64 registers; 16 of 128 where deep pipelines need the tiled evaluation).  Results and counters go
-// straight into the host's memory; the counters are put back to their starting values for the next search.
-template <bool DEEP> constexpr uint32_t MIXF_WARPS = DEEP ? 16 : 32;
+// Merge the blocks' lists; the winners are built and simulated again for the result records, a warp each.  DEEP: the
+// space has pipelines of more than 32 stages.  Results and counters go straight into the host's memory; the counters are
+// put back to their starting values for the next search.
+template <bool DEEP> constexpr uint32_t MIXF_WARPS = DEEP ? 4 : 16;
+template <bool DEEP>
+struct MixFinishWarp {                   // what a warp of it keeps in shared memory
+    static constexpr uint32_t STAGES = DEEP ? SAILOR_MIX_P_MAX : 32;
+    MixScratch<STAGES> scratch;
+    uint64_t plan[(offsetof(sailor_mixed_plan, stage) + STAGES * sizeof(sailor_mixed_stage)) / 8];   // the record, cut to STAGES stages
+};
 
 template <bool DEEP>
 __global__ void __launch_bounds__(32 * MIXF_WARPS<DEEP>) mixed_finish_kernel(const __grid_constant__ MixedSearchParams mp) {
@@ -586,14 +591,14 @@ __global__ void __launch_bounds__(32 * MIXF_WARPS<DEEP>) mixed_finish_kernel(con
     }
     TabView v;
     v.bind(dyn, mp.blob);
-    const uint32_t T = v.h->T, Z = v.h->Z, R = v.h->R;
-    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(dyn + static_bytes) + (size_t)warp * R;
-    sailor_mixed_plan* plan = reinterpret_cast<sailor_mixed_plan*>(dyn + static_bytes + sizeof(unsigned long long) * NW * R) + warp;
+    const uint32_t T = v.h->T, Z = v.h->Z;
+    MixFinishWarp<DEEP>& mine = reinterpret_cast<MixFinishWarp<DEEP>*>(dyn + static_bytes)[warp];
+    sailor_mixed_plan* plan = reinterpret_cast<sailor_mixed_plan*>(mine.plan);
     const uint32_t n = merge_block_lists<NW>(mp.partial, mp.n_partial, mp.k, s_hits, s_sel, &s_n);
     for (uint32_t j = warp; j < n; j += NW) {
         const uint64_t flat = s_hits[0][j].flat;
-        mixed_candidate(mp, T, Z, flat, plan, lane);
-        const SimOut o = DEEP ? simulate_mixed_plan(v, mp.avail, *plan, cnt, lane) : simulate_mixed_warp(v, mp.avail, *plan, cnt, lane);
+        mixed_candidate(mp, T, Z, flat, plan, MixFinishWarp<DEEP>::STAGES, lane);
+        const SimOut o = simulate_mixed_warp(v, mp.blob, mp.avail, *plan, mine.scratch, lane);
         __syncwarp();
         sailor_mixed_result* r = mp.out->results + j;
         if (lane == 0) {
@@ -603,7 +608,7 @@ __global__ void __launch_bounds__(32 * MIXF_WARPS<DEEP>) mixed_finish_kernel(con
         // the record, word by word
         const uint64_t* src = reinterpret_cast<const uint64_t*>(plan);
         uint64_t* dst = reinterpret_cast<uint64_t*>(&r->plan);
-        for (uint32_t x = lane; x < sizeof(sailor_mixed_plan) / 8; x += 32) dst[x] = src[x];
+        for (uint32_t x = lane; x < sizeof(sailor_mixed_plan) / 8; x += 32) dst[x] = x < sizeof(mine.plan) / 8 ? src[x] : 0ull;
         __syncwarp();
     }
     if (tid < MIXC_N) {
@@ -612,11 +617,6 @@ __global__ void __launch_bounds__(32 * MIXF_WARPS<DEEP>) mixed_finish_kernel(con
         live[tid] = tid == MIXC_MIN_COST ? COST_BITS_START : 0ull;
     }
     if (tid == 0) mp.out->span.end = device_ns();
-}
-
-// Shared memory of `warps` evaluating warps: the static tables, R counters and a record per warp.
-inline size_t mixed_smem(uint32_t static_bytes, uint32_t R, uint32_t warps) {
-    return static_bytes + (sizeof(unsigned long long) * R + sizeof(sailor_mixed_plan)) * warps;
 }
 
 }  // namespace sailor

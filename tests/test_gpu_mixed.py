@@ -194,3 +194,33 @@ def test_mixed_device_pointers_empty_and_bad_records():
         torch.cuda.synchronize()
         assert st.cpu().tolist()[1] == B.ST_BAD_RECORD and not (st.cpu().tolist()[0] & B.ST_BAD_RECORD)
         assert math.isnan(tt.cpu().tolist()[1])
+
+
+@pytest.mark.parametrize("D,stages", [(2, 1), (32, 5), (33, 32), (64, 31), (65, 33), (300, 96), (7, 64)])
+def test_mixed_interval_edges(D, stages):
+    """Intervals between group boundaries are found by one bit per replica up to D = 64 and boundary by boundary beyond;
+    items and pipelines take several rounds of 32 lanes when there are many: up to four groups a stage, cut differently."""
+    w = W.tiny(seed=37, n_types=4, n_zones=3, L=max(stages, 4), gbs=D * 4, d_values=(D,), p_values=[stages])
+    w.gpus_per_node[...] = [4, 64, 700, 2]
+    rng = W.SplitMix64(D * 131 + stages)
+    plans = []
+    for j in range(40):
+        st = []
+        for i in range(stages):
+            cuts = sorted({rng.randint(1, D - 1) for _ in range(rng.randint(0, 3))})
+            b = [0] + cuts + [D]
+            if j % 7 == 3 and i == stages // 2:
+                b[-1] += 1                                       # one replica too many: an invalid plan
+            st.append({"zone": rng.randint(0, 2) if j % 3 else 1,
+                       "groups": [(rng.randint(0, 3), rng.randint(0, 2), b[q + 1] - b[q]) for q in range(len(b) - 1)]})
+        plans.append({"P": stages, "mbs_idx": rng.randint(0, 2), "rc": j & 1, "D": D, "stages": st})
+    o = Oracle(w)
+    ctx = B.sailor_create(w, 0, 0)
+    try:
+        B.sailor_set_availability(ctx, w.avail)
+        t, m, c, s = B.sailor_simulate_mixed(ctx, B.pack_mixed_plans(plans))
+    finally:
+        B.sailor_destroy(ctx)
+    so, to, co, mo = o.simulate_mixed_batch(plans)
+    assert np.array_equal(s, so) and np.array_equal(m, mo)
+    assert np.array_equal(t, to, equal_nan=True) and np.array_equal(c, co, equal_nan=True)
