@@ -1053,6 +1053,7 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
         CUF(cudaGetLastError());
     }
     // both kernels stage the static tables in dynamic shared memory; the create-time limit is 96 KB
+    CUF(cudaFuncSetAttribute(simulate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
     CUF(cudaFuncSetAttribute(simulate_mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixScratch<MIX_STAGES<false>>) * MIX_WARPS<false>));
     CUF(cudaFuncSetAttribute(simulate_mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixScratch<MIX_STAGES<true>>) * MIX_WARPS<true>));
     CUF(cudaFuncSetAttribute(finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 8) * 1024));
@@ -1097,24 +1098,29 @@ int sailor_simulate(sailor_ctx* ctx, const sailor_plan_rec* plans, uint64_t n, i
     if ((uintptr_t)plans % 8 != 0) return SAILOR_E_ARG;
     DeviceGuard guard(ctx->device);
     auto launch = [ctx](const sailor_plan_rec* d_plans, uint64_t m, double* d_t, uint64_t* d_m, double* d_c, uint32_t* d_s,
-                        unsigned int* bad_flag) {
-        const uint64_t tiles = (m + BATCH_POOL - 1) / BATCH_POOL;
-        const uint64_t cap = (uint64_t)ctx->sm_count * BATCH_BLOCKS_PER_SM * 4;   // the resident blocks, four pools each at least
-        const uint32_t grid = (uint32_t)(tiles < cap ? tiles : cap);
-        simulate_kernel<<<grid, BATCH_THREADS, 0, ctx->stream>>>(ctx->d_blob, ctx->d_avail, d_plans, m, d_t, d_m, d_c, d_s, bad_flag);
+                        uint32_t report_bad) {
+        // as many pools for every SM, and no larger ones than that takes
+        const uint64_t turns = (m + (uint64_t)ctx->sm_count * BATCH_POOL - 1) / ((uint64_t)ctx->sm_count * BATCH_POOL);
+        const uint64_t share = (m + ctx->sm_count * turns - 1) / (ctx->sm_count * turns);
+        const uint32_t pool = (uint32_t)((share + 31) / 32 * 32);
+        const uint64_t pools = (m + pool - 1) / pool;
+        const uint32_t grid = (uint32_t)std::min<uint64_t>(pools, (uint64_t)ctx->sm_count);
+        const BatchParams p = batch_params(ctx->hdr, ctx->d_blob);
+        simulate_kernel<<<grid, BATCH_THREADS, p.smem, ctx->stream>>>(
+            p, ctx->d_avail, d_plans, m, pool, d_t, d_m, d_c, d_s, ctx->d_sim_error, report_bad);
         CU(ctx, cudaGetLastError());
         return (int)SAILOR_OK;
     };
     if (!on_device)                                               // records are checked by the kernel (SIM_ERR_BAD_RECORD)
         return host_batch(ctx, reinterpret_cast<const unsigned char*>(plans), sizeof(sailor_plan_rec), n, t_iter, peak_mem, cost,
                           status, [&](const unsigned char* d_recs, uint64_t m, double* d_t, uint64_t* d_m, double* d_c, uint32_t* d_s) {
-                              return launch(reinterpret_cast<const sailor_plan_rec*>(d_recs), m, d_t, d_m, d_c, d_s, ctx->d_sim_error);
+                              return launch(reinterpret_cast<const sailor_plan_rec*>(d_recs), m, d_t, d_m, d_c, d_s, 1u);
                           });
     {
         const int rc_up = upload_availability(ctx);
         if (rc_up) return rc_up;
     }
-    return launch(plans, n, t_iter, peak_mem, cost, status, nullptr);
+    return launch(plans, n, t_iter, peak_mem, cost, status, 0u);
 }
 
 int sailor_simulate_mixed(sailor_ctx* ctx, const sailor_mixed_plan* plans, uint64_t n, int on_device, double* t_iter,

@@ -154,6 +154,37 @@ def test_simulate_empty_and_bad_records(make_ctx, torch_cuda):
     assert L.sailor_simulate(cx.ctx, both.ctypes.data, 1, 0, out_t.ctypes.data, None, None, out_s.ctypes.data) == B.OK
 
 
+@pytest.mark.parametrize("n,L,kind", [(1, 8, "plain"), (33, 8, "poly"), (4737, 96, "plain"), (113700, 12, "bare"), (227333, 96, "plain"),
+                                      (9000, 420, "poly"), (9000, 420, "plain")])
+def test_simulate_batch_shapes(n, L, kind, make_ctx, torch_cuda):
+    """The batch kernel takes pools of 32 to 768 records, several a block when the batch is large, from device memory that
+    may start 8 bytes past a 16-byte line; gradient tables move out of shared memory for long models, and models may lack an
+    embedding or a head.  Up to 16 runs that repeat zones and types.  A record's results do not depend on its place."""
+    torch = torch_cuda
+    w = W.tiny(seed=41, n_types=2, n_zones=2, L=L, gbs=104, p_values=[p for p in (1, 2, 3, 24, 96) if p <= L], d_values=(1, 2, 3, 8))
+    w.avail[...] = [[60, 9], [300, 25]]
+    if kind == "poly":
+        w = W.with_bandwidth_polynomials(w, seed=5)
+    if kind == "bare":
+        w.has_embed = w.has_head = 0
+    base = 1500
+    recs = W.random_plans(w, base, seed=n)
+    expected = Oracle(w).simulate_records(recs)
+    pick = np.arange(n) * 7 % base
+    packed = B.pack_records(recs)[pick]
+    cx = make_ctx(w)
+    for shift in (0, 8):
+        d = torch.zeros(n * 72 + 16, dtype=torch.uint8, device="cuda")
+        d[shift:shift + n * 72] = torch.from_numpy(packed.view(np.uint8).reshape(-1).copy()).cuda()
+        t, c = torch.empty(n, dtype=torch.float64, device="cuda"), torch.empty(n, dtype=torch.float64, device="cuda")
+        m, s = torch.empty(n, dtype=torch.int64, device="cuda"), torch.empty(n, dtype=torch.int32, device="cuda")
+        B.sailor_simulate_device(cx.ctx, d.data_ptr() + shift, n, t.data_ptr(), m.data_ptr(), c.data_ptr(), s.data_ptr())
+        torch.cuda.synchronize()
+        gpu = (t.cpu().numpy(), m.cpu().numpy().view(np.uint64), c.cpu().numpy(), s.cpu().numpy().view(np.uint32))
+        assert_sim_equal(gpu, tuple(x[pick] for x in expected), (n, kind, shift))
+    assert_sim_equal(B.sailor_simulate(cx.ctx, packed), tuple(x[pick] for x in expected), (n, kind, "host"))
+
+
 def test_simulate_host_batch_in_chunks(make_ctx):
     """A host batch larger than what the library stages at a time (chunks of 2^19 records taking turns in three
     slots): every record's results are the oracle's, whichever chunk and slot it went through; a ragged last chunk."""
