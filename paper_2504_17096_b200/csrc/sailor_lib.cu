@@ -197,12 +197,15 @@ struct SpaceCache {
 };
 
 // What a context keeps in pinned host memory the device can write.
+constexpr size_t HOST_SMALL_BYTES = 192 * 1024;
+
 struct HostBlock {
     PlanOut out;                           // results of a search
     SurveyOut survey;                      // what the survey of a space found
     uint16_t avail[R_MAX];                 // the availability snapshot last set
     MixedOut mixed;                        // results of a search over plans with mixed replicas
     DpOut dp;                              // results of a search over per-stage GPU types
+    alignas(256) unsigned char batch[HOST_SMALL_BYTES];     // a small host batch: error word, results, records
 };
 
 constexpr size_t CFG_CACHE_MAX_BYTES = 512ull << 20;
@@ -348,7 +351,7 @@ int device_grow(sailor_ctx* ctx, unsigned char** p, size_t* have, size_t need) {
     return rc;
 }
 
-// Pinned host blocks (76 KB each): allocating one can cost a millisecond, so the process keeps a few that no context
+// Pinned host blocks (268 KB each): allocating one can cost a millisecond, so the process keeps a few that no context
 // uses at the moment.
 class HostBlocks {
   public:
@@ -762,15 +765,18 @@ int enqueue_pass(sailor_ctx* ctx, uint32_t obj, double budget, bool budget_from_
 // End of a host-side batch call: read the batch kernels' error word with the results, wait, and report (and
 // clear) a fault.  Device-side batch calls only enqueue work; a fault in one of them is reported here as well,
 // by the next host-side call.
+int host_batch_error(unsigned int err) {
+    return err == 0 ? SAILOR_OK : (err & SIM_ERR_DEVICE) ? SAILOR_E_DEVICE : SAILOR_E_RANGE;
+}
+
 int finish_host_batch(sailor_ctx* ctx) {
     unsigned int* h_err = &ctx->h_out->ctrl.error;               // pinned; no search is in flight on this context
     CU(ctx, cudaMemcpyAsync(h_err, ctx->d_sim_error, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
     CU(ctx, stream_sync(ctx));
     if (*h_err) {
         CU(ctx, cudaMemsetAsync(ctx->d_sim_error, 0, sizeof(unsigned int), ctx->stream));
-        return (*h_err & SIM_ERR_DEVICE) ? SAILOR_E_DEVICE : SAILOR_E_RANGE;
     }
-    return SAILOR_OK;
+    return host_batch_error(*h_err);
 }
 
 // A host-side batch: records of `rec_bytes` in, four result arrays out (any may be NULL).  The batch goes through
@@ -779,15 +785,50 @@ int finish_host_batch(sailor_ctx* ctx) {
 // directions of the host link carry data at the same time; a slot is filled again only after its results have
 // left.  The staging memory therefore does not grow with the batch beyond HOST_SLOTS chunks.  Records are checked
 // by the kernel that reads them (`launch` passes the error word along, and a record outside its tables sets
-// SIM_ERR_BAD_RECORD in it).  `launch(d_records, m, d_t, d_m, d_c, d_s)` enqueues the evaluation of m records on
+// SIM_ERR_BAD_RECORD in it).  `launch(d_records, m, d_t, d_m, d_c, d_s, error)` enqueues the evaluation of m records on
 // the context's stream.
 constexpr uint64_t HOST_CHUNK_RECORDS = 1u << 19, HOST_CHUNK_BYTES = 1u << 26;
 constexpr uint32_t HOST_SLOTS = 3;
 int upload_availability(sailor_ctx* ctx);
 
+// A host batch of up to HOST_SMALL_BYTES: its records go through the context's pinned block in one copy, the kernel writes
+// results and error word straight back into that block.  1 000 records: 96 us with pageable copies each way (four of results,
+// one of the error word), 61 with one copy back, 54 this way; a tenth of that is the host's own copying, which larger batches
+// would pay instead of the driver's.
+template <class Launch>
+int host_batch_small(sailor_ctx* ctx, const unsigned char* recs, size_t rec_bytes, uint64_t n, double* t_iter, uint64_t* peak_mem,
+                     double* cost, uint32_t* status, Launch launch) {
+    int rc = device_grow(ctx, &ctx->d_stage, &ctx->stage_bytes, HOST_SMALL_BYTES);
+    if (rc == SAILOR_OK) rc = upload_availability(ctx);
+    if (rc != SAILOR_OK) return rc;
+    unsigned char* const h_recs = ctx->host->batch;            // records, error word, t_iter, cost, peak_mem, status
+    unsigned char* const h_out = h_recs + (n * rec_bytes + 15) / 16 * 16;
+    unsigned char* out = nullptr;
+    CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&out), h_out, 0));
+    memcpy(h_recs, recs, n * rec_bytes);
+    memset(h_out, 0, 16);
+    CU(ctx, cudaMemcpyAsync(ctx->d_stage, h_recs, n * rec_bytes, cudaMemcpyHostToDevice, ctx->stream));
+    double* t = reinterpret_cast<double*>(out + 16);
+    rc = launch(ctx->d_stage, n, t_iter ? t : nullptr, peak_mem ? reinterpret_cast<uint64_t*>(t + 2 * n) : nullptr,
+                cost ? t + n : nullptr, status ? reinterpret_cast<uint32_t*>(t + 3 * n) : nullptr, reinterpret_cast<unsigned int*>(out));
+    const cudaError_t ce = stream_sync(ctx);                   // the pinned block is free again, whatever happened
+    if (rc != SAILOR_OK) return rc;
+    if (ce != cudaSuccess) { ctx->last_cuda = (int)ce; return SAILOR_E_CUDA; }
+    const unsigned char* r = h_out + 16;
+    if (t_iter) memcpy(t_iter, r, 8 * n);
+    if (cost) memcpy(cost, r + 8 * n, 8 * n);
+    if (peak_mem) memcpy(peak_mem, r + 16 * n, 8 * n);
+    if (status) memcpy(status, r + 24 * n, 4 * n);
+    unsigned int err;
+    memcpy(&err, h_out, sizeof(err));
+    return host_batch_error(err);
+}
+
 template <class Launch>
 int host_batch(sailor_ctx* ctx, const unsigned char* recs, size_t rec_bytes, uint64_t n, double* t_iter, uint64_t* peak_mem,
                double* cost, uint32_t* status, Launch launch) {
+    if (n <= (HOST_SMALL_BYTES - 32) / (rec_bytes + 28))
+        return host_batch_small(ctx, recs, rec_bytes, n, t_iter, peak_mem, cost, status, launch);
     uint64_t chunk = HOST_CHUNK_BYTES / rec_bytes;             // records per chunk: 64 MB of records, 2^19 at most
     chunk = chunk > HOST_CHUNK_RECORDS ? HOST_CHUNK_RECORDS : chunk;
     const bool split = n > chunk;
@@ -826,7 +867,7 @@ int host_batch(sailor_ctx* ctx, const unsigned char* recs, size_t rec_bytes, uin
             if ((ce = cudaStreamWaitEvent(ctx->stream, ctx->ev_slot[slot], 0)) != cudaSuccess) break;
         ce = cudaMemcpyAsync(d_recs, recs + off * rec_bytes, m * rec_bytes, cudaMemcpyHostToDevice, ctx->stream);
         if (ce != cudaSuccess) break;
-        rc = launch(d_recs, m, d_t, d_m, d_c, d_s);
+        rc = launch(d_recs, m, d_t, d_m, d_c, d_s, ctx->d_sim_error);
         if (rc != SAILOR_OK) break;
         if (split) {
             if ((ce = cudaEventRecord(ctx->ev_chunk, ctx->stream)) != cudaSuccess) break;
@@ -1098,7 +1139,7 @@ int sailor_simulate(sailor_ctx* ctx, const sailor_plan_rec* plans, uint64_t n, i
     if ((uintptr_t)plans % 8 != 0) return SAILOR_E_ARG;
     DeviceGuard guard(ctx->device);
     auto launch = [ctx](const sailor_plan_rec* d_plans, uint64_t m, double* d_t, uint64_t* d_m, double* d_c, uint32_t* d_s,
-                        uint32_t report_bad) {
+                        unsigned int* error, uint32_t report_bad) {
         // as many pools for every SM, and no larger ones than that takes
         const uint64_t turns = (m + (uint64_t)ctx->sm_count * BATCH_POOL - 1) / ((uint64_t)ctx->sm_count * BATCH_POOL);
         const uint64_t share = (m + ctx->sm_count * turns - 1) / (ctx->sm_count * turns);
@@ -1107,20 +1148,20 @@ int sailor_simulate(sailor_ctx* ctx, const sailor_plan_rec* plans, uint64_t n, i
         const uint32_t grid = (uint32_t)std::min<uint64_t>(pools, (uint64_t)ctx->sm_count);
         const BatchParams p = batch_params(ctx->hdr, ctx->d_blob);
         simulate_kernel<<<grid, BATCH_THREADS, p.smem, ctx->stream>>>(
-            p, ctx->d_avail, d_plans, m, pool, d_t, d_m, d_c, d_s, ctx->d_sim_error, report_bad);
+            p, ctx->d_avail, d_plans, m, pool, d_t, d_m, d_c, d_s, error, report_bad);
         CU(ctx, cudaGetLastError());
         return (int)SAILOR_OK;
     };
     if (!on_device)                                               // records are checked by the kernel (SIM_ERR_BAD_RECORD)
         return host_batch(ctx, reinterpret_cast<const unsigned char*>(plans), sizeof(sailor_plan_rec), n, t_iter, peak_mem, cost,
-                          status, [&](const unsigned char* d_recs, uint64_t m, double* d_t, uint64_t* d_m, double* d_c, uint32_t* d_s) {
-                              return launch(reinterpret_cast<const sailor_plan_rec*>(d_recs), m, d_t, d_m, d_c, d_s, 1u);
+                          status, [&](const unsigned char* d_recs, uint64_t m, double* d_t, uint64_t* d_m, double* d_c, uint32_t* d_s, unsigned int* error) {
+                              return launch(reinterpret_cast<const sailor_plan_rec*>(d_recs), m, d_t, d_m, d_c, d_s, error, 1u);
                           });
     {
         const int rc_up = upload_availability(ctx);
         if (rc_up) return rc_up;
     }
-    return launch(plans, n, t_iter, peak_mem, cost, status, 0u);
+    return launch(plans, n, t_iter, peak_mem, cost, status, ctx->d_sim_error, 0u);
 }
 
 int sailor_simulate_mixed(sailor_ctx* ctx, const sailor_mixed_plan* plans, uint64_t n, int on_device, double* t_iter,
@@ -1141,18 +1182,18 @@ int sailor_simulate_mixed_strided(sailor_ctx* ctx, const void* plans_v, uint64_t
     const uint32_t max_stages = (record_bytes - HEAD) / (uint32_t)sizeof(sailor_mixed_stage);
     DeviceGuard guard(ctx->device);
     auto launch = [ctx, record_bytes, max_stages](const unsigned char* d_plans, uint64_t m, double* d_t, uint64_t* d_m, double* d_c,
-                                                  uint32_t* d_s, uint32_t report_bad) {
+                                                  uint32_t* d_s, unsigned int* error, uint32_t report_bad) {
         // a warp per plan; blocks take several plans per warp in larger batches
         const uint64_t blocks = (m + MIX_WARPS<false> - 1) / MIX_WARPS<false>, cap = (uint64_t)ctx->sm_count * 32;
         unsigned int* deep_seen = ctx->d_sim_error + 1;
         if (max_stages > 32) CU(ctx, cudaMemsetAsync(deep_seen, 0, sizeof(unsigned int), ctx->stream));
         simulate_mixed_kernel<false><<<(uint32_t)std::min(blocks, cap), 32 * MIX_WARPS<false>, mixed_smem<false>(ctx->hdr), ctx->stream>>>(
-            ctx->d_blob, ctx->d_avail, d_plans, record_bytes, max_stages, m, d_t, d_m, d_c, d_s, ctx->d_sim_error, deep_seen, report_bad);
+            ctx->d_blob, ctx->d_avail, d_plans, record_bytes, max_stages, m, d_t, d_m, d_c, d_s, error, deep_seen, report_bad);
         CU(ctx, cudaGetLastError());
         if (max_stages > 32) {                                   // the plans of more than 32 stages, if the first launch saw any
             const uint64_t blocks2 = (m + MIX_WARPS<true> - 1) / MIX_WARPS<true>, cap2 = (uint64_t)ctx->sm_count * 16;
             simulate_mixed_kernel<true><<<(uint32_t)std::min(blocks2, cap2), 32 * MIX_WARPS<true>, mixed_smem<true>(ctx->hdr), ctx->stream>>>(
-                ctx->d_blob, ctx->d_avail, d_plans, record_bytes, max_stages, m, d_t, d_m, d_c, d_s, ctx->d_sim_error, deep_seen,
+                ctx->d_blob, ctx->d_avail, d_plans, record_bytes, max_stages, m, d_t, d_m, d_c, d_s, error, deep_seen,
                 report_bad);
             CU(ctx, cudaGetLastError());
         }
@@ -1160,14 +1201,14 @@ int sailor_simulate_mixed_strided(sailor_ctx* ctx, const void* plans_v, uint64_t
     };
     if (!on_device)                                               // records are checked by the kernel (SIM_ERR_BAD_RECORD)
         return host_batch(ctx, plans, record_bytes, n, t_iter, peak_mem, cost, status,
-                          [&](const unsigned char* d_recs, uint64_t m, double* d_t, uint64_t* d_m, double* d_c, uint32_t* d_s) {
-                              return launch(d_recs, m, d_t, d_m, d_c, d_s, 1u);
+                          [&](const unsigned char* d_recs, uint64_t m, double* d_t, uint64_t* d_m, double* d_c, uint32_t* d_s, unsigned int* error) {
+                              return launch(d_recs, m, d_t, d_m, d_c, d_s, error, 1u);
                           });
     {
         const int rc_up = upload_availability(ctx);
         if (rc_up) return rc_up;
     }
-    return launch(plans, n, t_iter, peak_mem, cost, status, 0u);
+    return launch(plans, n, t_iter, peak_mem, cost, status, ctx->d_sim_error, 0u);
 }
 
 int sailor_space_size(const sailor_ctx* ctx, const sailor_space* s, uint64_t* n_out) {

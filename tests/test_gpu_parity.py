@@ -185,6 +185,30 @@ def test_simulate_batch_shapes(n, L, kind, make_ctx, torch_cuda):
     assert_sim_equal(B.sailor_simulate(cx.ctx, packed), tuple(x[pick] for x in expected), (n, kind, "host"))
 
 
+@pytest.mark.parametrize("n", [1, 2, 1965, 1966, 1967])
+def test_simulate_small_host_batches(n, make_ctx):
+    """Host batches go through the context's pinned block up to 1 965 records, through pageable copies beyond; any output
+    array may be left out, and a bad record is reported in every case."""
+    w = W.tiny(seed=43, n_types=3, n_zones=2)
+    cx, L = make_ctx(w), B.load()
+    recs = W.random_plans(w, n, seed=n)
+    so, to, co, mo = Oracle(w).simulate_records(recs)
+    packed = B.pack_records(recs)
+    assert_sim_equal(B.sailor_simulate(cx.ctx, packed), (so, to, co, mo), n)
+    for keep in range(4):                                          # one output at a time
+        out = [np.full(n, 77, t) for t in (np.float64, np.uint64, np.float64, np.uint32)]
+        args = [o.ctypes.data if j == keep else None for j, o in enumerate(out)]
+        assert L.sailor_simulate(cx.ctx, packed.ctypes.data, n, 0, *args) == B.OK
+        assert np.array_equal(out[keep], (to, mo, co, so)[keep], equal_nan=keep in (0, 2))
+    packed["D"][n - 1] = 0
+    assert L.sailor_simulate(cx.ctx, packed.ctypes.data, n, 0, None, None, None, None) == B.E_RANGE
+    s = np.zeros(n, np.uint32)
+    assert L.sailor_simulate(cx.ctx, packed.ctypes.data, n, 0, None, None, None, s.ctypes.data) == B.E_RANGE
+    assert s[-1] == B.ST_BAD_RECORD and np.array_equal(s[:-1], so[:-1])
+    packed["D"][n - 1] = 1
+    assert L.sailor_simulate(cx.ctx, packed.ctypes.data, n, 0, None, None, None, None) == B.OK
+
+
 def test_simulate_host_batch_in_chunks(make_ctx):
     """A host batch larger than what the library stages at a time (chunks of 2^19 records taking turns in three
     slots): every record's results are the oracle's, whichever chunk and slot it went through; a ragged last chunk."""
