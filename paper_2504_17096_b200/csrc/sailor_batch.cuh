@@ -125,7 +125,7 @@ struct BatchRing {
     uint16_t rank[BATCH_POOL];                       // of a record among those of its bin
     uint32_t run[BATCH_WARPS][SAILOR_RUN_MAX][32];   // runs of the records that a warp is evaluating
     uint64_t loaded[BATCH_RING], ready[BATCH_RING], drained[BATCH_RING];     // barriers
-    uint32_t ticket;                                 // next group of 32 records, counted over all pools of the block
+    uint32_t ticket;                                 // next group of records, counted over all pools of the block
 };
 
 inline BatchParams batch_params(const TabHdr& h, const unsigned char* blob) {
@@ -384,7 +384,7 @@ __device__ __forceinline__ void order_pool(const uint64_t* rec, uint16_t* perm, 
 // 896 and 1 024 the same 411.  Results leave as four structure-of-arrays streams.
 __global__ void __launch_bounds__(BATCH_THREADS, 1)
 simulate_kernel(const __grid_constant__ BatchParams p, const uint16_t* __restrict__ avail,
-                const sailor_plan_rec* __restrict__ plans, uint64_t n, uint32_t pool_size, double* __restrict__ t_iter,
+                const sailor_plan_rec* __restrict__ plans, uint64_t n, uint32_t pool_size, uint32_t lanes, double* __restrict__ t_iter,
                 uint64_t* __restrict__ peak_mem, double* __restrict__ cost, uint32_t* __restrict__ status, unsigned int* error,
                 uint32_t report_bad) {                         // report_bad: set SIM_ERR_BAD_RECORD when a record is refused
     extern __shared__ __align__(16) unsigned char dyn[];
@@ -418,7 +418,7 @@ simulate_kernel(const __grid_constant__ BatchParams p, const uint16_t* __restric
         for (uint32_t s = 0; s < BATCH_RING; ++s) {
             bar_init(&ring.loaded[s], 1);
             bar_init(&ring.ready[s], 1);
-            bar_init(&ring.drained[s], pool_size / 32);
+            bar_init(&ring.drained[s], pool_size / lanes);
         }
         ring.ticket = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -483,17 +483,18 @@ simulate_kernel(const __grid_constant__ BatchParams p, const uint16_t* __restric
         return;
     }
     uint32_t* run = &ring.run[warp][0][lane];
+    const uint32_t groups = pool_size / lanes;
     for (uint32_t it = 0, base = 0;;) {
         uint32_t grp = 0;
         if (lane == 0) grp = atomicAdd(&ring.ticket, 1u);
         grp = __shfl_sync(FULL, grp, 0);
-        for (; grp - base >= pool_size / 32; base += pool_size / 32) ++it;
+        for (; grp - base >= groups; base += groups) ++it;
         if (it >= mine) break;
         const uint32_t slot = it % BATCH_RING;
         if (!bar_wait(&ring.ready[slot], (it / BATCH_RING) & 1u)) { if (lane == 0) atomicOr(error, SIM_ERR_DEVICE); return; }
         const uint64_t first = (blockIdx.x + (uint64_t)it * gridDim.x) * pool_size;
-        const uint32_t x = (grp - base) * 32 + lane;
-        const bool live = first + x < n;
+        const uint32_t x = (grp - base) * lanes + lane;
+        const bool live = lane < lanes && first + x < n;
         // take the records along, so that the slot can be filled again before they are evaluated
         uint64_t w0 = 0;
         uint32_t r = 0;

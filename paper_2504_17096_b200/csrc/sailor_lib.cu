@@ -1145,10 +1145,14 @@ int sailor_simulate(sailor_ctx* ctx, const sailor_plan_rec* plans, uint64_t n, i
         const uint64_t share = (m + ctx->sm_count * turns - 1) / (ctx->sm_count * turns);
         const uint32_t pool = (uint32_t)((share + 31) / 32 * 32);
         const uint64_t pools = (m + pool - 1) / pool;
+        // groups of fewer lanes diverge less: as few as leave every group a warp of its own (1 000 records in groups of 32:
+        // 32.3 us on the device, of 8: 30.9, of 4: 30.1; 45 000 records: no difference)
+        uint32_t lanes = 4;
+        while (lanes < 32 && pool > lanes * BATCH_WARPS) lanes *= 2;
         const uint32_t grid = (uint32_t)std::min<uint64_t>(pools, (uint64_t)ctx->sm_count);
         const BatchParams p = batch_params(ctx->hdr, ctx->d_blob);
         simulate_kernel<<<grid, BATCH_THREADS, p.smem, ctx->stream>>>(
-            p, ctx->d_avail, d_plans, m, pool, d_t, d_m, d_c, d_s, error, report_bad);
+            p, ctx->d_avail, d_plans, m, pool, lanes, d_t, d_m, d_c, d_s, error, report_bad);
         CU(ctx, cudaGetLastError());
         return (int)SAILOR_OK;
     };

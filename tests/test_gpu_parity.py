@@ -154,10 +154,10 @@ def test_simulate_empty_and_bad_records(make_ctx, torch_cuda):
     assert L.sailor_simulate(cx.ctx, both.ctypes.data, 1, 0, out_t.ctypes.data, None, None, out_s.ctypes.data) == B.OK
 
 
-@pytest.mark.parametrize("n,L,kind", [(1, 8, "plain"), (33, 8, "poly"), (4737, 96, "plain"), (113700, 12, "bare"), (227333, 96, "plain"),
+@pytest.mark.parametrize("n,L,kind", [(1, 8, "plain"), (33, 8, "poly"), (4737, 96, "plain"), (14800, 96, "plain"), (37000, 24, "bare"), (113700, 12, "bare"), (227333, 96, "plain"),
                                       (9000, 420, "poly"), (9000, 420, "plain")])
 def test_simulate_batch_shapes(n, L, kind, make_ctx, torch_cuda):
-    """The batch kernel takes pools of 32 to 768 records, several a block when the batch is large, from device memory that
+    """The batch kernel takes pools of 32 to 768 records, several a block when the batch is large, in groups of 4 to 32, from device memory that
     may start 8 bytes past a 16-byte line; gradient tables move out of shared memory for long models, and models may lack an
     embedding or a head.  Up to 16 runs that repeat zones and types.  A record's results do not depend on its place."""
     torch = torch_cuda
