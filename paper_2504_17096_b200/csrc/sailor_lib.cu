@@ -1500,7 +1500,7 @@ extern "C" int sailor_plan_noalloc(sailor_ctx* ctx, const sailor_space* s, const
     }
     if (ce == cudaSuccess && rc == SAILOR_OK) ce = cudaEventRecord(ctx->ev1, ctx->stream);
     if (ce == cudaSuccess && rc == SAILOR_OK)
-        ce = cudaMemcpyAsync(ctx->h_out, &sc->out, sizeof(Ctrl) + sizeof(sailor_result) * k, cudaMemcpyDeviceToHost, ctx->stream);
+        ce = cudaMemcpyAsync(ctx->h_out, &sc->out, offsetof(PlanOut, results) + sizeof(sailor_result) * k, cudaMemcpyDeviceToHost, ctx->stream);
     if (ce == cudaSuccess && rc == SAILOR_OK && stats) ce = cudaEventRecord(ctx->ev2, ctx->stream);
     {
         const cudaError_t se = stream_sync(ctx);               // on every path: the copies above read this thread's arrays

@@ -238,6 +238,7 @@ struct alignas(16) CfgShared {
     uint32_t g_magic[SAILOR_SEG_MAX];     // floor(2^32 / g_cnt) + 1, for division by g_cnt
     uint64_t live_items;         // product of g_cnt over the prefix segments
     uint8_t good_list[SAILOR_SEG_MAX][R_MAX];   // the usable digits of each segment, ascending
+    uint32_t need_last;                   // need of the last segment
     uint32_t seg_a[SAILOR_SEG_MAX + 1];   // first stage of each segment; seg_a[nseg] = P
     uint32_t need[SAILOR_SEG_MAX];        // GPUs a segment takes of its digit: D * tp * stages
     uint32_t n_run[SAILOR_SEG_MAX][N_RUNS];   // stages in each run (without a non-final segment's last stage)
@@ -398,6 +399,7 @@ static __device__ void build_config(const PlanParams& pp, const TabView& v, CfgS
             const uint32_t lo = (tid * P + nseg - 1) / nseg, end = ((tid + 1) * P + nseg - 1) / nseg;
             const uint32_t extra = h->n_blocks % P;
             cs.need[tid] = D * tp * (end - lo);
+            if (tid + 1 == nseg) cs.need_last = D * tp * (end - lo);
             cs.oom_mask[tid] = 0;
             for (uint32_t j = 0; j < SAILOR_TP_MAX; ++j) cs.lower_fit[j][tid] = 0;
             uint32_t hi = (tid + 1 < nseg) ? end - 1 : end;      // a non-final segment's last stage is kept apart
@@ -550,27 +552,47 @@ static __device__ void build_config(const PlanParams& pp, const TabView& v, CfgS
     __syncthreads();
 }
 
-// The tables of configuration `c` from the cache instead of building them: two straight copies, then the
-// availability mask of the last segment, which is the only part that follows the snapshot.  Called by the
-// whole block (after a barrier); ends synchronised.  `a.availv` holds the snapshot already.
+// The tables of configuration `c` from the cache instead of building them: two straight copies, then the availability mask
+// of the last segment, which is the only part that follows the snapshot, by the warp that copied the scalars.  Called by the
+// whole block; starts and ends synchronised.  `a.availv` holds the snapshot already.  (Bringing the next record into shared
+// memory by a bulk copy while a configuration is searched, with the claims of chunks a turn ahead, made searches 2 to 9 %
+// slower: what has to be worked out for it sits on the path that every warp waits for.)
 static __device__ void load_config(const PlanParams& pp, CfgShared& cs, CfgArrays& a, uint32_t R, uint32_t c) {
     const uint32_t tid = threadIdx.x;
     const uint4* src = pp.cfg_cache + (size_t)c * (pp.cache_head16 + pp.cache_arr16);
+    const CfgShared& rec = *reinterpret_cast<const CfgShared*>(src);                       // (its head)
+    uint32_t need_last = 0;
+    if (tid < 32) need_last = rec.need_last;
+    __syncthreads();                                       // the old tables are not used any more
     for (uint32_t x = tid; x < pp.cache_head16; x += PLAN_THREADS) reinterpret_cast<uint4*>(&cs)[x] = src[x];
     for (uint32_t x = tid; x < pp.cache_arr16; x += PLAN_THREADS) reinterpret_cast<uint4*>(a.rec)[x] = src[pp.cache_head16 + x];
-    __syncthreads();
     if (tid < 32) {
-        const uint32_t need_last = cs.need[cs.cfg.nseg - 1];
         const uint32_t a_lo = __ballot_sync(FULL, tid < R && need_last <= a.availv[tid < R ? tid : 0]);
         const uint32_t a_hi = __ballot_sync(FULL, tid + 32 < R && need_last <= a.availv[tid + 32 < R ? tid + 32 : 0]);
+        __syncwarp();
         if (tid == 0) {
             cs.avail_last = ((uint64_t)a_hi << 32) | a_lo;
-            cs.whole = cs.flat_base >= pp.flat_lo && cs.flat_base + cs.n_items * R <= pp.flat_hi;
-            cs.packed = cs.valid ? pp.live_mode : 0u;
+            cs.whole = rec.flat_base >= pp.flat_lo && rec.flat_base + rec.n_items * R <= pp.flat_hi;
+            cs.packed = cs.valid ? pp.live_mode : 0u;      // (this warp copied `valid`, and `packed`, which is replaced)
             cs.cur_config = c;
         }
     }
     __syncthreads();
+}
+static_assert(offsetof(CfgShared, packed) < 32 * 16 && offsetof(CfgShared, valid) < 32 * 16, "copied by warp 0");
+
+// The configuration of chunk `ch`: the last of the n whose first chunk is not beyond it.  By a whole warp, 32 offsets at a
+// time (thread by thread a binary search waits for its loads one after another).
+__device__ __forceinline__ uint32_t find_config(const uint32_t* chunk_start, uint32_t n, uint32_t ch, uint32_t lane) {
+    uint32_t lo = 0, span = n;
+    while (span > 1) {
+        const uint32_t step = (span + 31) / 32, at = lane * step;
+        const uint32_t below = __popc(__ballot_sync(FULL, at < span && chunk_start[lo + (at < span ? at : 0)] <= ch));
+        const uint32_t skip = (below - 1) * step;          // the first offset of the span never lies beyond ch
+        lo += skip;
+        span = min(step, span - skip);
+    }
+    return lo;
 }
 
 __device__ __forceinline__ uint64_t warp_or64(uint64_t x) {
@@ -1139,18 +1161,9 @@ __device__ __forceinline__ uint32_t merge_block_lists(const Hit* partial, uint32
         sc = raw.x;
         fl = (uint64_t)__double_as_longlong(raw.y);
     };
-    WarpTopK top, more;
+    constexpr uint32_t PER_WARP = (SAILOR_K_MAX + NW - 1) / NW;
+    WarpTopK top;
     top.init();
-    const uint32_t rounds = (n_lists + 32 * NW - 1) / (32 * NW);
-    for (uint32_t r = 0; r < rounds; ++r) {
-        const uint32_t b = r * 32 * NW + tid;
-        more.init();
-        if (b < n_lists) load_hit(b, 0, more.score, more.flat);
-        if (more.flat == ~0ull) more.score = make_inf();       // an empty list (only its first slot need be written)
-        more.sort(k, lane);
-        if (r == 0) top = more;
-        else top.merge_sorted(more.score, more.flat, k, lane);
-    }
     auto tree_merge = [&]() {          // the warps' lists into warp 0's, through shared memory
         s_hits[warp][lane].score = top.score;
         s_hits[warp][lane].flat = top.flat;
@@ -1164,29 +1177,46 @@ __device__ __forceinline__ uint32_t merge_block_lists(const Hit* partial, uint32
             __syncthreads();
         }
     };
+    WarpTopK more;
+    double hs[2];                                          // the heads of up to 64 * NW lists stay in registers
+    uint64_t hf[2];
+    const uint32_t rounds = (n_lists + 32 * NW - 1) / (32 * NW);
+    for (uint32_t r = 0; r < rounds; ++r) {
+        const uint32_t b = r * 32 * NW + tid;
+        more.init();
+        if (b < n_lists) load_hit(b, 0, more.score, more.flat);
+        if (more.flat == ~0ull) more.score = make_inf();   // an empty list (only its first slot need be written)
+        if (r == 0) { hs[0] = more.score; hf[0] = more.flat; }
+        if (r == 1) { hs[1] = more.score; hf[1] = more.flat; }
+        more.sort(k, lane);
+        if (r == 0) top = more;
+        else top.merge_sorted(more.score, more.flat, k, lane);
+    }
     tree_merge();
-    const double cut_s = s_hits[0][k - 1].score;             // the k-th best head (or (+inf, ~0): fewer than k lists hold anything)
+    const double cut_s = s_hits[0][k - 1].score;           // the k-th best head (or (+inf, ~0): fewer than k lists hold anything)
     const uint64_t cut_f = s_hits[0][k - 1].flat;
     if (tid == 0) *s_n = 0;
     __syncthreads();
     for (uint32_t r = 0; r < rounds; ++r) {
         const uint32_t b = r * 32 * NW + tid;
-        double hs = make_inf();
-        uint64_t hf = ~0ull;
-        if (b < n_lists) load_hit(b, 0, hs, hf);
-        if (hf != ~0ull && (hs < cut_s || (hs == cut_s && hf <= cut_f))) sel[atomicAdd(s_n, 1u)] = b;
+        double h_s = make_inf();
+        uint64_t h_f = ~0ull;
+        if (r == 0) { h_s = hs[0]; h_f = hf[0]; }
+        else if (r == 1) { h_s = hs[1]; h_f = hf[1]; }
+        else if (b < n_lists) load_hit(b, 0, h_s, h_f);
+        if (h_f != ~0ull && (h_s < cut_s || (h_s == cut_s && h_f <= cut_f))) sel[atomicAdd(s_n, 1u)] = b;
     }
     __syncthreads();
-    const uint32_t n_sel = *s_n;                               // at most k
     top.init();
-    constexpr uint32_t PER_WARP = (SAILOR_K_MAX + NW - 1) / NW;
+    const uint32_t n_sel = *s_n;                               // at most k
     double ls[PER_WARP];
     uint64_t lf[PER_WARP];
 #pragma unroll
     for (uint32_t x = 0; x < PER_WARP; ++x) {                  // all loads in flight before the first merge
+        const uint32_t y = warp + x * NW;
         ls[x] = make_inf();
         lf[x] = ~0ull;
-        if (warp + x * NW < n_sel && lane < k) load_hit(sel[warp + x * NW], lane, ls[x], lf[x]);
+        if (y < n_sel && lane < k) load_hit(sel[y], lane, ls[x], lf[x]);
     }
 #pragma unroll
     for (uint32_t x = 0; x < PER_WARP; ++x)
@@ -1202,11 +1232,21 @@ __device__ __forceinline__ uint32_t merge_block_lists(const Hit* partial, uint32
     return *s_n;
 }
 
-// The result record of candidate `hit.flat`: decoded, simulated and written by one warp, lane i taking stage i (then
-// i + 32, ...).  Per-stage terms are formed side by side; the sums whose order is part of the result run over the lanes'
-// terms in stage order, so the bits are those of simulate_runs.  Bound by latency: a thread alone waits for one table
-// after another (9.4 us from decoding to the record for plans of up to 24 stages, 5.0 us here).
-__device__ __forceinline__ void write_result(const PlanParams& pp, const TabView& v, const Hit& hit, sailor_result* out, uint32_t lane) {
+// The result records of the `n` winners, side by side: a group of G lanes per winner, lane i of it taking stage i (then
+// i + G, ...), G as large as lets every winner have a group.  Per-stage terms are formed side by side; the sums whose order is
+// part of the result run over the lanes' terms in stage order (a stage or message that is not there adds zero), so the bits
+// are those of simulate_runs.  Bound by latency: a thread alone waits for one table after another (9.4 us from decoding to the
+// record for plans of up to 24 stages, 5.0 us by a warp); 32 winners of up to 48 stages four to a warp, one after the other:
+// 19.5 us, side by side 8.  By the whole block.
+__device__ __forceinline__ void write_results(const PlanParams& pp, const TabView& v, const Hit* hits, uint32_t n, sailor_result* results) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t G = 32;
+    while (G > 1 && n > PLAN_WARPS * (32 / G)) G /= 2;
+    const uint32_t mine = lane & (G - 1), group = lane / G, j = warp * (32 / G) + group;
+    if (warp * (32 / G) >= n) return;
+    const bool real = j < n;
+    const Hit hit = hits[real ? j : n - 1];
+    sailor_result* out = results + j;
     const TabHdr* h = v.h;
     const SpaceDesc& sp = pp.sp;
     const uint32_t T = h->T, Z = h->Z, R = h->R;
@@ -1220,7 +1260,13 @@ __device__ __forceinline__ void write_result(const PlanParams& pp, const TabView
         const uint64_t up = __shfl_up_sync(FULL, end, o);
         if (lane >= (uint32_t)o) end += up;
     }
-    const uint32_t sub = __ffs(__ballot_sync(FULL, lane < sp.n_p && hit.flat < end)) - 1;
+    uint32_t sub = 0;
+#pragma unroll 1
+    for (uint32_t q = 0; q < 32 / G; ++q) {
+        const uint64_t flat = __shfl_sync(FULL, hit.flat, q * G);
+        const uint32_t at = __ffs(__ballot_sync(FULL, lane < sp.n_p && flat < end)) - 1;
+        if (group == q) sub = at;
+    }
     const uint64_t rem = hit.flat - __shfl_sync(FULL, end - size, sub);
     const uint32_t nseg = nseg_of(sp.p_values[sub], sp.seg_max);
     const uint32_t block = (uint32_t)ipow64(R, nseg);       // candidates of a configuration: at most 64^4
@@ -1258,8 +1304,9 @@ __device__ __forceinline__ void write_result(const PlanParams& pp, const TabView
     const double xbytes = (double)(2 * n_b * (uint64_t)D * v.p2p[mi]);
     double sum_t = 0.0, max_t = 0.0, max_sync = 0.0, max_u = 0.0, rate = 0.0, c_comm = 0.0;
     uint64_t peak = 0;
-    for (uint32_t at = 0; at < P; at += 32) {
-        const uint32_t i = at + lane;
+    const uint32_t P_most = __reduce_max_sync(FULL, P);
+    for (uint32_t at = 0; at < P_most; at += G) {
+        const uint32_t i = at + mine;
         double t = 0.0, gpu_rate = 0.0, comm = 0.0;
         bool crosses = false;
         if (i < P) {
@@ -1285,24 +1332,28 @@ __device__ __forceinline__ void write_result(const PlanParams& pp, const TabView
             }
             max_t = dmax(max_t, t);
         }
-        const uint32_t n = P - at < 32 ? P - at : 32;
-        for (uint32_t l = 0; l < n; ++l) {                   // in stage order
-            sum_t = add_rn(sum_t, __shfl_sync(FULL, t, l));
-            rate = add_rn(rate, __shfl_sync(FULL, gpu_rate, l));
+        const uint32_t m = P_most - at < G ? P_most - at : G;
+        for (uint32_t l = 0; l < m; ++l) {                   // in stage order
+            sum_t = add_rn(sum_t, __shfl_sync(FULL, t, l, G));
+            rate = add_rn(rate, __shfl_sync(FULL, gpu_rate, l, G));
         }
-        for (uint32_t m = __ballot_sync(FULL, crosses); m; m &= m - 1) c_comm = add_rn(c_comm, __shfl_sync(FULL, comm, __ffs(m) - 1));
+        uint32_t some = __ballot_sync(FULL, crosses);        // the stages at which any of the warp's plans changes zones
+        for (uint32_t o = 16; o >= G; o >>= 1) some |= some >> o;
+        for (some &= G == 32 ? FULL : (1u << G) - 1u; some; some &= some - 1)
+            c_comm = add_rn(c_comm, __shfl_sync(FULL, comm, __ffs(some) - 1, G));
     }
 #pragma unroll 1
-    for (int o = 16; o; o >>= 1) {
+    for (uint32_t o = G / 2; o; o >>= 1) {
         max_t = dmax(max_t, __shfl_xor_sync(FULL, max_t, o));
         max_sync = dmax(max_sync, __shfl_xor_sync(FULL, max_sync, o));
         max_u = dmax(max_u, __shfl_xor_sync(FULL, max_u, o));
         const uint64_t other = __shfl_xor_sync(FULL, peak, o);
         peak = other > peak ? other : peak;
+        status |= __shfl_xor_sync(FULL, status, o);
     }
-    status = __reduce_or_sync(FULL, status);
+    if (!real) return;
     const double t_iter = add_rn(add_rn(add_rn(sum_t, mul_rn((double)n_b, max_t)), max_sync), max_u);
-    if (lane == 0) {
+    if (mine == 0) {
         out->flat = hit.flat;
         out->score = hit.score;
         out->t_iter = t_iter;
@@ -1311,17 +1362,17 @@ __device__ __forceinline__ void write_result(const PlanParams& pp, const TabView
         out->status = status;
         out->_pad = 0;
     }
-    if (lane < sizeof(sailor_plan_rec) / 4) {                // the record word by word: header, then a run per segment
+    for (uint32_t y = mine; y < sizeof(sailor_plan_rec) / 4; y += G) {      // the record word by word: header, then a run per segment
         uint32_t word = 0;
-        if (lane == 0) word = P | mi << 8 | k.rc << 16 | nseg << 24;
-        else if (lane == 1) word = D;
-        else if (lane - 2 < nseg) {
-            const uint32_t q = lane - 2, x_q = q == 0 ? gz[0] : q == 1 ? gz[1] : q == 2 ? gz[2] : gz[3];
+        if (y == 0) word = P | mi << 8 | k.rc << 16 | nseg << 24;
+        else if (y == 1) word = D;
+        else if (y - 2 < nseg) {
+            const uint32_t q = y - 2, x_q = q == 0 ? gz[0] : q == 1 ? gz[1] : q == 2 ? gz[2] : gz[3];
             const uint32_t a = q == 0 ? 0u : q == 1 ? seg_end[0] : q == 2 ? seg_end[1] : seg_end[2];
             const uint32_t e = q == 0 ? seg_end[0] : q == 1 ? seg_end[1] : q == 2 ? seg_end[2] : seg_end[3];
             word = x_q | k.tpi << 16 | (e - a) << 24;
         }
-        reinterpret_cast<uint32_t*>(&out->plan)[lane] = word;
+        reinterpret_cast<uint32_t*>(&out->plan)[y] = word;
     }
 }
 
@@ -1354,37 +1405,27 @@ static __device__ __noinline__ void finish_pass(const PlanParams& pp, const TabV
         }
         return;
     }
+    // The counters as they stand (every block's contribution is in: atomics, then its blocks_done increment), a lane of the last
+    // warp per word; they are asked for now and looked at when the merge is done.
+    constexpr uint32_t WORDS = sizeof(Ctrl) / 4;
+    static_assert(WORDS <= 32, "a lane per word");
+    volatile uint32_t* live = reinterpret_cast<volatile uint32_t*>(pp.ctrl);
+    const bool counts = warp == PLAN_WARPS - 1 && lane < WORDS;
+    uint32_t word = 0;
+    if (counts) word = live[lane];
     const uint32_t n = merge_block_lists<PLAN_WARPS>(pp.partial, n_partial, pp.k, s_hits, s_cnt, s_n);
-    // the winners are simulated in full for the result records, a warp each
-    for (uint32_t j = warp; j < n; j += PLAN_WARPS) write_result(pp, v, s_hits[0][j], pp.out->results + j, lane);
-    if (tid == 0) {
-        // the counters as they stand (every block's contribution is in: atomics, then its blocks_done increment)
-        volatile Ctrl* live = pp.ctrl;
-        Ctrl c;
-        c.work_counter = live->work_counter;
-        c.blocks_done = live->blocks_done;
-        for (int q = 0; q < 7; ++q) c.stats[q] = live->stats[q];
-        c.wave_chunks = live->wave_chunks;
-        c.n_cfg_evaluated = live->n_cfg_evaluated;
-        c.min_cost_bits = live->min_cost_bits;
-        c.thr_bits = live->thr_bits;
-        c.error = live->error;
-        c.n_found = n;
-        pp.out->ctrl = c;
+    if (counts) {                      // to the host, and back to their starting values; the budget stays for the next pass
+        const uint32_t at = 4 * lane;
+        const bool cost = at >= offsetof(Ctrl, min_cost_bits) && at < offsetof(Ctrl, min_cost_bits) + 16;   // and thr_bits
+        if (at != offsetof(Ctrl, n_found)) reinterpret_cast<uint32_t*>(&pp.out->ctrl)[lane] = word;
+        if (!(at >= offsetof(Ctrl, budget) && at < offsetof(Ctrl, budget) + 8) && at != offsetof(Ctrl, blocks_done))
+            live[lane] = cost && (at & 4) ? (uint32_t)(COST_BITS_START >> 32) : 0u;
     }
-    __syncthreads();                   // the budget of the next pass is written (thread 0 or warp 0's lane 0)
+    if (n) write_results(pp, v, s_hits[0], n, pp.out->results);     // the winners are simulated in full for the result records
+    __syncthreads();
     if (tid == 0) {
-        pp.out->ctrl.budget = *reinterpret_cast<volatile double*>(&pp.ctrl->budget);
-        Ctrl* live = pp.ctrl;          // back to the starting values; the budget stays for the next pass
-        live->work_counter = 0;
-        for (int q = 0; q < 7; ++q) live->stats[q] = 0;
-        live->wave_chunks = 0;
-        live->n_cfg_evaluated = 0;
-        live->min_cost_bits = COST_BITS_START;
-        live->thr_bits = COST_BITS_START;
-        live->error = 0;               // (a cheapest-plan pass before this one kept the flag)
+        pp.out->ctrl.n_found = n;
         pp.out->span.end = device_ns();
-        live->n_found = 0;
     }
 }
 
@@ -1463,12 +1504,6 @@ __global__ void __launch_bounds__(PLAN_THREADS, SCREEN ? PLAN_SCREEN_BLOCKS : PL
             // first (a block then stays inside one configuration and changes its tables rarely), single chunks at
             // the end (even finish)
             const uint32_t n_chunks = chunk_hi - chunk_lo;
-            if (!first_round) {      // trade thresholds with the other blocks
-                const unsigned long long theirs = *reinterpret_cast<volatile unsigned long long*>(&pp.ctrl->thr_bits);
-                const unsigned long long ours = *reinterpret_cast<volatile unsigned long long*>(&cs.thr_bits);
-                if (ours < theirs) atomicMin(&pp.ctrl->thr_bits, ours);
-                else if (theirs < ours) atomicMin(&cs.thr_bits, theirs);
-            }
             if (first_round) {
                 cs.next_chunk = chunk_lo + min(blockIdx.x, n_chunks);
                 cs.batch_len = 1;
@@ -1481,6 +1516,11 @@ __global__ void __launch_bounds__(PLAN_THREADS, SCREEN ? PLAN_SCREEN_BLOCKS : PL
                 const uint32_t left = seen < rest ? rest - seen : 0u;
                 const uint32_t len = max(1u, left / (gridDim.x * 4u));
                 const uint32_t got = atomicAdd(&pp.ctrl->work_counter, len);
+                // trade thresholds with the other blocks in the meantime
+                const unsigned long long theirs = *reinterpret_cast<volatile unsigned long long*>(&pp.ctrl->thr_bits);
+                const unsigned long long ours = *reinterpret_cast<volatile unsigned long long*>(&cs.thr_bits);
+                if (ours < theirs) atomicMin(&pp.ctrl->thr_bits, ours);
+                else if (theirs < ours) atomicMin(&cs.thr_bits, theirs);
                 cs.next_chunk = got < rest ? chunk_lo + gridDim.x + got : chunk_hi;
                 cs.batch_len = len;
             }
@@ -1490,21 +1530,16 @@ __global__ void __launch_bounds__(PLAN_THREADS, SCREEN ? PLAN_SCREEN_BLOCKS : PL
         const uint32_t first = cs.next_chunk;
         if (first >= chunk_hi) break;
         const uint32_t end = min(first + cs.batch_len, chunk_hi);
-        {   // configuration of the first chunk: binary search (uniform)
-            uint32_t lo = 0, hi = pp.n_config;
-            while (hi - lo > 1) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (chunk_start[mid] <= first) lo = mid; else hi = mid;
-            }
-            c = lo;
-        }
+        c = find_config(chunk_start, pp.n_config, first, lane);
         for (uint32_t ch = first; ch < end; ++ch) {
             while (ch >= chunk_start[c + 1]) ++c;
             if (cs.cur_config != c) {
                 if (pp.cfg_best && cs.cur_config != 0xffffffffu) flush_cfg_best(pp, cnt, cs.cur_config, lane);
-                __syncthreads();
                 if (pp.cfg_cache) load_config(pp, cs, a, R, c);
-                else build_config(pp, v, cs, a, c);
+                else {
+                    __syncthreads();
+                    build_config(pp, v, cs, a, c);
+                }
                 if (SCREEN) round_config32(a, R, Z);
             }
             const uint32_t q = (ch - chunk_start[c]) * PLAN_THREADS + tid;    // < R^3 + 256 <= 2^18 + 256

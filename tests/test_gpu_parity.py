@@ -775,3 +775,20 @@ def test_every_candidate_over_zone_shapes(n_types, n_zones, zoned, poly, make_ct
         assert [r.flat for r in res] == [h["flat"] for h in hits] and st.n_total == hi - lo
         assert (st.n_invalid, st.n_oom, st.n_over_avail, st.n_feasible) == tuple(
             counts[k] for k in ("n_invalid", "n_oom", "n_over_avail", "n_feasible"))
+
+
+@pytest.mark.parametrize("k", [1, 7, 8, 9, 16, 17, 32])
+def test_result_records_side_by_side(k, make_ctx):
+    """Result records are written by groups of 32, 16 or 8 lanes, as the number of winners asks for, over pipelines of
+    different depths that cross zones in different places: the oracle's list and, record by record, the simulator's values."""
+    w = W.tiny(seed=47, n_types=2, n_zones=3, L=40, p_values=[1, 3, 9, 40], d_values=(1, 2), tp_values=(1, 2), mbs_values=(1,))
+    w.avail[...] = 60
+    o, ctx = Oracle(w), make_ctx(w).ctx
+    for kind in (0, 1, 2):
+        hits, _ = o.search(kind, k)
+        res, _ = B.sailor_plan(ctx, B.make_space(w), B.Objective(kind, 0, 0.0, 0.0, 0.0), k)
+        assert [(r.flat, r.score) for r in res] == [(h["flat"], h["score"]) for h in hits] and len(res) == k
+        recs = np.frombuffer(b"".join(bytes(r.plan) for r in res), dtype=B.REC_DTYPE)
+        t, m, c, s = B.sailor_simulate(ctx, recs)
+        assert [(r.t_iter, r.cost, r.peak_mem, r.status) for r in res] == list(zip(t.tolist(), c.tolist(), m.tolist(), s.tolist()))
+        assert [bytes(B.sailor_decode(ctx, B.make_space(w), r.flat)) for r in res] == [bytes(r.plan) for r in res]
