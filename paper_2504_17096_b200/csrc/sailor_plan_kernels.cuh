@@ -55,6 +55,7 @@ struct Ctrl {                       // one per context, device memory
 struct PlanOut {
     Ctrl ctrl;
     DeviceSpan span;
+    uint64_t ticket;                   // written last: which call the rest belongs to
     sailor_result results[SAILOR_K_MAX];
 };
 
@@ -82,6 +83,7 @@ struct PlanParams {
     const uint32_t* chunk_hi_dev;      // non-null: chunks [0, *chunk_hi_dev) instead of [chunk_lo, chunk_hi)
     unsigned long long* cfg_best;      // non-null: [n_config] best feasible score per configuration (ordered bits)
     PlanOut* out;                      // where the block that finishes the pass leaves the results
+    uint64_t ticket;                   // of the call
     uint32_t first;                    // this launch is the call's first: it stamps the start
     uint32_t finish;                   // this launch ends a pass: its last block merges the lists and writes `out`
     double next_budget_factor;         // > 0: the finishing block writes ctrl->budget = factor * best cost (next pass)
@@ -1426,6 +1428,8 @@ static __device__ __noinline__ void finish_pass(const PlanParams& pp, const TabV
     if (tid == 0) {
         pp.out->ctrl.n_found = n;
         pp.out->span.end = device_ns();
+        __threadfence_system();        // the host may be looking: everything above is there before the ticket is
+        *const_cast<volatile uint64_t*>(&pp.out->ticket) = pp.ticket;
     }
 }
 
