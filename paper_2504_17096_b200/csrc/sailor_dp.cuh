@@ -250,19 +250,37 @@ struct DpLevelParams {
     uint32_t dist;                   // stage i = P - 1 - dist
 };
 
-// Stage i of a job for the vector in `slot` of the stage, all its types at once (TM >= T types).  `here` and `then` are
-// the live rows of stages i and i + 1 (shared memory).
-template <uint32_t TM>
-__device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayout& L, const DpJob& job, const uint32_t* here,
-                                          const uint32_t* then, uint32_t i, uint32_t slot) {
-    const uint32_t T = lp.T, dist = job.P - 1 - i;
-    const double* tab = lp.tabs + (size_t)job.config * lp.lay.stride();
+// What a stage of a job reads of the job's tables, kept in shared memory (every vector of the stage reads it).
+struct DpStageTab {
+    double nb;
+    uint32_t ok, ok_next;            // types that fit the stage, and the next
+    double fb[SAILOR_T_MAX], upd[SAILOR_T_MAX], sync[R_MAX];
+};
+// Thread `x` of the block brings in its part of stage i's.
+__device__ __forceinline__ void dp_stage_tab(const DpLevelParams& lp, const double* tab, uint32_t P, uint32_t i, uint32_t x, DpStageTab& st) {
     const uint32_t* okv = reinterpret_cast<const uint32_t*>(tab + lp.lay.off_ok());
-    const double nb = (double)*reinterpret_cast<const uint64_t*>(tab + lp.lay.off_nb());
+    if (x < lp.lay.R) st.sync[x] = tab[lp.lay.off_sync() + (size_t)i * lp.lay.R + x];
+    else if (x >= 64 && x < 64 + lp.T) st.fb[x - 64] = tab[lp.lay.off_fb() + i * lp.T + (x - 64)];
+    else if (x >= 96 && x < 96 + lp.T) st.upd[x - 96] = tab[lp.lay.off_upd() + i * lp.T + (x - 96)];
+    else if (x == 128) st.ok = okv[i];
+    else if (x == 129) st.ok_next = i + 1 < P ? okv[i + 1] : 0u;
+    else if (x == 130) st.nb = (double)*reinterpret_cast<const uint64_t*>(tab + lp.lay.off_nb());
+}
+static_assert(R_MAX <= 64 && SAILOR_T_MAX <= 32 && DP_THREADS > 130, "a thread per entry");
+
+// Stage i of a job for the vector in `slot` of the stage, all its types at once (TM >= T types).  `here` and `then` are
+// the live rows of stages i and i + 1, `st` the stage's tables (shared memory).
+// AFTER_LEVEL: launched while the level it reads may still be running.
+template <uint32_t TM, bool AFTER_LEVEL>
+__device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayout& L, const DpJob& job, const uint32_t* here,
+                                          const uint32_t* then, const DpStageTab& st, uint32_t i, uint32_t slot) {
+    const uint32_t T = lp.T, dist = job.P - 1 - i;
+    const double* c2x = lp.tabs + (size_t)job.config * lp.lay.stride() + lp.lay.off_c2x();
+    const double nb = st.nb;
     uint32_t zp = 0;
     while (zp + 1 < L.nz && here[3 + 2 * (zp + 1)] <= slot) ++zp;
     const uint32_t v = here[2 + 2 * zp] + (slot - here[3 + 2 * zp]);
-    uint32_t nx[TM];
+    uint32_t nx[TM];                                         // (nothing so far depends on another stage)
     {
         const uint4* row = reinterpret_cast<const uint4*>(lp.nxt + (size_t)(L.nxt_off + v) * TM);
 #pragma unroll
@@ -271,6 +289,7 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
             nx[4 * q] = x.x; nx[4 * q + 1] = x.y; nx[4 * q + 2] = x.z; nx[4 * q + 3] = x.w;
         }
     }
+    if (AFTER_LEVEL) asm volatile("griddepcontrol.wait;" ::: "memory");       // the level after this stage is complete
     // what follows a stage of each type g2: the state it leads to (the same for every type of stage i) and its value
     const DpVal* nxt = lp.val[(dist & 1) ^ 1] + job.val_off;
     DpVal n[TM];
@@ -282,7 +301,7 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
         n[g2].sum = make_inf(); n[g2].mx = n[g2].sy = n[g2].up = 0.0;
     }
     if (dist != 0) {
-        const uint32_t ok_next = okv[i + 1];
+        const uint32_t ok_next = st.ok_next;
 #pragma unroll
         for (uint32_t g2 = 0; g2 < TM; ++g2) {
             if (g2 >= T || !((ok_next >> g2) & 1u)) continue;
@@ -300,7 +319,7 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
             n[g2] = nxt[code[g2]];
         }
     }
-    const uint32_t ok_here = okv[i];
+    const uint32_t ok_here = st.ok;
     DpVal* cur = lp.val[dist & 1] + job.val_off + (size_t)slot * T;
     uint32_t* succ = lp.succ + job.succ_off + (size_t)(here[1] + slot) * T;
 #pragma unroll
@@ -309,8 +328,7 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
         // a state holds stage i itself: its type must fit the stage and, when counted, be counted at least once
         if (!((ok_here >> g) & 1u) || !(nx[g] & DP_SELF)) continue;
         const uint32_t d = L.zone[zp] * T + g;
-        const double fb = tab[lp.lay.off_fb() + i * T + g], upd = tab[lp.lay.off_upd() + i * T + g];
-        const double sync = tab[lp.lay.off_sync() + (size_t)i * lp.lay.R + d];
+        const double fb = st.fb[g], upd = st.upd[g], sync = st.sync[d];
         DpVal best;
         uint32_t pick = DP_NO_STATE;
         if (dist == 0) {                                     // the last stage sends nothing
@@ -321,7 +339,7 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
 #pragma unroll
             for (uint32_t g2 = 0; g2 < TM; ++g2) {
                 if (code[g2] == DP_NO_STATE || !(n[g2].sum < make_inf())) continue;
-                const double t = add_rn(fb, tab[lp.lay.off_c2x() + (size_t)d2[g2] * lp.lay.R + d]);
+                const double t = add_rn(fb, c2x[d2[g2] * lp.lay.R + d]);
                 DpVal c;
                 c.sum = add_rn(t, n[g2].sum);
                 c.mx = dmax(t, n[g2].mx);
@@ -342,9 +360,11 @@ __global__ void __launch_bounds__(DP_THREADS, TM <= 4 ? 3 : 2) dp_level_kernel(c
     __shared__ DpLayout L;
     __shared__ DpJob job;
     __shared__ uint32_t rows[2][DP_LIVE_WORDS_MAX];
+    __shared__ DpStageTab st;
     __shared__ uint32_t s_lo;
     const uint32_t tid = threadIdx.x;
     uint32_t which = 0;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // the next stage's blocks may find their way meanwhile
     // the job whose blocks include this one: a search with DP_THREADS probes per round, so that a block waits for one or
     // two loads, not for a chain of them
     {
@@ -374,8 +394,9 @@ __global__ void __launch_bounds__(DP_THREADS, TM <= 4 ? 3 : 2) dp_level_kernel(c
         rows[0][tid] = row[0];
         rows[1][tid] = lp.dist ? row[words] : 0u;
     }
+    dp_stage_tab(lp, lp.tabs + (size_t)gj.config * lp.lay.stride(), gj.P, i, tid, st);
     __syncthreads();
-    if (slot < rows[0][0]) dp_vector<TM>(lp, L, job, rows[0], rows[1], i, slot);
+    if (slot < rows[0][0]) dp_vector<TM, true>(lp, L, job, rows[0], rows[1], st, i, slot);
 }
 
 // Small problems: a block takes one job through all its stages, from the last to the first, with a barrier between
@@ -384,7 +405,8 @@ template <uint32_t TM>
 __global__ void __launch_bounds__(DP_THREADS, TM <= 4 ? 3 : 2) dp_problem_kernel(const __grid_constant__ DpLevelParams lp) {
     __shared__ DpLayout L;
     __shared__ DpJob job;
-    __shared__ uint32_t rows[2][DP_LIVE_WORDS_MAX];
+    __shared__ uint32_t rows[3][DP_LIVE_WORDS_MAX];          // of this stage, the one after it and the one before it: one
+    __shared__ DpStageTab st[2];                             // barrier a stage
     const uint32_t tid = threadIdx.x;
     const DpJob& gj = lp.jobs[blockIdx.x];
     const DpLayout* gl = lp.layouts + gj.layout;
@@ -393,19 +415,102 @@ __global__ void __launch_bounds__(DP_THREADS, TM <= 4 ? 3 : 2) dp_problem_kernel
         reinterpret_cast<uint32_t*>(&L)[x] = reinterpret_cast<const uint32_t*>(gl)[x];
     __syncthreads();
     const uint32_t words = dp_live_words(L.nz);
+    const double* tab = lp.tabs + (size_t)job.config * lp.lay.stride();
     for (uint32_t dist = 0; dist < job.P; ++dist) {
         const uint32_t i = job.P - 1 - dist;
-        uint32_t* here = rows[dist & 1];
+        uint32_t* here = rows[dist % 3];
         if (tid < words) here[tid] = lp.live[L.live_off + (size_t)i * words + tid];
+        dp_stage_tab(lp, tab, job.P, i, tid, st[dist & 1]);
         __syncthreads();                                     // the row, and the values of the stage after this one
         for (uint32_t slot = tid; slot < here[0]; slot += DP_THREADS)
-            dp_vector<TM>(lp, L, job, here, rows[(dist & 1) ^ 1], i, slot);
-        __syncthreads();
+            dp_vector<TM, false>(lp, L, job, here, rows[(dist + 2) % 3], st[dist & 1], i, slot);
     }
 }
 
-// Stage 0 and the walk through the kept successors: one thread per job.  The walk is a chain of one dependent load per
-// stage (a successor is the next state's own address).
+// A plan of one degree simulated by a warp, lane i taking stage i (then i + 32, ...): `gz` holds type | zone << 8 of every
+// stage, `cnt` a counter per (zone, type) (both shared memory, the warp's own).  Per-stage terms are formed side by side; the
+// sums whose order is part of the result run over the lanes' terms in stage order, so the bits are those of simulate_runs.
+// Every lane returns the same.
+__device__ __forceinline__ SimOut simulate_stages(const TabView& v, const uint16_t* __restrict__ avail, const Config& k,
+                                                  const uint16_t* gz, uint32_t* cnt, uint32_t lane) {
+    const TabHdr* h = v.h;
+    const uint32_t T = h->T, Z = h->Z, P = k.P, D = k.D, mi = k.mi, tp = h->tp_values[k.tpi];
+    SimOut o;
+    o.t_iter = o.cost = make_nan();
+    for (uint32_t d = lane; d < h->R; d += 32) cnt[d] = 0;
+    __syncwarp();
+    for (uint32_t i = lane; i < P; i += 32) atomicAdd(&cnt[(gz[i] >> 8) * T + (gz[i] & 0xffu)], 1u);       // stages
+    __syncwarp();
+    const uint64_t dm = (uint64_t)D * h->mbs_values[mi], n_b = h->gbs / dm;
+    uint32_t status = (n_b * dm != h->gbs || h->heads % tp != 0) ? SAILOR_ST_INVALID : 0u;
+    const uint32_t base = h->n_blocks / P, extra = h->n_blocks - base * P;
+    const double msg = (double)v.p2p[mi], steps = (double)(2 * (uint64_t)(D - 1)), coef = steps / (double)D;
+    const double xbytes = (double)(2 * n_b * (uint64_t)D * v.p2p[mi]);
+    double sum_t = 0.0, max_t = 0.0, max_sync = 0.0, max_u = 0.0, rate = 0.0, c_comm = 0.0;
+    uint64_t peak = 0;
+    for (uint32_t at = 0; at < P; at += 32) {
+        const uint32_t i = at + lane;
+        double t = 0.0, gpu_rate = 0.0, comm = 0.0;
+        bool crosses = false;
+        if (i < P) {
+            const uint32_t g = gz[i] & 0xffu, z = gz[i] >> 8, d = z * T + g;
+            const bool e = (i == 0) && h->has_embed, hd = (i == P - 1) && h->has_head;
+            const size_t comp = (size_t)((e ? 2u : 0u) + (hd ? 1u : 0u)) * h->chain_len + base + (i < extra ? 1u : 0u);
+            const size_t ct = comp * h->n_tp + k.tpi;
+            t = v.cmp_fb[(((comp * T + g) * h->n_tp + k.tpi) * h->n_mbs + mi) * 2 + k.rc];
+            max_u = dmax(max_u, v.cmp_upd[(comp * T + g) * h->n_tp + k.tpi]);
+            const uint64_t* mm = v.cmp_mem + ((ct * h->n_mbs + mi) * 2 + k.rc) * 2;
+            const uint64_t inflight = (uint64_t)(P - i) < n_b ? (uint64_t)(P - i) : n_b;
+            const uint64_t m = mm[0] + h->reserved[g] + inflight * mm[1];
+            if (m > h->capacity[g]) status |= SAILOR_ST_OOM;
+            if (tp > h->gpn[g]) status |= SAILOR_ST_INVALID;
+            if ((uint64_t)cnt[d] * D * tp > avail[d]) status |= SAILOR_ST_OVER_AVAIL;
+            peak = m > peak ? m : peak;
+            if (D > 1) max_sync = dmax(max_sync, allreduce_bytes_time(v, d, (uint64_t)D * tp <= h->gpn[g], v.cmp_grad[ct], D, steps, coef));
+            gpu_rate = mul_rn((double)(D * tp), v.price_s[d]);
+            if (i + 1 < P) {
+                const uint32_t gn = gz[i + 1] & 0xffu, zn = gz[i + 1] >> 8;
+                t = add_rn(t, mul_rn(2.0, boundary_time(v, g, z, tp, gn, zn, tp, D, msg)));
+                crosses = zn != z;
+                if (crosses) comm = mul_rn(xbytes, v.egress[z * Z + zn]);
+            }
+            max_t = dmax(max_t, t);
+        }
+        const uint32_t n = P - at < 32 ? P - at : 32;
+        for (uint32_t l = 0; l < n; ++l) {                   // in stage order
+            sum_t = add_rn(sum_t, __shfl_sync(FULL, t, l));
+            rate = add_rn(rate, __shfl_sync(FULL, gpu_rate, l));
+        }
+        for (uint32_t m = __ballot_sync(FULL, crosses); m; m &= m - 1) c_comm = add_rn(c_comm, __shfl_sync(FULL, comm, __ffs(m) - 1));
+    }
+#pragma unroll 1
+    for (int x = 16; x; x >>= 1) {
+        max_t = dmax(max_t, __shfl_xor_sync(FULL, max_t, x));
+        max_sync = dmax(max_sync, __shfl_xor_sync(FULL, max_sync, x));
+        max_u = dmax(max_u, __shfl_xor_sync(FULL, max_u, x));
+        const uint64_t other = __shfl_xor_sync(FULL, peak, x);
+        peak = other > peak ? other : peak;
+    }
+    o.peak_mem = peak;
+    o.status = __reduce_or_sync(FULL, status);
+    if (o.status & SAILOR_ST_INVALID) return o;
+    o.t_iter = add_rn(add_rn(add_rn(sum_t, mul_rn((double)n_b, max_t)), max_sync), max_u);
+    o.cost = add_rn(mul_rn(rate, o.t_iter), c_comm);
+    return o;
+}
+
+// What a warp of the kernels that end a search keeps in shared memory.
+struct DpFinishWarp {
+    uint32_t code[SAILOR_P_MAX];     // state of every stage
+    uint16_t gz[SAILOR_P_MAX];       // its type | zone << 8
+    uint32_t cnt[R_MAX];
+    uint8_t used[SAILOR_T_MAX];
+};
+constexpr int DP_FINISH_WARPS = 4, DP_FINISH_THREADS = 32 * DP_FINISH_WARPS;
+
+// Stage 0 and the walk through the kept successors, a warp per job.  The walk is a chain of one dependent load per stage (a
+// successor is the next state's own address) and what the kernel's time is; types, zones and the simulation are the lanes'.
+// 520 jobs of up to 48 stages: 107 us by a thread each, 33 this way.
 struct DpFinishParams {
     const unsigned char* blob;
     const uint16_t* avail;
@@ -422,11 +527,11 @@ struct DpFinishParams {
     uint32_t n_jobs, T;
 };
 
-constexpr int DP_FINISH_THREADS = 32;
-
 __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_finish_kernel(const __grid_constant__ DpFinishParams fp) {
-    const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ DpFinishWarp warps[DP_FINISH_WARPS];
+    const uint32_t lane = threadIdx.x & 31, x = blockIdx.x * DP_FINISH_WARPS + (threadIdx.x >> 5);
     if (x >= fp.n_jobs) return;
+    DpFinishWarp& w = warps[threadIdx.x >> 5];
     const DpJob job = fp.jobs[x];
     const DpLayout& L = fp.layouts[job.layout];
     DpResult& out = fp.results[job.index];
@@ -436,50 +541,62 @@ __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_finish_kernel(const __gr
     const uint32_t* okv = reinterpret_cast<const uint32_t*>(tab + fp.lay.off_ok());
     const double nb = (double)*reinterpret_cast<const uint64_t*>(tab + fp.lay.off_nb());
     const DpVal* lvl0 = fp.val[(P - 1) & 1] + job.val_off;
+    double mine_v = make_inf();
+    uint32_t mine = DP_NO_STATE;
+    if (lane < T && ((okv[0] >> lane) & 1u)) {               // stage 0 by first fit from the first zone of the order, a lane per type
+        const uint32_t p = L.cap[0][lane] >= 1 ? 0u : L.first_later[0][lane];
+        if (p != DP_NONE) {
+            const uint32_t slot = live[3 + 2 * p] + (L.first_vec[p][lane] - live[2 + 2 * p]);
+            if (slot < live[0]) {
+                const DpVal v = lvl0[slot * T + lane];
+                if (v.sum < make_inf()) {
+                    mine_v = add_rn(add_rn(add_rn(v.sum, mul_rn(nb, v.mx)), v.sy), v.up);
+                    mine = slot * T + lane;
+                }
+            }
+        }
+    }
     double best_v = make_inf();
     uint32_t code = DP_NO_STATE;
-    for (uint32_t g0 = 0; g0 < T; ++g0) {                    // stage 0 by first fit from the first zone of the order
-        if (!((okv[0] >> g0) & 1u)) continue;
-        const uint32_t p = L.cap[0][g0] >= 1 ? 0u : L.first_later[0][g0];
-        if (p == DP_NONE) continue;
-        const uint32_t slot = live[3 + 2 * p] + (L.first_vec[p][g0] - live[2 + 2 * p]);
-        if (slot >= live[0]) continue;
-        const DpVal v = lvl0[slot * T + g0];
-        if (!(v.sum < make_inf())) continue;
-        const double val = add_rn(add_rn(add_rn(v.sum, mul_rn(nb, v.mx)), v.sy), v.up);
-        if (code == DP_NO_STATE || val < best_v) { best_v = val; code = slot * T + g0; }
+    for (uint32_t g0 = 0; g0 < T; ++g0) {                    // the first of the best
+        const double val = __shfl_sync(FULL, mine_v, g0);
+        const uint32_t c = __shfl_sync(FULL, mine, g0);
+        if (c != DP_NO_STATE && (code == DP_NO_STATE || val < best_v)) { best_v = val; code = c; }
     }
     if (code == DP_NO_STATE) return;                         // the value stays at "no plan"
-    fp.value[job.index] = best_v;
+    if (lane == 0) fp.value[job.index] = best_v;
     const Config k = config_of(fp.sp, job.config);
-    sailor_run runs[SAILOR_P_MAX];
-    uint32_t n_runs = 0;
     const uint32_t* succ = fp.succ + job.succ_off;
-    for (uint32_t i = 0; i < P; ++i) {
+    for (uint32_t at = 0; at < P; at += 32) {
+        const uint32_t first = at + lane < P ? live[(size_t)(at + lane) * words + 1] : 0u;     // states before the stage's
+        const uint32_t n = P - at < 32 ? P - at : 32;
+        for (uint32_t l = 0; l < n; ++l) {
+            if (lane == 0) w.code[at + l] = code;
+            if (at + l + 1 < P) code = succ[(size_t)__shfl_sync(FULL, first, l) * T + code];
+        }
+    }
+    __syncwarp();
+    for (uint32_t i = lane; i < P; i += 32) {
         const uint32_t* row = live + (size_t)i * words;
-        const uint32_t now = code, slot = now / T, g = now - slot * T;
-        if (i + 1 < P) code = succ[(size_t)row[1] * T + now];
+        const uint32_t slot = w.code[i] / T, g = w.code[i] - slot * T;
         uint32_t zp = 0;
         while (zp + 1 < nz && row[3 + 2 * (zp + 1)] <= slot) ++zp;
         const uint8_t z = L.zone[zp];
         out.type[i] = (uint8_t)g;
         out.zone[i] = z;
-        if (n_runs && runs[n_runs - 1].type == g && runs[n_runs - 1].zone == z) runs[n_runs - 1].n_stages++;
-        else {
-            runs[n_runs].type = (uint8_t)g; runs[n_runs].zone = z;
-            runs[n_runs].tp_idx = (uint8_t)k.tpi; runs[n_runs].n_stages = 1;
-            ++n_runs;
-        }
+        w.gz[i] = (uint16_t)(g | z << 8);
     }
+    __syncwarp();
     // the plan written out, through the simulator (Sec. 4.3): what a caller compares with a constraint
     TabView v;
     v.bind(fp.blob, fp.blob);
-    uint32_t cnt[R_MAX];
-    const SimOut so = simulate_runs(v, fp.avail, P, n_runs, k.D, k.mi, k.rc, runs, SAILOR_P_MAX, cnt, 1);
-    out.t_iter = so.t_iter;
-    out.cost = so.cost;
-    out.peak_mem = so.peak_mem;
-    out.status = so.status;
+    const SimOut so = simulate_stages(v, fp.avail, k, w.gz, w.cnt, lane);
+    if (lane == 0) {
+        out.t_iter = so.t_iter;
+        out.cost = so.cost;
+        out.peak_mem = so.peak_mem;
+        out.status = so.status;
+    }
 }
 
 // The k best problems by (value, problem index), then the simulator's figures for their plans.

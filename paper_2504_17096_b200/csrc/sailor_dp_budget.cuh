@@ -240,10 +240,12 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
     for (uint32_t j = 0; j < P; ++j) root.type[j] = fr[0].b_type[j];
 }
 
-// Per problem the best of its first stage's types (the lowest among equals), written out and simulated; one thread each.
+// Per problem the best of its first stage's types (the lowest among equals), written out and simulated; a warp each.
 __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_budget_finish_kernel(const __grid_constant__ DpBudgetParams bp) {
-    const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ DpFinishWarp warps[DP_FINISH_WARPS];
+    const uint32_t lane = threadIdx.x & 31, x = blockIdx.x * DP_FINISH_WARPS + (threadIdx.x >> 5);
     if (x >= bp.n_problems) return;
+    DpFinishWarp& w = warps[threadIdx.x >> 5];
     const DpProblem& pb = bp.problems[x];
     const uint32_t T = bp.T, P = pb.P;
     const DpbRoot* roots = bp.roots + (size_t)x * T;
@@ -254,43 +256,43 @@ __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_budget_finish_kernel(con
         nodes += roots[g].nodes;
         if (roots[g].value < best_v) { best_v = roots[g].value; best = g; }
     }
-    if (nodes) atomicAdd(&bp.counters[4], nodes);
-    if (nodes > bp.node_limit) { atomicAdd(&bp.counters[3], 1ull); return; }
+    if (lane == 0 && nodes) atomicAdd(&bp.counters[4], nodes);
+    if (nodes > bp.node_limit) {
+        if (lane == 0) atomicAdd(&bp.counters[3], 1ull);
+        return;
+    }
     if (best == DP_NONE) return;
-    bp.value[pb.index] = best_v;
+    if (lane == 0) bp.value[pb.index] = best_v;
     const uint8_t* best_type = roots[best].type;
     DpResult& out = bp.results[pb.index];
     TabView v;
     v.bind(bp.blob, bp.blob);
     const Config k = config_of(bp.sp, pb.config);
     // zones by first fit, as the recursion placed them; then the plan through the simulator (Sec. 4.3)
-    sailor_run runs[DP_BUDGET_P_MAX];
-    uint32_t n_runs = 0, zp = 0;
-    uint8_t u[SAILOR_T_MAX];
-    for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) u[t] = 0;
-    for (uint32_t i = 0; i < P; ++i) {
-        const uint32_t g = best_type[i];
-        uint32_t zp2 = zp;
-        if (!(u[g] < pb.cap[zp][g])) zp2 = pb.first_later[zp][g];
-        if (zp2 != zp) for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) u[t] = 0;
-        u[g]++;
+    const uint32_t my_type = lane < P ? best_type[lane] : 0u;
+    static_assert(DP_BUDGET_P_MAX <= 32, "a lane per stage");
+    if (lane < SAILOR_T_MAX) w.used[lane] = 0;
+    __syncwarp();
+    for (uint32_t i = 0, zp = 0; i < P; ++i) {
+        const uint32_t g = __shfl_sync(FULL, my_type, i);
+        const uint32_t zp2 = w.used[g] < pb.cap[zp][g] ? zp : (uint32_t)pb.first_later[zp][g];
+        __syncwarp();
+        if (lane < SAILOR_T_MAX) w.used[lane] = (uint8_t)((zp2 != zp ? 0u : w.used[lane]) + (lane == g ? 1u : 0u));
         zp = zp2;
-        const uint8_t z = pb.zone[zp];
-        out.type[i] = (uint8_t)g;
-        out.zone[i] = z;
-        if (n_runs && runs[n_runs - 1].type == g && runs[n_runs - 1].zone == z) runs[n_runs - 1].n_stages++;
-        else {
-            runs[n_runs].type = (uint8_t)g; runs[n_runs].zone = z;
-            runs[n_runs].tp_idx = (uint8_t)k.tpi; runs[n_runs].n_stages = 1;
-            ++n_runs;
-        }
+        if (lane == i) w.gz[i] = (uint16_t)(g | pb.zone[zp] << 8);
+        __syncwarp();
     }
-    uint32_t cnt[R_MAX];
-    const SimOut so = simulate_runs(v, bp.avail, P, n_runs, k.D, k.mi, k.rc, runs, DP_BUDGET_P_MAX, cnt, 1);
-    out.t_iter = so.t_iter;
-    out.cost = so.cost;
-    out.peak_mem = so.peak_mem;
-    out.status = so.status;
+    if (lane < P) {
+        out.type[lane] = (uint8_t)my_type;
+        out.zone[lane] = (uint8_t)(w.gz[lane] >> 8);
+    }
+    const SimOut so = simulate_stages(v, bp.avail, k, w.gz, w.cnt, lane);
+    if (lane == 0) {
+        out.t_iter = so.t_iter;
+        out.cost = so.cost;
+        out.peak_mem = so.peak_mem;
+        out.status = so.status;
+    }
 }
 
 }  // namespace sailor

@@ -199,6 +199,7 @@ struct SpaceCache {
 // What a context keeps in pinned host memory the device can write.
 constexpr size_t HOST_SMALL_BYTES = 192 * 1024;
 
+
 struct HostBlock {
     PlanOut out;                           // results of a search
     SurveyOut survey;                      // what the survey of a space found
@@ -852,6 +853,15 @@ int host_batch_small(sailor_ctx* ctx, const unsigned char* recs, size_t rec_byte
     return host_batch_error(err);
 }
 
+// A second stream of the context and the events around it, made when a call first needs them.
+int side_stream(sailor_ctx* ctx) {
+    if (ctx->out_stream) return SAILOR_OK;
+    for (cudaEvent_t* e : {&ctx->ev_chunk, &ctx->ev_join, &ctx->ev_slot[0], &ctx->ev_slot[1], &ctx->ev_slot[2]})
+        if (!*e) CU(ctx, cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    CU(ctx, cudaStreamCreateWithFlags(&ctx->out_stream, cudaStreamNonBlocking));
+    return SAILOR_OK;
+}
+
 template <class Launch>
 int host_batch(sailor_ctx* ctx, const unsigned char* recs, size_t rec_bytes, uint64_t n, double* t_iter, uint64_t* peak_mem,
                double* cost, uint32_t* status, Launch launch) {
@@ -868,11 +878,9 @@ int host_batch(sailor_ctx* ctx, const unsigned char* recs, size_t rec_bytes, uin
         const int rc_mem = device_grow(ctx, &ctx->d_stage, &ctx->stage_bytes, need);
         if (rc_mem) return rc_mem;
     }
-    if (split && !ctx->out_stream) {       // made when the first batch that needs them arrives
-        CU(ctx, cudaEventCreateWithFlags(&ctx->ev_chunk, cudaEventDisableTiming));
-        CU(ctx, cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
-        for (cudaEvent_t& e : ctx->ev_slot) CU(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        CU(ctx, cudaStreamCreateWithFlags(&ctx->out_stream, cudaStreamNonBlocking));
+    if (split) {
+        const int rc_side = side_stream(ctx);
+        if (rc_side) return rc_side;
     }
     {
         const int rc_up = upload_availability(ctx);
@@ -1810,7 +1818,7 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     bp.node_limit = 1ull << 24;
     dp_budget_kernel<<<(uint32_t)((n_problems * T + DPB_WARPS - 1) / DPB_WARPS), 32 * DPB_WARPS, dpb_smem(p_max), ctx->stream>>>(bp);
     CU(ctx, cudaGetLastError());
-    dp_budget_finish_kernel<<<(uint32_t)((n_problems + DP_FINISH_THREADS - 1) / DP_FINISH_THREADS), DP_FINISH_THREADS, 0, ctx->stream>>>(bp);
+    dp_budget_finish_kernel<<<(uint32_t)((n_problems + DP_FINISH_WARPS - 1) / DP_FINISH_WARPS), DP_FINISH_THREADS, 0, ctx->stream>>>(bp);
     CU(ctx, cudaGetLastError());
     launches += 2;
     DpSelectParams sel;
@@ -2072,31 +2080,54 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
         else dp_layout_kernel<SAILOR_T_MAX><<<lay_blk.back(), DP_THREADS, 0, ctx->stream>>>(yp);
         CU(ctx, cudaGetLastError());
         ++launches;
+        // The small problems' blocks take each a problem through all its stages and mostly wait for one another: they run beside
+        // the levels of the large ones, on a second stream (five zones, 48 stages: 300 us of a search's 2 315; joining in only
+        // when levels have become small, as late as they hide, 1 984 instead of 1 809).
         const uint32_t n_small = (uint32_t)jobs.size() - n_big;
+        const bool fork = n_small && n_big;
+        auto joined = [&](cudaError_t e) {                       // nothing is left running there after a failure
+            if (e != cudaSuccess && fork) cudaStreamSynchronize(ctx->out_stream);
+            return e;
+        };
+        if (fork) {
+            const int rc_side = side_stream(ctx);
+            if (rc_side) return rc_side;
+            CU(ctx, cudaEventRecord(ctx->ev_chunk, ctx->stream));
+            CU(ctx, cudaStreamWaitEvent(ctx->out_stream, ctx->ev_chunk, 0));
+        }
         if (n_small) {
             DpLevelParams sp = lp;
             sp.jobs = lp.jobs + n_big;
-            if (TM == 4) dp_problem_kernel<4><<<n_small, DP_THREADS, 0, ctx->stream>>>(sp);
-            else dp_problem_kernel<SAILOR_T_MAX><<<n_small, DP_THREADS, 0, ctx->stream>>>(sp);
-            CU(ctx, cudaGetLastError());
+            cudaStream_t stream = fork ? ctx->out_stream : ctx->stream;
+            if (TM == 4) dp_problem_kernel<4><<<n_small, DP_THREADS, 0, stream>>>(sp);
+            else dp_problem_kernel<SAILOR_T_MAX><<<n_small, DP_THREADS, 0, stream>>>(sp);
+            CU(ctx, joined(cudaGetLastError()));
             ++launches;
+            if (fork) CU(ctx, joined(cudaEventRecord(ctx->ev_join, ctx->out_stream)));
         }
         for (uint32_t dist = 0; dist + 1 < dist_off.size(); ++dist) {
             lp.dist = dist;
             lp.blk_prefix = d_prefix + dist_off[dist];
             lp.n_active = (uint32_t)(dist_off[dist + 1] - dist_off[dist] - 1);
             const uint32_t n_blk = prefix[dist_off[dist + 1] - 1];
-            if (TM == 4) dp_level_kernel<4><<<n_blk, DP_THREADS, 0, ctx->stream>>>(lp);
-            else dp_level_kernel<SAILOR_T_MAX><<<n_blk, DP_THREADS, 0, ctx->stream>>>(lp);
-            CU(ctx, cudaGetLastError());
+            // a level's blocks may start (and find their job and its tables) while the level before it ends
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr = {};
+            attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr.val.programmaticStreamSerializationAllowed = dist ? 1 : 0;
+            cfg.gridDim = dim3(n_blk); cfg.blockDim = dim3(DP_THREADS); cfg.stream = ctx->stream;
+            cfg.attrs = &attr; cfg.numAttrs = 1;
+            CU(ctx, joined(TM == 4 ? cudaLaunchKernelEx(&cfg, dp_level_kernel<4>, (const DpLevelParams)lp)
+                                   : cudaLaunchKernelEx(&cfg, dp_level_kernel<SAILOR_T_MAX>, (const DpLevelParams)lp)));
             ++launches;
         }
+        if (fork) CU(ctx, joined(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0)));
         DpFinishParams fp;
         memset(&fp, 0, sizeof(fp));
         fp.blob = ctx->d_blob; fp.avail = ctx->d_avail; fp.sp = d; fp.layouts = lp.layouts; fp.jobs = lp.jobs; fp.live = lp.live;
         fp.tabs = d_tabs; fp.val[0] = lp.val[0]; fp.val[1] = lp.val[1]; fp.succ = lp.succ; fp.value = d_value;
         fp.results = d_results; fp.lay = lay; fp.n_jobs = (uint32_t)jobs.size(); fp.T = T;
-        dp_finish_kernel<<<(fp.n_jobs + DP_FINISH_THREADS - 1) / DP_FINISH_THREADS, DP_FINISH_THREADS, 0, ctx->stream>>>(fp);
+        dp_finish_kernel<<<(fp.n_jobs + DP_FINISH_WARPS - 1) / DP_FINISH_WARPS, DP_FINISH_THREADS, 0, ctx->stream>>>(fp);
         CU(ctx, cudaGetLastError());
         ++launches;
         up.clear();
