@@ -1598,7 +1598,8 @@ struct LayoutInfo {
 
 // The layout of pipelines of P stages of `need` GPUs each over the zones of `order`, with the types of `usable`.
 // Returns SAILOR_E_RANGE when a position has more than 2^31 vectors; a stage without live vectors leaves max_live at 0.
-int build_layout(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_zone_order& order, uint32_t usable, LayoutInfo& info) {
+int build_layout(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_zone_order& order, uint32_t usable,
+                 std::vector<uint64_t>& W, LayoutInfo& info) {
     const uint32_t T = ctx->hdr.T, w = P + 1;
     DpLayout& l = info.l;
     memset(&l, 0, sizeof(l));
@@ -1607,7 +1608,8 @@ int build_layout(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_
     uint64_t lo = 0, mx = 0;               // stages before a position: at least, at most
     uint64_t lo_of[SAILOR_Z_MAX], mx_of[SAILOR_Z_MAX], n_vec = 0;
     bool uncounted_of[SAILOR_Z_MAX], hosts[SAILOR_Z_MAX];
-    std::vector<uint64_t> W((size_t)(T + 1) * w), first_sum(order.n, 0);
+    W.resize((size_t)(T + 1) * w);         // (scratch)
+    info.w.reserve((size_t)order.n * (T + 1) * w);
     for (uint32_t zp = 0; zp < order.n && lo < P; ++zp) {
         l.nz = zp + 1;
         l.zone[zp] = order.zone[zp];
@@ -1644,7 +1646,9 @@ int build_layout(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_
         }
         if (W[most] > (1ull << 31)) return SAILOR_E_RANGE;
         l.w_off[zp] = (uint32_t)info.w.size();
-        for (size_t x = 0; x < (size_t)(m + 1) * w; ++x) info.w.push_back((uint32_t)(W[x] < 0xffffffffull ? W[x] : 0xffffffffull));
+        info.w.resize(info.w.size() + (size_t)(m + 1) * w);
+        uint32_t* out = info.w.data() + l.w_off[zp];
+        for (size_t x = 0; x < (size_t)(m + 1) * w; ++x) out[x] = (uint32_t)(W[x] < 0xffffffffull ? W[x] : 0xffffffffull);
         l.vec_base[zp] = (uint32_t)n_vec;
         for (uint32_t j = 0; j < m; ++j)
             l.first_vec[zp][types[j]] = (uint32_t)(n_vec + W[0] + (P >= 1 ? W[(size_t)(j + 1) * w + 1] - W[(size_t)(j + 1) * w] : 0));
@@ -1694,31 +1698,47 @@ int build_layout(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_
     return SAILOR_OK;
 }
 
-// The GPU types that fit the memory of some stage of a configuration; 0 when a stage fits none.  Inside a stretch of
-// stages of one make-up the first keeps the most microbatches and the last the fewest.
-uint32_t usable_types(const sailor_ctx* ctx, const TabView& v, const Config& k, uint64_t n_b) {
-    const TabHdr& h = ctx->hdr;
-    const uint32_t P = k.P, base = h.n_blocks / P, extra = h.n_blocks % P, tp = h.tp_values[k.tpi];
-    auto fits = [&](uint32_t i) {
-        const bool e = (i == 0) && h.has_embed, hd = (i == P - 1) && h.has_head;
-        const uint64_t inflight = (uint64_t)(P - i) < n_b ? (uint64_t)(P - i) : n_b;
-        const StageMem sm = stage_memory(v, k.tpi, k.mi, k.rc, base + (i < extra ? 1u : 0u), e, hd, inflight);
+// The stretches of stages of one make-up in a pipeline, with what a stage of each needs of the memory: bytes without a
+// microbatch in flight, bytes per microbatch.  The same for every data-parallel degree.
+struct Stretches {
+    uint32_t n = 0, first[4], last[4];
+    uint64_t fixed[4], kept[4];
+    Stretches(const TabHdr& h, const TabView& v, const Config& k) {
+        const uint32_t P = k.P, base = h.n_blocks / P, extra = h.n_blocks % P;
+        for (uint32_t i = 0; i < P;) {
+            uint32_t end = P;
+            if (i == 0 && h.has_embed) end = 1;
+            else {
+                if (i < extra && extra < end) end = extra;
+                if (h.has_head && i < P - 1 && P - 1 < end) end = P - 1;
+            }
+            const bool e = (i == 0) && h.has_embed, hd = (i == P - 1) && h.has_head;
+            const uint32_t nb = base + (i < extra ? 1u : 0u);
+            first[n] = i;
+            last[n] = end - 1;
+            fixed[n] = stage_memory(v, k.tpi, k.mi, k.rc, nb, e, hd, 0).mem;
+            kept[n] = stage_memory(v, k.tpi, k.mi, k.rc, nb, e, hd, 1).mem - fixed[n];
+            ++n;
+            i = end;
+        }
+    }
+};
+
+// The GPU types that fit the memory of some stage of a configuration; 0 when a stage fits none.  Inside a stretch the first
+// stage keeps the most microbatches and the last the fewest.
+uint32_t usable_types(const TabHdr& h, const Stretches& st, const Config& k, uint64_t n_b) {
+    const uint32_t tp = h.tp_values[k.tpi];
+    auto fits = [&](uint32_t q, uint32_t i) {
+        const uint64_t inflight = (uint64_t)(k.P - i) < n_b ? (uint64_t)(k.P - i) : n_b, mem = st.fixed[q] + inflight * st.kept[q];
         uint32_t mask = 0;
         for (uint32_t g = 0; g < h.T; ++g)
-            if (sm.mem + h.reserved[g] <= h.capacity[g] && tp <= h.gpn[g]) mask |= 1u << g;
+            if (mem + h.reserved[g] <= h.capacity[g] && tp <= h.gpn[g]) mask |= 1u << g;
         return mask;
     };
     uint32_t all = 0;
-    for (uint32_t i = 0; i < P;) {
-        uint32_t end = P;
-        if (i == 0 && h.has_embed) end = 1;
-        else {
-            if (i < extra && extra < end) end = extra;
-            if (h.has_head && i < P - 1 && P - 1 < end) end = P - 1;
-        }
-        if (!fits(i)) return 0;
-        all |= fits(end - 1);
-        i = end;
+    for (uint32_t q = 0; q < st.n; ++q) {
+        if (!fits(q, st.first[q])) return 0;
+        all |= fits(q, st.last[q]);
     }
     return all;
 }
@@ -1896,6 +1916,10 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
     std::vector<Problem> by_depth[SAILOR_P_MAX + 1];         // deepest first, so that a stage's launch covers a prefix
     std::vector<uint8_t> wanted(n_config, 0);                // configurations whose per-configuration tables are needed
     uint64_t n_states = 0;
+    std::unique_ptr<Stretches> stretches;
+    uint64_t stretches_end = 0;
+    std::vector<uint64_t> scratch;
+    layouts.reserve(512);
     for (uint64_t c = 0; c < n_config; ++c) {
         const Config cf = config_of(d, (uint32_t)c);
         const uint32_t tp = h.tp_values[cf.tpi];
@@ -1905,14 +1929,18 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
         if (o->flags & SAILOR_DP_FLAG_INDEX_DENSE)
             for (uint32_t q = 0; q < n_orders; ++q)
                 if (dense_fits(ctx, cf.P, need, orders[q], workspace_bytes) != SAILOR_OK) return SAILOR_E_RANGE;
-        const uint32_t usable = usable_types(ctx, hv, cf, h.gbs / dm);
+        if (!stretches || c >= stretches_end) {              // the degree varies fastest
+            stretches.reset(new Stretches(h, hv, cf));
+            stretches_end = c - c % d.n_d + d.n_d;
+        }
+        const uint32_t usable = usable_types(h, *stretches, cf, h.gbs / dm);
         if (!usable) continue;                               // some stage fits no type
         for (uint32_t q = 0; q < n_orders; ++q) {
             const std::pair<uint64_t, uint64_t> key((uint64_t)q << 8 | cf.P, need << SAILOR_T_MAX | usable);
             const auto seen = layout_of.emplace(key, (uint32_t)layouts.size());
             if (seen.second) {
                 layouts.emplace_back();
-                const int rc_lay = build_layout(ctx, cf.P, need, orders[q], usable, layouts.back());
+                const int rc_lay = build_layout(ctx, cf.P, need, orders[q], usable, scratch, layouts.back());
                 if (rc_lay) return rc_lay;
             }
             const LayoutInfo& info = layouts[seen.first->second];
