@@ -288,9 +288,9 @@ inline void cpu_relax() {
 }
 
 // Waits until the kernel that ends a call has left its results, with `ticket` behind them, in the context's pinned memory:
-// the host sees them some microseconds before the stream counts as idle (a search of one zone with new availability 55.2 us by
-// cudaStreamSynchronize, 52.5 this way).  Everything enqueued earlier on the stream is done by then.  A stream that ends, or fails, without
-// the ticket is found out by asking it now and then.
+// the host sees them some microseconds before the stream counts as idle (a search of one zone with new availability:
+// 55.2 us by cudaStreamSynchronize, 52.5 this way).  Everything enqueued earlier on the stream is done by then.  A stream
+// that ends, or fails, without the ticket is found out by asking it now and then.
 cudaError_t wait_ticket(sailor_ctx* ctx, const uint64_t* slot, uint64_t ticket) {
     const volatile uint64_t* seen = slot;
     for (uint32_t spin = 1;; ++spin) {
@@ -1761,7 +1761,7 @@ int dense_fits(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_zo
 
 }  // namespace
 
-// The recursion steered by the budget (Sec. 4.2.3): one thread per problem, depth first.
+// The recursion steered by the budget (Sec. 4.2.3): a warp per problem and type of its first stage, depth first.
 static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor_zone_order* orders, uint32_t n_orders,
                                const sailor_objective* o, uint64_t workspace_bytes, uint32_t k, sailor_dp_result* topk,
                                uint32_t* n_found, sailor_dp_stats* stats) {
