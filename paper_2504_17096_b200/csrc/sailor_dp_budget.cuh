@@ -35,10 +35,14 @@ struct DpbFrame {                    // one call of the recursion: stage `level`
     double b_sum, b_mx, b_sy, b_up, b_cost;      // best plan of stages level.. so far (b_found)
     uint8_t g, zp, g2, zp2;          // g2: type tried for the next stage, zp2: where first fit puts it
     uint8_t b_found, _pad[3];
-    uint8_t u[SAILOR_T_MAX];         // stages per type in zone position zp, this stage included
-    uint8_t u2[SAILOR_T_MAX];        // the same for the next stage's position after the move
-    uint8_t b_type[DP_BUDGET_P_MAX]; // types of stages level.. of the best plan (indexed by stage)
+    uint64_t u;                      // stages per type (a byte each) in zone position zp, this stage included
+    uint64_t u2;                     // the same for the next stage's position after the move
+    union {                          // types of stages level.. of the best plan (indexed by stage)
+        uint8_t b_type[DP_BUDGET_P_MAX];
+        uint64_t b_word[DP_BUDGET_P_MAX / 8];
+    };
 };
+static_assert(SAILOR_T_MAX <= 8 && DP_BUDGET_P_MAX < 256, "a byte per type holds every count");
 
 struct DpbRoot {                     // what the walk from one type of stage 0 found
     double value;                    // +inf: no plan
@@ -71,6 +75,7 @@ __device__ __forceinline__ double dpb_value(double nb, double sum, double mx, do
 // Bound by the latency of one chain of calls.  Workload 2, pipelines of up to eight stages, all orders, budget 1.2 x
 // cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.64 ms a call.
 constexpr int DPB_WARPS = 4;
+constexpr size_t DPB_NEAR_BYTES = 16 * 1024;      // a block's four tables of this size leave L1 room for the rest
 
 __host__ __device__ inline size_t dpb_smem(uint32_t p_max) {
     return DPB_WARPS * (p_max * sizeof(DpbFrame) + (p_max + 1) * sizeof(double));
@@ -108,6 +113,17 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
     const double* synct = tab + bp.lay.off_sync();
     const double* c2x = tab + bp.lay.off_c2x();
 
+    // one thread walks below: what it reads is brought near by all of them first (a walk of a few dozen calls otherwise
+    // waits for one line after another)
+    auto bring = [&](const void* first, size_t bytes) {
+        const uintptr_t at = reinterpret_cast<uintptr_t>(first) & ~(uintptr_t)127, end = reinterpret_cast<uintptr_t>(first) + bytes;
+        for (uintptr_t a = at + 128 * lane; a < end; a += 128 * 32) asm volatile("prefetch.global.L1 [%0];" ::"l"(a));
+    };
+    bring(&pb, sizeof(pb));
+    bring(v.price_s, R * sizeof(double));
+    bring(v.egress, Z * Z * sizeof(double));
+    if (bp.lay.stride() * sizeof(double) <= DPB_NEAR_BYTES) bring(tab, bp.lay.stride() * sizeof(double));
+
     // the least any plan of stages j.. can be charged: every stage alone on the cheapest GPUs it fits, for its own
     // compute time; added up from the last stage backwards, as the recursion adds its charges
     if (lane < P) {
@@ -136,8 +152,7 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
     {
         DpbFrame& f = fr[0];
         f.g = (uint8_t)g0; f.zp = (uint8_t)p0; f.limit = bp.limit;
-        for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) f.u[t] = 0;
-        f.u[g0] = 1;
+        f.u = 1ull << (8 * g0);
     }
     enum { ENTER, NEXT_TYPE, CHARGE, RESUME } state = ENTER;
     while (level >= 0) {
@@ -169,11 +184,10 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
                 if ((okv[i + 1] >> g2) & 1u) {
                     // first fit: this zone while it has room for one more stage of the type, else the next that has
                     uint32_t zp2 = f.zp;
-                    if (!(f.u[g2] < pb.cap[f.zp][g2])) zp2 = pb.first_later[f.zp][g2];
+                    if (!(((uint32_t)(f.u >> (8 * g2)) & 0xffu) < pb.cap[f.zp][g2])) zp2 = pb.first_later[f.zp][g2];
                     if (zp2 != DP_NONE) {
                         f.zp2 = (uint8_t)zp2;
-                        for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) f.u2[t] = zp2 == f.zp ? f.u[t] : 0;
-                        f.u2[g2]++;
+                        f.u2 = (zp2 == f.zp ? f.u : 0ull) + (1ull << (8 * g2));
                         const uint32_t z2 = pb.zone[zp2], dn = z2 * T + g2;
                         f.t = add_rn(f.fb, c2x[dn * R + d]);
                         f.comm = z2 != z ? mul_rn(xbytes, v.egress[z * Z + z2]) : 0.0;
@@ -203,7 +217,7 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
             }
             DpbFrame& c = fr[level + 1];
             c.g = f.g2; c.zp = f.zp2; c.limit = rest;
-            for (uint32_t t = 0; t < SAILOR_T_MAX; ++t) c.u[t] = f.u2[t];
+            c.u = f.u2;
             ++level;
             state = ENTER;
             continue;
@@ -223,7 +237,8 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
                     f.b_found = 1;
                     f.b_sum = c_sum; f.b_mx = c_mx; f.b_sy = c_sy; f.b_up = c_up; f.b_cost = all;
                     const DpbFrame& c = fr[level + 1];
-                    for (uint32_t j = i + 1; j < P; ++j) f.b_type[j] = c.b_type[j];
+#pragma unroll
+                    for (uint32_t j = 0; j < DP_BUDGET_P_MAX / 8; ++j) f.b_word[j] = c.b_word[j];
                     f.b_type[i] = (uint8_t)g;
                 }
             }
