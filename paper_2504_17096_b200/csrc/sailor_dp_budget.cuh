@@ -28,6 +28,39 @@ struct DpProblem {                   // what first fit needs of a (configuration
     uint8_t first_later[SAILOR_Z_MAX][SAILOR_T_MAX];   // first position after zp that can host a stage of the type
 };
 
+// What first fit needs of every problem, from the availability last set.  A thread per problem (formed and copied by the
+// host it took 60 us for 1 344).
+__global__ void __launch_bounds__(128)
+dp_budget_problems_kernel(const unsigned char* __restrict__ blob, const uint16_t* __restrict__ avail, SpaceDesc sp,
+                          const sailor_zone_order* __restrict__ orders, uint32_t n_orders, uint32_t n_problems, DpProblem* __restrict__ out,
+                          unsigned long long* counters) {
+    const TabHdr* h = reinterpret_cast<const TabHdr*>(blob);
+    const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x, T = h->T;
+    if (x < 5) counters[x] = 0;
+    if (x >= n_problems) return;
+    const uint32_t c = x / n_orders, q = x - c * n_orders;
+    const Config k = config_of(sp, c);
+    const uint64_t need = (uint64_t)k.D * h->tp_values[k.tpi];
+    const sailor_zone_order& order = orders[q];
+    DpProblem& pb = out[x];
+    pb.config = c; pb.order = q; pb.index = x;
+    pb.P = k.P; pb.nz = order.n; pb.need = (uint32_t)(need > 0xffffffffull ? 0xffffffffull : need);
+    uint32_t later = 0;                                      // per type (4 bits each): the first position after this one, or none
+    for (uint32_t g = 0; g < T; ++g) later |= 15u << (4 * g);
+    for (uint32_t zp = pb.nz; zp-- > 0;) {
+        const uint32_t z = order.zone[zp];
+        pb.zone[zp] = (uint8_t)z;
+        for (uint32_t g = 0; g < T; ++g) {
+            const uint32_t a = avail[z * T + g], first = (later >> (4 * g)) & 15u;
+            const uint32_t cap = need > a ? 0u : a / (uint32_t)need;
+            pb.cap[zp][g] = (uint8_t)(cap > 255 ? 255 : cap);
+            pb.first_later[zp][g] = first == 15u ? DP_NONE : (uint8_t)first;
+            if (cap >= 1) later = (later & ~(15u << (4 * g))) | zp << (4 * g);
+        }
+    }
+}
+static_assert(SAILOR_Z_MAX < 15 && SAILOR_T_MAX * 4 <= 32, "a position fits four bits");
+
 struct DpbFrame {                    // one call of the recursion: stage `level` on type g at zone position zp
     double limit;                    // what stages level.. may be charged
     double rate, sync, fb, upd;      // of this stage on its GPUs

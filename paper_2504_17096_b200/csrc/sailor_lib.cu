@@ -1770,37 +1770,13 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     const uint64_t n_config = (uint64_t)d.n_p * d.n_mbs * d.n_tp * d.n_rc * d.n_d, n_problems = n_config * n_orders;
     uint32_t p_max = 0;
     for (uint32_t j = 0; j < d.n_p; ++j) p_max = d.p_values[j] > p_max ? d.p_values[j] : p_max;
-    // what first fit needs of every problem, from the availability last set (host copy)
-    std::vector<DpProblem> prob(n_problems);
-    for (uint64_t c = 0; c < n_config; ++c) {
-        const Config cf = config_of(d, (uint32_t)c);
-        const uint64_t need = (uint64_t)cf.D * h.tp_values[cf.tpi];
-        for (uint32_t q = 0; q < n_orders; ++q) {
-            DpProblem& pb = prob[c * n_orders + q];
-            memset(&pb, 0, sizeof(pb));
-            pb.config = (uint32_t)c; pb.order = q; pb.index = (uint32_t)(c * n_orders + q);
-            pb.P = cf.P; pb.nz = orders[q].n; pb.need = (uint32_t)(need > 0xffffffffull ? 0xffffffffull : need);
-            memset(pb.first_later, DP_NONE, sizeof(pb.first_later));
-            for (uint32_t zp = 0; zp < pb.nz; ++zp) {
-                pb.zone[zp] = orders[q].zone[zp];
-                for (uint32_t g = 0; g < T; ++g) {
-                    const uint64_t cap = ctx->h_avail[pb.zone[zp] * T + g] / need;
-                    pb.cap[zp][g] = (uint8_t)(cap > 255 ? 255 : cap);
-                }
-            }
-            for (uint32_t zp = 0; zp < pb.nz; ++zp)
-                for (uint32_t g = 0; g < T; ++g)
-                    for (uint32_t later = zp + 1; later < pb.nz; ++later)
-                        if (pb.cap[later][g] >= 1) { pb.first_later[zp][g] = (uint8_t)later; break; }
-        }
-    }
     DeviceGuard guard(ctx->device);
     DpTabLayout lay;
     lay.p_max = p_max; lay.T = T; lay.R = h.R;
     const size_t tab_bytes = (size_t)n_config * lay.stride() * sizeof(double);
     const size_t total = padded(tab_bytes) + padded(n_problems * sizeof(DpResult)) + padded(n_problems * sizeof(DpProblem)) +
                          padded(n_problems * T * sizeof(DpbRoot)) + padded(n_problems * sizeof(double)) +
-                         padded(40) + 4096;
+                         padded(40) + std::max<size_t>(padded(n_orders * sizeof(sailor_zone_order)), 4096);
     if (total > workspace_bytes) return SAILOR_E_RANGE;
     {
         const int rc_mem = device_grow(ctx, &ctx->d_dp, &ctx->dp_bytes, total);
@@ -1813,6 +1789,7 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     DpbRoot* d_roots = bump.take<DpbRoot>(n_problems * T);
     double* d_value = bump.take<double>(n_problems);
     unsigned long long* d_counters = bump.take<unsigned long long>(5);
+    sailor_zone_order* d_orders = bump.take<sailor_zone_order>(n_orders);
     DpOut* d_out = nullptr;
     CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&d_out), &ctx->host->dp, 0));
 
@@ -1821,14 +1798,17 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
         const int rc_up = upload_availability(ctx);
         if (rc_up) return rc_up;
     }
-    CU(ctx, cudaMemsetAsync(d_counters, 0, 40, ctx->stream));
-    CU(ctx, cudaMemcpyAsync(d_problems, prob.data(), n_problems * sizeof(DpProblem), cudaMemcpyHostToDevice, ctx->stream));
+    CU(ctx, cudaMemcpyAsync(d_orders, orders, n_orders * sizeof(sailor_zone_order), cudaMemcpyHostToDevice, ctx->stream));
     {
         const uint32_t grid = (uint32_t)(n_config < 4096 ? n_config : 4096);
         dp_tables_kernel<<<grid, DP_THREADS, 0, ctx->stream>>>(ctx->d_blob, d, (uint32_t)n_config, n_orders, lay, nullptr, d_tabs, d_value, &d_out->span);
         CU(ctx, cudaGetLastError());
         ++launches;
     }
+    dp_budget_problems_kernel<<<(uint32_t)((n_problems + 127) / 128), 128, 0, ctx->stream>>>(
+        ctx->d_blob, ctx->d_avail, d, d_orders, n_orders, (uint32_t)n_problems, d_problems, d_counters);
+    CU(ctx, cudaGetLastError());
+    ++launches;
     DpBudgetParams bp;
     memset(&bp, 0, sizeof(bp));
     bp.blob = ctx->d_blob; bp.avail = ctx->d_avail; bp.sp = d; bp.problems = d_problems; bp.tabs = d_tabs;
@@ -1849,7 +1829,7 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     dp_select_kernel<<<1, DP_SELECT_THREADS, 0, ctx->stream>>>(sel);
     CU(ctx, cudaGetLastError());
     ++launches;
-    CU(ctx, stream_sync(ctx));                                 // also: `prob` is pageable
+    CU(ctx, stream_sync(ctx));
     const unsigned long long* counters = ctx->host->dp.counters;
     if (counters[1] > k) return SAILOR_E_DEVICE;
     *n_found = (uint32_t)counters[1];

@@ -161,3 +161,19 @@ def test_budget_loop_argument_checks():
         with pytest.raises(B.SailorError) as e:
             B.sailor_plan_dp(cx.ctx, cx.space, [[0]], 4, budget=1.0, budget_loop=True)
         assert e.value.code == B.E_RANGE
+
+
+@pytest.mark.parametrize("orders", [[[3]], [[7, 6, 5, 4, 3, 2, 1, 0], [2, 5], [0]]])
+def test_first_fit_tables_up_to_the_limits(orders):
+    """What first fit needs of a problem is formed on the device, positions in four bits: eight types in up to eight zones,
+    zones without GPUs of a type or fewer than a stage takes, orders of unlike length."""
+    w = W.tiny(seed=53, n_types=8, n_zones=8, L=4, p_values=[1, 3], d_values=(1, 3), tp_values=(1, 2), mbs_values=(1,), rc_values=(0,))
+    w.avail[...] = np.arange(64).reshape(8, 8) * 7 % 9
+    w.avail[3] = 12
+    o = Oracle(w)
+    kept, _, _ = oracle_limited(w, o, orders, 1e9)
+    limit = 1.5 * min(x[3].cost for x in kept)
+    want, solved, over = oracle_limited(w, o, orders, limit)
+    with Ctx(w) as cx:
+        res, st = B.sailor_plan_dp(cx.ctx, cx.space, orders, 16, budget=limit, budget_loop=True)
+        assert_same(res, st, want, solved, over, w, orders, 16, str(orders))
