@@ -106,7 +106,8 @@ __device__ __forceinline__ double dpb_value(double nb, double sum, double mx, do
 // A warp per (problem, type of stage 0).  The walk is one lane's: problems differ too much in what they try to share
 // instructions (a thread per problem ran a warp's 32 walks one after the other), and its stack sits in shared memory.
 // Bound by the latency of one chain of calls.  Workload 2, pipelines of up to eight stages, all orders, budget 1.2 x
-// cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.64 ms a call.
+// cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.44 ms a call; a frame's counts as
+// bytes of one word and the walk's tables brought near beforehand took its share from 459 to 408 us.
 constexpr int DPB_WARPS = 4;
 constexpr size_t DPB_NEAR_BYTES = 16 * 1024;      // a block's four tables of this size leave L1 room for the rest
 
