@@ -67,7 +67,9 @@ extern "C" {
 #define SAILOR_E_NOMEM    (-4)  /* host or device allocation failed                          */
 #define SAILOR_E_DEVICE   (-5)  /* a kernel reported an internal fault (bounded wait ran out)
                                    during THIS call; the flag is cleared with the call, the
-                                   context stays usable and the next call starts clean        */
+                                   context stays usable and the next call starts clean.  A
+                                   batch of device pointers only enqueues work: its fault is
+                                   returned by the context's next batch of host pointers      */
 
 /* ---- status bits of one simulated plan ------------------------------------------------- */
 #define SAILOR_ST_INVALID          1u   /* gbs % (D*mbs) != 0, tp > gpus_per_node, heads % tp != 0 (H1) */

@@ -204,9 +204,10 @@ struct HostBlock {
     PlanOut out;                           // results of a search
     SurveyOut survey;                      // what the survey of a space found
     uint16_t avail[R_MAX];                 // the availability snapshot last set
+    unsigned int sim_error;                // error word of the explicit-batch kernels: read and cleared by the next host-side batch
     MixedOut mixed;                        // results of a search over plans with mixed replicas
     DpOut dp;                              // results of a search over per-stage GPU types
-    alignas(256) unsigned char batch[HOST_SMALL_BYTES];     // a small host batch: error word, results, records
+    alignas(256) unsigned char batch[HOST_SMALL_BYTES];     // a small host batch: records, results
 };
 
 constexpr size_t CFG_CACHE_MAX_BYTES = 512ull << 20;
@@ -231,7 +232,8 @@ struct sailor_ctx {
     bool avail_dirty = false;              // d_avail is older than h_avail
     PlanOut* d_out_mapped = nullptr;       // device address of h_out (mapped pinned memory)
     Ctrl* d_ctrl = nullptr;
-    unsigned int* d_sim_error = nullptr;   // error word of the explicit-batch kernels, then the "deep plans seen" word
+    unsigned int* d_sim_error = nullptr;   // device address of host->sim_error
+    unsigned int* d_deep_seen = nullptr;   // mixed batches: "deep plans seen"
     PlanOut* h_out = nullptr;              // &host->out
     bool ctrl_dirty = true;                // the counters must be cleared from the host (first call, or after a failed one)
     uint64_t ticket = 0;                   // calls that ended with one (wait_ticket)
@@ -791,21 +793,15 @@ int enqueue_pass(sailor_ctx* ctx, uint32_t obj, double budget, bool budget_from_
     return SAILOR_OK;
 }
 
-// End of a host-side batch call: read the batch kernels' error word with the results, wait, and report (and
-// clear) a fault.  Device-side batch calls only enqueue work; a fault in one of them is reported here as well,
-// by the next host-side call.
-int host_batch_error(unsigned int err) {
-    return err == 0 ? SAILOR_OK : (err & SIM_ERR_DEVICE) ? SAILOR_E_DEVICE : SAILOR_E_RANGE;
-}
-
+// End of a host-side batch call: wait, and report (and clear) what the batch kernels left in their error word.  The word
+// is pinned host memory that they write on a fault only, so looking at it costs nothing.  Device-side batch calls only
+// enqueue work; a fault in one of them is reported here as well, by the next host-side call of whatever size.
 int finish_host_batch(sailor_ctx* ctx) {
-    unsigned int* h_err = &ctx->h_out->ctrl.error;               // pinned; no search is in flight on this context
-    CU(ctx, cudaMemcpyAsync(h_err, ctx->d_sim_error, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
     CU(ctx, stream_sync(ctx));
-    if (*h_err) {
-        CU(ctx, cudaMemsetAsync(ctx->d_sim_error, 0, sizeof(unsigned int), ctx->stream));
-    }
-    return host_batch_error(*h_err);
+    volatile unsigned int* word = &ctx->host->sim_error;
+    const unsigned int err = *word;
+    *word = 0;
+    return err == 0 ? SAILOR_OK : (err & SIM_ERR_DEVICE) ? SAILOR_E_DEVICE : SAILOR_E_RANGE;
 }
 
 // A host-side batch: records of `rec_bytes` in, four result arrays out (any may be NULL).  The batch goes through
@@ -821,7 +817,7 @@ constexpr uint32_t HOST_SLOTS = 3;
 int upload_availability(sailor_ctx* ctx);
 
 // A host batch of up to HOST_SMALL_BYTES: its records go through the context's pinned block in one copy, the kernel writes
-// results and error word straight back into that block.  1 000 records: 96 us with pageable copies each way (four of results,
+// the results straight back into that block.  1 000 records: 96 us with pageable copies each way (four of results,
 // one of the error word), 61 with one copy back, 54 this way; a tenth of that is the host's own copying, which larger batches
 // would pay instead of the driver's.
 template <class Launch>
@@ -830,27 +826,22 @@ int host_batch_small(sailor_ctx* ctx, const unsigned char* recs, size_t rec_byte
     int rc = device_grow(ctx, &ctx->d_stage, &ctx->stage_bytes, HOST_SMALL_BYTES);
     if (rc == SAILOR_OK) rc = upload_availability(ctx);
     if (rc != SAILOR_OK) return rc;
-    unsigned char* const h_recs = ctx->host->batch;            // records, error word, t_iter, cost, peak_mem, status
+    unsigned char* const h_recs = ctx->host->batch;            // records, t_iter, cost, peak_mem, status
     unsigned char* const h_out = h_recs + (n * rec_bytes + 15) / 16 * 16;
-    unsigned char* out = nullptr;
-    CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&out), h_out, 0));
+    double* t = nullptr;
+    CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&t), h_out, 0));
     memcpy(h_recs, recs, n * rec_bytes);
-    memset(h_out, 0, 16);
     CU(ctx, cudaMemcpyAsync(ctx->d_stage, h_recs, n * rec_bytes, cudaMemcpyHostToDevice, ctx->stream));
-    double* t = reinterpret_cast<double*>(out + 16);
     rc = launch(ctx->d_stage, n, t_iter ? t : nullptr, peak_mem ? reinterpret_cast<uint64_t*>(t + 2 * n) : nullptr,
-                cost ? t + n : nullptr, status ? reinterpret_cast<uint32_t*>(t + 3 * n) : nullptr, reinterpret_cast<unsigned int*>(out));
-    const cudaError_t ce = stream_sync(ctx);                   // the pinned block is free again, whatever happened
+                cost ? t + n : nullptr, status ? reinterpret_cast<uint32_t*>(t + 3 * n) : nullptr, ctx->d_sim_error);
+    const int rc_end = finish_host_batch(ctx);                 // the pinned block is free again, whatever happened
     if (rc != SAILOR_OK) return rc;
-    if (ce != cudaSuccess) { ctx->last_cuda = (int)ce; return SAILOR_E_CUDA; }
-    const unsigned char* r = h_out + 16;
-    if (t_iter) memcpy(t_iter, r, 8 * n);
-    if (cost) memcpy(cost, r + 8 * n, 8 * n);
-    if (peak_mem) memcpy(peak_mem, r + 16 * n, 8 * n);
-    if (status) memcpy(status, r + 24 * n, 4 * n);
-    unsigned int err;
-    memcpy(&err, h_out, sizeof(err));
-    return host_batch_error(err);
+    if (rc_end == SAILOR_E_CUDA) return rc_end;
+    if (t_iter) memcpy(t_iter, h_out, 8 * n);
+    if (cost) memcpy(cost, h_out + 8 * n, 8 * n);
+    if (peak_mem) memcpy(peak_mem, h_out + 16 * n, 8 * n);
+    if (status) memcpy(status, h_out + 24 * n, 4 * n);
+    return rc_end;
 }
 
 // A second stream of the context and the events around it, made when a call first needs them.
@@ -1096,11 +1087,12 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
     ctx->h_avail = ctx->host->avail;
     ctx->h_out = &ctx->host->out;
     CUF(cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->d_out_mapped), ctx->h_out, 0));
+    CUF(cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->d_sim_error), &ctx->host->sim_error, 0));
     auto carve_ctx = [&](unsigned char* base) {              // returns (bytes that start from zero, all bytes)
         Bump bump{base};
         ctx->d_avail = bump.take<uint16_t>(R_MAX);
         ctx->d_ctrl = bump.take<Ctrl>(1);
-        ctx->d_sim_error = bump.take<unsigned int>(2);
+        ctx->d_deep_seen = bump.take<unsigned int>(1);
         const size_t zeroed = bump.at;
         ctx->d_blob = bump.take<unsigned char>(h.total_bytes);
         ctx->d_partial = bump.take<Hit>((size_t)SAILOR_K_MAX * ctx->max_grid);
@@ -1225,7 +1217,7 @@ int sailor_simulate_mixed_strided(sailor_ctx* ctx, const void* plans_v, uint64_t
                                                   uint32_t* d_s, unsigned int* error, uint32_t report_bad) {
         // a warp per plan; blocks take several plans per warp in larger batches
         const uint64_t blocks = (m + MIX_WARPS<false> - 1) / MIX_WARPS<false>, cap = (uint64_t)ctx->sm_count * 32;
-        unsigned int* deep_seen = ctx->d_sim_error + 1;
+        unsigned int* deep_seen = ctx->d_deep_seen;
         if (max_stages > 32) CU(ctx, cudaMemsetAsync(deep_seen, 0, sizeof(unsigned int), ctx->stream));
         simulate_mixed_kernel<false><<<(uint32_t)std::min(blocks, cap), 32 * MIX_WARPS<false>, mixed_smem<false>(ctx->hdr), ctx->stream>>>(
             ctx->d_blob, ctx->d_avail, d_plans, record_bytes, max_stages, m, d_t, d_m, d_c, d_s, error, deep_seen, report_bad);
@@ -2406,6 +2398,14 @@ extern "C" int sailor_plan_mixed(sailor_ctx* ctx, const sailor_mixed_space* s, c
     try {
         return plan_mixed_impl(ctx, s, o, k, topk, n_found, stats);
     } catch (const std::bad_alloc&) { return SAILOR_E_NOMEM; } catch (...) { return SAILOR_E_ARG; }
+}
+
+// What a device-side batch leaves behind when a bounded wait in it ran out.  No input makes one run out, so tests of how
+// the fault is reported put it there from the host; not part of the interface.
+extern "C" int sailor_internal_post_batch_fault(sailor_ctx* ctx) {
+    if (!ctx) return SAILOR_E_ARG;
+    *const_cast<volatile unsigned int*>(&ctx->host->sim_error) = SIM_ERR_DEVICE;
+    return SAILOR_OK;
 }
 
 // ---- sustained issue rates (measurement) ---------------------------------------------------------------

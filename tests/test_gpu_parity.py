@@ -792,3 +792,24 @@ def test_result_records_side_by_side(k, make_ctx):
         t, m, c, s = B.sailor_simulate(ctx, recs)
         assert [(r.t_iter, r.cost, r.peak_mem, r.status) for r in res] == list(zip(t.tolist(), c.tolist(), m.tolist(), s.tolist()))
         assert [bytes(B.sailor_decode(ctx, B.make_space(w), r.flat)) for r in res] == [bytes(r.plan) for r in res]
+
+
+@pytest.mark.parametrize("n", [1, 700, 5000])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_fault_of_a_device_batch_is_reported_by_the_next_host_batch(mixed, n, make_ctx):
+    """A batch of device pointers only enqueues work, so what went wrong in it is returned by the next batch of host
+    pointers, small (results through pinned memory) or large, exactly once.  The fault is put there from the host."""
+    w = W.tiny(seed=6, n_types=2, n_zones=2)
+    ctx = make_ctx(w).ctx
+    if mixed:
+        plans = W.random_mixed_plans(w, n, seed=8)
+        run, want = lambda: B.sailor_simulate_mixed(ctx, B.pack_mixed_plans(plans)), Oracle(w).simulate_mixed_batch(plans)
+    else:
+        plans = W.random_plans(w, n, seed=8)
+        run, want = lambda: B.sailor_simulate(ctx, B.pack_records(plans)), Oracle(w).simulate_records(plans)
+    assert_sim_equal(run(), want)
+    assert B.load().sailor_internal_post_batch_fault(ctx) == B.OK
+    with pytest.raises(B.SailorError) as e:
+        run()
+    assert e.value.code == B.E_DEVICE
+    assert_sim_equal(run(), want)                            # reported once; the context stays usable
