@@ -615,15 +615,16 @@ int prepare_space(sailor_ctx* ctx, const sailor_space* s) {
     return SAILOR_OK;
 }
 
-// Configuration that contains flat index f (f < n_total).
-uint32_t config_at(const sailor_ctx* ctx, uint64_t f) {
+// Chunk that contains flat index f (f < n_total) of a configuration whose items are taken in flat order.
+uint32_t chunk_of(const sailor_ctx* ctx, uint64_t f) {
     const SpaceCache& sc = ctx->space;
     uint32_t lo = 0, hi = sc.n_config;
     while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) / 2;
         if (sc.flat_base[mid] <= f) lo = mid; else hi = mid;
     }
-    return lo;
+    const uint64_t item = (f - sc.flat_base[lo]) / ctx->hdr.R;
+    return sc.chunk_start[lo] + (uint32_t)(item / PLAN_THREADS);
 }
 
 constexpr int PLAN_VARIANTS = 30;      // (objective x constraint x fused, then the three screened kernels) x every candidate or not
@@ -713,9 +714,9 @@ int enqueue_pass(sailor_ctx* ctx, uint32_t obj, double budget, bool budget_from_
         pp.live_mode = 1;
         pp.chunk_lo = 0;
         pp.chunk_hi = sc.live_chunks;
-    } else if (hi > lo) {                 // a range: whole configurations, whose items are not in flat order (run_items)
-        pp.chunk_lo = sc.chunk_start[config_at(ctx, lo)];
-        pp.chunk_hi = sc.chunk_start[config_at(ctx, hi - 1) + 1];
+    } else if (hi > lo) {                 // a configuration that a range holds a part of is taken in flat order (run_items)
+        pp.chunk_lo = chunk_of(ctx, lo);
+        pp.chunk_hi = chunk_of(ctx, hi - 1) + 1;
     }
     if (pp.chunk_hi > pp.chunk_lo) {
         const uint32_t n_chunks = waves ? sc.live_chunks : pp.chunk_hi - pp.chunk_lo;

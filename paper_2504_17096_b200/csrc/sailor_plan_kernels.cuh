@@ -942,28 +942,37 @@ __device__ __forceinline__ void run_items(const PlanParams& pp, const CfgShared&
     constexpr uint32_t last = NSEG - 1;
     // ---- prefix: segments 0 .. NSEG-2 --------------------------------------------------------
     // EVAL: the digit of the prefix's last segment varies slowest over the items of a configuration, so that the lanes of
-    // a warp nearly always send to the last segment from one zone (evaluate_only relies on it).  Otherwise it varies
-    // fastest: the lanes' prefixes then share their first digits, and with them most of what makes a prefix fail.
-    constexpr int SLOWEST = EVAL && NSEG > 1 ? NSEG - 2 : 0, FASTEST = EVAL ? NSEG - 3 : NSEG - 2;
+    // a warp nearly always send to the last segment from one zone (evaluate_only relies on it).  Otherwise, and in a
+    // configuration that the range holds only a part of (its other chunks are not launched), the items are in flat order
+    // and it varies fastest: the lanes' prefixes then share their first digits, and with them most of what makes a prefix fail.
     uint32_t dg[NSEG > 1 ? NSEG - 1 : 1];
     {
         uint32_t x = active ? q : 0;
-        auto peel = [&](int s, bool rest) {                // mixed radix, over the usable digits of each segment when packed
-            if (cs.packed) {
-                const uint32_t n = cs.g_cnt[s];
-                const uint32_t y = rest ? 0u : n > 1 ? __umulhi(x, cs.g_magic[s]) : x;   // x / n
-                dg[s] = active ? cs.good_list[s][x - y * n] : 0u;
-                x = y;
-            } else {
-                const uint32_t y = rest ? 0u : R == 1 ? x : __umulhi(x, cs.magic);     // x / R
-                dg[s] = x - y * R;
-                x = y;
-            }
+        auto by_radix = [&]() {                            // the next digit over all digits
+            const uint32_t y = R == 1 ? x : __umulhi(x, cs.magic), digit = x - y * R;      // x / R
+            x = y;
+            return digit;
         };
-        if (NSEG > 1) {
+        if constexpr (EVAL && NSEG > 1) {                  // (every candidate is wanted: never packed)
+            uint32_t o[NSEG - 1];
 #pragma unroll
-            for (int s = FASTEST; s >= (EVAL ? 0 : 1); --s) peel(s, false);
-            peel(SLOWEST, true);
+            for (int j = 0; j < NSEG - 2; ++j) o[j] = by_radix();
+            o[NSEG - 2] = x;
+            const bool whole = cs.whole;
+#pragma unroll
+            for (int s = 0; s < NSEG - 1; ++s) dg[s] = whole ? o[s == NSEG - 2 ? s : NSEG - 3 - s] : o[NSEG - 2 - s];
+        } else if (NSEG > 1) {
+#pragma unroll
+            for (int s = NSEG - 2; s >= 0; --s) {
+                if (cs.packed) {                           // mixed radix, over the usable digits of each segment
+                    const uint32_t n = cs.g_cnt[s];
+                    const uint32_t y = s == 0 ? 0u : n > 1 ? __umulhi(x, cs.g_magic[s]) : x;   // x / n
+                    dg[s] = active ? cs.good_list[s][x - y * n] : 0u;
+                    x = y;
+                } else {
+                    dg[s] = s == 0 ? x : by_radix();
+                }
+            }
         }
     }
     uint64_t item_flat = cs.flat_base;                     // the item's flat index follows from its digits

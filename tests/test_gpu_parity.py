@@ -813,3 +813,27 @@ def test_fault_of_a_device_batch_is_reported_by_the_next_host_batch(mixed, n, ma
         run()
     assert e.value.code == B.E_DEVICE
     assert_sim_equal(run(), want)                            # reported once; the context stays usable
+
+
+@pytest.mark.parametrize("flags", [0, B.FLAG_EVAL_ALL, B.FLAG_EVAL_ALL | B.FLAG_F32_SCREEN])
+def test_a_short_range_costs_its_own_candidates(flags, make_ctx):
+    """A range inside one configuration of 1.7e7 candidates (64 digits, four segments of 24 stages): a few candidates,
+    or a sixteenth of the configuration, must not take the time of the whole configuration.  Same results as the oracle."""
+    w = W.tiny(seed=31, n_types=8, n_zones=8, L=96, p_values=[96], d_values=(1,), tp_values=(1,), mbs_values=(1,), rc_values=(0,))
+    w.avail[...] = 200
+    w.capacity[:] = np.uint64(1 << 50)
+    cx, o = make_ctx(w), Oracle(w)
+    n = B.sailor_space_size(cx.ctx, cx.space)
+    assert n == 64 ** 4
+    obj = B.Objective(0, flags, 0.0, 0.0, 0.0)
+
+    def best_ms(lo, hi):
+        return min(B.sailor_plan_range(cx.ctx, cx.space, obj, lo, hi, 4)[1].kernel_ms for _ in range(20))
+
+    whole = best_ms(0, n)
+    assert best_ms(n // 2 + 77, n // 2 + 1077) < 0.5 * whole
+    assert best_ms(n // 2 + 77, n // 2 + 77 + n // 16) < 0.5 * whole
+    lo, hi = n // 2 + 77, n // 2 + 70_077
+    hits, counts = o.search(0, 4, lo=lo, hi=hi)
+    res, st = B.sailor_plan_range(cx.ctx, cx.space, obj, lo, hi, 4)
+    assert_plan_equal(res, st, hits, counts, o, f"flags={flags}")
