@@ -253,8 +253,7 @@ struct alignas(16) CfgShared {
     uint32_t lower_tpi[SAILOR_TP_MAX];    // their tp indices
     uint64_t lower_fit[SAILOR_TP_MAX][SAILOR_SEG_MAX];   // digit d: every stage of the segment fits at that degree
     uint64_t flat_base;          // flat index of the configuration's first candidate
-    uint32_t zone_alike;         // the last segment's records of a type are the same bits in every zone: bit 0 all but
-                                 // the price rate, bit 1 the price rate (what evaluate_zones may share between zones)
+    uint32_t by_zone;            // sweeps take the last segment's digits zone by zone (see zones_pay)
     uint32_t _pad_head;
     // ---- everything above depends on the configuration and the context only, not on availability: it is what a
     // ---- cached record holds (with the arrays rec .. fb_last); everything below belongs to the block or the snapshot
@@ -363,6 +362,19 @@ __device__ __forceinline__ uint32_t run_of(const TabHdr* h, uint32_t P, uint32_t
     return i < extra ? 1 : 2;                              // extra = n_blocks % P
 }
 
+// Zones that evaluate_only's first group takes besides the prefix's own.
+__device__ __forceinline__ uint32_t zone_group(uint32_t Z) { return Z > 7 ? 7u : 4u; }
+// Where a type's records are alike in all zones (price rate included), taking a sweep's last digits zone by zone pays if the
+// first group is full; the zones beyond it go one at a time, a chain of additions each, which pays for last segments of up
+// to five stages.  Sweeps of pipelines of one depth over 8 types, zone by zone against digit by digit, ms, last segments of
+// 1, 4, 5, 6, 12 and 24 stages: 5 zones 2.9 4.2, 3.3 5.1, 4.8 7.0, 5.1 6.8, 7.4 8.8, 12.3 12.4; 7 zones 11.6 14.7,
+// 17.8 18.1, 23.3 25.0, 25.7 24.3, 41.8 31.5, 74 45; 8 zones 14.7 24.2, 17.6 30.2, 23.3 41.9, 24.8 40.7, 35.8 52.7,
+// 57.8 75.5.  Up to 4 zones, one at a time, 1.5 times the digits' time; with a price rate per zone 1.1 (5 zones), 1.06 (8).
+__device__ __forceinline__ bool zones_pay(uint32_t Z, uint32_t stages) {
+    const uint32_t group = zone_group(Z);
+    return Z > group && (Z == group + 1 || stages <= 5);
+}
+
 // Build the tables of configuration `c`.  Called by the whole block; ends synchronised.
 static __device__ void build_config(const PlanParams& pp, const TabView& v, CfgShared& cs, CfgArrays& a, uint32_t c) {
     const TabHdr* h = v.h;
@@ -382,7 +394,7 @@ static __device__ void build_config(const PlanParams& pp, const TabView& v, CfgS
             cs.ar_coef = k.D > 0 ? cs.ar_steps / (double)k.D : 0.0;
             cs.n_items = ipow64(R, k.nseg - 1);
             cs.flat_base = pp.cfg_flat_base[c];
-            cs.zone_alike = 0;
+            cs.by_zone = 0;
             cs._pad_head = 0;
             cs.packed = 0;             // decided at the end of the build, and only for valid configurations
             cs.cur_config = c;
@@ -510,15 +522,14 @@ static __device__ void build_config(const PlanParams& pp, const TabView& v, CfgS
     __syncthreads();                   // the memory masks and the records are complete
     {
         const SegRec* recs = a.rec + (k.nseg - 1) * R;
-        bool time_alike = true, rate_alike = true;
+        bool alike = true;             // the last segment's records of a type are the same bits in every zone
         for (uint32_t d = tid; d < R; d += PLAN_THREADS) {
             const SegRec &x = recs[d], &y = recs[d % T];
-            for (int q = 0; q < N_RUNS; ++q) time_alike &= x.v[q] == y.v[q];
-            time_alike &= x.tmax == y.tmax && x.sync == y.sync && x.upd == y.upd;
-            rate_alike &= x.rate == y.rate;
+            for (int q = 0; q < N_RUNS; ++q) alike &= x.v[q] == y.v[q];
+            alike &= x.tmax == y.tmax && x.sync == y.sync && x.upd == y.upd && x.rate == y.rate;
         }
-        const int t_all = __syncthreads_and(time_alike), r_all = __syncthreads_and(rate_alike);
-        if (tid == 0) cs.zone_alike = (t_all ? 1u : 0u) | (r_all ? 2u : 0u);
+        const int all = __syncthreads_and(alike);
+        if (tid == 0) cs.by_zone = all && zones_pay(Z, cs.seg_a[k.nseg] - cs.seg_a[k.nseg - 1]) ? 1u : 0u;
     }
     if (tid < 32) {
         const uint32_t last = k.nseg - 1;
@@ -802,15 +813,15 @@ __device__ __forceinline__ void evaluated(uint32_t& signs, float t, float c) { s
 // The candidates of W zones that are not the prefix's own and (OWN) of the one that is.  A digit is a (zone, type) pair:
 // the message from the prefix, and with it the running sum, the maximum and the transfer cost up to the last segment,
 // depend on the zone alone unless it is the prefix's own, so these heads are formed once per zone and kept in registers;
-// where a type's record is alike in all zones (CfgShared::zone_alike) it is read once for all of them, and the maxima over
-// synchronisation and update times and (RATE) the price-rate sum are formed once.  n_b x max(a, b) is taken as
+// a type's record is alike in all zones here (CfgShared::by_zone): it is read once for all of them, and the maxima over
+// synchronisation and update times and the price-rate sum are formed once.  n_b x max(a, b) is taken as
 // max(n_b x a, n_b x b): rounding is monotone, so these are the same bits; a transfer cost of zero is not added.  Every
 // candidate still takes its own additions over the segment's stages, in stage order, and its own closing terms: the bits
 // are those of eval_candidates.  N2 >= 0: the segment is N2 plain stages and the final stage (straight code); -1: any.
 // Bound: issue slots (64 % busy) and the FP64 pipe (52 %): 6 + (stages of the segment) FP64 instructions a candidate
 // against 14 + 2 x (stages) digit by digit.  Workload 5, 6.4e9 candidates: 13.89 -> 7.30 ms, 55.9 -> 26.9
 // lane-instructions a candidate, about 7 of them what an item costs before its candidates (digits, masks, prefix sums).
-template <int N2, int W, bool RATE, bool OWN, typename F>
+template <int N2, int W, bool OWN, typename F>
 __device__ __forceinline__ void evaluate_zones(const CfgShared& cs, const ItemState<F>& it, uint32_t T, uint32_t Z, uint32_t R,
                                                uint32_t z_own, uint32_t first, F nb, uint32_t& signs) {
     constexpr uint32_t last = SAILOR_SEG_MAX - 1;
@@ -848,9 +859,8 @@ __device__ __forceinline__ void evaluate_zones(const CfgShared& cs, const ItemSt
                 for (int j = 0; j < N2; ++j) t_sum[w] = add_rn(t_sum[w], v2);
                 t_sum[w] = add_rn(t_sum[w], v3);
             }
-            if (RATE)
 #pragma unroll
-                for (int j = 0; j <= N2; ++j) r = add_rn(r, rc->rate);
+            for (int j = 0; j <= N2; ++j) r = add_rn(r, rc->rate);
         } else {
             const F v0 = n1 ? v1 : n2 ? v2 : v3;
 #pragma unroll
@@ -861,13 +871,12 @@ __device__ __forceinline__ void evaluate_zones(const CfgShared& cs, const ItemSt
 #pragma unroll
                 for (int w = 0; w < S; ++w) t_sum[w] = add_rn(t_sum[w], v);
             }
-            if (RATE) r = add_n(r, rc->rate, n);
+            r = add_n(r, rc->rate, n);
         }
         const F tm = mul_rn(nb, rc->tmax), sy = dmax(it.sy, rc->sync), up = dmax(it.up, rc->upd);
 #pragma unroll
         for (int w = 0; w < S; ++w) {
             const F t = add_rn(add_rn(add_rn(t_sum[w], dmax(hm[w], tm)), sy), up);
-            if (!RATE) r = add_n(it.rate, rc[dz[w]].rate, n);
             evaluated(signs, t, add_rn(mul_rn(r, t), hc[w]));
         }
     }
@@ -882,34 +891,23 @@ __device__ __forceinline__ uint32_t evaluate_only(const CfgShared& cs, const Ite
     const F nb = (F)cs.n_b;
     const uint32_t lanes = __ballot_sync(FULL, active);
     const uint32_t z_own = __shfl_sync(FULL, z_prev, lanes ? __ffs(lanes) - 1 : 0);
-    const bool by_zone = (cs.zone_alike & 1u) && __all_sync(FULL, !active || z_prev == z_own);
     uint32_t signs = 0;
-    if (!by_zone || Z == 1) {
-        constexpr uint32_t U = PLAN_DIGITS_PER_STEP;       // (the tables are padded)
-        for (uint32_t d = 0; d < R; d += U) {
-            F t[U], c[U];
-            eval_candidates<NSEG, -1, (int)U>(cs, it, Z, R, d, nb, t, c);
+    if (!cs.by_zone || __any_sync(FULL, active && z_prev != z_own)) {
+        by_shape<NSEG>(cs, [&](auto shape) {
+            constexpr uint32_t U = PLAN_DIGITS_PER_STEP;   // (the tables are padded)
+            for (uint32_t d = 0; d < R; d += U) {
+                F t[U], c[U];
+                eval_candidates<NSEG, decltype(shape)::value, (int)U>(cs, it, Z, R, d, nb, t, c);
 #pragma unroll
-            for (uint32_t u = 0; u < U; ++u) evaluated(signs, t[u], c[u]);
-        }
+                for (uint32_t u = 0; u < U; ++u) evaluated(signs, t[u], c[u]);
+            }
+        });
         return signs;
     }
-    // the first group takes the prefix's own zone along
-    const bool rate = (cs.zone_alike & 2u) != 0;
-    uint32_t j;
-    if (Z > 7) {
-        if (rate) by_shape<NSEG>(cs, [&](auto shape) { evaluate_zones<decltype(shape)::value, 7, true, true>(cs, it, T, Z, R, z_own, 0, nb, signs); });
-        else evaluate_zones<-1, 7, false, true>(cs, it, T, Z, R, z_own, 0, nb, signs);
-        j = 7;
-    } else if (Z > 4) {
-        if (rate) by_shape<NSEG>(cs, [&](auto shape) { evaluate_zones<decltype(shape)::value, 4, true, true>(cs, it, T, Z, R, z_own, 0, nb, signs); });
-        else evaluate_zones<-1, 4, false, true>(cs, it, T, Z, R, z_own, 0, nb, signs);
-        j = 4;
-    } else {
-        evaluate_zones<-1, 1, false, true>(cs, it, T, Z, R, z_own, 0, nb, signs);
-        j = 1;
-    }
-    for (; j + 1 < Z; ++j) evaluate_zones<-1, 1, false, false>(cs, it, T, Z, R, z_own, j, nb, signs);
+    const uint32_t group = zone_group(Z);                  // the first group takes the prefix's own zone along
+    if (group == 7) by_shape<NSEG>(cs, [&](auto shape) { evaluate_zones<decltype(shape)::value, 7, true>(cs, it, T, Z, R, z_own, 0, nb, signs); });
+    else by_shape<NSEG>(cs, [&](auto shape) { evaluate_zones<decltype(shape)::value, 4, true>(cs, it, T, Z, R, z_own, 0, nb, signs); });
+    for (uint32_t j = group; j + 1 < Z; ++j) evaluate_zones<-1, 1, false>(cs, it, T, Z, R, z_own, j, nb, signs);
     return signs;
 }
 

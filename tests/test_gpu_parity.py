@@ -837,3 +837,26 @@ def test_a_short_range_costs_its_own_candidates(flags, make_ctx):
     hits, counts = o.search(0, 4, lo=lo, hi=hi)
     res, st = B.sailor_plan_range(cx.ctx, cx.space, obj, lo, hi, 4)
     assert_plan_equal(res, st, hits, counts, o, f"flags={flags}")
+
+
+def test_sweeps_cost_no_more_where_zones_are_alike(make_ctx):
+    """A sweep may take zones that are alike together, and may evaluate in binary32 first: neither may cost more than the
+    plain way, which is what links that differ between zones (bandwidth polynomials) get."""
+    def sweep_ms(w, flags):
+        cx = make_ctx(w)
+        return min(B.sailor_plan(cx.ctx, cx.space, B.Objective(0, flags, 0.0, 0.0, 0.0), 8)[1].kernel_ms for _ in range(7))
+
+    def workload(n_zones):
+        w = W.tiny(seed=33, n_types=8, n_zones=n_zones, L=48, p_values=[8, 16, 48], d_values=(1, 2, 4, 8), tp_values=(1, 2),
+                   mbs_values=(1, 2), rc_values=(0, 1))
+        w.avail[...] = 1                                     # nothing is feasible: every item is evaluated only
+        return w
+
+    for n_zones in (3, 4, 7):
+        alike, differ = workload(n_zones), W.with_bandwidth_polynomials(workload(n_zones), seed=5)
+        zoned = workload(n_zones)
+        zoned.price_per_hour = zoned.price_per_hour * np.linspace(0.8, 1.2, n_zones)[:, None]
+        plain = sweep_ms(differ, B.FLAG_EVAL_ALL)
+        for w in (alike, zoned):
+            assert sweep_ms(w, B.FLAG_EVAL_ALL) < 1.08 * plain, n_zones
+        assert sweep_ms(differ, B.FLAG_EVAL_ALL | B.FLAG_F32_SCREEN) < 0.95 * plain, n_zones
