@@ -545,7 +545,7 @@ typedef struct sailor_dp_stats {
     uint64_t n_solved;                  /* problems that have a plan                                  */
     uint64_t n_over_constraint;         /* of which the plan is over the budget or under the throughput */
     uint64_t n_states;                  /* table entries filled (all problems, all stages)            */
-    uint64_t workspace_used;            /* bytes of the largest batch                                 */
+    uint64_t workspace_used;            /* bytes of the largest batch (tables and moves)              */
     float    kernel_ms;
     uint32_t n_launches, n_batches;
     uint32_t n_unfinished;              /* SAILOR_DP_FLAG_BUDGET_LOOP: problems given up (too many calls)   */
@@ -554,10 +554,13 @@ typedef struct sailor_dp_stats {
 /* Solve every problem of `s` x `orders` and return the k best plans within the constraint by
  * (value, problem index = config * n_orders + order) ascending; *n_found <= k.  `topk` is a HOST array of k records;
  * `stats` may be NULL.  Uses the availability last set.  `workspace_bytes` bounds the device memory
- * of the tables (0 = 8 GiB); it is allocated on first use and kept by the context (grow-only).
+ * of the tables of a batch (0 = 8 GiB); it is allocated on first use and kept by the context (grow-only).  A problem's
+ * own tables take at most 64 + P bytes per GPU type and count vector of at most P stages (within what every zone of the
+ * order can host), and a problem whose own tables fit is never refused: its table of moves, 16 or 32 bytes per count
+ * vector (up to four types, or more), may then come on top.
  * Errors: E_ARG (null, k == 0, n_orders == 0, a zone twice or out of range, an objective other
  * than plain MAX_THROUGHPUT, the budget loop without a budget), E_RANGE (k >
- * SAILOR_K_MAX, space limits as sailor_plan, a single problem whose tables exceed the workspace or
+ * SAILOR_K_MAX, space limits as sailor_plan, a single problem whose own tables exceed the workspace or
  * 2^31 entries per stage), E_NOMEM, E_CUDA. */
 int sailor_plan_dp(sailor_ctx* ctx, const sailor_space* s, const sailor_zone_order* orders, uint32_t n_orders,
                    const sailor_objective* o, uint64_t workspace_bytes, uint32_t k, sailor_dp_result* topk,

@@ -58,14 +58,17 @@ struct DpLayout {
     uint8_t first_later[SAILOR_Z_MAX][SAILOR_T_MAX];    // first position after zp that can host a stage of the type
 };
 static_assert(sizeof(DpLayout) % 4 == 0, "copied word by word");
-// A live row (one per stage): count of live vectors, count before this stage, then per position (first vector, slot of
-// that vector); a vector's slot is its place among the live vectors of the stage.
-__host__ __device__ inline uint32_t dp_live_words(uint32_t nz) { return 2 + 2 * nz; }
-constexpr uint32_t DP_LIVE_WORDS_MAX = 2 + 2 * SAILOR_Z_MAX;
+// A live row (one per stage): count of live vectors, count before this stage (two words), then per position (first vector,
+// slot of that vector); a vector's slot is its place among the live vectors of the stage.
+__host__ __device__ inline uint32_t dp_live_words(uint32_t nz) { return 3 + 2 * nz; }
+constexpr uint32_t DP_LIVE_WORDS_MAX = 3 + 2 * SAILOR_Z_MAX;
+__host__ __device__ inline uint64_t live_before(const uint32_t* row) { return (uint64_t)row[2] << 32 | row[1]; }
+__host__ __device__ inline uint32_t live_vec(const uint32_t* row, uint32_t zp) { return row[3 + 2 * zp]; }
+__host__ __device__ inline uint32_t live_slot(const uint32_t* row, uint32_t zp) { return row[4 + 2 * zp]; }
 
 struct DpJob {                       // a problem that has tables
     uint64_t val_off;                // first entry of its two level buffers
-    uint64_t succ_off;               // first word of its successors: [stage][slot][type]
+    uint64_t succ_off;               // first byte of its successors: [stage][slot][type]
     uint32_t config, index, layout, P;   // index = config * n_orders + order
 };
 
@@ -243,7 +246,7 @@ struct DpLevelParams {
     const uint32_t* nxt;
     const double* tabs;
     DpVal* val[2];                   // level buffers [slot][type]; stage i lives in val[(P - 1 - i) & 1]
-    uint32_t* succ;                  // [stage][slot][type]: slot * T + type of the best next state
+    uint8_t* succ;                   // [stage][slot][type]: type of the next stage in the best plan (DP_NONE: there is none)
     const uint32_t* blk_prefix;      // per-stage launches: [n_active + 1] blocks before each job of this launch
     DpTabLayout lay;
     uint32_t T, n_active;
@@ -278,8 +281,8 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
     const double* c2x = lp.tabs + (size_t)job.config * lp.lay.stride() + lp.lay.off_c2x();
     const double nb = st.nb;
     uint32_t zp = 0;
-    while (zp + 1 < L.nz && here[3 + 2 * (zp + 1)] <= slot) ++zp;
-    const uint32_t v = here[2 + 2 * zp] + (slot - here[3 + 2 * zp]);
+    while (zp + 1 < L.nz && live_slot(here, zp + 1) <= slot) ++zp;
+    const uint32_t v = live_vec(here, zp) + (slot - live_slot(here, zp));
     uint32_t nx[TM];                                         // (nothing so far depends on another stage)
     {
         const uint4* row = reinterpret_cast<const uint4*>(lp.nxt + (size_t)(L.nxt_off + v) * TM);
@@ -312,7 +315,7 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
                 if (zp2 == DP_NONE) continue;
                 id = L.first_vec[zp2][g2];
             }
-            const uint32_t slot2 = then[3 + 2 * zp2] + (id - then[2 + 2 * zp2]);
+            const uint32_t slot2 = live_slot(then, zp2) + (id - live_vec(then, zp2));
             if (slot2 >= then[0]) continue;                  // (a move of a live state leads to a live state)
             code[g2] = slot2 * T + g2;
             d2[g2] = L.zone[zp2] * T + g2;
@@ -321,7 +324,10 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
     }
     const uint32_t ok_here = st.ok;
     DpVal* cur = lp.val[dist & 1] + job.val_off + (size_t)slot * T;
-    uint32_t* succ = lp.succ + job.succ_off + (size_t)(here[1] + slot) * T;
+    uint8_t* succ = lp.succ + job.succ_off + (live_before(here) + slot) * T;
+    uint32_t picks[TM / 4];                                  // a byte per type, written together where T allows it
+#pragma unroll
+    for (uint32_t q = 0; q < TM / 4; ++q) picks[q] = 0xffffffffu;
 #pragma unroll
     for (uint32_t g = 0; g < TM; ++g) {
         if (g >= T) break;
@@ -330,7 +336,7 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
         const uint32_t d = L.zone[zp] * T + g;
         const double fb = st.fb[g], upd = st.upd[g], sync = st.sync[d];
         DpVal best;
-        uint32_t pick = DP_NO_STATE;
+        uint32_t pick = DP_NONE;
         if (dist == 0) {                                     // the last stage sends nothing
             best.sum = fb; best.mx = fb; best.sy = sync; best.up = upd;
         } else {
@@ -346,11 +352,19 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
                 c.sy = dmax(sync, n[g2].sy);
                 c.up = dmax(upd, n[g2].up);
                 const double val = add_rn(add_rn(add_rn(c.sum, mul_rn(nb, c.mx)), c.sy), c.up);
-                if (pick == DP_NO_STATE || val < best_v) { best = c; best_v = val; pick = code[g2]; }
+                if (pick == DP_NONE || val < best_v) { best = c; best_v = val; pick = g2; }
             }
         }
         cur[g] = best;
-        succ[g] = pick;
+        picks[g / 4] = (picks[g / 4] & ~(0xffu << (8 * (g % 4)))) | pick << (8 * (g % 4));
+    }
+    if (T == TM) {                                           // (every problem's successors start on a 64-byte line)
+        if (TM == 4) *reinterpret_cast<uint32_t*>(succ) = picks[0];
+        else *reinterpret_cast<uint2*>(succ) = make_uint2(picks[0], picks[TM / 4 - 1]);
+    } else {
+#pragma unroll
+        for (uint32_t g = 0; g < TM; ++g)
+            if (g < T) succ[g] = (uint8_t)(picks[g / 4] >> (8 * (g % 4)));
     }
 }
 
@@ -501,16 +515,16 @@ __device__ __forceinline__ SimOut simulate_stages(const TabView& v, const uint16
 
 // What a warp of the kernels that end a search keeps in shared memory.
 struct DpFinishWarp {
-    uint32_t code[SAILOR_P_MAX];     // state of every stage
-    uint16_t gz[SAILOR_P_MAX];       // its type | zone << 8
+    uint16_t gz[SAILOR_P_MAX];       // type | zone << 8 of every stage
     uint32_t cnt[R_MAX];
     uint8_t used[SAILOR_T_MAX];
 };
 constexpr int DP_FINISH_WARPS = 4, DP_FINISH_THREADS = 32 * DP_FINISH_WARPS;
 
-// Stage 0 and the walk through the kept successors, a warp per job.  The walk is a chain of one dependent load per stage (a
-// successor is the next state's own address) and what the kernel's time is; types, zones and the simulation are the lanes'.
-// 520 jobs of up to 48 stages: 107 us by a thread each, 33 this way.
+// Stage 0 and the walk through the kept successors, a warp per job.  The walk is a chain of one round of loads per stage (the
+// successor's type, and next to it the moves of the state's vector for every type it can be) and what the kernel's time is;
+// the simulation is the lanes'.  520 jobs of up to 48 stages: 107 us by a thread each, 43 this way (34 where a successor is
+// the next state's four-byte number, which costs the levels more than that: 1 525 us against 1 489, and memory).
 struct DpFinishParams {
     const unsigned char* blob;
     const uint16_t* avail;
@@ -520,73 +534,86 @@ struct DpFinishParams {
     const uint32_t* live;
     const double* tabs;
     const DpVal* val[2];
-    const uint32_t* succ;
+    const uint8_t* succ;
+    const uint32_t* nxt;             // [vector][TM]
     double* value;                   // indexed by problem index
     DpResult* results;               // indexed by problem index
     DpTabLayout lay;
-    uint32_t n_jobs, T;
+    uint32_t n_jobs, T, TM;
 };
 
 __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_finish_kernel(const __grid_constant__ DpFinishParams fp) {
     __shared__ DpFinishWarp warps[DP_FINISH_WARPS];
+    __shared__ uint32_t s_rows[DP_FINISH_WARPS][33 * DP_LIVE_WORDS_MAX];    // live rows of 32 stages and the one after them
     const uint32_t lane = threadIdx.x & 31, x = blockIdx.x * DP_FINISH_WARPS + (threadIdx.x >> 5);
     if (x >= fp.n_jobs) return;
     DpFinishWarp& w = warps[threadIdx.x >> 5];
+    uint32_t* rows = s_rows[threadIdx.x >> 5];
     const DpJob job = fp.jobs[x];
     const DpLayout& L = fp.layouts[job.layout];
     DpResult& out = fp.results[job.index];
-    const uint32_t T = fp.T, P = job.P, nz = L.nz, words = dp_live_words(nz);
+    const uint32_t T = fp.T, P = job.P, words = dp_live_words(L.nz);
     const uint32_t* live = fp.live + L.live_off;
     const double* tab = fp.tabs + (size_t)job.config * fp.lay.stride();
     const uint32_t* okv = reinterpret_cast<const uint32_t*>(tab + fp.lay.off_ok());
     const double nb = (double)*reinterpret_cast<const uint64_t*>(tab + fp.lay.off_nb());
     const DpVal* lvl0 = fp.val[(P - 1) & 1] + job.val_off;
     double mine_v = make_inf();
-    uint32_t mine = DP_NO_STATE;
+    uint32_t mine = DP_NO_STATE, mine_p = 0;
     if (lane < T && ((okv[0] >> lane) & 1u)) {               // stage 0 by first fit from the first zone of the order, a lane per type
         const uint32_t p = L.cap[0][lane] >= 1 ? 0u : L.first_later[0][lane];
         if (p != DP_NONE) {
-            const uint32_t slot = live[3 + 2 * p] + (L.first_vec[p][lane] - live[2 + 2 * p]);
+            const uint32_t slot = live_slot(live, p) + (L.first_vec[p][lane] - live_vec(live, p));
             if (slot < live[0]) {
                 const DpVal v = lvl0[slot * T + lane];
                 if (v.sum < make_inf()) {
                     mine_v = add_rn(add_rn(add_rn(v.sum, mul_rn(nb, v.mx)), v.sy), v.up);
-                    mine = slot * T + lane;
+                    mine = slot;
+                    mine_p = p;
                 }
             }
         }
     }
     double best_v = make_inf();
-    uint32_t code = DP_NO_STATE;
+    uint32_t slot = DP_NO_STATE, g = 0;                      // the state of the stage that the walk is at: slot, type, position
     for (uint32_t g0 = 0; g0 < T; ++g0) {                    // the first of the best
         const double val = __shfl_sync(FULL, mine_v, g0);
         const uint32_t c = __shfl_sync(FULL, mine, g0);
-        if (c != DP_NO_STATE && (code == DP_NO_STATE || val < best_v)) { best_v = val; code = c; }
+        if (c != DP_NO_STATE && (slot == DP_NO_STATE || val < best_v)) { best_v = val; slot = c; g = g0; }
     }
-    if (code == DP_NO_STATE) return;                         // the value stays at "no plan"
+    if (slot == DP_NO_STATE) return;                         // the value stays at "no plan"
     if (lane == 0) fp.value[job.index] = best_v;
+    uint32_t zp = __shfl_sync(FULL, mine_p, g);
     const Config k = config_of(fp.sp, job.config);
-    const uint32_t* succ = fp.succ + job.succ_off;
+    const uint8_t* succ = fp.succ + job.succ_off;
+    const uint32_t* nxt = fp.nxt + (size_t)L.nxt_off * fp.TM;
     for (uint32_t at = 0; at < P; at += 32) {
-        const uint32_t first = at + lane < P ? live[(size_t)(at + lane) * words + 1] : 0u;     // states before the stage's
         const uint32_t n = P - at < 32 ? P - at : 32;
+        __syncwarp();
+        for (uint32_t y = lane; y < (n + (at + n < P ? 1u : 0u)) * words; y += 32) rows[y] = live[(size_t)at * words + y];
+        __syncwarp();
         for (uint32_t l = 0; l < n; ++l) {
-            if (lane == 0) w.code[at + l] = code;
-            if (at + l + 1 < P) code = succ[(size_t)__shfl_sync(FULL, first, l) * T + code];
+            const uint32_t *here = rows + l * words, *then = here + words;
+            if (lane == 0) w.gz[at + l] = (uint16_t)(g | L.zone[zp] << 8);
+            if (at + l + 1 == P) break;
+            const uint32_t v = live_vec(here, zp) + (slot - live_slot(here, zp));
+            uint32_t got = 0;
+            if (lane < fp.TM) got = nxt[(size_t)v * fp.TM + lane];
+            else if (lane == 31) got = succ[(live_before(here) + slot) * T + g];
+            g = __shfl_sync(FULL, got, 31);
+            uint32_t id = __shfl_sync(FULL, got, g) & DP_NO_VEC;
+            if (id == DP_NO_VEC) {                           // no room left in this position: the next that has
+                zp = L.first_later[zp][g];
+                id = L.first_vec[zp][g];
+            }
+            slot = live_slot(then, zp) + (id - live_vec(then, zp));
         }
     }
     __syncwarp();
     for (uint32_t i = lane; i < P; i += 32) {
-        const uint32_t* row = live + (size_t)i * words;
-        const uint32_t slot = w.code[i] / T, g = w.code[i] - slot * T;
-        uint32_t zp = 0;
-        while (zp + 1 < nz && row[3 + 2 * (zp + 1)] <= slot) ++zp;
-        const uint8_t z = L.zone[zp];
-        out.type[i] = (uint8_t)g;
-        out.zone[i] = z;
-        w.gz[i] = (uint16_t)(g | z << 8);
+        out.type[i] = (uint8_t)(w.gz[i] & 0xffu);
+        out.zone[i] = (uint8_t)(w.gz[i] >> 8);
     }
-    __syncwarp();
     // the plan written out, through the simulator (Sec. 4.3): what a caller compares with a constraint
     TabView v;
     v.bind(fp.blob, fp.blob);

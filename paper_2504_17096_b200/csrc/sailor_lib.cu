@@ -1583,7 +1583,7 @@ struct LayoutInfo {
     DpLayout l;
     std::vector<uint32_t> w;           // rank tables, position after position
     std::vector<uint32_t> live;        // [P][dp_live_words(nz)]
-    uint64_t total_live = 0;           // live vectors of all stages
+    uint64_t total_live = 0;           // live vectors of all stages (a byte of successors per type each)
     uint32_t max_live = 0;
     int batch = -1;                    // the last batch it was put into, and its place there
     uint32_t place = 0;
@@ -1662,6 +1662,7 @@ int build_layout(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_
     for (uint32_t i = 0; i < P; ++i) {
         uint32_t* row = &info.live[(size_t)i * words];
         row[1] = (uint32_t)info.total_live;
+        row[2] = (uint32_t)(info.total_live >> 32);
         uint64_t slots = 0;
         for (uint32_t zp = 0; zp < l.nz; ++zp) {
             const uint32_t* W0 = &info.w[l.w_off[zp]];
@@ -1675,13 +1676,13 @@ int build_layout(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_
                     count = W0[top] - first;
                 }
             }
-            row[2 + 2 * zp] = (uint32_t)(l.vec_base[zp] + first);
-            row[3 + 2 * zp] = (uint32_t)slots;
+            row[3 + 2 * zp] = (uint32_t)(l.vec_base[zp] + first);
+            row[4 + 2 * zp] = (uint32_t)slots;
             slots += count;
         }
         row[0] = (uint32_t)slots;
         info.total_live += slots;
-        if (slots == 0 || (slots + 1) * ctx->hdr.T >= 0xffffffffull || info.total_live >= 0xffffffffull) {
+        if (slots == 0 || (slots + 1) * ctx->hdr.T >= 0xffffffffull) {
             const bool none = slots == 0;
             info.max_live = 0;
             return none ? SAILOR_OK : SAILOR_E_RANGE;
@@ -1926,16 +1927,16 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
     std::vector<Problem> todo;
     for (uint32_t P = SAILOR_P_MAX; P > 0; --P) todo.insert(todo.end(), by_depth[P].begin(), by_depth[P].end());
 
-    // cut into batches that fit the workspace: per problem two level buffers and its successors (padded to 256 bytes
-    // each), per layout its moves
+    // cut into batches that fit the workspace: per problem two level buffers and its successors, per layout its moves.  What
+    // bounds a problem alone is its own tables, (64 + stages) bytes a state at most; its moves may then come on top.
     const uint32_t TM = T <= 4 ? 4 : SAILOR_T_MAX;
     struct Batch {
         size_t first, count;
-        uint64_t val_entries, succ_words, nxt_rows;
+        uint64_t val_entries, succ_bytes, nxt_rows;
         std::vector<std::pair<uint32_t, uint32_t>> layouts;  // layout, its first row of moves in this batch
     };
     std::vector<Batch> batches;
-    uint64_t largest = 0, max_val = 0, max_succ = 0, max_rows = 0;
+    size_t largest = 0;
     auto pad8 = [](uint64_t x) { return (x + 7) / 8 * 8; };
     auto pad64 = [](uint64_t x) { return (x + 63) / 64 * 64; };
     for (size_t j = 0; j < todo.size();) {
@@ -1945,11 +1946,9 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
             LayoutInfo& info = layouts[todo[j].layout];
             const uint64_t val = pad8((uint64_t)info.max_live * T), succ = pad64(info.total_live * T);
             const uint64_t rows = info.batch == (int)batches.size() ? 0 : info.l.vec_base[info.l.nz];
-            const uint64_t more = val * 2 * sizeof(DpVal) + succ * 4 + rows * TM * 4;
-            if (bytes + more > workspace_bytes || b.nxt_rows + rows >= (1ull << 32)) {
-                if (b.count == 0) return SAILOR_E_RANGE;     // one problem alone does not fit
-                break;
-            }
+            const uint64_t tables = val * 2 * sizeof(DpVal) + succ, moves = rows * TM * 4;
+            if (b.count && (bytes + tables + moves > workspace_bytes || b.nxt_rows + rows >= (1ull << 32))) break;
+            if (tables > workspace_bytes) return SAILOR_E_RANGE;     // one problem alone does not fit
             if (rows) {
                 info.batch = (int)batches.size();
                 info.place = (uint32_t)b.layouts.size();
@@ -1957,15 +1956,12 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
                 b.nxt_rows += rows;
             }
             todo[j].place = info.place;
-            bytes += more;
+            bytes += tables + moves;
             b.val_entries += val;
-            b.succ_words += succ;
+            b.succ_bytes += succ;
             ++b.count;
         }
-        largest = std::max(largest, bytes);
-        max_val = std::max(max_val, b.val_entries);
-        max_succ = std::max(max_succ, b.succ_words);
-        max_rows = std::max(max_rows, b.nxt_rows);
+        largest = std::max(largest, 2 * padded(b.val_entries * sizeof(DpVal)) + padded(b.succ_bytes) + padded(b.nxt_rows * TM * 4));
         batches.push_back(std::move(b));
     }
 
@@ -1979,8 +1975,7 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
     const size_t tab_bytes = (size_t)n_config * lay.stride() * sizeof(double);
     DpOut* d_out = nullptr;
     CU(ctx, cudaHostGetDevicePointer(reinterpret_cast<void**>(&d_out), &ctx->host->dp, 0));
-    const size_t total = padded(tab_bytes) + padded(n_problems * sizeof(DpResult)) + padded(n_problems * sizeof(double)) +
-                         padded(max_rows * TM * 4) + 2 * padded(max_val * sizeof(DpVal)) + padded(max_succ * 4);
+    const size_t total = padded(tab_bytes) + padded(n_problems * sizeof(DpResult)) + padded(n_problems * sizeof(double)) + largest;
     {
         const int rc_mem = device_grow(ctx, &ctx->d_dp, &ctx->dp_bytes, total);
         if (rc_mem) return rc_mem;
@@ -1991,11 +1986,7 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
     double* d_value = bump.take<double>(n_problems);
     DpLevelParams lp;
     memset(&lp, 0, sizeof(lp));
-    uint32_t* d_nxt = bump.take<uint32_t>(max_rows * TM);
-    lp.nxt = d_nxt;
-    lp.val[0] = bump.take<DpVal>(max_val);
-    lp.val[1] = bump.take<DpVal>(max_val);
-    lp.succ = bump.take<uint32_t>(max_succ);
+    const size_t arena = bump.at;                            // the batches take turns in what follows
     lp.tabs = d_tabs; lp.lay = lay; lp.T = T;
 
     uint32_t launches = 0;
@@ -2067,6 +2058,12 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
             ++launches;
         }
         if (!b) break;
+        bump.at = arena;
+        uint32_t* d_nxt = bump.take<uint32_t>(b->nxt_rows * TM);
+        lp.nxt = d_nxt;
+        lp.val[0] = bump.take<DpVal>(b->val_entries);
+        lp.val[1] = bump.take<DpVal>(b->val_entries);
+        lp.succ = bump.take<uint8_t>(b->succ_bytes);
         lp.layouts = reinterpret_cast<const DpLayout*>(ctx->d_dp_up + off_lay);
         lp.live = reinterpret_cast<const uint32_t*>(ctx->d_dp_up + off_live);
         lp.jobs = reinterpret_cast<const DpJob*>(ctx->d_dp_up + off_jobs);
@@ -2126,8 +2123,8 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
         DpFinishParams fp;
         memset(&fp, 0, sizeof(fp));
         fp.blob = ctx->d_blob; fp.avail = ctx->d_avail; fp.sp = d; fp.layouts = lp.layouts; fp.jobs = lp.jobs; fp.live = lp.live;
-        fp.tabs = d_tabs; fp.val[0] = lp.val[0]; fp.val[1] = lp.val[1]; fp.succ = lp.succ; fp.value = d_value;
-        fp.results = d_results; fp.lay = lay; fp.n_jobs = (uint32_t)jobs.size(); fp.T = T;
+        fp.tabs = d_tabs; fp.val[0] = lp.val[0]; fp.val[1] = lp.val[1]; fp.succ = lp.succ; fp.nxt = d_nxt; fp.value = d_value;
+        fp.results = d_results; fp.lay = lay; fp.n_jobs = (uint32_t)jobs.size(); fp.T = T; fp.TM = TM;
         dp_finish_kernel<<<(fp.n_jobs + DP_FINISH_WARPS - 1) / DP_FINISH_WARPS, DP_FINISH_THREADS, 0, ctx->stream>>>(fp);
         CU(ctx, cudaGetLastError());
         ++launches;

@@ -289,3 +289,36 @@ def test_dp_argument_checks():
         B.sailor_set_availability(cx.ctx, np.zeros_like(w.avail))
         res, st = B.sailor_plan_dp(cx.ctx, cx.space, [[0, 1]], 4)
         assert res == [] and st.n_solved == 0
+
+
+def _count_vectors(caps, P):
+    """Vectors of stage counts within `caps` (types that can host some but not all stages) that add up to at most P."""
+    ways = np.zeros(P + 1, dtype=object)
+    ways[0] = 1
+    for c in caps:
+        if 1 <= c < P:
+            ways = np.array([sum(ways[s - x] for x in range(min(c, s) + 1)) for s in range(P + 1)], dtype=object)
+    return int(ways.sum())
+
+
+@pytest.mark.parametrize("P,caps", [(24, [[1, 3, 1, 2], [3, 2, 1, 1], [3, 1, 2, 1], [3, 3, 2, 2]]),
+                                    (32, [[1, 4, 3, 1, 2], [3, 2, 3, 1, 4], [5, 2, 3, 4, 5]]),
+                                    (48, [[5, 3, 2, 1], [3, 5, 4, 1], [5, 4, 5, 5], [1, 1, 4, 5]]),
+                                    (24, [[2, 1, 3, 3, 1, 2, 3, 1], [1, 1, 3, 2, 3, 1, 3, 2], [2, 1, 1, 1, 2, 3, 3, 3], [2, 3, 1, 3, 2, 3, 3, 1],
+                                          [3, 1, 2, 1, 1, 3, 2, 2], [3, 3, 1, 2, 3, 3, 2, 1]])])
+def test_dp_tables_fit_what_the_interface_says(P, caps, _index_mode):
+    """A problem's own tables take at most 64 + P bytes per type and count vector: with that much workspace it is solved,
+    with the same plans as with the default workspace, however many of its vectors are live at most stages."""
+    if _index_mode == "dense":
+        return                                               # (tables in mixed radix take more)
+    T, Z = len(caps[0]), len(caps)
+    w = W.tiny(seed=61, n_types=T, n_zones=Z, L=P, p_values=[P], d_values=(1,), tp_values=(1,), mbs_values=(1,), rc_values=(0,))
+    w.avail = np.array(caps, dtype=np.uint16)
+    w.capacity[:] = np.uint64(1 << 44)
+    limit = T * sum(_count_vectors(c, P) for c in caps) * (64 + P) + 512
+    orders = [list(range(Z))]
+    with Ctx(w) as cx:
+        want, st = B.sailor_plan_dp(cx.ctx, cx.space, orders, 4)
+        got, st2 = B.sailor_plan_dp(cx.ctx, cx.space, orders, 4, workspace_bytes=limit)
+    assert len(want) == 1 and st.n_solved == 1
+    assert [bytes(r) for r in got] == [bytes(r) for r in want] and st2.n_states == st.n_states
