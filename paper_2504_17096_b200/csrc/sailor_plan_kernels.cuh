@@ -47,6 +47,8 @@ struct Ctrl {                       // one per context, device memory
     double budget;                  // written by the cheapest-plan pass for the next pass
     unsigned int error;             // non-zero: a kernel gave up during this call (bounded wait ran out)
     unsigned int n_found;
+    unsigned int no_number;         // a candidate that cannot be chosen cost 0 x infinity: never read (see evaluated())
+    unsigned int _pad;
 };
 
 // What a pass leaves for the host (one device-to-host copy: the counters, then the k records).  The block that
@@ -803,8 +805,9 @@ __device__ __forceinline__ void by_shape(const CfgShared& cs, Walk walk) {
 //
 // SAILOR_FLAG_EVAL_ALL wants the time and the cost of every candidate formed, also of those that are invalid, out of
 // memory or over the availability.  Where no lane of the warp has a feasible candidate (98 % of workload 5) nothing is
-// selected from them, so no masks and no minima are formed; the values are only checked for what non-negative tables
-// cannot give, a set sign bit (one three-input OR a candidate).
+// selected from them, so no masks and no minima are formed; the values are only looked at for what non-negative tables
+// nearly never give, a set sign bit (one three-input OR a candidate): a price rate of zero over an infinite time is a NaN,
+// whose sign is set.  It is noted where nobody reads it, as the walk that selects passes over such a candidate too.
 __device__ __forceinline__ void evaluated(uint32_t& signs, double t, double c) {
     signs |= (uint32_t)__double2hiint(t) | (uint32_t)__double2hiint(c);
 }
@@ -1100,7 +1103,7 @@ __device__ __forceinline__ void run_items(const PlanParams& pp, const CfgShared&
         s32.c2x_col = a.c2x32 + d_prev;
         s32.comm_col = a.commx32 + z_prev;
         if (EVAL && NSEG == SAILOR_SEG_MAX && none_ok) {
-            if ((int)evaluate_only(cs, s32, T, Z, R, active, z_prev) < 0) pp.ctrl->error = 1u;
+            if ((int)evaluate_only(cs, s32, T, Z, R, active, z_prev) < 0) pp.ctrl->no_number = 1u;
             return;
         }
         const float f_inf = __int_as_float(0x7f800000);
@@ -1126,7 +1129,7 @@ __device__ __forceinline__ void run_items(const PlanParams& pp, const CfgShared&
         return;
     }
     if (EVAL && NSEG == SAILOR_SEG_MAX && none_ok) {
-        if ((int)evaluate_only(cs, it, T, Z, R, active, z_prev) < 0) pp.ctrl->error = 1u;      // cannot happen
+        if ((int)evaluate_only(cs, it, T, Z, R, active, z_prev) < 0) pp.ctrl->no_number = 1u;
         return;
     }
     // fast pass: no votes, no list updates; each lane keeps its item's best score

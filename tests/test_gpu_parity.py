@@ -860,3 +860,21 @@ def test_sweeps_cost_no_more_where_zones_are_alike(make_ctx):
         for w in (alike, zoned):
             assert sweep_ms(w, B.FLAG_EVAL_ALL) < 1.08 * plain, n_zones
         assert sweep_ms(differ, B.FLAG_EVAL_ALL | B.FLAG_F32_SCREEN) < 0.95 * plain, n_zones
+
+
+@pytest.mark.parametrize("n_zones", [1, 5])
+def test_every_candidate_where_times_overflow(n_zones, make_ctx):
+    """Tables are finite, sums of them need not be: on GPUs that cost nothing a candidate of infinite time costs 0 x inf.
+    Looking at every candidate must neither choose it nor fail on it."""
+    w = W.tiny(seed=37, n_types=2, n_zones=n_zones, L=8, p_values=[4, 8], d_values=(1, 8), tp_values=(1,), mbs_values=(1, 4), rc_values=(0,))
+    w.fwd[:, 1] = w.bwd[:, 1] = 1e308
+    w.price_per_hour[:, 1] = 0.0
+    w.avail[:] = 0
+    w.avail[:, 0] = 9                                        # eight replicas of a stage fit nowhere next to another stage
+    w.capacity[:] = np.uint64(1 << 44)
+    cx, o = make_ctx(w), Oracle(w)
+    for kind in (0, 1, 2):
+        hits, counts = o.search(kind, 8)
+        for flags in (0, B.FLAG_EVAL_ALL, B.FLAG_EVAL_ALL | B.FLAG_F32_SCREEN):
+            res, st = B.sailor_plan(cx.ctx, cx.space, B.Objective(kind, flags, 0.0, 0.0, 0.0), 8)
+            assert_plan_equal(res, st, hits, counts, o, f"kind={kind} flags={flags}")
