@@ -34,8 +34,11 @@
  *   C_iter= rate * T_iter + C_comm                                      (Sec. 4.3, Sec. 4.2.3)
  *
  * Threading.  A context is not thread-safe; use one context per host thread.  Different
- * contexts may be used from different threads at the same time (the library's few process-wide
- * flags are atomic).  The library reads no environment variable and keeps no other global state.
+ * contexts may be used from different threads at the same time (what they share is guarded).  The
+ * library reads no environment variable.  What it keeps between contexts: per device a memory pool
+ * of at most 256 MB that no context uses, in the process up to eight blocks of pinned host memory
+ * (270 KB each), and per device which kernels have been prepared.  The stream given to sailor_create
+ * must outlive the context.
  */
 #ifndef SAILOR_H
 #define SAILOR_H
@@ -317,13 +320,13 @@ int sailor_plan_range(sailor_ctx* ctx, const sailor_space* s, const sailor_objec
 /* Search without allocating.  (The paper has no counterpart: this entry point exists for the
  * sake of callers, not of the method.)
  *
- * sailor_plan allocates device memory whenever it meets a space it has not cached (two
- * cudaMalloc / cudaFree pairs for the per-configuration index arrays).  Some callers cannot
- * afford or are not allowed that: a re-planning loop inside a training process whose memory
- * pool already owns the whole GPU, where a further cudaMalloc fails; a latency-critical
- * controller for which cudaMalloc's device-wide synchronisation stalls every other stream;
- * a thread that runs while another thread of the process captures a stream in the global
- * capture mode, during which cudaMalloc is an error.  This variant computes exactly what
+ * sailor_plan allocates device memory whenever it meets a space it has not cached (one piece, from
+ * the library's pool, for the per-configuration tables; the pool takes more from the device when it
+ * has none left).  Some callers cannot afford or are not allowed that: a re-planning loop inside a
+ * training process whose memory pool already owns the whole GPU, where a further allocation fails; a
+ * latency-critical controller that cannot wait for the device to map more memory; a thread that
+ * runs while another thread of the process captures a stream in the global capture mode, during
+ * which allocating is an error.  This variant computes exactly what
  * sailor_plan computes (whole space, same results, same statistics) but calls no cudaMalloc,
  * cudaFree or any other allocating routine: all of its working memory (work counter,
  * statistics, per-block top-k lists, result records, per-configuration index arrays) lies in

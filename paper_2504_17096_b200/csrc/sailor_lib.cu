@@ -324,8 +324,9 @@ size_t padded(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
 
 // Device memory comes from one memory pool per device that the library owns: a context's first buffers then cost
 // microseconds where cudaMalloc and cudaFree of a megabyte cost 0.3 ms each (up to 12 ms seen).  The pool keeps at most
-// POOL_KEEP bytes that no context uses (what is beyond goes back to the device when a stream is next synchronised).
-// Allocation and release are ordered on the context's stream; the pool itself is safe to use from any thread.
+// POOL_KEEP bytes that no context uses; what a living context gives up beyond that goes back to the device at the
+// synchronisation that ends the call, what a destroyed one leaves at once.  While a context lives, allocation and release
+// are ordered on its stream; the pool itself is safe to use from any thread.
 constexpr uint64_t POOL_KEEP = 256ull << 20;
 constexpr int POOL_DEVICES_MAX = 64;
 
@@ -1138,7 +1139,9 @@ int sailor_destroy(sailor_ctx* ctx) {
     if (!ctx) return SAILOR_OK;
     DeviceGuard guard(ctx->device);
     if (ctx->d_mem) cudaStreamSynchronize(ctx->stream);
-    for (unsigned char* p : {ctx->d_mem, ctx->space.d_mem, ctx->d_stage, ctx->d_mix, ctx->d_dp, ctx->d_dp_up}) device_free(ctx, p);
+    // nothing uses the memory any more: freed in no stream's order, so that what the pool does not keep goes back to the
+    // device here, and not when some stream is next synchronised (another allocator of the process may need it before)
+    for (unsigned char* p : {ctx->d_mem, ctx->space.d_mem, ctx->d_stage, ctx->d_mix, ctx->d_dp, ctx->d_dp_up}) cudaFree(p);
     g_host_blocks.give_back(ctx->host);
     delete ctx->mix;
     for (cudaEvent_t e : {ctx->ev0, ctx->ev1, ctx->ev2, ctx->evh0, ctx->evh1, ctx->ev_chunk, ctx->ev_join, ctx->ev_slot[0],

@@ -878,3 +878,19 @@ def test_every_candidate_where_times_overflow(n_zones, make_ctx):
         for flags in (0, B.FLAG_EVAL_ALL, B.FLAG_EVAL_ALL | B.FLAG_F32_SCREEN):
             res, st = B.sailor_plan(cx.ctx, cx.space, B.Objective(kind, flags, 0.0, 0.0, 0.0), 8)
             assert_plan_equal(res, st, hits, counts, o, f"kind={kind} flags={flags}")
+
+
+def test_a_destroyed_context_gives_its_memory_back(torch_cuda):
+    """The memory pool behind the contexts keeps at most 256 MB that none of them uses: after sailor_destroy the rest is the
+    device's again, without waiting for some other synchronisation of the process."""
+    torch = torch_cuda
+    w = W.config3()
+    ctx = B.sailor_create(w, 0, 0)
+    B.sailor_set_availability(ctx, w.avail)
+    before = torch.cuda.mem_get_info()[0]
+    orders = [[0, 1, 2, 3, 4], [4, 3, 2, 1, 0], [2, 0, 1, 4, 3], [1, 3, 0, 2, 4]]
+    _, st = B.sailor_plan_dp(ctx, B.make_space(w), orders, 4, workspace_bytes=1 << 30)
+    during = torch.cuda.mem_get_info()[0]
+    assert st.workspace_used > 700 << 20 and before - during > 600 << 20
+    B.sailor_destroy(ctx)
+    assert before - torch.cuda.mem_get_info()[0] <= 256 << 20
