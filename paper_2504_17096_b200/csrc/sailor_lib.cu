@@ -2,6 +2,7 @@
 // Every simulation step runs in the kernels; the host only validates, packs tables and
 // enqueues work on the caller's stream.
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstddef>
 #include <cstdlib>
@@ -291,16 +292,19 @@ inline void cpu_relax() {
 
 // Waits until the kernel that ends a call has left its results, with `ticket` behind them, in the context's pinned memory:
 // the host sees them some microseconds before the stream counts as idle (a search of one zone with new availability:
-// 55.2 us by cudaStreamSynchronize, 52.5 this way).  Everything enqueued earlier on the stream is done by then.  A stream
-// that ends, or fails, without the ticket is found out by asking it now and then.
+// 55.2 us by cudaStreamSynchronize, 52.5 this way).  Everything enqueued earlier on the stream is done by then.  Longer
+// searches, of which those microseconds are a small part, wait in cudaStreamSynchronize after a millisecond, the way the
+// application has chosen for the device (blocking, yielding); it also finds out a stream that fails.
+constexpr std::chrono::microseconds TICKET_SPIN(1000);
+
 cudaError_t wait_ticket(sailor_ctx* ctx, const uint64_t* slot, uint64_t ticket) {
     const volatile uint64_t* seen = slot;
-    for (uint32_t spin = 1;; ++spin) {
-        if (*seen == ticket) break;
-        if (spin % 4096 == 0) {
-            const cudaError_t e = cudaStreamQuery(ctx->stream);
-            if (e == cudaSuccess) break;                       // (what is missing now never comes)
-            if (e != cudaErrorNotReady) return e;
+    const auto until = std::chrono::steady_clock::now() + TICKET_SPIN;
+    for (uint32_t spin = 1; *seen != ticket; ++spin) {
+        if (spin % 256 == 0 && std::chrono::steady_clock::now() > until) {
+            const cudaError_t e = cudaStreamSynchronize(ctx->stream);
+            if (e != cudaSuccess) return e;
+            break;                                             // (what is missing now never comes)
         }
         cpu_relax();
     }

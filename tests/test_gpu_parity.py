@@ -894,3 +894,33 @@ def test_a_destroyed_context_gives_its_memory_back(torch_cuda):
     assert st.workspace_used > 700 << 20 and before - during > 600 << 20
     B.sailor_destroy(ctx)
     assert before - torch.cuda.mem_get_info()[0] <= 256 << 20
+
+
+def test_long_searches_wait_as_the_application_chose(torch_cuda):
+    """An application that asked for blocking synchronisation (cudaDeviceScheduleBlockingSync) gets its processor back
+    during a search of several milliseconds."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import ctypes, time
+cuda = ctypes.CDLL("libcuda.so.1")
+assert cuda.cuInit(0) == 0 and cuda.cuDevicePrimaryCtxSetFlags_v2(0, 4) == 0     # CU_CTX_SCHED_BLOCKING_SYNC
+from paper_2504_17096_b200 import binding as B, workloads as W
+w = W.config5()
+ctx = B.sailor_create(w, 0, 0)
+B.sailor_set_availability(ctx, w.avail)
+space, obj = B.make_space(w), B.make_objective(w, flags=B.FLAG_EVAL_ALL)
+B.sailor_plan(ctx, space, obj, 4)
+wall, cpu = time.perf_counter(), time.thread_time()
+for _ in range(40):
+    B.sailor_plan(ctx, space, obj, 4)
+wall, cpu = time.perf_counter() - wall, time.thread_time() - cpu
+B.sailor_destroy(ctx)
+print(wall, cpu)
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    wall, cpu = map(float, out.stdout.split())
+    assert cpu < 0.5 * wall, (wall, cpu)
