@@ -377,7 +377,9 @@ __device__ __forceinline__ bool zones_pay(uint32_t Z, uint32_t stages) {
     return Z > group && (Z == group + 1 || stages <= 5);
 }
 
-// Build the tables of configuration `c`.  Called by the whole block; ends synchronised.
+// Build the tables of configuration `c`.  Called by the whole block; ends synchronised.  SWEEP: with `by_zone`, which only
+// sweeps of every candidate read.
+template <bool SWEEP>
 static __device__ void build_config(const PlanParams& pp, const TabView& v, CfgShared& cs, CfgArrays& a, uint32_t c) {
     const TabHdr* h = v.h;
     const uint32_t T = h->T, Z = h->Z, R = h->R, tid = threadIdx.x;
@@ -522,7 +524,7 @@ static __device__ void build_config(const PlanParams& pp, const TabView& v, CfgS
                 atomicOr(reinterpret_cast<unsigned long long*>(&cs.lower_fit[j][s]), 1ull << d);
     }
     __syncthreads();                   // the memory masks and the records are complete
-    {
+    if constexpr (SWEEP) {
         const SegRec* recs = a.rec + (k.nseg - 1) * R;
         bool alike = true;             // the last segment's records of a type are the same bits in every zone
         for (uint32_t d = tid; d < R; d += PLAN_THREADS) {
@@ -1552,7 +1554,7 @@ __global__ void __launch_bounds__(PLAN_THREADS, SCREEN ? PLAN_SCREEN_BLOCKS : PL
                 if (pp.cfg_cache) load_config(pp, cs, a, R, c);
                 else {
                     __syncthreads();
-                    build_config(pp, v, cs, a, c);
+                    build_config<EVAL>(pp, v, cs, a, c);
                 }
                 if (SCREEN) round_config32(a, R, Z);
             }

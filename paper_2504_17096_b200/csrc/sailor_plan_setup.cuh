@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(PLAN_THREADS, PLAN_MIN_BLOCKS) cfg_cache_kerne
     __syncthreads();
     for (uint32_t c = blockIdx.x; c < pp.n_config; c += gridDim.x) {
         __syncthreads();
-        build_config(pp, v, cs, a, c);
+        build_config<true>(pp, v, cs, a, c);
         __syncthreads();
         uint4* dst = cache + (size_t)c * (pp.cache_head16 + pp.cache_arr16);
         for (uint32_t x = tid; x < pp.cache_head16; x += PLAN_THREADS) dst[x] = reinterpret_cast<const uint4*>(&cs)[x];
