@@ -1143,9 +1143,14 @@ int sailor_destroy(sailor_ctx* ctx) {
     if (!ctx) return SAILOR_OK;
     DeviceGuard guard(ctx->device);
     if (ctx->d_mem) cudaStreamSynchronize(ctx->stream);
-    // nothing uses the memory any more: freed in no stream's order, so that what the pool does not keep goes back to the
-    // device here, and not when some stream is next synchronised (another allocator of the process may need it before)
-    for (unsigned char* p : {ctx->d_mem, ctx->space.d_mem, ctx->d_stage, ctx->d_mix, ctx->d_dp, ctx->d_dp_up}) cudaFree(p);
+    for (unsigned char* p : {ctx->d_mem, ctx->space.d_mem, ctx->d_stage, ctx->d_mix, ctx->d_dp, ctx->d_dp_up}) device_free(ctx, p);
+    // what the pool does not keep goes back to the device here, and not when some stream is next synchronised: another
+    // allocator of the process may need it before
+    cudaMemPool_t pool;
+    uint64_t reserved = 0;
+    if (ctx->d_mem && device_pool(ctx, &pool) == SAILOR_OK &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess && reserved > POOL_KEEP)
+        cudaStreamSynchronize(ctx->stream);
     g_host_blocks.give_back(ctx->host);
     delete ctx->mix;
     for (cudaEvent_t e : {ctx->ev0, ctx->ev1, ctx->ev2, ctx->evh0, ctx->evh1, ctx->ev_chunk, ctx->ev_join, ctx->ev_slot[0],
