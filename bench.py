@@ -365,7 +365,8 @@ def explicit_batches(B, torch, dev) -> dict:
             out[key].update({"host_call_ms": statistics.median(ts) * 1e3, "host_plans_per_s": n / statistics.median(ts),
                              "host_pcie_gb_per_s": n * 100 / statistics.median(ts) / 1e9, "host_equals_device": same})
             del d_plans, t, c, m, st, h_plans, ht, hc, hm, hs
-        # plans whose stages mix GPU types among their replicas, up to 32 stages each: 648 B in + 28 B out per plan
+        # plans whose stages mix GPU types among their replicas, up to 32 stages each: 8 B and 20 B a stage in,
+        # 28 B out per plan (stages past the last are not read)
         base = B.pack_mixed_plans(W.random_mixed_plans(w, 1 << 14, seed=13), stages=32)
         reps = 64
         n = base.size * reps                                           # 1.05e6 plans, 680 MB: larger than L2
@@ -387,7 +388,7 @@ def explicit_batches(B, torch, dev) -> dict:
         ms = e0.elapsed_time(e1) / 5
         out["simulate_mixed_cfg5"] = {"plans": n, "mean_stages": float(base["P"].astype(np.float64).mean()),
                                       "kernel_ms": ms, "plans_per_s": n / ms * 1e3,
-                                      "hbm_gb_per_s": n * (base.itemsize + 28) / ms / 1e6}
+                                      "hbm_gb_per_s": reps * float((8 + 20 * base["P"].astype(np.int64) + 28).sum()) / ms / 1e6}
         del d_plans, t, c, m, st
     finally:
         B.sailor_destroy(ctx)

@@ -1,7 +1,7 @@
 // Explicit batches of plan records (Sailor Sec. 4.3): the kernel behind sailor_simulate.
 //
 // A record costs 72 bytes in and 28 bytes out; what bounds the batch is the instructions a record takes (issue slots 64 %
-// busy, HBM 12 %).  4.2e6 random records of workload 5 (19 stages, 4.3 runs, 5.7 pieces on average): 850 us -> 411 us
+// busy, HBM 12 %).  4.2e6 random records of workload 5 (19 stages, 4.3 runs, 5.7 pieces on average): 850 us -> 396 us
 // (110 -> 67 warp-instructions a record).  What keeps them few:
 //   - everything a stretch of equal stages needs (f + b, update time, memory with and without an in-flight microbatch)
 //     sits in ONE 32-byte table entry (one memory sector, one load) per (stage make-up, GPU type, tp, mbs, rc), the gradient
@@ -380,8 +380,8 @@ __device__ __forceinline__ void order_pool(const uint64_t* rec, uint16_t* perm, 
 // a ring in shared memory (one bulk copy each) and orders them by work; the others take groups of 32 similar records, longest
 // first, copy their runs aside and hand the slot on before they evaluate them, so that nobody waits for the slowest group (an
 // order of 512 records with barriers around it cost 3 of 11 stall cycles an instruction; slots held until evaluated: 626 us).
-// 19 warps of 96 registers: 23 of 80 spill (461 us), 15 of 107 leave latencies open (461); pools of 768: 512 446 us, 640 419,
-// 896 and 1 024 the same 411.  Results leave as four structure-of-arrays streams.
+// 19 warps of 96 registers: 23 of 80 spill (461 us), 15 of 107 leave latencies open (461); pools of 768: 411 us when
+// this was tried, 512 446, 640 419, 896 and 1 024 the same.  Results leave as four structure-of-arrays streams.
 __global__ void __launch_bounds__(BATCH_THREADS, 1)
 simulate_kernel(const __grid_constant__ BatchParams p, const uint16_t* __restrict__ avail,
                 const sailor_plan_rec* __restrict__ plans, uint64_t n, uint32_t pool_size, uint32_t lanes, double* __restrict__ t_iter,

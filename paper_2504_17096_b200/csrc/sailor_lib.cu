@@ -328,9 +328,9 @@ size_t padded(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
 
 // Device memory comes from one memory pool per device that the library owns: a context's first buffers then cost
 // microseconds where cudaMalloc and cudaFree of a megabyte cost 0.3 ms each (up to 12 ms seen).  The pool keeps at most
-// POOL_KEEP bytes that no context uses; what a living context gives up beyond that goes back to the device at the
-// synchronisation that ends the call, what a destroyed one leaves at once.  While a context lives, allocation and release
-// are ordered on its stream; the pool itself is safe to use from any thread.
+// POOL_KEEP bytes that no context uses; what is beyond goes back to the device at the synchronisation that ends a call, or
+// one at the end of sailor_destroy.  Allocation and release are ordered on the context's stream; the pool itself is safe to
+// use from any thread.
 constexpr uint64_t POOL_KEEP = 256ull << 20;
 constexpr int POOL_DEVICES_MAX = 64;
 

@@ -12,7 +12,7 @@
 // transfer cost: stage after stage).
 // Bound: issue slots (67 % busy).  Random plans of workload 5 (mean 9.4 stages, 1.9 groups a stage, 5.4 pipelines), 2.6e5
 // of them: 1 003 us with a lane per stage throughout and one pipeline after the other (2 960 warp-instructions a plan);
-// 479 us this way (1 440).  Four blocks of 64 registers an SM: with 80 registers and three blocks 540 us.
+// 479 us this way (1 424).  Four blocks of 64 registers an SM: with 80 registers and three blocks 540 us.
 #pragma once
 
 #include "sailor_batch.cuh"
