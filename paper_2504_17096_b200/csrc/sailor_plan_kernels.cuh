@@ -823,8 +823,8 @@ __device__ __forceinline__ void evaluated(uint32_t& signs, float t, float c) { s
 // max(n_b x a, n_b x b): rounding is monotone, so these are the same bits; a transfer cost of zero is not added.  Every
 // candidate still takes its own additions over the segment's stages, in stage order, and its own closing terms: the bits
 // are those of eval_candidates.  N2 >= 0: the segment is N2 plain stages and the final stage (straight code); -1: any.
-// Bound: issue slots (64 % busy) and the FP64 pipe (52 %): 6 + (stages of the segment) FP64 instructions a candidate
-// against 14 + 2 x (stages) digit by digit.  Workload 5, 6.4e9 candidates: 13.89 -> 7.30 ms, 55.9 -> 26.9
+// Bound: issue slots (63 % busy) and the FP64 pipe (52 %): 6 + (stages of the segment) FP64 instructions a candidate
+// against 14 + 2 x (stages) digit by digit.  Workload 5, 6.4e9 candidates: 13.89 -> 7.19 ms, 55.9 -> 26.4
 // lane-instructions a candidate, about 7 of them what an item costs before its candidates (digits, masks, prefix sums).
 template <int N2, int W, bool OWN, typename F>
 __device__ __forceinline__ void evaluate_zones(const CfgShared& cs, const ItemState<F>& it, uint32_t T, uint32_t Z, uint32_t R,
