@@ -20,6 +20,7 @@
 #include "sailor_dp.cuh"
 #include "sailor_dp_budget.cuh"
 #include "sailor_mixed.cuh"
+#include "sailor_mixed_batch.cuh"
 #include "sailor_mixed_search.cuh"
 #include "sailor_peaks.cuh"
 #include "sailor_plan_setup.cuh"
@@ -102,56 +103,47 @@ __global__ void compose_kernel(unsigned char* blob) {
     }
 }
 
-// One warp per plan with mixed replicas (records `stride` bytes apart holding `max_stages` stages, read in place).
-// Tables in shared memory, then a scratch area per warp.  Plans of up to 32 stages are evaluated by the DEEP = false
-// launch, which leaves deeper ones alone and notes in `deep_seen` that there are some; the DEEP = true launch that follows
-// returns at once when there are none and evaluates only those otherwise (three times the scratch per warp).
+// A warp per plan with mixed replicas (records `stride` bytes apart holding `max_stages` stages, read in place): all plans of up
+// to 32 stages of a small batch (DEEP = false; see mixb_least), or the deeper ones of any batch.  The launch for shallow plans,
+// this or simulate_mixed_kernel, notes in `deep_seen` that there are deep ones; the DEEP launch that follows returns at once when
+// there are none (three times the scratch per warp).
 template <bool DEEP> constexpr uint32_t MIX_WARPS = DEEP ? 4 : 8;
-template <bool DEEP> constexpr uint32_t MIX_STAGES = DEEP ? SAILOR_MIX_P_MAX : 32;
+template <bool DEEP> constexpr uint32_t MIX_STAGES = DEEP ? SAILOR_MIX_P_MAX : MIXB_P_MAX;
 
 template <bool DEEP>
 __global__ void __launch_bounds__(32 * MIX_WARPS<DEEP>, 4)
-simulate_mixed_kernel(const unsigned char* __restrict__ blob, const uint16_t* __restrict__ avail,
-                      const unsigned char* __restrict__ plans, uint32_t stride, uint32_t max_stages, uint64_t n,
-                      double* __restrict__ t_iter, uint64_t* __restrict__ peak_mem, double* __restrict__ cost,
-                      uint32_t* __restrict__ status, unsigned int* error, unsigned int* deep_seen, uint32_t report_bad) {
+simulate_mixed_each_kernel(const __grid_constant__ MixbParams p) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ uint64_t mbar;
-    if (DEEP && *reinterpret_cast<volatile unsigned int*>(deep_seen) == 0) return;
+    if (DEEP && *reinterpret_cast<const volatile unsigned int*>(p.deep_seen) == 0) return;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     constexpr uint32_t WARPS = MIX_WARPS<DEEP>;
-    const uint32_t static_bytes = reinterpret_cast<const TabHdr*>(blob)->static_bytes;
-    if (!bulk_load(dyn, blob, static_bytes, &mbar)) {
-        if (tid == 0) atomicOr(error, SIM_ERR_DEVICE);
+    const uint32_t static_bytes = reinterpret_cast<const TabHdr*>(p.blob)->static_bytes;
+    if (!bulk_load(dyn, p.blob, static_bytes, &mbar)) {
+        if (tid == 0) atomicOr(p.error, SIM_ERR_DEVICE);
         for (uint32_t x = tid; x < static_bytes / 16; x += 32 * WARPS)
-            reinterpret_cast<uint4*>(dyn)[x] = reinterpret_cast<const uint4*>(blob)[x];
+            reinterpret_cast<uint4*>(dyn)[x] = reinterpret_cast<const uint4*>(p.blob)[x];
         __syncthreads();
     }
     TabView v;
-    v.bind(dyn, blob);
+    v.bind(dyn, p.blob);
     auto& scratch = reinterpret_cast<MixScratch<MIX_STAGES<DEEP>>*>(dyn + static_bytes)[warp];
-    for (uint64_t j = (uint64_t)blockIdx.x * WARPS + warp; j < n; j += (uint64_t)gridDim.x * WARPS) {
-        const sailor_mixed_plan& r = *reinterpret_cast<const sailor_mixed_plan*>(plans + j * stride);
+    for (uint64_t j = (uint64_t)blockIdx.x * WARPS + warp; j < p.n; j += (uint64_t)gridDim.x * WARPS) {
+        const sailor_mixed_plan& r = *reinterpret_cast<const sailor_mixed_plan*>(p.plans + j * p.stride);
         const uint32_t P = r.P;
         SimOut o;
-        if (DEEP && (P <= 32 || P > max_stages)) continue;       // done by the first launch
-        if (P > max_stages) {                                    // more stages than the record has room for
+        if (DEEP && (P <= MIXB_P_MAX || P > p.max_stages)) continue;     // done by the first launch
+        if (P > p.max_stages) {                                  // more stages than the record has room for
             o.t_iter = o.cost = make_nan();
             o.peak_mem = 0;
             o.status = SAILOR_ST_BAD_RECORD;
-        } else if (!DEEP && P > 32) {
-            if (lane == 0) *reinterpret_cast<volatile unsigned int*>(deep_seen) = 1u;
+        } else if (!DEEP && P > MIXB_P_MAX) {
+            if (lane == 0) *reinterpret_cast<volatile unsigned int*>(p.deep_seen) = 1u;
             continue;
         } else {
-            o = simulate_mixed_warp(v, blob, avail, r, scratch, lane);
+            o = simulate_mixed_warp(v, p.blob, p.avail, r, scratch, lane);
         }
-        if (lane == 0) {
-            if (t_iter) t_iter[j] = o.t_iter;
-            if (peak_mem) peak_mem[j] = o.peak_mem;
-            if (cost) cost[j] = o.cost;
-            if (status) status[j] = o.status;
-            if (report_bad && (o.status & SAILOR_ST_BAD_RECORD)) atomicOr(error, SIM_ERR_BAD_RECORD);
-        }
+        if (lane == 0) mixb_store(p, j, o);
         __syncwarp();
     }
 }
@@ -1129,8 +1121,9 @@ static int create_impl(const sailor_model* m, const sailor_profile* p, const sai
     }
     // both kernels stage the static tables in dynamic shared memory; the create-time limit is 96 KB
     CUF(cudaFuncSetAttribute(simulate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    CUF(cudaFuncSetAttribute(simulate_mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixScratch<MIX_STAGES<false>>) * MIX_WARPS<false>));
-    CUF(cudaFuncSetAttribute(simulate_mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixScratch<MIX_STAGES<true>>) * MIX_WARPS<true>));
+    CUF(cudaFuncSetAttribute(simulate_mixed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(MixbShared) + 2 * R_MAX * SAILOR_MBS_MAX * sizeof(double))));
+    CUF(cudaFuncSetAttribute(simulate_mixed_each_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixScratch<MIX_STAGES<false>>) * MIX_WARPS<false>));
+    CUF(cudaFuncSetAttribute(simulate_mixed_each_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixScratch<MIX_STAGES<true>>) * MIX_WARPS<true>));
     CUF(cudaFuncSetAttribute(finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (96 + 8) * 1024));
     CUF(cudaFuncSetAttribute(mixed_finish_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixFinishWarp<false>) * MIXF_WARPS<false>));
     CUF(cudaFuncSetAttribute(mixed_finish_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)sizeof(MixFinishWarp<true>) * MIXF_WARPS<true>));
@@ -1228,18 +1221,20 @@ int sailor_simulate_mixed_strided(sailor_ctx* ctx, const void* plans_v, uint64_t
     DeviceGuard guard(ctx->device);
     auto launch = [ctx, record_bytes, max_stages](const unsigned char* d_plans, uint64_t m, double* d_t, uint64_t* d_m, double* d_c,
                                                   uint32_t* d_s, unsigned int* error, uint32_t report_bad) {
-        // a warp per plan; blocks take several plans per warp in larger batches
-        const uint64_t blocks = (m + MIX_WARPS<false> - 1) / MIX_WARPS<false>, cap = (uint64_t)ctx->sm_count * 32;
-        unsigned int* deep_seen = ctx->d_deep_seen;
-        if (max_stages > 32) CU(ctx, cudaMemsetAsync(deep_seen, 0, sizeof(unsigned int), ctx->stream));
-        simulate_mixed_kernel<false><<<(uint32_t)std::min(blocks, cap), 32 * MIX_WARPS<false>, mixed_smem<false>(ctx->hdr), ctx->stream>>>(
-            ctx->d_blob, ctx->d_avail, d_plans, record_bytes, max_stages, m, d_t, d_m, d_c, d_s, error, deep_seen, report_bad);
+        MixbParams p = mixb_params(ctx->hdr, ctx->d_blob);
+        p.avail = ctx->d_avail;
+        p.plans = d_plans; p.n = m; p.stride = record_bytes; p.max_stages = max_stages;
+        p.t_iter = d_t; p.peak_mem = d_m; p.cost = d_c; p.status = d_s;
+        p.error = error; p.deep_seen = ctx->d_deep_seen; p.report_bad = report_bad;
+        if (max_stages > MIXB_P_MAX) CU(ctx, cudaMemsetAsync(ctx->d_deep_seen, 0, sizeof(unsigned int), ctx->stream));
+        if (m < mixb_least(ctx->hdr))
+            simulate_mixed_each_kernel<false><<<(uint32_t)((m + MIX_WARPS<false> - 1) / MIX_WARPS<false>), 32 * MIX_WARPS<false>, mixed_smem<false>(ctx->hdr), ctx->stream>>>(p);
+        else
+            simulate_mixed_kernel<<<(uint32_t)std::min<uint64_t>(m, MIXB_BLOCKS * (uint64_t)ctx->sm_count), MIXB_THREADS, mixb_smem(ctx->hdr), ctx->stream>>>(p);
         CU(ctx, cudaGetLastError());
-        if (max_stages > 32) {                                   // the plans of more than 32 stages, if the first launch saw any
-            const uint64_t blocks2 = (m + MIX_WARPS<true> - 1) / MIX_WARPS<true>, cap2 = (uint64_t)ctx->sm_count * 16;
-            simulate_mixed_kernel<true><<<(uint32_t)std::min(blocks2, cap2), 32 * MIX_WARPS<true>, mixed_smem<true>(ctx->hdr), ctx->stream>>>(
-                ctx->d_blob, ctx->d_avail, d_plans, record_bytes, max_stages, m, d_t, d_m, d_c, d_s, error, deep_seen,
-                report_bad);
+        if (max_stages > MIXB_P_MAX) {                           // the plans of more than 32 stages, if the first launch saw any
+            const uint64_t blocks = (m + MIX_WARPS<true> - 1) / MIX_WARPS<true>, cap = (uint64_t)ctx->sm_count * 16;
+            simulate_mixed_each_kernel<true><<<(uint32_t)std::min(blocks, cap), 32 * MIX_WARPS<true>, mixed_smem<true>(ctx->hdr), ctx->stream>>>(p);
             CU(ctx, cudaGetLastError());
         }
         return (int)SAILOR_OK;

@@ -224,3 +224,45 @@ def test_mixed_interval_edges(D, stages):
     so, to, co, mo = o.simulate_mixed_batch(plans)
     assert np.array_equal(s, so) and np.array_equal(m, mo)
     assert np.array_equal(t, to, equal_nan=True) and np.array_equal(c, co, equal_nan=True)
+
+
+@pytest.mark.parametrize("D,stages,n,node", [(6, 3, 16, 8), (6, 3, 17, 8),           # either side of the smallest batch of the batch kernel
+                                             (127, 32, 700, 8), (128, 32, 700, 8),   # the largest replica numbers that fit its bytes; more
+                                             (129, 32, 40, 8),                       # items than a batch has room for (four groups a stage)
+                                             (4, 8, 3000, 8190), (4, 8, 300, 8191),  # the largest node its items can tell apart, and a larger one
+                                             (3, 1, 5000, 8), (2, 33, 50, 8)])       # one stage: the most plans at a time; deep plans
+def test_mixed_batches_at_their_edges(D, stages, n, node):
+    """Plans of one depth (and some shallower), most stages with four groups, refused records in between: the same bits as
+    the oracle, and the refused ones flagged."""
+    import torch
+    w = W.tiny(seed=51, n_types=4, n_zones=3, L=max(stages, 4), gbs=D * 4, d_values=(D,), p_values=[stages])
+    w.gpus_per_node[...] = [4, node, 700, 2]
+    rng = W.SplitMix64(D * 977 + stages)
+    plans = []
+    for j in range(n):
+        P = stages if j % 5 else rng.randint(1, stages)
+        st = []
+        for i in range(P):
+            cuts = sorted({rng.randint(1, D - 1) for _ in range(3 if j % 3 else rng.randint(0, 3))})
+            b = [0] + cuts + [D]
+            st.append({"zone": rng.randint(0, 2) if j % 3 else 1,
+                       "groups": [(rng.randint(0, 3), rng.randint(0, 2), b[q + 1] - b[q]) for q in range(len(b) - 1)]})
+        plans.append({"P": P, "mbs_idx": rng.randint(0, 2), "rc": j & 1, "D": D, "stages": st})
+    so, to, co, mo = Oracle(w).simulate_mixed_batch(plans)
+    packed = B.pack_mixed_plans(plans)
+    refused = np.arange(n) % 11 == 5
+    for j in np.flatnonzero(refused):
+        if j % 2:
+            packed["stage"]["group"]["type"][j, int(packed["P"][j]) - 1, 0] = 4
+        else:
+            packed["stage"]["n_groups"][j, 0] = 0
+    so[refused], mo[refused], to[refused], co[refused] = B.ST_BAD_RECORD, 0, math.nan, math.nan
+    with Ctx(w) as cx:
+        d = torch.from_numpy(packed.view(np.uint8).reshape(n, packed.itemsize).copy()).cuda()
+        dt = torch.empty(n, dtype=torch.float64, device="cuda"); dc = torch.empty(n, dtype=torch.float64, device="cuda")
+        dm = torch.empty(n, dtype=torch.int64, device="cuda"); ds = torch.empty(n, dtype=torch.int32, device="cuda")
+        B.sailor_simulate_mixed_device(cx.ctx, d.data_ptr(), n, dt.data_ptr(), dm.data_ptr(), dc.data_ptr(), ds.data_ptr(),
+                                       record_bytes=packed.itemsize)
+        torch.cuda.synchronize()
+    gpu = (dt.cpu().numpy(), dm.cpu().numpy().view(np.uint64), dc.cpu().numpy(), ds.cpu().numpy().view(np.uint32))
+    assert_equal(gpu, (so, to, co, mo), f"D {D}, {stages} stages, {n} plans")
