@@ -70,7 +70,11 @@ struct DpJob {                       // a problem that has tables
     uint64_t val_off;                // first entry of its two level buffers
     uint64_t succ_off;               // first byte of its successors: [stage][slot][type]
     uint32_t config, index, layout, P;   // index = config * n_orders + order
+    uint32_t slots, _pad;            // most live vectors of a stage: a type's values are this many entries, slot after slot (a
+                                     // warp's gathers then fall into a few lines instead of one each: workload 3 1 700 -> 1 622
+                                     // us a call, workload 5 496 -> 468)
 };
+static_assert(sizeof(DpJob) % 8 == 0, "copied by eight bytes");
 
 struct DpResult {                    // per problem that has a plan, written by dp_finish_kernel
     double t_iter, cost;             // the simulator's figures for the plan (stage order)
@@ -245,13 +249,23 @@ struct DpLevelParams {
     const uint32_t* live;
     const uint32_t* nxt;
     const double* tabs;
-    DpVal* val[2];                   // level buffers [slot][type]; stage i lives in val[(P - 1 - i) & 1]
+    DpVal* val[2];                   // level buffers [type][slot]; stage i lives in val[(P - 1 - i) & 1]
     uint8_t* succ;                   // [stage][slot][type]: type of the next stage in the best plan (DP_NONE: there is none)
     const uint32_t* blk_prefix;      // per-stage launches: [n_active + 1] blocks before each job of this launch
     DpTabLayout lay;
     uint32_t T, n_active;
     uint32_t dist;                   // stage i = P - 1 - dist
 };
+
+// A value in one 32-byte load or store.
+__device__ __forceinline__ DpVal load_val(const DpVal* p) {
+    DpVal v;
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v.sum), "=d"(v.mx), "=d"(v.sy), "=d"(v.up) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void store_val(DpVal* p, const DpVal& v) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v.sum), "d"(v.mx), "d"(v.sy), "d"(v.up) : "memory");
+}
 
 // What a stage of a job reads of the job's tables, kept in shared memory (every vector of the stage reads it).
 struct DpStageTab {
@@ -296,10 +310,9 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
     // what follows a stage of each type g2: the state it leads to (the same for every type of stage i) and its value
     const DpVal* nxt = lp.val[(dist & 1) ^ 1] + job.val_off;
     DpVal n[TM];
-    uint32_t code[TM], d2[TM];
+    uint32_t d2[TM];
 #pragma unroll
     for (uint32_t g2 = 0; g2 < TM; ++g2) {
-        code[g2] = DP_NO_STATE;
         d2[g2] = 0;
         n[g2].sum = make_inf(); n[g2].mx = n[g2].sy = n[g2].up = 0.0;
     }
@@ -317,13 +330,12 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
             }
             const uint32_t slot2 = live_slot(then, zp2) + (id - live_vec(then, zp2));
             if (slot2 >= then[0]) continue;                  // (a move of a live state leads to a live state)
-            code[g2] = slot2 * T + g2;
             d2[g2] = L.zone[zp2] * T + g2;
-            n[g2] = nxt[code[g2]];
+            n[g2] = load_val(nxt + (size_t)g2 * job.slots + slot2);
         }
     }
     const uint32_t ok_here = st.ok;
-    DpVal* cur = lp.val[dist & 1] + job.val_off + (size_t)slot * T;
+    DpVal* cur = lp.val[dist & 1] + job.val_off + slot;
     uint8_t* succ = lp.succ + job.succ_off + (live_before(here) + slot) * T;
     uint32_t picks[TM / 4];                                  // a byte per type, written together where T allows it
 #pragma unroll
@@ -344,7 +356,7 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
             double best_v = make_inf();
 #pragma unroll
             for (uint32_t g2 = 0; g2 < TM; ++g2) {
-                if (code[g2] == DP_NO_STATE || !(n[g2].sum < make_inf())) continue;
+                if (!(n[g2].sum < make_inf())) continue;     // (also where there is no such state)
                 const double t = add_rn(fb, c2x[d2[g2] * lp.lay.R + d]);
                 DpVal c;
                 c.sum = add_rn(t, n[g2].sum);
@@ -355,7 +367,7 @@ __device__ __forceinline__ void dp_vector(const DpLevelParams& lp, const DpLayou
                 if (pick == DP_NONE || val < best_v) { best = c; best_v = val; pick = g2; }
             }
         }
-        cur[g] = best;
+        store_val(cur + (size_t)g * job.slots, best);
         picks[g / 4] = (picks[g / 4] & ~(0xffu << (8 * (g % 4)))) | pick << (8 * (g % 4));
     }
     if (T == TM) {                                           // (every problem's successors start on a 64-byte line)
@@ -565,7 +577,7 @@ __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_finish_kernel(const __gr
         if (p != DP_NONE) {
             const uint32_t slot = live_slot(live, p) + (L.first_vec[p][lane] - live_vec(live, p));
             if (slot < live[0]) {
-                const DpVal v = lvl0[slot * T + lane];
+                const DpVal v = lvl0[(size_t)lane * job.slots + slot];
                 if (v.sum < make_inf()) {
                     mine_v = add_rn(add_rn(add_rn(v.sum, mul_rn(nb, v.mx)), v.sy), v.up);
                     mine = slot;

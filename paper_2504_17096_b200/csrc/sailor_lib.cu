@@ -2035,6 +2035,8 @@ static int plan_dp_impl(sailor_ctx* ctx, const sailor_space* s, const sailor_zon
                 job.val_off = val_off;
                 job.succ_off = succ_off;
                 job.config = pr.config; job.index = pr.index; job.layout = pr.place; job.P = info.l.P;
+                job.slots = info.max_live;
+                job._pad = 0;
                 val_off += pad8((uint64_t)info.max_live * T);
                 succ_off += pad64(info.total_live * T);
             }
