@@ -77,7 +77,7 @@ struct DpbFrame {                    // one call of the recursion: stage `level`
 };
 static_assert(SAILOR_T_MAX <= 8 && DP_BUDGET_P_MAX < 256, "a byte per type holds every count");
 
-struct DpbRoot {                     // what the walk from one type of stage 0 found
+struct DpbRoot {                     // what the walk from one type of stage 0 (and one of stage 1, see `split`) found
     double value;                    // +inf: no plan
     unsigned long long nodes;        // calls of the recursion; above the limit: given up
     uint8_t type[DP_BUDGET_P_MAX];
@@ -91,10 +91,11 @@ struct DpBudgetParams {
     const double* tabs;
     double* value;                   // indexed by problem index; +inf: no plan
     DpResult* results;
-    DpbRoot* roots;                  // [n_problems][T]
+    DpbRoot* roots;                  // [n_problems][T][split]
     unsigned long long* counters;    // [3] += problems given up, [4] += calls of the recursion
     DpTabLayout lay;
     uint32_t n_problems, T, p_max;
+    uint32_t split;                  // T: a walk per type of stage 1 as well; 1: one walk for all of them
     double limit;
     unsigned long long node_limit;
 };
@@ -103,12 +104,18 @@ __device__ __forceinline__ double dpb_value(double nb, double sum, double mx, do
     return add_rn(add_rn(add_rn(sum, mul_rn(nb, mx)), sy), up);
 }
 
-// A warp per (problem, type of stage 0).  The walk is one lane's: problems differ too much in what they try to share
+// A warp per (problem, type of stage 0, type of stage 1): what the first stage has to give to a type of the second does not
+// depend on the others, so the best of them is found afterwards (dp_budget_finish_kernel), the lowest among equals as in one walk.
+// The walk is one lane's: problems differ too much in what they try to share
 // instructions (a thread per problem ran a warp's 32 walks one after the other), and its stack sits in shared memory.
 // Bound by the latency of one chain of calls.  Workload 2, pipelines of up to eight stages, all orders, budget 1.2 x
-// cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.44 ms a call; a frame's counts as
+// cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.44 ms a call with a warp per first type; a frame's counts as
 // bytes of one word and the walk's tables brought near beforehand took its share from 459 to 408 us.
 constexpr int DPB_WARPS = 4;
+// Most walks that a search is split into.  Where few run at once the longest decides, and it gets shorter: workload 2, 1 344
+// problems of up to 8 stages 413 -> 345 us a call, 504 of up to 16 stages 3.33 -> 2.48 ms.  Where they no longer fit the device
+// together each costs its beginning: workload 3 up to 4 stages, 2.0e4 walks 118 -> 108 us, 8.2e4 121 -> 120, 3.3e5 164 -> 220.
+constexpr uint64_t DPB_SPLIT_WALKS = 1u << 16;
 constexpr size_t DPB_NEAR_BYTES = 16 * 1024;      // a block's four tables of this size leave L1 room for the rest
 
 __host__ __device__ inline size_t dpb_smem(uint32_t p_max) {
@@ -119,8 +126,9 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
     extern __shared__ __align__(16) unsigned char dyn[];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t unit = blockIdx.x * DPB_WARPS + warp, T = bp.T;
-    if (unit >= bp.n_problems * T) return;
-    const uint32_t x = unit / T, g0 = unit - x * T;
+    if (unit >= bp.n_problems * T * bp.split) return;
+    const uint32_t x = unit / (T * bp.split), walk = unit - x * T * bp.split, g0 = walk / bp.split, g1 = walk - g0 * bp.split;
+    const uint32_t g1_end = bp.split > 1 ? g1 + 1 : T;           // types of stage 1 that this walk tries
     DpbFrame* const fr = reinterpret_cast<DpbFrame*>(dyn) + warp * bp.p_max;
     double* const lb = reinterpret_cast<double*>(reinterpret_cast<DpbFrame*>(dyn) + DPB_WARPS * bp.p_max) + warp * (bp.p_max + 1);
     const DpProblem& pb = bp.problems[x];
@@ -135,6 +143,7 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
     const uint32_t R = h->R, Z = h->Z;
     const uint32_t* okv = reinterpret_cast<const uint32_t*>(tab + bp.lay.off_ok());
     if (!((okv[0] >> g0) & 1u)) return;
+    if (g1 && (P == 1 || !((okv[1] >> g1) & 1u))) return;
     const uint32_t p0 = pb.cap[0][g0] >= 1 ? 0u : pb.first_later[0][g0];     // by first fit from the first zone of the order
     if (p0 == DP_NONE) return;
     const uint64_t n_b = *reinterpret_cast<const uint64_t*>(tab + bp.lay.off_nb());
@@ -177,7 +186,7 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
     for (uint32_t j = P; j-- > 0;) lb[j] = add_rn(lb[j], lb[j + 1]);
     if (bp.limit < lb[0]) return;
 
-    unsigned long long nodes = 0;
+    unsigned long long nodes = g1 ? ~0ull : 0ull;                // (the call for the first stage counts once)
     bool gave_up = false;
     // result of the call that has just returned
     bool r_found = false;
@@ -208,12 +217,12 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
                 state = RESUME;
                 continue;
             }
-            f.g2 = 0;
+            f.g2 = (uint8_t)(level ? 0u : g1);
             state = NEXT_TYPE;
         }
         if (state == NEXT_TYPE) {
             bool placed = false;
-            while (f.g2 < T) {
+            for (const uint32_t g2_end = level ? T : g1_end; f.g2 < g2_end;) {
                 const uint32_t g2 = f.g2;
                 if ((okv[i + 1] >> g2) & 1u) {
                     // first fit: this zone while it has room for one more stage of the type, else the next that has
@@ -289,7 +298,7 @@ __global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_
     for (uint32_t j = 0; j < P; ++j) root.type[j] = fr[0].b_type[j];
 }
 
-// Per problem the best of its first stage's types (the lowest among equals), written out and simulated; a warp each.
+// Per problem the best of its walks (the lowest types among equals), written out and simulated; a warp each.
 __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_budget_finish_kernel(const __grid_constant__ DpBudgetParams bp) {
     __shared__ DpFinishWarp warps[DP_FINISH_WARPS];
     const uint32_t lane = threadIdx.x & 31, x = blockIdx.x * DP_FINISH_WARPS + (threadIdx.x >> 5);
@@ -297,11 +306,12 @@ __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_budget_finish_kernel(con
     DpFinishWarp& w = warps[threadIdx.x >> 5];
     const DpProblem& pb = bp.problems[x];
     const uint32_t T = bp.T, P = pb.P;
-    const DpbRoot* roots = bp.roots + (size_t)x * T;
+    const uint32_t n_roots = T * bp.split;
+    const DpbRoot* roots = bp.roots + (size_t)x * n_roots;
     unsigned long long nodes = 0;
     double best_v = make_inf();
     uint32_t best = DP_NONE;
-    for (uint32_t g = 0; g < T; ++g) {
+    for (uint32_t g = 0; g < n_roots; ++g) {
         nodes += roots[g].nodes;
         if (roots[g].value < best_v) { best_v = roots[g].value; best = g; }
     }

@@ -1775,9 +1775,12 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     DpTabLayout lay;
     lay.p_max = p_max; lay.T = T; lay.R = h.R;
     const size_t tab_bytes = (size_t)n_config * lay.stride() * sizeof(double);
-    const size_t total = padded(tab_bytes) + padded(n_problems * sizeof(DpResult)) + padded(n_problems * sizeof(DpProblem)) +
-                         padded(n_problems * T * sizeof(DpbRoot)) + padded(n_problems * sizeof(double)) +
-                         padded(40) + std::max<size_t>(padded(n_orders * sizeof(sailor_zone_order)), 4096);
+    const size_t others = padded(tab_bytes) + padded(n_problems * sizeof(DpResult)) + padded(n_problems * sizeof(DpProblem)) +
+                          padded(n_problems * sizeof(double)) + padded(40) + std::max<size_t>(padded(n_orders * sizeof(sailor_zone_order)), 4096);
+    // a walk per pair of first types, as long as they are few enough to run at once (and the workspace holds them)
+    uint32_t split = T;
+    if (n_problems * T * T > DPB_SPLIT_WALKS || others + padded(n_problems * T * T * sizeof(DpbRoot)) > workspace_bytes) split = 1;
+    const size_t total = others + padded(n_problems * T * split * sizeof(DpbRoot));
     if (total > workspace_bytes) return SAILOR_E_RANGE;
     {
         const int rc_mem = device_grow(ctx, &ctx->d_dp, &ctx->dp_bytes, total);
@@ -1787,7 +1790,7 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     double* d_tabs = bump.take<double>(tab_bytes / sizeof(double));
     DpResult* d_results = bump.take<DpResult>(n_problems);
     DpProblem* d_problems = bump.take<DpProblem>(n_problems);
-    DpbRoot* d_roots = bump.take<DpbRoot>(n_problems * T);
+    DpbRoot* d_roots = bump.take<DpbRoot>(n_problems * T * split);
     double* d_value = bump.take<double>(n_problems);
     unsigned long long* d_counters = bump.take<unsigned long long>(5);
     sailor_zone_order* d_orders = bump.take<sailor_zone_order>(n_orders);
@@ -1814,10 +1817,10 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     memset(&bp, 0, sizeof(bp));
     bp.blob = ctx->d_blob; bp.avail = ctx->d_avail; bp.sp = d; bp.problems = d_problems; bp.tabs = d_tabs;
     bp.value = d_value; bp.results = d_results; bp.roots = d_roots; bp.counters = d_counters; bp.lay = lay;
-    bp.n_problems = (uint32_t)n_problems; bp.T = T; bp.p_max = p_max;
+    bp.n_problems = (uint32_t)n_problems; bp.T = T; bp.p_max = p_max; bp.split = split;
     bp.limit = o->budget_usd_per_iter;
     bp.node_limit = 1ull << 24;
-    dp_budget_kernel<<<(uint32_t)((n_problems * T + DPB_WARPS - 1) / DPB_WARPS), 32 * DPB_WARPS, dpb_smem(p_max), ctx->stream>>>(bp);
+    dp_budget_kernel<<<(uint32_t)((n_problems * T * split + DPB_WARPS - 1) / DPB_WARPS), 32 * DPB_WARPS, dpb_smem(p_max), ctx->stream>>>(bp);
     CU(ctx, cudaGetLastError());
     dp_budget_finish_kernel<<<(uint32_t)((n_problems + DP_FINISH_WARPS - 1) / DP_FINISH_WARPS), DP_FINISH_THREADS, 0, ctx->stream>>>(bp);
     CU(ctx, cudaGetLastError());
