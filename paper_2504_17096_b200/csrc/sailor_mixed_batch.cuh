@@ -10,11 +10,11 @@
 //   a pipeline (of any of them): a walk over its plan's stages;
 //   a plan.
 // Bound: issue slots (45 % busy, 470 warp-instructions a plan, 24 of 32 lanes) and barriers between steps.  Random plans of
-// workload 5, 2.6e5 of them: 478 us with a warp per plan (1 424 warp-instructions), 250 us this way; 6.0e4 plans of workloads
-// 1, 2, 3, 5: 110 144 152 129 -> 56 80 83 63 us.  A warp with plans of its
-// own, 64 stages at a time without barriers, took 328 us (steps with a lane per plan ran a few lanes wide); the same with the
-// batch's plans in input order 281 (each batch waits for its deepest plan).  Two blocks of 384 threads 250 us, three of 256
-// 254, three of 320 271.
+// workload 5, 2.6e5 of them: 481 us with a warp per plan (1 424 warp-instructions), 245 us this way; 6.0e4 plans of workloads
+// 1, 2, 3, 5: 110 144 152 129 -> 56 79 82 63 us.  A warp with plans of its own, 64 stages at a time without barriers, took 328 us
+// (steps with a lane per plan ran a few lanes wide); blocks with the batch's plans in input order 281 (each batch waits for its
+// deepest plan).  Two blocks of 384 threads 250 us, three of 256 254, three of 320 271, two of 512 262; four steps of a walk side by
+// side instead of three, and the window's records asked for at its beginning, 250 -> 245.
 // Replica numbers are below 128 (MIXB_D_MAX), so the three group boundaries of a stage are bytes of a word, and the group
 // that replica k falls into is one subtraction and a population count.  Plans with more replicas, and those of a context
 // with larger nodes than the packed items can tell apart, are evaluated by a warp each (simulate_mixed_warp).
@@ -38,7 +38,7 @@ constexpr uint32_t MIXB_COUNTERS = 48 * MIXB_PLANS;          // GPUs taken per (
 constexpr uint32_t MIXB_PIPES = MIXB_ITEMS + MIXB_PLANS;
 constexpr uint32_t MIXB_PIPE_WORDS = (MIXB_PIPES + 31) / 32;
 constexpr uint32_t MIXB_GPUS_MAX = 8191;         // of an item, saturating: 13 bits; a node has fewer
-constexpr uint32_t MIXB_AHEAD = 3;               // steps of a walk whose loads are in flight together
+constexpr uint32_t MIXB_AHEAD = 4;               // steps of a walk whose loads are in flight together
 constexpr uint32_t MIXB_WIDE_WARPS = 4;          // warps that take a plan each
 static_assert(MIXB_ITEMS >= SAILOR_MIX_GROUPS_MAX * MIXB_P_MAX && MIXB_STAGES >= MIXB_P_MAX && MIXB_COUNTERS >= R_MAX, "a plan fits");
 static_assert(SAILOR_T_MAX * SAILOR_TP_MAX <= MIXB_THREADS && SAILOR_T_MAX <= 8 && MIXB_WARPS <= 32 && MIXB_PIPE_WORDS <= 32 && MIXB_PLANS <= 64, "bits and lanes");
@@ -276,6 +276,8 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
             } else {
                 P = P0;
                 rank = atomicAdd(&s.bin_n[MIXB_P_MAX - P], 1u);
+                for (uint32_t x = 0; x < 8 + 20 * P; x += 128)       // its stages are read some batches later
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(plans + (size_t)at * p.stride + x));
             }
         }
         __syncthreads();
