@@ -106,17 +106,17 @@ __device__ __forceinline__ double dpb_value(double nb, double sum, double mx, do
 
 // A warp per (problem, type of stage 0, type of stage 1): what the first stage has to give to a type of the second does not
 // depend on the others, so the best of them is found afterwards (dp_budget_finish_kernel), the lowest among equals as in one walk.
-// The walk is one lane's: problems differ too much in what they try to share
-// instructions (a thread per problem ran a warp's 32 walks one after the other), and its stack sits in shared memory.
+// The walk is one lane's: problems differ too much in what they try to share instructions (a thread per problem ran a warp's 32
+// walks one after the other), and its stack sits in shared memory.
 // Bound by the latency of one chain of calls.  Workload 2, pipelines of up to eight stages, all orders, budget 1.2 x
-// cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.44 ms a call with a warp per first type; a frame's counts as
-// bytes of one word and the walk's tables brought near beforehand took its share from 459 to 408 us.
-constexpr int DPB_WARPS = 4;
+// cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.44 ms a call with a warp per first type; a
+// frame's counts as bytes of one word and the walk's tables brought near beforehand took its share from 459 to 408 us.
+constexpr int DPB_WARPS = 1;                      // a block lasts as long as its longest walk: 342 -> 326 us, 2.48 -> 2.34 ms (4 -> 1)
 // Most walks that a search is split into.  Where few run at once the longest decides, and it gets shorter: workload 2, 1 344
-// problems of up to 8 stages 413 -> 345 us a call, 504 of up to 16 stages 3.33 -> 2.48 ms.  Where they no longer fit the device
+// problems of up to 8 stages 413 -> 345 us a call, 420 of up to 16 stages 3.33 -> 2.48 ms.  Where they no longer fit the device
 // together each costs its beginning: workload 3 up to 4 stages, 2.0e4 walks 118 -> 108 us, 8.2e4 121 -> 120, 3.3e5 164 -> 220.
 constexpr uint64_t DPB_SPLIT_WALKS = 1u << 16;
-constexpr size_t DPB_NEAR_BYTES = 16 * 1024;      // a block's four tables of this size leave L1 room for the rest
+constexpr size_t DPB_NEAR_BYTES = 16 * 1024;      // tables of up to this size are brought near before a walk
 
 __host__ __device__ inline size_t dpb_smem(uint32_t p_max) {
     return DPB_WARPS * (p_max * sizeof(DpbFrame) + (p_max + 1) * sizeof(double));
