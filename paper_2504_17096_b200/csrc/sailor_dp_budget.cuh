@@ -111,26 +111,29 @@ __device__ __forceinline__ double dpb_value(double nb, double sum, double mx, do
 // Bound by the latency of one chain of calls.  Workload 2, pipelines of up to eight stages, all orders, budget 1.2 x
 // cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.44 ms a call with a warp per first type; a
 // frame's counts as bytes of one word and the walk's tables brought near beforehand took its share from 459 to 408 us.
-constexpr int DPB_WARPS = 1;                      // a block lasts as long as its longest walk: 342 -> 326 us, 2.48 -> 2.34 ms (4 -> 1)
+// Warps of a block where the walks are many; where they are split a block is one warp and the kernel compiled for that (345 ->
+// 326 us and 2.48 -> 2.34 ms in the searches below; the kernel for four launched with one: no difference).
+constexpr uint32_t DPB_WARPS = 4;
 // Most walks that a search is split into.  Where few run at once the longest decides, and it gets shorter: workload 2, 1 344
 // problems of up to 8 stages 413 -> 345 us a call, 420 of up to 16 stages 3.33 -> 2.48 ms.  Where they no longer fit the device
 // together each costs its beginning: workload 3 up to 4 stages, 2.0e4 walks 118 -> 108 us, 8.2e4 121 -> 120, 3.3e5 164 -> 220.
 constexpr uint64_t DPB_SPLIT_WALKS = 1u << 16;
 constexpr size_t DPB_NEAR_BYTES = 16 * 1024;      // tables of up to this size are brought near before a walk
 
-__host__ __device__ inline size_t dpb_smem(uint32_t p_max) {
-    return DPB_WARPS * (p_max * sizeof(DpbFrame) + (p_max + 1) * sizeof(double));
+inline size_t dpb_smem(uint32_t p_max, uint32_t warps) {
+    return warps * (p_max * sizeof(DpbFrame) + (p_max + 1) * sizeof(double));
 }
 
-__global__ void __launch_bounds__(32 * DPB_WARPS) dp_budget_kernel(const __grid_constant__ DpBudgetParams bp) {
+template <uint32_t WARPS>
+__global__ void __launch_bounds__(32 * WARPS) dp_budget_kernel(const __grid_constant__ DpBudgetParams bp) {
     extern __shared__ __align__(16) unsigned char dyn[];
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t unit = blockIdx.x * DPB_WARPS + warp, T = bp.T;
+    const uint32_t lane = threadIdx.x & 31u, warp = WARPS > 1 ? threadIdx.x >> 5 : 0u;
+    const uint32_t unit = blockIdx.x * WARPS + warp, T = bp.T;
     if (unit >= bp.n_problems * T * bp.split) return;
     const uint32_t x = unit / (T * bp.split), walk = unit - x * T * bp.split, g0 = walk / bp.split, g1 = walk - g0 * bp.split;
     const uint32_t g1_end = bp.split > 1 ? g1 + 1 : T;           // types of stage 1 that this walk tries
     DpbFrame* const fr = reinterpret_cast<DpbFrame*>(dyn) + warp * bp.p_max;
-    double* const lb = reinterpret_cast<double*>(reinterpret_cast<DpbFrame*>(dyn) + DPB_WARPS * bp.p_max) + warp * (bp.p_max + 1);
+    double* const lb = reinterpret_cast<double*>(reinterpret_cast<DpbFrame*>(dyn) + WARPS * bp.p_max) + warp * (bp.p_max + 1);
     const DpProblem& pb = bp.problems[x];
     DpbRoot& root = bp.roots[unit];
     if (lane == 0) { root.value = make_inf(); root.nodes = 0; }

@@ -1820,7 +1820,8 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     bp.n_problems = (uint32_t)n_problems; bp.T = T; bp.p_max = p_max; bp.split = split;
     bp.limit = o->budget_usd_per_iter;
     bp.node_limit = 1ull << 24;
-    dp_budget_kernel<<<(uint32_t)((n_problems * T * split + DPB_WARPS - 1) / DPB_WARPS), 32 * DPB_WARPS, dpb_smem(p_max), ctx->stream>>>(bp);
+    if (split > 1) dp_budget_kernel<1><<<(uint32_t)(n_problems * T * split), 32, dpb_smem(p_max, 1), ctx->stream>>>(bp);
+    else dp_budget_kernel<DPB_WARPS><<<(uint32_t)((n_problems * T + DPB_WARPS - 1) / DPB_WARPS), 32 * DPB_WARPS, dpb_smem(p_max, DPB_WARPS), ctx->stream>>>(bp);
     CU(ctx, cudaGetLastError());
     dp_budget_finish_kernel<<<(uint32_t)((n_problems + DP_FINISH_WARPS - 1) / DP_FINISH_WARPS), DP_FINISH_THREADS, 0, ctx->stream>>>(bp);
     CU(ctx, cudaGetLastError());
