@@ -104,7 +104,7 @@ __global__ void compose_kernel(unsigned char* blob) {
 }
 
 // A warp per plan with mixed replicas (records `stride` bytes apart holding `max_stages` stages, read in place): all plans of up
-// to 32 stages of a small batch (DEEP = false; see mixb_least), or the deeper ones of any batch.  The launch for shallow plans,
+// to 32 stages of a small batch (DEEP = false; see mixb_takes), or the deeper ones of any batch.  The launch for shallow plans,
 // this or simulate_mixed_kernel, notes in `deep_seen` that there are deep ones; the DEEP launch that follows returns at once when
 // there are none (three times the scratch per warp).
 template <bool DEEP> constexpr uint32_t MIX_WARPS = DEEP ? 4 : 8;
@@ -1227,10 +1227,12 @@ int sailor_simulate_mixed_strided(sailor_ctx* ctx, const void* plans_v, uint64_t
         p.t_iter = d_t; p.peak_mem = d_m; p.cost = d_c; p.status = d_s;
         p.error = error; p.deep_seen = ctx->d_deep_seen; p.report_bad = report_bad;
         if (max_stages > MIXB_P_MAX) CU(ctx, cudaMemsetAsync(ctx->d_deep_seen, 0, sizeof(unsigned int), ctx->stream));
-        if (m < mixb_least(ctx->hdr))
-            simulate_mixed_each_kernel<false><<<(uint32_t)((m + MIX_WARPS<false> - 1) / MIX_WARPS<false>), 32 * MIX_WARPS<false>, mixed_smem<false>(ctx->hdr), ctx->stream>>>(p);
-        else
+        if (mixb_takes(ctx->hdr, m)) {
             simulate_mixed_kernel<<<(uint32_t)std::min<uint64_t>(m, MIXB_BLOCKS * (uint64_t)ctx->sm_count), MIXB_THREADS, mixb_smem(ctx->hdr), ctx->stream>>>(p);
+        } else {                                                 // (blocks take several plans per warp in larger batches)
+            const uint64_t blocks = (m + MIX_WARPS<false> - 1) / MIX_WARPS<false>, cap = (uint64_t)ctx->sm_count * 32;
+            simulate_mixed_each_kernel<false><<<(uint32_t)std::min(blocks, cap), 32 * MIX_WARPS<false>, mixed_smem<false>(ctx->hdr), ctx->stream>>>(p);
+        }
         CU(ctx, cudaGetLastError());
         if (max_stages > MIXB_P_MAX) {                           // the plans of more than 32 stages, if the first launch saw any
             const uint64_t blocks = (m + MIX_WARPS<true> - 1) / MIX_WARPS<true>, cap = (uint64_t)ctx->sm_count * 16;

@@ -9,15 +9,17 @@
 //   a sum or a maximum over a plan's items or stages, in order;
 //   a pipeline (of any of them): a walk over its plan's stages;
 //   a plan.
-// Bound: issue slots (45 % busy, 470 warp-instructions a plan, 24 of 32 lanes) and barriers between steps.  Random plans of
+// Bound: issue slots (44 % busy, 456 warp-instructions a plan, 25 of 32 lanes) and barriers between steps.  Random plans of
 // workload 5, 2.6e5 of them: 481 us with a warp per plan (1 424 warp-instructions), 245 us this way; 6.0e4 plans of workloads
 // 1, 2, 3, 5: 110 144 152 129 -> 56 79 82 63 us.  A warp with plans of its own, 64 stages at a time without barriers, took 328 us
 // (steps with a lane per plan ran a few lanes wide); blocks with the batch's plans in input order 281 (each batch waits for its
 // deepest plan).  Two blocks of 384 threads 250 us, three of 256 254, three of 320 271, two of 512 262; four steps of a walk side by
 // side instead of three, and the window's records asked for at its beginning, 250 -> 245.
 // Replica numbers are below 128 (MIXB_D_MAX), so the three group boundaries of a stage are bytes of a word, and the group
-// that replica k falls into is one subtraction and a population count.  Plans with more replicas, and those of a context
-// with larger nodes than the packed items can tell apart, are evaluated by a warp each (simulate_mixed_warp).
+// that replica k falls into is one subtraction and a population count.  Of a plan with more replicas only the order of its
+// boundaries matters to the pipelines: each takes its place among them as its number (96 at most), after two more barriers
+// where such a plan is among those evaluated together (6.0e4 plans of workload 3 with 256 replicas: 175 us by a warp each,
+// 117 this way; left to a few warps of the block 436).  Contexts with larger nodes than the packed items can tell apart keep a warp per plan.
 // Sums whose order of additions is part of the result are one thread's, term after term, as in simulate_mixed_warp.
 #pragma once
 
@@ -29,7 +31,7 @@ constexpr uint32_t MIXB_THREADS = 384;
 constexpr uint32_t MIXB_WARPS = MIXB_THREADS / 32;
 constexpr uint32_t MIXB_BLOCKS = 2;              // of an SM
 constexpr uint32_t MIXB_P_MAX = 32;              // stages of a plan
-constexpr uint32_t MIXB_D_MAX = 128;             // replicas of a stage
+constexpr uint32_t MIXB_D_MAX = 128;             // replicas of a stage whose numbers are kept; of more, boundaries are numbered in order
 constexpr uint32_t MIXB_WINDOW = 256;   // plans ordered at a time
 constexpr uint32_t MIXB_STAGES = MIXB_THREADS;   // stages evaluated at a time
 constexpr uint32_t MIXB_PLANS = 60;              // their plans, at most
@@ -37,11 +39,12 @@ constexpr uint32_t MIXB_ITEMS = 5 * MIXB_STAGES / 2;         // their items (sta
 constexpr uint32_t MIXB_COUNTERS = 48 * MIXB_PLANS;          // GPUs taken per (plan, zone, type)
 constexpr uint32_t MIXB_PIPES = MIXB_ITEMS + MIXB_PLANS;
 constexpr uint32_t MIXB_PIPE_WORDS = (MIXB_PIPES + 31) / 32;
+constexpr uint32_t MIXB_WIDE = 1u << 16;         // with a stage's items: its plan has more than MIXB_D_MAX replicas
 constexpr uint32_t MIXB_GPUS_MAX = 8191;         // of an item, saturating: 13 bits; a node has fewer
 constexpr uint32_t MIXB_AHEAD = 4;               // steps of a walk whose loads are in flight together
-constexpr uint32_t MIXB_WIDE_WARPS = 4;          // warps that take a plan each
 static_assert(MIXB_ITEMS >= SAILOR_MIX_GROUPS_MAX * MIXB_P_MAX && MIXB_STAGES >= MIXB_P_MAX && MIXB_COUNTERS >= R_MAX, "a plan fits");
 static_assert(SAILOR_T_MAX * SAILOR_TP_MAX <= MIXB_THREADS && SAILOR_T_MAX <= 8 && MIXB_WARPS <= 32 && MIXB_PIPE_WORDS <= 32 && MIXB_PLANS <= 64, "bits and lanes");
+static_assert((SAILOR_MIX_GROUPS_MAX - 1) * MIXB_P_MAX < MIXB_D_MAX, "a plan's boundaries, numbered from 1, fit where replica numbers do");
 
 struct alignas(16) MixbHead {        // of a plan of the window, deepest first
     double nb, xbytes;
@@ -70,17 +73,13 @@ struct alignas(16) MixbDigit {       // of a (zone, type)
     uint32_t avail, _pad;
 };
 struct alignas(16) MixbShared {
-    union {
-        struct {
-            MixbItem item[MIXB_ITEMS];
-            MixbStage stage[MIXB_STAGES];
-            double term[4][MIXB_STAGES];             // of a stage: transfer cost, synchronisation, update, memory (bytes)
-            double rate[MIXB_ITEMS];
-        };
-        MixScratch<MIXB_P_MAX> one[MIXB_WIDE_WARPS]; // plans that take a warp each
-    };
+    MixbItem item[MIXB_ITEMS];
+    MixbStage stage[MIXB_STAGES];
+    double term[4][MIXB_STAGES];                     // of a stage: transfer cost, synchronisation, update, memory (bytes)
+    double rate[MIXB_ITEMS];
     double pp[MIXB_PIPES];                           // times of the pipelines
     MixbHead head[MIXB_WINDOW];
+    double2 ring[MIXB_WINDOW];                       // 2 (D - 1), 2 (D - 1) / D of its plans
     MixbPlan plan[MIXB_PLANS];
     double total[MIXB_PLANS][5];                     // price rate, transfer cost, synchronisation, update, memory
     uint32_t counter[MIXB_COUNTERS];                 // zero between batches
@@ -88,16 +87,19 @@ struct alignas(16) MixbShared {
     MixbDigit digit[R_MAX];
     uint4 tp[SAILOR_T_MAX * SAILOR_TP_MAX];          // per (type, tp index): tp (bit 31: the type cannot host it), table entry, GPUs per node
     uint64_t capacity[SAILOR_T_MAX];
-    double2 ring[MIXB_D_MAX + 1];                    // 2 (D - 1), 2 (D - 1) / D
     uint64_t p2p[SAILOR_MBS_MAX];
     uint32_t mbs[SAILOR_MBS_MAX];
     uint32_t blocks[MIXB_P_MAX + 1];
     uint32_t pipe_bits[MIXB_PIPE_WORDS];             // bit t: a plan's first pipeline
     uint32_t bin_n[32], bin_plan[32], bin_stage[32]; // by depth, deepest first
     uint32_t warp_sum[MIXB_WARPS];
-    uint32_t n_listed, n_stages, n_pipes, n_wide, fit;
+    uint32_t n_listed, n_stages, n_pipes, fit;
+    // The block's share of the batch.  Here and not in registers, which the steps below need (3 to 5 % of a large batch).
+    uint64_t lo;                                     // first plan
+    const unsigned char* plans;                      // its record
+    uint32_t share, windows, pos, size;              // plans, windows left, the next one
+    uint64_t next_head[MIXB_WINDOW];                 // its records' heads, each for the thread that asked for it
     uint8_t has_pipes[MIXB_PLANS];                   // the plans that have any
-    uint8_t wide[MIXB_WINDOW];                       // places in the window
 };
 static_assert(MIXB_PLANS <= 256 && MIXB_WINDOW <= 256 && MIXB_WINDOW <= MIXB_THREADS, "bytes; a thread per plan");
 static_assert(offsetof(MixbShared, starts) % 16 == 0, "read as words of 16 bytes");
@@ -106,7 +108,12 @@ static_assert(offsetof(MixbShared, starts) % 16 == 0, "read as words of 16 bytes
 // fewer barriers.  us a call by a warp per plan and by blocks: workload 2, 1 plan 7.2 9.7, 17 12.3 10.3, 1 000 16.4 12.3; workload 5
 // 7.9 9.5, 11.3 10.5, 14.9 12.3.  In workload 1's context of one zone with two types plans are lighter: 17 9.7 10.2, 300 10.5
 // 10.9, 1 000 10.8 12.3, 2 500 12.3 12.3, 9 001 24.1 16.9.
-inline uint64_t mixb_least(const TabHdr& h) { return h.R <= 2 ? 2048 : 17; }
+// Contexts with nodes too large for the packed items keep it for batches of any size.
+inline bool mixb_takes(const TabHdr& h, uint64_t n) {
+    for (uint32_t g = 0; g < h.T; ++g)
+        if (h.gpn[g] >= MIXB_GPUS_MAX) return false;
+    return n >= (h.R <= 2 ? 2048 : 17);
+}
 
 struct MixbParams {
     const unsigned char* blob;
@@ -125,7 +132,6 @@ struct MixbParams {
     uint32_t stride, max_stages, report_bad;
     uint32_t n_blocks, T, Z, R, n_tp, n_mbs, chain_len, has_embed, has_head, piece_stride;
     uint32_t plans_max;              // plans at a time
-    uint32_t packed;                 // nodes are small enough for the packed items
 };
 
 inline size_t mixb_smem(const TabHdr& h) { return sizeof(MixbShared) + 2 * (size_t)h.R * h.n_mbs * sizeof(double); }
@@ -150,8 +156,6 @@ inline MixbParams mixb_params(const TabHdr& h, const unsigned char* blob) {
     p.has_embed = h.has_embed; p.has_head = h.has_head;
     p.piece_stride = h.T * h.n_tp * h.n_mbs * 2;
     p.plans_max = MIXB_COUNTERS / h.R < MIXB_PLANS ? MIXB_COUNTERS / h.R : MIXB_PLANS;
-    p.packed = 1;
-    for (uint32_t g = 0; g < h.T; ++g) p.packed &= h.gpn[g] < MIXB_GPUS_MAX ? 1u : 0u;
     return p;
 }
 
@@ -193,13 +197,29 @@ __device__ __noinline__ double mixb_poly_ring(const double* poly, uint32_t d, do
     return poly ? volume / poly_bw(poly + 4 * d, grad / (double)D) : without;
 }
 
-__device__ __noinline__ void mixb_one(const MixbParams& p, uint64_t j, MixScratch<MIXB_P_MAX>& scratch) {
-    const uint32_t lane = threadIdx.x & 31u;
-    TabView v;
-    v.bind(p.blob, p.blob);
-    const SimOut o = simulate_mixed_warp(v, p.blob, p.avail, *reinterpret_cast<const sailor_mixed_plan*>(p.plans + j * p.stride), scratch, lane);
-    if (lane == 0) mixb_store(p, j, o);
-    __syncwarp();
+// Boundaries of a stage as mixb_bounds packs them, numbered from 1 by their place among those of the plan's stages: the
+// places in the form of MixbStage::ends, their bits set in `starts`.  Equal ones have one place.
+__device__ __noinline__ uint32_t mixb_places(const uint2* of_plan, uint32_t P, uint2 mine, uint32_t* starts) {
+    const uint32_t b[3] = {mine.x & 0xffffu, mine.x >> 16, mine.y};
+    uint32_t place[3] = {1, 1, 1}, ends = 0;
+    for (uint32_t y = 0; y < P; ++y) {
+        const uint2 o = of_plan[y];
+#pragma unroll
+        for (uint32_t q = 0; q < 3; ++q) place[q] += ((o.x & 0xffffu) < b[q]) + ((o.x >> 16) < b[q]) + (o.y < b[q]);
+    }
+#pragma unroll
+    for (uint32_t q = 0; q < 3; ++q)
+        if (b[q] != 0xffffu) {
+            ends |= (place[q] | 0x80u) << (8 * q);
+            atomicOr(&starts[place[q] >> 5], 1u << (place[q] & 31u));
+        }
+    return ends;
+}
+
+// The replicas before a stage's second, third and fourth group, 16 bits each (0xffff: there is none; a valid plan has fewer).
+__device__ __forceinline__ uint2 mixb_bounds(const uint32_t (&g)[SAILOR_MIX_GROUPS_MAX], uint32_t ng) {
+    const uint32_t b1 = g[0] >> 16, b2 = b1 + (g[1] >> 16), b3 = b2 + (g[2] >> 16);
+    return make_uint2((ng > 1 ? b1 : 0xffffu) | (ng > 2 ? b2 & 0xffffu : 0xffffu) << 16, ng > 3 ? b3 & 0xffffu : 0xffffu);
 }
 
 __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kernel(const __grid_constant__ MixbParams p) {
@@ -210,15 +230,18 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     constexpr uint32_t NO_TIME = SAILOR_ST_INVALID | SAILOR_ST_BAD_RECORD;
 
-    // The block's share of the batch, a window at a time.
+    // The block's share of the batch, a window at a time (of equal parts).
     const uint64_t lo = p.n / gridDim.x * blockIdx.x + (blockIdx.x < p.n % gridDim.x ? blockIdx.x : p.n % gridDim.x);
     const uint32_t share = (uint32_t)(p.n / gridDim.x) + (blockIdx.x < p.n % gridDim.x ? 1u : 0u);
-    const unsigned char* const plans = p.plans + lo * p.stride;
-    uint32_t windows = (share + MIXB_WINDOW - 1) / MIXB_WINDOW, size = share / windows;       // (equal parts)
-    auto read_head = [&](uint32_t x, uint32_t n) {
-        return tid < n ? *reinterpret_cast<const uint64_t*>(plans + (size_t)(x + tid) * p.stride) : 0ull;
+    const unsigned char* const first_plan = p.plans + lo * p.stride;
+    const uint32_t n_windows = (share + MIXB_WINDOW - 1) / MIXB_WINDOW, first_size = share / n_windows;
+    auto read_head = [&](const unsigned char* plans, uint32_t x, uint32_t n) {     // (records start at multiples of 8 bytes)
+        if (tid < n)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(&s.next_head[tid])),
+                         "l"(plans + (size_t)(x + tid) * p.stride) : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    uint64_t next_head = read_head(0, size);
+    read_head(first_plan, 0, first_size);
     {                                                              // (all addresses and small tables are launch parameters: no load waits for another)
         for (uint32_t x = tid; x < p.R * p.n_mbs; x += MIXB_THREADS) {
             const uint32_t d = x / p.n_mbs, to = (x - d * p.n_mbs) * p.R + d;
@@ -240,26 +263,32 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
                                        (g * p.n_tp + ti) * p.n_mbs * 2, gpn, 0u);
             }
         }
+        if (tid == 0) {
+            s.plans = first_plan;
+            s.lo = lo;
+            s.pos = 0;
+            s.size = first_size;
+            s.windows = n_windows;
+            s.share = share;
+        }
         if (tid < SAILOR_T_MAX) s.capacity[tid] = p.capacity[tid];
         if (tid < p.n_mbs) { s.p2p[tid] = p.p2p[tid]; s.mbs[tid] = p.mbs_values[tid]; }
-        for (uint32_t x = tid + 1; x <= MIXB_D_MAX; x += MIXB_THREADS) {
-            const double steps = (double)(2 * (x - 1));
-            s.ring[x] = make_double2(steps, steps / (double)x);
-        }
         if (tid >= 1 && tid <= MIXB_P_MAX) { const uint32_t b = p.n_blocks / tid; s.blocks[tid] = b << 8 | (p.n_blocks - b * tid); }
         for (uint32_t x = tid; x < MIXB_COUNTERS; x += MIXB_THREADS) s.counter[x] = 0;
         if (tid < 2 * MIXB_PLANS) reinterpret_cast<uint4*>(s.starts)[tid] = make_uint4(1, 0, 0, 0);
     }
 
     uint32_t turn = 0;
-    for (uint32_t pos = 0; windows; --windows) {
+    __syncthreads();
+    for (;;) {
         // ---- a thread per plan: sort out and order, deepest first (a counting sort; any order gives the same results) ---------
-        const uint64_t head = next_head;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        const uint32_t size = s.size, pos = s.pos;
+        const uint64_t head = tid < size ? s.next_head[tid] : 0ull;
         const uint32_t P0 = (uint32_t)head & 0xff, mi = (uint32_t)(head >> 8) & 0xff, D = (uint32_t)(head >> 32) & 0xffff;
         const bool have = tid < size;
         const uint32_t at = pos + tid;
         if (tid < 32) s.bin_n[tid] = 0;
-        if (tid == 32) s.n_wide = 0;
         __syncthreads();
         uint32_t P = 0, rank = 0;
         if (have) {
@@ -268,16 +297,14 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
                 o.t_iter = o.cost = make_nan();
                 o.peak_mem = 0;
                 o.status = SAILOR_ST_BAD_RECORD;
-                mixb_store(p, lo + at, o);
+                mixb_store(p, s.lo + at, o);
             } else if (P0 > MIXB_P_MAX) {
                 *reinterpret_cast<volatile unsigned int*>(p.deep_seen) = 1u;             // left to the launch for deep plans
-            } else if (D > MIXB_D_MAX || !p.packed) {
-                s.wide[atomicAdd(&s.n_wide, 1u)] = (uint8_t)tid;
             } else {
                 P = P0;
                 rank = atomicAdd(&s.bin_n[MIXB_P_MAX - P], 1u);
                 for (uint32_t x = 0; x < 8 + 20 * P; x += 128)       // its stages are read some batches later
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(plans + (size_t)at * p.stride + x));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(s.plans + (size_t)at * p.stride + x));
             }
         }
         __syncthreads();
@@ -301,11 +328,10 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
                 if (n_b * dm != p.gbs) status0 = SAILOR_ST_INVALID;
             }
         }
-        const uint32_t window = pos;
-        pos += size;
-        if (windows > 1) size = (share - pos) / (windows - 1);
-        next_head = read_head(pos, windows > 1 ? size : 0u);
+        const uint32_t left = s.windows - 1, next_size = left ? (s.share - pos - size) / left : 0u;
+        read_head(s.plans, pos + size, next_size);
         __syncthreads();
+        if (tid == 0) { s.windows = left; s.pos = pos + size; s.size = next_size; }
         if (P) {
             const uint32_t bin = MIXB_P_MAX - P;
             MixbHead hd;
@@ -320,12 +346,14 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
             hd.status = status0;
             hd.at = at;
             s.head[s.bin_plan[bin] + rank] = hd;
+            const double steps = (double)(2 * (D - 1));
+            s.ring[s.bin_plan[bin] + rank] = make_double2(steps, steps / (double)D);
         }
         __syncthreads();
 
         // ---- as many plans at a time as have a stage per thread together --------------------------------------------------------
-        const uint32_t n_listed = s.n_listed, all_stages = s.n_stages;
-        for (uint32_t r0 = 0; r0 < n_listed; turn ^= 1u) {
+        for (uint32_t r0 = 0; r0 < s.n_listed; turn ^= 1u) {
+            const uint32_t n_listed = s.n_listed, all_stages = s.n_stages;
             uint32_t (*const starts)[MIXB_D_MAX / 32] = s.starts[turn];
             // how many of the plans from r0 on, and which plan a thread's stage belongs to: a lane per plan (and per plan + 32)
             const uint32_t base = s.head[r0].s0;
@@ -343,11 +371,11 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
             }
             // ---- a thread per stage: its record, checked -----------------------------------------------------------------------------
             const uint32_t rel = earlier + __popc(begins & (MIX_FULL >> (31u - lane))) - 1u;
-            uint32_t i = 0, zones = 0, ng = 0, ends = 0, tpi_least = 0, g[SAILOR_MIX_GROUPS_MAX] = {0, 0, 0, 0};
+            uint32_t i = 0, zones = 0, ng = 0, ends = 0, tpi_least = 0, wide = 0, g[SAILOR_MIX_GROUPS_MAX] = {0, 0, 0, 0};
             if (tid < n_stages) {
                 MixbHead& hd = s.head[r0 + rel];
                 i = tid - (hd.s0 - base);
-                const uint32_t* rec = reinterpret_cast<const uint32_t*>(plans + (size_t)hd.at * p.stride + 8) + 5 * i;
+                const uint32_t* rec = reinterpret_cast<const uint32_t*>(s.plans + (size_t)hd.at * p.stride + 8) + 5 * i;
                 const uint32_t w0 = rec[0], zone = w0 & 0xff, next = i + 1 < hd.P ? rec[5] & 0xff : zone;
 #pragma unroll
                 for (uint32_t q = 0; q < SAILOR_MIX_GROUPS_MAX; ++q) g[q] = rec[1 + q];
@@ -357,12 +385,14 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
                 for (uint32_t q = 0; q < SAILOR_MIX_GROUPS_MAX; ++q) refuse |= q < ng && ((g[q] & 0xff) >= p.T || ((g[q] >> 8) & 0xff) >= p.n_tp);
                 if (refuse) ng = 0;
                 uint32_t status = refuse ? SAILOR_ST_BAD_RECORD : 0u, run = 0, tp_least = 0xffffffffu;
+                wide = hd.D > MIXB_D_MAX ? MIXB_WIDE : 0u;
+                const uint32_t kept = wide ? 0u : MIXB_D_MAX;
                 zones = zone | (next < p.Z ? next : zone) << 8;                // (the next is checked by the thread that has that stage)
 #pragma unroll
                 for (uint32_t q = 0; q < SAILOR_MIX_GROUPS_MAX; ++q) {
                     if (q >= ng) break;
                     const uint32_t ty = g[q] & 0xff, ti = (g[q] >> 8) & 0xff, cn = g[q] >> 16, tpw = s.tp[ty * SAILOR_TP_MAX + ti].x;
-                    if (q && run < MIXB_D_MAX) {                             // (a valid plan's are)
+                    if (q && run < kept) {                                   // (a valid plan's are)
                         ends |= (run | 0x80u) << (8 * (q - 1));
                         atomicOr(&starts[rel][run >> 5], 1u << (run & 31u));
                     }
@@ -373,17 +403,27 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
                 if (run != hd.D) status |= SAILOR_ST_INVALID;
                 if (status) atomicOr(&hd.status, status);
             }
-            const uint32_t items = warp_scan(ng, lane);
+            const uint32_t items = warp_scan(ng + wide, lane);
             if (lane == 31) s.warp_sum[warp] = items;
             if (tid < MIXB_PIPE_WORDS) s.pipe_bits[tid] = 0;
             if (tid == 0) s.fit = np;
             __syncthreads();
             const uint32_t of_warp = lane < MIXB_WARPS ? s.warp_sum[lane] : 0u;
-            const uint32_t first = __reduce_add_sync(MIX_FULL, lane < warp ? of_warp : 0u) + items - ng;
-            if (__reduce_add_sync(MIX_FULL, of_warp) > MIXB_ITEMS) {         // fewer plans, then (the same for all threads; rare)
-                if (first + ng > MIXB_ITEMS) atomicMin(&s.fit, rel);
+            const uint32_t first = (__reduce_add_sync(MIX_FULL, lane < warp ? of_warp : 0u) + items - ng) % MIXB_WIDE;
+            const uint32_t all_items = __reduce_add_sync(MIX_FULL, of_warp);
+            if (all_items > MIXB_ITEMS) {                          // (the same for all threads; rare)
+                if (first + ng > MIXB_ITEMS) atomicMin(&s.fit, rel);         // fewer plans, then
+                uint2* const bounds = reinterpret_cast<uint2*>(s.term[0]);   // (not in use at this time)
+                if (all_items >= MIXB_WIDE && tid < n_stages) bounds[tid] = mixb_bounds(g, ng);
                 __syncthreads();
                 np = s.fit;
+                if (all_items >= MIXB_WIDE) {                      // numbers its boundaries by their order
+                    if (wide) {
+                        const MixbHead& hd = s.head[r0 + rel];
+                        ends = mixb_places(bounds + (hd.s0 - base), hd.P, bounds[tid], starts[rel]);
+                    }
+                    __syncthreads();
+                }
             }
             if (tid < MIXB_PLANS) *reinterpret_cast<uint4*>(s.starts[turn ^ 1u][tid]) = make_uint4(1, 0, 0, 0);
             if (warp == MIXB_WARPS - 1) {                          // counts the pipelines of the valid plans
@@ -426,7 +466,7 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
                         cross2 = __ldg(&p.zone2[(zone * p.Z + next) * p.n_mbs + (mr >> 1)]);
                         comm = mul_rn(hd.xbytes, __ldg(&p.egress[zone * p.Z + next]));
                     }
-                    const double2 rg = s.ring[D];
+                    const double2 rg = s.ring[r0 + rel];
                     const double steps = rg.x, volume = mul_rn(rg.y, grad);
                     const uint32_t left = P - i, inflight = left < hd.nb_cap ? left : hd.nb_cap;
                     double sync = 0.0, upd = 0.0;
@@ -576,20 +616,12 @@ __global__ void __launch_bounds__(MIXB_THREADS, MIXB_BLOCKS) simulate_mixed_kern
                         o.cost = add_rn(mul_rn(s.total[tid][0], o.t_iter), s.total[tid][1]);
                     }
                 }
-                mixb_store(p, lo + hd.at, o);
+                mixb_store(p, s.lo + hd.at, o);
             }
             for (uint32_t x = tid; x < np * p.R; x += MIXB_THREADS) s.counter[x] = 0;
             r0 += np;
         }
-
-        // ---- plans with many replicas: a warp each ---------------------------------------------------------------------------
-        const uint32_t n_wide = s.n_wide;
-        if (n_wide) {
-            __syncthreads();
-            if (warp < MIXB_WIDE_WARPS)
-                for (uint32_t x = warp; x < n_wide; x += MIXB_WIDE_WARPS) mixb_one(p, lo + window + s.wide[x], s.one[warp]);
-            __syncthreads();
-        }
+        if (s.windows == 0) break;
     }
 }
 

@@ -266,3 +266,122 @@ def test_mixed_batches_at_their_edges(D, stages, n, node):
         torch.cuda.synchronize()
     gpu = (dt.cpu().numpy(), dm.cpu().numpy().view(np.uint64), dc.cpu().numpy(), ds.cpu().numpy().view(np.uint32))
     assert_equal(gpu, (so, to, co, mo), f"D {D}, {stages} stages, {n} plans")
+
+
+def _run_on_device(w, packed):
+    """t_iter, peak_mem, cost and status of the records, which are copied to the device."""
+    import torch
+    n = packed.size
+    with Ctx(w) as cx:
+        d = torch.from_numpy(packed.view(np.uint8).reshape(n, packed.itemsize).copy()).cuda()
+        dt = torch.empty(n, dtype=torch.float64, device="cuda"); dc = torch.empty(n, dtype=torch.float64, device="cuda")
+        dm = torch.empty(n, dtype=torch.int64, device="cuda"); ds = torch.empty(n, dtype=torch.int32, device="cuda")
+        B.sailor_simulate_mixed_device(cx.ctx, d.data_ptr(), n, dt.data_ptr(), dm.data_ptr(), dc.data_ptr(), ds.data_ptr(),
+                                       record_bytes=packed.itemsize)
+        torch.cuda.synchronize()
+    return dt.cpu().numpy(), dm.cpu().numpy().view(np.uint64), dc.cpu().numpy(), ds.cpu().numpy().view(np.uint32)
+
+
+def _plans_of_degrees(rng, n, degrees, depths):
+    """Plans with a degree and a depth of the lists in turn, up to four groups a stage; some boundaries are equal to the
+    stage's before, some plans have a replica too many (or too few) or a group without any."""
+    plans = []
+    for j in range(n):
+        D, P, st = degrees[j % len(degrees)], depths[j // 3 % len(depths)], []
+        cuts = []
+        for i in range(P):
+            if not (cuts and rng.randint(0, 3) == 0):
+                near = rng.randint(0, 1)                             # boundaries among the first, or anywhere
+                cuts = sorted({rng.randint(1, min(D - 1, 9) if near else D - 1) for _ in range(rng.randint(0, 3))}) if D > 1 else []
+            b = [0] + cuts + [D]
+            if j % 13 == 7 and i == P // 2:
+                b[-1] += 1 if D < 65_535 else -1
+            groups = [(rng.randint(0, 3), rng.randint(0, 1), b[q + 1] - b[q]) for q in range(len(b) - 1)]
+            if j % 17 == 9 and i == P - 1 and len(groups) < 4:
+                groups.insert(0, (0, 0, 0))
+            st.append({"zone": rng.randint(0, 2) if j % 3 else 1, "groups": groups})
+        plans.append({"P": P, "mbs_idx": rng.randint(0, 2), "rc": j & 1, "D": D, "stages": st})
+    return plans
+
+
+@pytest.mark.parametrize("degrees,gbs,n,poly", [((4, 128, 129, 300), 4 * 412_800, 900, False),
+                                                ((129, 300), 4 * 412_800, 400, True),
+                                                ((65_535, 17, 257, 1), 4 * 65_535, 400, False),
+                                                ((256,), 1024, 30_000, False)])        # windows of a hundred plans
+def test_mixed_batches_of_unlike_degrees(degrees, gbs, n, poly):
+    """Degrees either side of 128 in one batch: of the larger ones a boundary is known by its place among the plan's."""
+    w = W.tiny(seed=52, n_types=4, n_zones=3, L=32, gbs=gbs, d_values=(4,), p_values=[32], tp_values=(1, 2))
+    w.gpus_per_node[...] = [4, 64, 700, 2]
+    w.avail[...] = 60_000
+    w.capacity[:] = np.uint64(1 << 44)
+    if poly:
+        w = W.with_bandwidth_polynomials(w, seed=3)
+    few = min(n, 900)
+    plans = _plans_of_degrees(W.SplitMix64(len(degrees) * 31 + n), few, degrees, [32, 1, 7, 31, 2, 16, 5])
+    so, to, co, mo = Oracle(w).simulate_mixed_batch(plans)
+    for D in degrees:
+        assert sum(1 for j, p in enumerate(plans) if p["D"] == D and not np.isnan(to[j])) > few // len(degrees) // 2
+    idx = np.arange(n) % few
+    gpu = _run_on_device(w, B.pack_mixed_plans(plans)[idx])
+    assert_equal(gpu, (so[idx], to[idx], co[idx], mo[idx]), f"degrees {degrees}")
+
+
+def test_mixed_batches_of_large_degrees_keep_pace():
+    """6e4 plans of 256 replicas take no longer than twice those of 128 (left to a few warps of a block they took four
+    times as long)."""
+    import torch
+    w = W.config3()
+    n, took = 60_000, {}
+    with Ctx(w) as cx:
+        outs = [torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(3)] + [torch.empty(n, dtype=torch.int32, device="cuda")]
+        batches = {}
+        for D in (128, 256):
+            w.d_values = [D]
+            packed = B.pack_mixed_plans(W.random_mixed_plans(w, 2000, seed=77), stages=32)[np.arange(n) % 2000]
+            batches[D] = torch.from_numpy(packed.view(np.uint8).reshape(n, -1).copy()).cuda()
+        for _ in range(6):                                           # in turn, the fastest of each
+            for D, d in batches.items():
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                torch.cuda.synchronize()
+                a.record()
+                for _ in range(5):
+                    B.sailor_simulate_mixed_device(cx.ctx, d.data_ptr(), n, *(o.data_ptr() for o in outs), record_bytes=d.shape[1])
+                b.record()
+                torch.cuda.synchronize()
+                took[D] = min(took.get(D, math.inf), a.elapsed_time(b))
+    assert took[256] <= 2.0 * took[128], took
+
+
+@pytest.mark.parametrize("what", ["items", "plans", "windows"])
+def test_mixed_batches_of_full_blocks(what):
+    """What a block meets only in large batches, two blocks an SM: twelve plans of 32 stages with four groups each have
+    1 536 items, more than the 960 that are evaluated together, so some are put back; plans of one stage, more than the 60
+    that are; and more plans than the 256 that are ordered together, degrees either side of 128 among them."""
+    import torch
+    blocks = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    rng = W.SplitMix64(len(what))
+    w = W.tiny(seed=54, n_types=4, n_zones=3, L=32, gbs=4 * 300 * 127, d_values=(4,), p_values=[32], tp_values=(1, 2))
+    w.gpus_per_node[...] = [4, 64, 700, 2]
+    w.avail[...] = 60_000
+    w.capacity[:] = np.uint64(1 << 44)
+    if what == "items":
+        n, plans = 25 * blocks + 7, []
+        for j in range(60):
+            st = []
+            for i in range(32):
+                b = [0] + sorted(rng.randint(0, 40) * 3 + q for q in (1, 2, 3)) + [127]
+                st.append({"zone": rng.randint(0, 2), "groups": [(rng.randint(0, 3), rng.randint(0, 1), b[q + 1] - b[q]) for q in range(4)]})
+            plans.append({"P": 32, "mbs_idx": rng.randint(0, 2), "rc": j & 1, "D": 127, "stages": st})
+    elif what == "plans":
+        n, plans = 150 * blocks + 11, _plans_of_degrees(rng, 901, [4, 127, 1], [1, 2, 1])
+    else:
+        n, plans = 600 * blocks + 13, _plans_of_degrees(rng, 2003, [4, 127, 300, 1], [3, 1, 6, 2])
+    so, to, co, mo = Oracle(w).simulate_mixed_batch(plans)
+    idx = np.arange(n) % len(plans)
+    packed = B.pack_mixed_plans(plans)[idx]
+    refused = np.arange(n) % 997 == 500
+    packed["stage"]["n_groups"][refused, 0] = 5
+    so, to, co, mo = so[idx], to[idx], co[idx], mo[idx]
+    so[refused], mo[refused], to[refused], co[refused] = B.ST_BAD_RECORD, 0, math.nan, math.nan
+    assert np.count_nonzero(~np.isnan(to)) > n // 2
+    assert_equal(_run_on_device(w, packed), (so, to, co, mo), what)
