@@ -6,7 +6,7 @@
 // slower the stage is charged again with that one and they are solved again, until the assumption holds,
 // nothing is left, or they have no plan.  The remaining limit is an argument of the recursion, so a state has no
 // single value and the tables of the unlimited search do not apply: every problem (configuration x zone order) is
-// walked depth-first with an explicit stack.  Problems, and the types of a problem's first stage, are independent, which
+// walked depth-first with an explicit stack.  Problems, and the types of a problem's first two stages, are independent, which
 // is where the parallelism is; a walk itself is sequential by nature (each call's limit depends on the charges before
 // it).  A branch is cut when what is left cannot pay even the cheapest conceivable rest of the
 // pipeline (every later stage alone on its cheapest GPUs, charged for its own compute time): such a branch has no
@@ -77,7 +77,7 @@ struct DpbFrame {                    // one call of the recursion: stage `level`
 };
 static_assert(SAILOR_T_MAX <= 8 && DP_BUDGET_P_MAX < 256, "a byte per type holds every count");
 
-struct DpbRoot {                     // what the walk from one type of stage 0 (and one of stage 1, see `split`) found
+struct DpbRoot {                     // what the walk from one type of stage 0 (and one of stage 1, where it is split) found
     double value;                    // +inf: no plan
     unsigned long long nodes;        // calls of the recursion; above the limit: given up
     uint8_t type[DP_BUDGET_P_MAX];
@@ -91,32 +91,49 @@ struct DpBudgetParams {
     const double* tabs;
     double* value;                   // indexed by problem index; +inf: no plan
     DpResult* results;
-    DpbRoot* roots;                  // [n_problems][T][split]
+    DpbRoot* roots;                  // [n_walks]
     unsigned long long* counters;    // [3] += problems given up, [4] += calls of the recursion
     DpTabLayout lay;
     uint32_t n_problems, T, p_max;
-    uint32_t split;                  // T: a walk per type of stage 1 as well; 1: one walk for all of them
+    uint32_t n_walks;
+    uint32_t per_length;             // problems of each pipeline length in the space's list: problem / per_length is its place there
+    uint32_t split;                  // bit: problems of this length have a walk per type of stage 1 as well
+    uint32_t first[SAILOR_NP_MAX];   // the first walk of a length (deep ones first; all in the problems' order where none is split)
     double limit;
     unsigned long long node_limit;
+
+    __host__ __device__ uint32_t walks_of_type(uint32_t length) const { return (split >> length) & 1u ? T : 1u; }
 };
+static_assert(SAILOR_NP_MAX <= 32, "a bit per length");
 
 __device__ __forceinline__ double dpb_value(double nb, double sum, double mx, double sy, double up) {
     return add_rn(add_rn(add_rn(sum, mul_rn(nb, mx)), sy), up);
 }
 
-// A warp per (problem, type of stage 0, type of stage 1): what the first stage has to give to a type of the second does not
-// depend on the others, so the best of them is found afterwards (dp_budget_finish_kernel), the lowest among equals as in one walk.
+// A warp per (problem, type of stage 0) or, where walks are split, (problem, type of stage 0, type of stage 1): what the first stage
+// has to give to a type of the second does not depend on the others, so the best of them is found afterwards
+// (dp_budget_finish_kernel), the lowest among equals as in one walk.
 // The walk is one lane's: problems differ too much in what they try to share instructions (a thread per problem ran a warp's 32
 // walks one after the other), and its stack sits in shared memory.
 // Bound by the latency of one chain of calls.  Workload 2, pipelines of up to eight stages, all orders, budget 1.2 x
 // cheapest (1 344 problems, up to 4 700 calls, hundreds of them in one walk): 2.76 -> 0.44 ms a call with a warp per first type; a
 // frame's counts as bytes of one word and the walk's tables brought near beforehand took its share from 459 to 408 us.
-// Warps of a block where the walks are many; where they are split a block is one warp and the kernel compiled for that (345 ->
-// 326 us and 2.48 -> 2.34 ms in the searches below; the kernel for four launched with one: no difference).
-constexpr uint32_t DPB_WARPS = 4;
-// Most walks that a search is split into.  Where few run at once the longest decides, and it gets shorter: workload 2, 1 344
-// problems of up to 8 stages 413 -> 345 us a call, 420 of up to 16 stages 3.33 -> 2.48 ms.  Where they no longer fit the device
-// together each costs its beginning: workload 3 up to 4 stages, 2.0e4 walks 118 -> 108 us, 8.2e4 121 -> 120, 3.3e5 164 -> 220.
+// Warps of a block.  Where walks are split a block is one warp and the kernel compiled for that: the longest walk decides then
+// (workload 2, up to 8 stages, and up to 16: 324 us and 13.7 ms a call; blocks of four 347 us and 14.7 ms, of two 361 us and 15.4
+// ms; frames of a block's warps side by side instead of each warp's own in one piece 367 us).
+template <bool SPLIT> constexpr uint32_t DPB_WARPS = SPLIT ? 1 : 4;
+// Where walks are split, by the length of their pipelines, deepest first: as long as the walks this adds, for all lengths split so
+// far, are at most DPB_SPLIT_WORTH times the calls that one walk from a first type can make without charging again.  A walk costs
+// about 0.5 ns (its block, and reading that there is nothing to do), and where the limit is tight most of them end at once; what a
+// long one saves grows with its calls.  us a call, unsplit and split, limits of 1.2 and 1.01 x the cheapest plan:
+//   workload 3, up to 4 stages (85 calls):  7 680 walks more 117 97, 79 80; 11 520 more 119 102, 84 83; 19 200 more 128 111, 90 93
+//   workload 3, up to 3 stages (21 calls):  3 840 more 73 70, 65 66; 15 360 more 86 85, 75 80
+//   workload 5, up to 4 stages: the deepest (259 calls), 14 400 more 97 85, 82 80; with the second (43 calls), 28 800 more 89, 87
+//   eight types, up to 3 stages (73 calls): 16 128 more 153 102
+// All lengths split (workload 3, up to 2 stages, 51 000 walks): 75 -> 95 us.  Fewer than DPB_SPLIT_CALLS calls (two types, three
+// stages: 7; three types: 13) are not worth a walk of their own; two types, four stages, 15 calls: 89 -> 76 us.
+constexpr uint64_t DPB_SPLIT_CALLS = 15, DPB_SPLIT_WORTH = 224;
+// Most walks of a search that splits any (their records' memory).
 constexpr uint64_t DPB_SPLIT_WALKS = 1u << 16;
 constexpr size_t DPB_NEAR_BYTES = 16 * 1024;      // tables of up to this size are brought near before a walk
 
@@ -124,14 +141,21 @@ inline size_t dpb_smem(uint32_t p_max, uint32_t warps) {
     return warps * (p_max * sizeof(DpbFrame) + (p_max + 1) * sizeof(double));
 }
 
-template <uint32_t WARPS>
-__global__ void __launch_bounds__(32 * WARPS) dp_budget_kernel(const __grid_constant__ DpBudgetParams bp) {
+template <bool SPLIT>
+__global__ void __launch_bounds__(32 * DPB_WARPS<SPLIT>) dp_budget_kernel(const __grid_constant__ DpBudgetParams bp) {
     extern __shared__ __align__(16) unsigned char dyn[];
+    constexpr uint32_t WARPS = DPB_WARPS<SPLIT>;
     const uint32_t lane = threadIdx.x & 31u, warp = WARPS > 1 ? threadIdx.x >> 5 : 0u;
     const uint32_t unit = blockIdx.x * WARPS + warp, T = bp.T;
-    if (unit >= bp.n_problems * T * bp.split) return;
-    const uint32_t x = unit / (T * bp.split), walk = unit - x * T * bp.split, g0 = walk / bp.split, g1 = walk - g0 * bp.split;
-    const uint32_t g1_end = bp.split > 1 ? g1 + 1 : T;           // types of stage 1 that this walk tries
+    if (unit >= bp.n_walks) return;
+    uint32_t length = 0, split = SPLIT ? bp.walks_of_type(0) : 1u, first = 0;
+    if (SPLIT) {
+        while (unit - bp.first[length] >= bp.per_length * T * split) split = bp.walks_of_type(++length);
+        first = bp.first[length];
+    }
+    const uint32_t nth = (unit - first) / split, of_length = nth / T, x = length * bp.per_length + of_length;
+    const uint32_t g0 = nth - of_length * T, g1 = unit - first - nth * split;
+    const uint32_t g1_end = split > 1 ? g1 + 1 : T;              // types of stage 1 that this walk tries
     DpbFrame* const fr = reinterpret_cast<DpbFrame*>(dyn) + warp * bp.p_max;
     double* const lb = reinterpret_cast<double*>(reinterpret_cast<DpbFrame*>(dyn) + WARPS * bp.p_max) + warp * (bp.p_max + 1);
     const DpProblem& pb = bp.problems[x];
@@ -309,8 +333,8 @@ __global__ void __launch_bounds__(DP_FINISH_THREADS) dp_budget_finish_kernel(con
     DpFinishWarp& w = warps[threadIdx.x >> 5];
     const DpProblem& pb = bp.problems[x];
     const uint32_t T = bp.T, P = pb.P;
-    const uint32_t n_roots = T * bp.split;
-    const DpbRoot* roots = bp.roots + (size_t)x * n_roots;
+    const uint32_t length = x / bp.per_length, n_roots = T * bp.walks_of_type(length);
+    const DpbRoot* roots = bp.roots + bp.first[length] + (size_t)(x - length * bp.per_length) * n_roots;
     unsigned long long nodes = 0;
     double best_v = make_inf();
     uint32_t best = DP_NONE;

@@ -1764,7 +1764,7 @@ int dense_fits(const sailor_ctx* ctx, uint32_t P, uint64_t need, const sailor_zo
 
 }  // namespace
 
-// The recursion steered by the budget (Sec. 4.2.3): a warp per problem and type of its first stage, depth first.
+// The recursion steered by the budget (Sec. 4.2.3): a warp per problem and type of its first stage, or of its first two, depth first.
 static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor_zone_order* orders, uint32_t n_orders,
                                const sailor_objective* o, uint64_t workspace_bytes, uint32_t k, sailor_dp_result* topk,
                                uint32_t* n_found, sailor_dp_stats* stats) {
@@ -1779,11 +1779,35 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     const size_t tab_bytes = (size_t)n_config * lay.stride() * sizeof(double);
     const size_t others = padded(tab_bytes) + padded(n_problems * sizeof(DpResult)) + padded(n_problems * sizeof(DpProblem)) +
                           padded(n_problems * sizeof(double)) + padded(40) + std::max<size_t>(padded(n_orders * sizeof(sailor_zone_order)), 4096);
-    // a walk per pair of first types, as long as they are few enough to run at once (and the workspace holds them)
-    uint32_t split = T;
-    if (n_problems * T * T > DPB_SPLIT_WALKS || others + padded(n_problems * T * T * sizeof(DpbRoot)) > workspace_bytes) split = 1;
-    const size_t total = others + padded(n_problems * T * split * sizeof(DpbRoot));
+    DpBudgetParams bp;
+    memset(&bp, 0, sizeof(bp));
+    bp.T = T; bp.p_max = p_max;
+    const uint64_t per_length = n_problems / d.n_p, per_first = per_length * T;
+    // A length has a walk per pair of first types where that is worth it and the workspace holds them all.
+    uint8_t order[SAILOR_NP_MAX];
+    for (uint32_t j = 0; j < d.n_p; ++j) order[j] = (uint8_t)j;
+    std::sort(order, order + d.n_p, [&](uint8_t a, uint8_t b) { return d.p_values[a] != d.p_values[b] ? d.p_values[a] > d.p_values[b] : a < b; });
+    uint64_t extra = 0;
+    for (uint32_t x = 0; x < d.n_p; ++x) {
+        uint64_t calls = 1;                                  // that a walk from one type of stage 0 can make without charging again
+        for (uint32_t i = 1; i < d.p_values[order[x]] && calls < (1u << 20); ++i) calls = calls * T + 1;
+        if (T < 2 || calls < DPB_SPLIT_CALLS || extra + per_first * (T - 1) > DPB_SPLIT_WORTH * calls) continue;
+        extra += per_first * (T - 1);
+        bp.split |= 1u << order[x];
+    }
+    uint64_t n_walks = n_problems * T + extra;
+    if (n_walks > DPB_SPLIT_WALKS || others + padded(n_walks * sizeof(DpbRoot)) > workspace_bytes) {
+        bp.split = 0;
+        n_walks = n_problems * T;
+    }
+    if (!bp.split)
+        for (uint32_t j = 0; j < d.n_p; ++j) order[j] = (uint8_t)j;
+    const size_t total = others + padded(n_walks * sizeof(DpbRoot));
     if (total > workspace_bytes) return SAILOR_E_RANGE;
+    bp.n_walks = (uint32_t)n_walks;
+    bp.per_length = (uint32_t)per_length;
+    for (uint32_t x = 1; x < d.n_p; ++x)
+        bp.first[order[x]] = bp.first[order[x - 1]] + (uint32_t)per_first * bp.walks_of_type(order[x - 1]);
     {
         const int rc_mem = device_grow(ctx, &ctx->d_dp, &ctx->dp_bytes, total);
         if (rc_mem) return rc_mem;
@@ -1792,7 +1816,7 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
     double* d_tabs = bump.take<double>(tab_bytes / sizeof(double));
     DpResult* d_results = bump.take<DpResult>(n_problems);
     DpProblem* d_problems = bump.take<DpProblem>(n_problems);
-    DpbRoot* d_roots = bump.take<DpbRoot>(n_problems * T * split);
+    DpbRoot* d_roots = bump.take<DpbRoot>(n_walks);
     double* d_value = bump.take<double>(n_problems);
     unsigned long long* d_counters = bump.take<unsigned long long>(5);
     sailor_zone_order* d_orders = bump.take<sailor_zone_order>(n_orders);
@@ -1815,15 +1839,16 @@ static int plan_dp_budget_impl(sailor_ctx* ctx, const SpaceDesc& d, const sailor
         ctx->d_blob, ctx->d_avail, d, d_orders, n_orders, (uint32_t)n_problems, d_problems, d_counters);
     CU(ctx, cudaGetLastError());
     ++launches;
-    DpBudgetParams bp;
-    memset(&bp, 0, sizeof(bp));
     bp.blob = ctx->d_blob; bp.avail = ctx->d_avail; bp.sp = d; bp.problems = d_problems; bp.tabs = d_tabs;
     bp.value = d_value; bp.results = d_results; bp.roots = d_roots; bp.counters = d_counters; bp.lay = lay;
-    bp.n_problems = (uint32_t)n_problems; bp.T = T; bp.p_max = p_max; bp.split = split;
+    bp.n_problems = (uint32_t)n_problems;
     bp.limit = o->budget_usd_per_iter;
     bp.node_limit = 1ull << 24;
-    if (split > 1) dp_budget_kernel<1><<<(uint32_t)(n_problems * T * split), 32, dpb_smem(p_max, 1), ctx->stream>>>(bp);
-    else dp_budget_kernel<DPB_WARPS><<<(uint32_t)((n_problems * T + DPB_WARPS - 1) / DPB_WARPS), 32 * DPB_WARPS, dpb_smem(p_max, DPB_WARPS), ctx->stream>>>(bp);
+    auto launch = [&](auto kernel, uint32_t warps) {
+        kernel<<<(bp.n_walks + warps - 1) / warps, 32 * warps, dpb_smem(p_max, warps), ctx->stream>>>(bp);
+    };
+    if (bp.split) launch(dp_budget_kernel<true>, DPB_WARPS<true>);
+    else launch(dp_budget_kernel<false>, DPB_WARPS<false>);
     CU(ctx, cudaGetLastError());
     dp_budget_finish_kernel<<<(uint32_t)((n_problems + DP_FINISH_WARPS - 1) / DP_FINISH_WARPS), DP_FINISH_THREADS, 0, ctx->stream>>>(bp);
     CU(ctx, cudaGetLastError());

@@ -177,3 +177,43 @@ def test_first_fit_tables_up_to_the_limits(orders):
     with Ctx(w) as cx:
         res, st = B.sailor_plan_dp(cx.ctx, cx.space, orders, 16, budget=limit, budget_loop=True)
         assert_same(res, st, want, solved, over, w, orders, 16, str(orders))
+
+
+def _limit(w, orders, factor):
+    """A limit relative to the cheapest of the plans that the unlimited recursion finds."""
+    o = Oracle(w)
+    costs = [o.simulate(r["plan"]).cost for c in configs_of(w) for r in [o.solve_dp(*c, orders[0])] if r is not None]
+    return factor * min(costs)
+
+
+def _walked():
+    eight = W.tiny(seed=14, n_types=8, n_zones=2, L=12, p_values=[3, 1, 2], d_values=(1, 2, 4), tp_values=(1, 2), mbs_values=(1, 2, 4))
+    eight.avail[...] = eight.avail * 3
+    yield eight, [[1, 0], [0]], True                             # the deepest length has walks of its own, the list is not in order
+    many = W.tiny(seed=14, n_types=8, n_zones=4, L=12, p_values=[1, 3], d_values=(1, 2, 4), tp_values=(1, 2), mbs_values=(1, 2, 4))
+    many.avail[...] = many.avail * 3
+    yield many, B.all_zone_orders(4)[:40], False                 # too many problems for that
+    yield W.tiny(seed=9, n_types=3, n_zones=2, L=8, p_values=[4, 8, 2, 5], d_values=(1, 2)), [[0, 1], [1]], True
+    yield W.tiny(seed=3, n_types=3, n_zones=2, L=6, p_values=[2, 1]), [[0, 1], [1, 0], [1]], False         # walks of a few calls
+
+
+@pytest.mark.parametrize("w,orders,split", list(_walked()), ids=["eight-types", "many-problems", "list-out-of-order", "shallow"])
+def test_budget_walks_split_and_whole(w, orders, split):
+    """Long walks are split by the second stage's type where that adds few walks and the workspace holds their records: with a
+    byte less than it took, the same plans from whole walks, or a refusal where walks were whole already."""
+    o = Oracle(w)
+    limit = _limit(w, orders, 1.5)
+    want, solved, over = oracle_limited(w, o, orders, limit)
+    assert len(want) > 8
+    with Ctx(w) as cx:
+        res, st = B.sailor_plan_dp(cx.ctx, cx.space, orders, 16, budget=limit, budget_loop=True)
+        assert_same(res, st, want, solved, over, w, orders, 16, "first")
+        if not split:
+            with pytest.raises(B.SailorError) as e:
+                B.sailor_plan_dp(cx.ctx, cx.space, orders, 16, int(st.workspace_used) - 1, budget=limit, budget_loop=True)
+            assert e.value.code == B.E_RANGE
+            return
+        whole, st2 = B.sailor_plan_dp(cx.ctx, cx.space, orders, 16, int(st.workspace_used) - 1, budget=limit, budget_loop=True)
+        assert_same(whole, st2, want, solved, over, w, orders, 16, "whole walks")
+        assert st2.workspace_used < st.workspace_used and st2.n_states == st.n_states
+        assert [bytes(r) for r in whole] == [bytes(r) for r in res]
