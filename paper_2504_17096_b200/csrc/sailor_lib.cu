@@ -1227,7 +1227,7 @@ int sailor_simulate_mixed_strided(sailor_ctx* ctx, const void* plans_v, uint64_t
         p.t_iter = d_t; p.peak_mem = d_m; p.cost = d_c; p.status = d_s;
         p.error = error; p.deep_seen = ctx->d_deep_seen; p.report_bad = report_bad;
         if (max_stages > MIXB_P_MAX) CU(ctx, cudaMemsetAsync(ctx->d_deep_seen, 0, sizeof(unsigned int), ctx->stream));
-        if (mixb_takes(ctx->hdr, m)) {
+        if (mixb_takes(ctx->hdr, max_stages, m)) {
             simulate_mixed_kernel<<<(uint32_t)std::min<uint64_t>(m, MIXB_BLOCKS * (uint64_t)ctx->sm_count), MIXB_THREADS, mixb_smem(ctx->hdr), ctx->stream>>>(p);
         } else {                                                 // (blocks take several plans per warp in larger batches)
             const uint64_t blocks = (m + MIX_WARPS<false> - 1) / MIX_WARPS<false>, cap = (uint64_t)ctx->sm_count * 32;

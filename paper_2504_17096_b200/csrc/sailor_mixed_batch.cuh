@@ -104,15 +104,22 @@ struct alignas(16) MixbShared {
 static_assert(MIXB_PLANS <= 256 && MIXB_WINDOW <= 256 && MIXB_WINDOW <= MIXB_THREADS, "bytes; a thread per plan");
 static_assert(offsetof(MixbShared, starts) % 16 == 0, "read as words of 16 bytes");
 
-// Batches of fewer plans are evaluated by a warp per plan (simulate_mixed_each_kernel): its blocks lay out fewer tables and pass
-// fewer barriers.  us a call by a warp per plan and by blocks: workload 2, 1 plan 7.2 9.7, 17 12.3 10.3, 1 000 16.4 12.3; workload 5
-// 7.9 9.5, 11.3 10.5, 14.9 12.3.  In workload 1's context of one zone with two types plans are lighter: 17 9.7 10.2, 300 10.5
-// 10.9, 1 000 10.8 12.3, 2 500 12.3 12.3, 9 001 24.1 16.9.
-// Contexts with nodes too large for the packed items keep it for batches of any size.
-inline bool mixb_takes(const TabHdr& h, uint64_t n) {
+// Other batches are evaluated by a warp per plan (simulate_mixed_each_kernel): its blocks lay out fewer tables and pass fewer
+// barriers.  What decides is how deep plans can be: a record's room and the model's blocks bound it.  us a call by a warp per
+// plan and by blocks, three types, plans of up to so many stages, degrees up to 32 (up to 128):
+//    4:  17 6.3 9.3 (6.7 9.3), 1 000 7.2 10.3 (8.2 10.3), 3 500 8.3 10.3 (8.3 10.3)
+//    8:  17 8.3 10.3 (8.2 10.3), 2 047 8.3 10.3 (8.3 10.3), 3 500 9.2 10.3 (10.3 10.3)
+//   12: 100 8.3 10.3 (8.3 10.3), 1 000 8.3 10.3 (10.3 10.3), 2 047 10.3 10.5 (10.3 10.3)
+//   16: 100 9.3 10.3 (10.3 10.3), 1 500 10.3 10.7 (11.0 10.8), 2 500 10.8 11.3 (12.4 11.3)
+//   24: 300 10.3 10.3 (14.4 10.6), 1 000 10.7 12.3 (14.9 12.3), 2 500 12.4 12.4 (16.4 12.4)
+//   32:  17 12.4 10.3 (16.4 10.3), 1 000 12.4 12.4 (18.3 12.4), 2 500 14.4 12.4 (20.5 12.7)
+// Workload 1 (24 blocks, degrees up to 32, one zone with two types) keeps a warp per plan for longer.  Contexts with nodes too
+// large for the packed items keep it for batches of any size.
+inline bool mixb_takes(const TabHdr& h, uint32_t max_stages, uint64_t n) {
     for (uint32_t g = 0; g < h.T; ++g)
         if (h.gpn[g] >= MIXB_GPUS_MAX) return false;
-    return n >= (h.R <= 2 ? 2048 : 17);
+    const uint32_t deepest = max_stages < h.n_blocks ? max_stages : h.n_blocks;
+    return n >= (deepest <= 8 ? 4096 : deepest <= 16 ? 1536 : deepest <= 24 && h.R <= 2 ? 2048 : 17);
 }
 
 struct MixbParams {

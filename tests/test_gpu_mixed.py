@@ -226,16 +226,16 @@ def test_mixed_interval_edges(D, stages):
     assert np.array_equal(t, to, equal_nan=True) and np.array_equal(c, co, equal_nan=True)
 
 
-@pytest.mark.parametrize("D,stages,n,node", [(6, 3, 16, 8), (6, 3, 17, 8),           # either side of the smallest batch of the batch kernel
-                                             (127, 32, 700, 8), (128, 32, 700, 8),   # the largest replica numbers that fit its bytes; more
-                                             (129, 32, 40, 8),                       # items than a batch has room for (four groups a stage)
+@pytest.mark.parametrize("D,stages,n,node", [(6, 3, 16, 8), (6, 3, 17, 8),           # either side of the smallest batch that blocks take
+                                             (127, 32, 700, 8), (128, 32, 700, 8),   # the largest replica numbers that are kept,
+                                             (129, 32, 40, 8),                       # and boundaries numbered in order
                                              (4, 8, 3000, 8190), (4, 8, 300, 8191),  # the largest node its items can tell apart, and a larger one
-                                             (3, 1, 5000, 8), (2, 33, 50, 8)])       # one stage: the most plans at a time; deep plans
+                                             (3, 1, 5000, 8), (2, 33, 50, 8)])       # one stage; deep plans, and shallow ones among them
 def test_mixed_batches_at_their_edges(D, stages, n, node):
-    """Plans of one depth (and some shallower), most stages with four groups, refused records in between: the same bits as
-    the oracle, and the refused ones flagged."""
+    """Plans of one depth (and some shallower) in records of 32 stages and more, most stages with four groups, refused records
+    in between: the same bits as the oracle, and the refused ones flagged."""
     import torch
-    w = W.tiny(seed=51, n_types=4, n_zones=3, L=max(stages, 4), gbs=D * 4, d_values=(D,), p_values=[stages])
+    w = W.tiny(seed=51, n_types=4, n_zones=3, L=max(stages, 32), gbs=D * 4, d_values=(D,), p_values=[stages])
     w.gpus_per_node[...] = [4, node, 700, 2]
     rng = W.SplitMix64(D * 977 + stages)
     plans = []
@@ -249,7 +249,7 @@ def test_mixed_batches_at_their_edges(D, stages, n, node):
                        "groups": [(rng.randint(0, 3), rng.randint(0, 2), b[q + 1] - b[q]) for q in range(len(b) - 1)]})
         plans.append({"P": P, "mbs_idx": rng.randint(0, 2), "rc": j & 1, "D": D, "stages": st})
     so, to, co, mo = Oracle(w).simulate_mixed_batch(plans)
-    packed = B.pack_mixed_plans(plans)
+    packed = B.pack_mixed_plans(plans, stages=max(32, stages + stages % 2))
     refused = np.arange(n) % 11 == 5
     for j in np.flatnonzero(refused):
         if j % 2:
@@ -385,3 +385,17 @@ def test_mixed_batches_of_full_blocks(what):
     so[refused], mo[refused], to[refused], co[refused] = B.ST_BAD_RECORD, 0, math.nan, math.nan
     assert np.count_nonzero(~np.isnan(to)) > n // 2
     assert_equal(_run_on_device(w, packed), (so, to, co, mo), what)
+
+
+@pytest.mark.parametrize("stages,blocks,types,n", [(8, 8, 3, 4095), (8, 8, 3, 4096), (8, 40, 3, 4096), (32, 8, 3, 4095),   # room, or the model, for few stages
+                                                   (16, 16, 3, 1535), (10, 40, 3, 1536), (32, 16, 3, 1536),
+                                                   (24, 40, 2, 2047), (24, 24, 2, 2048), (32, 40, 2, 17), (24, 24, 3, 17)])
+def test_mixed_batches_either_side_of_their_kernels(stages, blocks, types, n):
+    """How many plans blocks take depends on how deep they can be, the records' room and the model's blocks: same bits on
+    both sides."""
+    w = W.tiny(seed=57, n_types=types, n_zones=1 if types == 2 else 2, L=blocks, gbs=768, d_values=(1, 3, 16, 128),
+               p_values=[p for p in (1, 2, 5, 8, 13, 24, 32) if p <= min(stages, blocks)], tp_values=(1, 2))
+    w.avail[...] = 60_000
+    w.capacity[:] = np.uint64(1 << 44)
+    plans = W.random_mixed_plans(w, n, seed=n, p_max=min(stages, blocks))
+    assert_equal(_run_on_device(w, B.pack_mixed_plans(plans, stages=stages)), Oracle(w).simulate_mixed_batch(plans), f"{stages} of {blocks}")
