@@ -112,7 +112,7 @@ template <bool DEEP> constexpr uint32_t MIX_STAGES = DEEP ? SAILOR_MIX_P_MAX : M
 
 template <bool DEEP>
 __global__ void __launch_bounds__(32 * MIX_WARPS<DEEP>, 4)
-simulate_mixed_each_kernel(const __grid_constant__ MixbParams p) {
+simulate_mixed_each_kernel(const __grid_constant__ MixbCall p) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ uint64_t mbar;
     if (DEEP && *reinterpret_cast<const volatile unsigned int*>(p.deep_seen) == 0) return;
@@ -1221,14 +1221,14 @@ int sailor_simulate_mixed_strided(sailor_ctx* ctx, const void* plans_v, uint64_t
     DeviceGuard guard(ctx->device);
     auto launch = [ctx, record_bytes, max_stages](const unsigned char* d_plans, uint64_t m, double* d_t, uint64_t* d_m, double* d_c,
                                                   uint32_t* d_s, unsigned int* error, uint32_t report_bad) {
-        MixbParams p = mixb_params(ctx->hdr, ctx->d_blob);
-        p.avail = ctx->d_avail;
+        MixbCall p = {};
+        p.blob = ctx->d_blob; p.avail = ctx->d_avail;
         p.plans = d_plans; p.n = m; p.stride = record_bytes; p.max_stages = max_stages;
         p.t_iter = d_t; p.peak_mem = d_m; p.cost = d_c; p.status = d_s;
         p.error = error; p.deep_seen = ctx->d_deep_seen; p.report_bad = report_bad;
         if (max_stages > MIXB_P_MAX) CU(ctx, cudaMemsetAsync(ctx->d_deep_seen, 0, sizeof(unsigned int), ctx->stream));
         if (mixb_takes(ctx->hdr, max_stages, m)) {
-            simulate_mixed_kernel<<<(uint32_t)std::min<uint64_t>(m, MIXB_BLOCKS * (uint64_t)ctx->sm_count), MIXB_THREADS, mixb_smem(ctx->hdr), ctx->stream>>>(p);
+            simulate_mixed_kernel<<<(uint32_t)std::min<uint64_t>(m, MIXB_BLOCKS * (uint64_t)ctx->sm_count), MIXB_THREADS, mixb_smem(ctx->hdr), ctx->stream>>>(mixb_params(p, ctx->hdr));
         } else {                                                 // (blocks take several plans per warp in larger batches)
             const uint64_t blocks = (m + MIX_WARPS<false> - 1) / MIX_WARPS<false>, cap = (uint64_t)ctx->sm_count * 32;
             simulate_mixed_each_kernel<false><<<(uint32_t)std::min(blocks, cap), 32 * MIX_WARPS<false>, mixed_smem<false>(ctx->hdr), ctx->stream>>>(p);

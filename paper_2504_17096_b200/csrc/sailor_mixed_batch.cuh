@@ -122,31 +122,39 @@ inline bool mixb_takes(const TabHdr& h, uint32_t max_stages, uint64_t n) {
     return n >= (deepest <= 8 ? 4096 : deepest <= 16 ? 1536 : deepest <= 24 && h.R <= 2 ? 2048 : 17);
 }
 
-struct MixbParams {
+// All that the kernels with a warp per plan are given: launches take longer with more (one plan, calls back to back: 6.4 to 7.7 us
+// with the tables' addresses and small tables as well, 6.2 to 7.2 without).
+struct MixbCall {
     const unsigned char* blob;
     const uint16_t* avail;
     const unsigned char* plans;
-    uint64_t n, gbs;
-    const PieceRec* piece;
-    const double *zone2, *egress, *grad, *intra_p, *inter_p, *inter_a, *inter_i, *intra_a, *intra_i, *price_s, *inter2, *intra2;
-    const uint64_t* p2p;
-    uint64_t capacity[SAILOR_T_MAX];
-    uint32_t tp_values[SAILOR_TP_MAX], mbs_values[SAILOR_MBS_MAX], gpn[SAILOR_T_MAX], heads_ok;
+    uint64_t n;
     double *t_iter, *cost;
     uint64_t* peak_mem;
     uint32_t* status;
     unsigned int *error, *deep_seen;
     uint32_t stride, max_stages, report_bad;
+};
+static_assert(sizeof(MixbCall) <= 128, "few launch parameters");
+
+struct MixbParams : MixbCall {
+    uint64_t gbs;
+    const PieceRec* piece;
+    const double *zone2, *egress, *grad, *intra_p, *inter_p, *inter_a, *inter_i, *intra_a, *intra_i, *price_s, *inter2, *intra2;
+    const uint64_t* p2p;
+    uint64_t capacity[SAILOR_T_MAX];
+    uint32_t tp_values[SAILOR_TP_MAX], mbs_values[SAILOR_MBS_MAX], gpn[SAILOR_T_MAX], heads_ok;
     uint32_t n_blocks, T, Z, R, n_tp, n_mbs, chain_len, has_embed, has_head, piece_stride;
     uint32_t plans_max;              // plans at a time
 };
 
 inline size_t mixb_smem(const TabHdr& h) { return sizeof(MixbShared) + 2 * (size_t)h.R * h.n_mbs * sizeof(double); }
 
-inline MixbParams mixb_params(const TabHdr& h, const unsigned char* blob) {
+inline MixbParams mixb_params(const MixbCall& call, const TabHdr& h) {
     MixbParams p = {};
+    static_cast<MixbCall&>(p) = call;
+    const unsigned char* blob = call.blob;
     auto table = [&](uint32_t off) { return off ? reinterpret_cast<const double*>(blob + off) : nullptr; };
-    p.blob = blob;
     p.gbs = h.gbs;
     p.piece = reinterpret_cast<const PieceRec*>(blob + h.off_piece);
     p.zone2 = table(h.off_lnk_zone2); p.egress = table(h.off_egress); p.grad = table(h.off_cmp_grad);
@@ -190,7 +198,7 @@ __device__ __forceinline__ uint32_t nth_bit(uint4 w, uint32_t n) {
     return at;
 }
 
-__device__ __forceinline__ void mixb_store(const MixbParams& p, uint64_t j, const SimOut& o) {
+__device__ __forceinline__ void mixb_store(const MixbCall& p, uint64_t j, const SimOut& o) {
     if (p.t_iter) p.t_iter[j] = o.t_iter;
     if (p.peak_mem) p.peak_mem[j] = o.peak_mem;
     if (p.cost) p.cost[j] = o.cost;
