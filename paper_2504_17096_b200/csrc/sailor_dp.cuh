@@ -257,10 +257,11 @@ struct DpLevelParams {
     uint32_t dist;                   // stage i = P - 1 - dist
 };
 
-// A value in one 32-byte load or store.
+// A value in one 32-byte load or store.  Both are memory accesses to the compiler: a block reads values it wrote before its last
+// barrier, and kernels launched early read after griddepcontrol.wait.
 __device__ __forceinline__ DpVal load_val(const DpVal* p) {
     DpVal v;
-    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v.sum), "=d"(v.mx), "=d"(v.sy), "=d"(v.up) : "l"(p));
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v.sum), "=d"(v.mx), "=d"(v.sy), "=d"(v.up) : "l"(p) : "memory");
     return v;
 }
 __device__ __forceinline__ void store_val(DpVal* p, const DpVal& v) {

@@ -324,20 +324,23 @@ def test_dp_tables_fit_what_the_interface_says(P, caps, _index_mode):
     assert [bytes(r) for r in got] == [bytes(r) for r in want] and st2.n_states == st.n_states
 
 
-@pytest.mark.parametrize("T,P", [(4, 20), (4, 22), (4, 25), (3, 63), (3, 70), (8, 7), (8, 9), (5, 14)])
-def test_dp_levels_and_what_a_block_takes_over(T, P, _index_mode):
-    """Problems whose stages have up to 1 771, 2 300 or 6 435 count vectors: either side of what one block takes from the
-    last stage on (2 048), and, in the larger ones, stages either side of where a block takes over (512)."""
-    if _index_mode == "dense":
-        return                                               # (tables in mixed radix of eight types are refused)
+@pytest.mark.parametrize("T,P", [(4, 20), (4, 22), (4, 25), (3, 62), (3, 63), (3, 70), (8, 7), (8, 9), (5, 14)])
+def test_dp_problems_either_side_of_one_block(T, P, _index_mode):
+    """Problems whose last stage has C(P + T - 1, T - 1) count vectors, 1 771 to 11 440: a block takes those of up to 2 048
+    (2 016 and 2 080 with three types and 62 or 63 stages) through all stages, levels together take the others."""
     w = W.tiny(seed=70 + T, n_types=T, n_zones=2, L=max(P, 4), p_values=[P, max(1, P // 2)], d_values=(1, 2), tp_values=(1,),
                mbs_values=(1, 2), rc_values=(0,), gbs=64)
     w.avail[...] = np.array([[P - 1] * T, [2] * T], dtype=np.uint16)
     w.capacity[:] = np.uint64(1 << 44)
     orders = [[0], [0, 1]]
+    with Ctx(w) as cx:
+        if _index_mode == "dense" and (T, P) == (8, 9):          # 9^8 vectors of eight types in mixed radix: 25 GB
+            with pytest.raises(B.SailorError) as e:
+                B.sailor_plan_dp(cx.ctx, cx.space, orders, 16)
+            assert e.value.code == B.E_RANGE
+            return
+        res, st = B.sailor_plan_dp(cx.ctx, cx.space, orders, 16)
     o = Oracle(w)
     want = oracle_all(w, o, orders)
     assert len(want) >= 4
-    with Ctx(w) as cx:
-        res, st = B.sailor_plan_dp(cx.ctx, cx.space, orders, 16)
     assert_dp_equal(res, st, want, w, o, orders, 16, f"{T} types, {P} stages")
