@@ -198,8 +198,9 @@ def test_mixed_device_pointers_empty_and_bad_records():
 
 @pytest.mark.parametrize("D,stages", [(2, 1), (32, 5), (33, 32), (64, 31), (65, 33), (300, 96), (7, 64)])
 def test_mixed_interval_edges(D, stages):
-    """Intervals between group boundaries are found by one bit per replica up to D = 64 and boundary by boundary beyond;
-    items and pipelines take several rounds of 32 lanes when there are many: up to four groups a stage, cut differently."""
+    """Up to four groups a stage, cut differently.  A warp per plan (calls with 16 plans, plans of more than 32 stages) finds
+    intervals between boundaries by one bit per replica up to D = 64 and boundary by boundary beyond, and takes items and
+    pipelines in several rounds of 32 lanes when there are many; blocks (40 plans that can be deep) have other ways."""
     w = W.tiny(seed=37, n_types=4, n_zones=3, L=max(stages, 4), gbs=D * 4, d_values=(D,), p_values=[stages])
     w.gpus_per_node[...] = [4, 64, 700, 2]
     rng = W.SplitMix64(D * 131 + stages)
@@ -218,12 +219,15 @@ def test_mixed_interval_edges(D, stages):
     ctx = B.sailor_create(w, 0, 0)
     try:
         B.sailor_set_availability(ctx, w.avail)
-        t, m, c, s = B.sailor_simulate_mixed(ctx, B.pack_mixed_plans(plans))
+        packed = B.pack_mixed_plans(plans)
+        whole = B.sailor_simulate_mixed(ctx, packed)
+        parts = [B.sailor_simulate_mixed(ctx, packed[j : j + 16]) for j in range(0, len(plans), 16)]
     finally:
         B.sailor_destroy(ctx)
     so, to, co, mo = o.simulate_mixed_batch(plans)
-    assert np.array_equal(s, so) and np.array_equal(m, mo)
-    assert np.array_equal(t, to, equal_nan=True) and np.array_equal(c, co, equal_nan=True)
+    for t, m, c, s in (whole, tuple(np.concatenate(x) for x in zip(*parts))):
+        assert np.array_equal(s, so) and np.array_equal(m, mo)
+        assert np.array_equal(t, to, equal_nan=True) and np.array_equal(c, co, equal_nan=True)
 
 
 @pytest.mark.parametrize("D,stages,n,node", [(6, 3, 16, 8), (6, 3, 17, 8),           # either side of the smallest batch that blocks take
