@@ -71,8 +71,8 @@ struct DpJob {                       // a problem that has tables
     uint64_t succ_off;               // first byte of its successors: [stage][slot][type]
     uint32_t config, index, layout, P;   // index = config * n_orders + order
     uint32_t slots, _pad;            // most live vectors of a stage: a type's values are this many entries, slot after slot (a
-                                     // warp's gathers then fall into a few lines instead of one each: workload 3 1 700 -> 1 622
-                                     // us a call, workload 5 496 -> 468)
+                                     // warp's gathers then fall into a few lines instead of one each: workload 3 1 853 -> 1 764
+                                     // us a call, workload 5 432 -> 412)
 };
 static_assert(sizeof(DpJob) % 8 == 0, "copied by eight bytes");
 
