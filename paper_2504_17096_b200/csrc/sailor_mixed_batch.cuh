@@ -19,7 +19,8 @@
 // that replica k falls into is one subtraction and a population count.  Of a plan with more replicas only the order of its
 // boundaries matters to the pipelines: each takes its place among them as its number (96 at most), after two more barriers
 // where such a plan is among those evaluated together (6.0e4 plans of workload 3 with 256 replicas: 175 us by a warp each,
-// 117 this way; left to a few warps of the block 436).  Contexts with larger nodes than the packed items can tell apart keep a warp per plan.
+// 117 this way; left to a few warps of the block 436).  Contexts with larger nodes than the packed items can tell apart keep a
+// warp per plan.
 // Sums whose order of additions is part of the result are one thread's, term after term, as in simulate_mixed_warp.
 #pragma once
 
